@@ -54,7 +54,7 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NBARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const uint32_t smem_base = smem_u32(smem);
@@ -80,7 +80,7 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     __syncthreads();
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int kblocks = args.d / TC_BK;
     const int tiles_n = (args.E + 255) / 256, tiles_m = (args.T + 255) / 256;
@@ -112,7 +112,8 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
 
     if (warp == 0) {
         // ===================================================================== TMA producer (both CTAs)
-        if (lane == 0) {
+        {
+            const bool el = elect_one();
             int sa = 0, sb = 0; uint32_t pa = 0, pb = 0; bool alive = true;
             for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
                 const Unit u = decode(t);
@@ -123,14 +124,18 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                 const CUtensorMap* mw = half_cols == 128 ? &tmW2 : &tmW1;
                 for (int kb = u.kb0; kb < u.kb1 && alive; ++kb) {
                     if (!mbar_wait(emptyA(sa), pa ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
-                    if (leader) mbar_expect_tx(fullA(sa), 2 * RS_SLOT);
-                    tma2_load_2d(slotA(sa), &tmX, fullA(sa) & T2_PEER_MASK, kb * TC_BK, row0);
+                    if (el) {
+                        if (leader) mbar_expect_tx(fullA(sa), 2 * RS_SLOT);
+                        tma2_load_2d(slotA(sa), &tmX, fullA(sa) & T2_PEER_MASK, kb * TC_BK, row0);
+                    }
                     if (++sa == RS_SA) { sa = 0; pa ^= 1u; }
                     for (int ph = 0; ph < 3; ++ph) {
                         if (!mbar_wait(emptyB(sb), pb ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
-                        if (leader) mbar_expect_tx(fullB(sb), 2 * half_cols * TC_BK * 2);
-                        // chunked map {64 columns, d rows, E/64 chunks, 3 pieces}
-                        tma2_load_4d(slotB(sb), mw, fullB(sb) & T2_PEER_MASK, 0, kb * TC_BK, chunk0, ph);
+                        if (el) {
+                            if (leader) mbar_expect_tx(fullB(sb), 2 * half_cols * TC_BK * 2);
+                            // chunked map {64 columns, d rows, E/64 chunks, 3 pieces}
+                            tma2_load_4d(slotB(sb), mw, fullB(sb) & T2_PEER_MASK, 0, kb * TC_BK, chunk0, ph);
+                        }
                         if (++sb == RS_SB) { sb = 0; pb ^= 1u; }
                     }
                 }
@@ -138,7 +143,8 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
         }
     } else if (warp == 1) {
         // ===================================================================== MMA issuer (leader CTA)
-        if (leader && lane == 0) {
+        if (leader) {
+            const bool el = elect_one();
             // kind::f16, bf16 x bf16 -> fp32, A K-major, B N-major, M = 256 over the pair; N per tile
             constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(256 >> 4) << 24);
             const uint64_t desc_a = smem_desc(0, 0, 1024);
@@ -160,18 +166,20 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         if (!mbar_wait(fullB(sb), pb, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
                         tc_fence_after();
                         const uint64_t db = desc_b | (uint64_t)((slotB(sb) & 0x3ffffu) >> 4);
+                        if (el) {
 #pragma unroll
-                        for (int k4 = 0; k4 < TC_BK / 16; ++k4)
-                            umma2_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kseg | ph | k4) != 0 ? 1u : 0u);
-                        umma2_commit_both(emptyB(sb));
+                            for (int k4 = 0; k4 < TC_BK / 16; ++k4)
+                                umma2_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kseg | ph | k4) != 0 ? 1u : 0u);
+                            umma2_commit_both(emptyB(sb));
+                        }
                         if (++sb == RS_SB) { sb = 0; pb ^= 1u; }
                     }
                     if (!alive) break;
-                    umma2_commit_both(emptyA(sa));
+                    if (el) umma2_commit_both(emptyA(sa));
                     if (++sa == RS_SA) { sa = 0; pa ^= 1u; }
                     if (++kseg == RS_SEG && kb + 1 < u.kb1) {
                         // segment done: hand this accumulator to the epilogue and go on in the other one
-                        umma2_commit_both(tfull_bar(it & 1));
+                        if (el) umma2_commit_both(tfull_bar(it & 1));
                         ++it;
                         kseg = 0;
                         if (!mbar_wait(tempty_bar(it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
@@ -181,7 +189,7 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     }
                 }
                 if (!alive) break;
-                umma2_commit_both(tfull_bar(it & 1));
+                if (el) umma2_commit_both(tfull_bar(it & 1));
                 ++it;
             }
         }

@@ -81,6 +81,17 @@ struct TcArgs {
 };
 
 // ------------------------------------------------------------------------------------------ PTX
+// The producer and MMA warps run their loops with all 32 lanes and let one elected lane issue: the loop's state is then the
+// same in every lane and the compiler keeps it in uniform registers, which is where TMA and tcgen05 instructions take their
+// operands from.  With `if (lane == 0)` around the loop a K block of four pair MMAs cost 535 cycles of issue whatever N; in this
+// form 237, less than the tensor core needs from N = 112 on (64 of K, N = 176 with its copies: 416 -> 352 cycles).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x / 32), 0); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -101,15 +112,25 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
         : "memory");
     return ok;
 }
+// The same with a time hint: the thread sleeps until the phase completes or the time (ns) has passed.
+__device__ __forceinline__ uint32_t mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(ns)
+        : "memory");
+    return ok;
+}
 // Bounded wait.  Returns false if the CTA is aborting (this wait or another one ran out).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           int code, long long limit = TC_WAIT_CYCLES) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 32; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
+        // asleep instead of polling: the poll's instructions took issue slots and power from the epilogue warps (data gradient
+        // of the down-projection with its SwiGLU, d = 2048, 384 rows per expert: 318 -> 300 us)
+        if (mbar_try_wait_for(bar, parity, 20000)) return true;
         if (*abort_flag) return false;
         if (clock64() - t0 > limit) {
             *abort_flag = 1;
@@ -511,7 +532,7 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * TC_STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t bar_base = smem_u32(bars);
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -532,7 +553,7 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     int total_tiles;
     if constexpr (Tr::RAGGED_K) total_tiles = args.E * args.tiles_m_fixed * args.tiles_n;
@@ -540,28 +561,29 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
 
     if (warp == 0) {
         // ===================================================================== TMA producer
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0; bool alive = true;
-            const uint64_t keep = l2_policy_evict_last();
-            (void)keep;
-            // the next tile's descriptor is fetched one tile ahead so that its latency is hidden
-            TileInfo nxt = decode_tile<KIND>(args, min((int)blockIdx.x, max(total_tiles - 1, 0)));
-            for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
-                const TileInfo ti = nxt;
-                if (t + (int)gridDim.x < total_tiles) nxt = decode_tile<KIND>(args, t + gridDim.x);
-                if (ti.skip) continue;
-                const int n0 = ti.nt * Tr::N_PER_TILE + (KIND == TC_VP ? args.n_base : 0);
-                const int nkb = Tr::RAGGED_K ? (ti.rows + TC_BK - 1) / TC_BK : Tr::PHASES * args.kblocks;
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
-                        alive = false; break;
-                    }
-                    const uint32_t fb = full_bar(stage);
+        const bool el = elect_one();
+        int stage = 0; uint32_t phase = 0; bool alive = true;
+        const uint64_t keep = l2_policy_evict_last();
+        (void)keep;
+        // the next tile's descriptor is fetched one tile ahead so that its latency is hidden
+        TileInfo nxt = decode_tile<KIND>(args, min((int)blockIdx.x, max(total_tiles - 1, 0)));
+        for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
+            const TileInfo ti = nxt;
+            if (t + (int)gridDim.x < total_tiles) nxt = decode_tile<KIND>(args, t + gridDim.x);
+            if (ti.skip) continue;
+            const int n0 = ti.nt * Tr::N_PER_TILE + (KIND == TC_VP ? args.n_base : 0);
+            const int nkb = Tr::RAGGED_K ? (ti.rows + TC_BK - 1) / TC_BK : Tr::PHASES * args.kblocks;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                    alive = false; break;
+                }
+                const uint32_t fb = full_bar(stage);
+                const uint32_t sA = smem_base + stage * TC_STAGE_BYTES;
+                const uint32_t sB = sA + TC_A_BYTES;
+                const int ph = Tr::PHASES > 1 ? kb / args.kblocks : 0;
+                const int k0 = (kb - ph * args.kblocks) * TC_BK;
+                if (el) {
                     mbar_expect_tx(fb, TC_STAGE_BYTES);
-                    const uint32_t sA = smem_base + stage * TC_STAGE_BYTES;
-                    const uint32_t sB = sA + TC_A_BYTES;
-                    const int ph = Tr::PHASES > 1 ? kb / args.kblocks : 0;
-                    const int k0 = (kb - ph * args.kblocks) * TC_BK;
                     if constexpr (!Tr::A_MN) {
                         tma_load_2d(sA, (KIND == TC_B4 && ph) ? &tmA1 : &tmA0, fb, k0, ti.row0);
                     } else {
@@ -581,8 +603,8 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
                             tma_load_3d_hint(sB, (Tr::SEL_B && ti.sel) ? &tmB1 : &tmB0, fb, 0, krow, n0 >> 6, keep);
                         }
                     }
-                    if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
                 }
+                if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
@@ -591,55 +613,55 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
         // MN-major operand: 64-wide chunks are TC_CHUNK_BYTES apart (leading offset), groups of
         // 8 K rows are 1024 bytes apart (stride offset); K-major: 8-row groups 1024 bytes apart.
         constexpr uint32_t mn_lbo = TC_CHUNK_BYTES, mn_sbo = 1024u;
+        const bool el = elect_one();
         int stage = 0; uint32_t phase = 0; int it = 0; bool alive = true;
-        TileInfo nxt = decode_tile<KIND>(args, min((int)blockIdx.x, max(total_tiles - 1, 0)));
         if constexpr (!Tr::RAGGED_K) {
-            // Token-row kinds: one thread runs the whole issue loop (wait, fence, four MMAs, commit) with
-            // descriptors that only need the stage's start address added, so the tensor pipe's queue stays fed.
-            if (lane == 0) {
-                const uint64_t desc_a = smem_desc(0, 0, 1024);
-                const uint64_t desc_b = Tr::B_MN ? smem_desc(0, mn_lbo, mn_sbo) : smem_desc(0, 0, 1024);
-                constexpr uint32_t b_step = (Tr::B_MN ? 2048 : 32) >> 4;
-                const int nkb = Tr::PHASES * args.kblocks;
-                for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
-                    if (t + (int)gridDim.x < total_tiles) nxt = decode_tile<KIND>(args, t + gridDim.x);
-                    const int buf = it & 1;
-                    const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
-                    if (!mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
+            // Token-row kinds: descriptors that only need the stage's start address added
+            const uint64_t desc_a = smem_desc(0, 0, 1024);
+            const uint64_t desc_b = Tr::B_MN ? smem_desc(0, mn_lbo, mn_sbo) : smem_desc(0, 0, 1024);
+            constexpr uint32_t b_step = (Tr::B_MN ? 2048 : 32) >> 4;
+            const int nkb = Tr::PHASES * args.kblocks;
+            for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
+                const int buf = it & 1;
+                const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
+                if (!mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)buf * TC_BN;
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) {
+                        alive = false; break;
+                    }
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)buf * TC_BN;
-                    for (int kb = 0; kb < nkb; ++kb) {
-                        if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) {
-                            alive = false; break;
-                        }
-                        tc_fence_after();
-                        const uint32_t sA = smem_base + stage * TC_STAGE_BYTES;
-                        const uint64_t da = desc_a | (uint64_t)((sA & 0x3ffffu) >> 4);
-                        const uint64_t db = desc_b | (uint64_t)(((sA + TC_A_BYTES) & 0x3ffffu) >> 4);
+                    const uint32_t sA = smem_base + stage * TC_STAGE_BYTES;
+                    const uint64_t da = desc_a | (uint64_t)((sA & 0x3ffffu) >> 4);
+                    const uint64_t db = desc_b | (uint64_t)(((sA + TC_A_BYTES) & 0x3ffffu) >> 4);
+                    if (el) {
 #pragma unroll
                         for (int k4 = 0; k4 < TC_BK / 16; ++k4)
                             umma_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kb | k4) != 0 ? 1u : 0u);
                         umma_commit(empty_bar(stage));
-                        if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
                     }
-                    if (!alive) break;
-                    umma_commit(tfull_bar(buf));
-                    ++it;
+                    if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
                 }
+                if (!alive) break;
+                if (el) umma_commit(tfull_bar(buf));
+                ++it;
             }
-        } else
+        } else {
+        TileInfo nxt = decode_tile<KIND>(args, min((int)blockIdx.x, max(total_tiles - 1, 0)));
         for (int t = blockIdx.x; t < total_tiles && alive; t += gridDim.x) {
             const TileInfo ti = nxt;
             if (t + (int)gridDim.x < total_tiles) nxt = decode_tile<KIND>(args, t + gridDim.x);
             if (ti.skip) continue;
             const int buf = it & 1;
             const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
-            if (!mbar_wait_warp(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY, lane)) break;
+            // the lanes meet again at the K tail below: they give up together or not at all
+            if (!__all_sync(0xffffffffu, mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)buf * TC_BN;
             const int nkb = Tr::RAGGED_K ? (ti.rows + TC_BK - 1) / TC_BK : Tr::PHASES * args.kblocks;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL, lane)) {
+                if (!__all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL))) {
                     alive = false; break;
                 }
                 tc_fence_after();
@@ -666,25 +688,20 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
                         __syncwarp();
                     }
                 }
-                if (lane == 0) {
+                const uint64_t da = smem_desc(0, mn_lbo, mn_sbo) | (uint64_t)((sA & 0x3ffffu) >> 4);
+                const uint64_t db = smem_desc(0, mn_lbo, mn_sbo) | (uint64_t)((sB & 0x3ffffu) >> 4);
+                if (el) {
 #pragma unroll
-                    for (int k4 = 0; k4 < TC_BK / 16; ++k4) {
-                        if (k4 >= n_k4) break;
-                        const uint64_t ad = Tr::A_MN ? smem_desc(sA + k4 * 2048, mn_lbo, mn_sbo)
-                                                     : smem_desc(sA + k4 * 32, 0, 1024);
-                        const uint64_t bd = Tr::B_MN ? smem_desc(sB + k4 * 2048, mn_lbo, mn_sbo)
-                                                     : smem_desc(sB + k4 * 32, 0, 1024);
-                        umma_bf16(d_tmem, ad, bd, idesc, (kb | k4) != 0 ? 1u : 0u);
-                    }
+                    for (int k4 = 0; k4 < TC_BK / 16; ++k4)
+                        if (k4 < n_k4) umma_bf16(d_tmem, da + k4 * (2048 >> 4), db + k4 * (2048 >> 4), idesc, (kb | k4) != 0 ? 1u : 0u);
                     umma_commit(empty_bar(stage));
                 }
-                __syncwarp();
                 if (++stage == TC_STAGES) { stage = 0; phase ^= 1u; }
             }
             if (!alive) break;
-            if (lane == 0) umma_commit(tfull_bar(buf));
-            __syncwarp();
+            if (el) umma_commit(tfull_bar(buf));
             ++it;
+        }
         }
     } else {
         // ===================================================================== epilogue (4 warps)

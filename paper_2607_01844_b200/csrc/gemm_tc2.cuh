@@ -163,7 +163,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const uint32_t smem_base = smem_u32(smem);
@@ -187,7 +187,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     __syncthreads();
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int total_tiles = (*args.n_mtiles) * args.tiles_n;
     const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
@@ -204,24 +204,25 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
 
     if (warp == 0) {
         // ===================================================================== TMA producer (both CTAs)
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0; bool alive = true;
-            TileInfo nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
-            for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
-                const TileInfo ti = nxt;
-                if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
-                const int n0 = ti.nt * Tr::N_PER_TILE + (KIND == TC_VP ? args.n_base : 0);
-                const int nkb = Tr::PHASES * args.kblocks;
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
-                        alive = false; break;
-                    }
-                    const uint32_t fb = full_bar(stage) & T2_PEER_MASK;    // the leader's barrier
+        const bool el = elect_one();
+        int stage = 0; uint32_t phase = 0; bool alive = true;
+        TileInfo nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
+        for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
+            const TileInfo ti = nxt;
+            if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
+            const int n0 = ti.nt * Tr::N_PER_TILE + (KIND == TC_VP ? args.n_base : 0);
+            const int nkb = Tr::PHASES * args.kblocks;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                    alive = false; break;
+                }
+                const uint32_t fb = full_bar(stage) & T2_PEER_MASK;    // the leader's barrier
+                const uint32_t sA = smem_base + stage * T2_STAGE_BYTES;
+                const uint32_t sB = sA + T2_A_BYTES;
+                const int ph = (Tr::PHASES == 2 && kb >= args.kblocks) ? 1 : 0;
+                const int k0 = (kb - ph * args.kblocks) * TC_BK;
+                if (el) {
                     if (leader) mbar_expect_tx(full_bar(stage), 2 * T2_STAGE_BYTES);
-                    const uint32_t sA = smem_base + stage * T2_STAGE_BYTES;
-                    const uint32_t sB = sA + T2_A_BYTES;
-                    const int ph = (Tr::PHASES == 2 && kb >= args.kblocks) ? 1 : 0;
-                    const int k0 = (kb - ph * args.kblocks) * TC_BK;
                     tma2_load_2d(sA, ph ? &tmA1 : &tmA0, fb, k0, ti.row0);
                     if constexpr (!Tr::B_MN) {
                         // K-major weights: this CTA's 128 output columns are 128 rows of the [E, N, K] tensor
@@ -234,14 +235,14 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                         const int nb = Tr::DUAL_B ? n0 : n0 + 128 * (int)rank;
                         tma2_load_4d(sB, mp, fb, 0, k0, nb >> 6, ti.e);   // chunked map, two chunks per copy
                     }
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
+                if (++stage == S) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
         // ===================================================================== MMA issuer (leader CTA)
-        // one thread runs the whole loop (wait, fence, four MMAs, commit) with precomputed descriptors
-        if (leader && lane == 0) {
+        if (leader) {
+            const bool el = elect_one();
             constexpr uint32_t idesc = make_idesc2(Tr::B_MN);
             const uint64_t desc_a = smem_desc(0, 0, 1024);
             const uint64_t desc_b = Tr::B_MN ? smem_desc(0, TC_CHUNK_BYTES, 1024) : smem_desc(0, 0, 1024);
@@ -262,14 +263,16 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                     const uint32_t sA = smem_base + stage * T2_STAGE_BYTES;
                     const uint64_t da = desc_a | (uint64_t)((sA & 0x3ffffu) >> 4);
                     const uint64_t db = desc_b | (uint64_t)(((sA + T2_A_BYTES) & 0x3ffffu) >> 4);
+                    if (el) {
 #pragma unroll
-                    for (int k4 = 0; k4 < TC_BK / 16; ++k4)
-                        umma2_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kb | k4) != 0 ? 1u : 0u);
-                    umma2_commit_both(empty_bar(stage));
+                        for (int k4 = 0; k4 < TC_BK / 16; ++k4)
+                            umma2_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kb | k4) != 0 ? 1u : 0u);
+                        umma2_commit_both(empty_bar(stage));
+                    }
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
                 if (!alive) break;
-                umma2_commit_both(tfull_bar(buf));
+                if (el) umma2_commit_both(tfull_bar(buf));
                 ++it;
             }
         }
