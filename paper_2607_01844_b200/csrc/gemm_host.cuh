@@ -63,33 +63,28 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     // Tokens-on-N kernels: fwd_tn bit 0 = up-projection, bit 1 = down-projection (see tc_plan_policy)
     const bool gather = a.x_gather != nullptr;
     const bool tn_f1 = gather || (p->fwd_tn & 1), tn_f2 = p->fwd_tn & 2;
-    int32_t* ttiles_fwd = tiles + 2 * (tc_tile_table_bytes(s.T * s.k, s.E) / 4);
-    if ((tn_f1 != tn_f2) && p->pairs == 0) {   // one GEMM on each kind of kernel: both tables in one launch
-        if ((r = build_both_tiles(p, a.offsets, tiles, ttiles_fwd, st)) != MOP_OK) return r;
+    if (tn_f1 || tn_f2) {
+        if ((r = tn_build_tiles(p, a.offsets, tiles, !(tn_f1 && tn_f2) && p->pairs == 0, st)) != MOP_OK) return r;
         ++*launches;
-    } else {
-        if (tn_f1 || tn_f2) {
-            if ((r = tn_build_tiles(p, a.offsets, ttiles_fwd, st)) != MOP_OK) return r;
-            ++*launches;
-        }
-        if (!tn_f1 || !tn_f2) {
-            if ((r = tc_build_row_tiles(p, a.offsets, tiles, st)) != MOP_OK) return r;
-            ++*launches;
-        }
+    }
+    if (!(tn_f1 && tn_f2) && !((tn_f1 || tn_f2) && p->pairs == 0)) {
+        if ((r = tc_build_row_tiles(p, a.offsets, tiles, st)) != MOP_OK) return r;
+        ++*launches;
     }
     // N-major weights as chunked maps: one-CTA tiles take 2 chunks per tensor (gate | up) or 4 (down);
     // a pair CTA takes 2 chunks
     CUtensorMap mXp, mWg, mWu, mH, mWd, mWdp;
-    if ((!tn_f1 && !tc_map_2d(p, &mXp, a.Xp, M, s.d, 128)) || !tc_map_chunked_3d(p, &mWg, a.W_gate, s.E, s.d, s.f, 2) ||
-        !tc_map_chunked_3d(p, &mWu, a.W_up, s.E, s.d, s.f, 2) || !tc_map_2d(p, &mH, a.H, M, s.f, 128) ||
-        !tc_map_chunked_3d(p, &mWd, a.W_down, s.E, s.f, s.d, 4) ||
-        !tc_map_chunked_3d(p, &mWdp, a.W_down, s.E, s.f, s.d, 2))
+    if (!tn_f1 && (!tc_map_2d(p, &mXp, a.Xp, M, s.d, 128) || !tc_map_chunked_3d(p, &mWg, a.W_gate, s.E, s.d, s.f, 2) ||
+                   !tc_map_chunked_3d(p, &mWu, a.W_up, s.E, s.d, s.f, 2)))
+        return MOP_ERR_CUDA;
+    if (with_down && !tn_f2 && (!tc_map_2d(p, &mH, a.H, M, s.f, 128) || !tc_map_chunked_3d(p, &mWd, a.W_down, s.E, s.f, s.d, 4) ||
+                                !tc_map_chunked_3d(p, &mWdp, a.W_down, s.E, s.f, s.d, 2)))
         return MOP_ERR_CUDA;
     if (gather) {
-        if ((r = tn_up_swiglu_gather(p, a.x_gather, a, tiles + 2 * (tc_tile_table_bytes(s.T * s.k, s.E) / 4), status, st)) != MOP_OK) return r;
+        if ((r = tn_up_swiglu_gather(p, a.x_gather, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else if (tn_f1) {
-        if ((r = tn_up_swiglu(p, a, tiles + 2 * (tc_tile_table_bytes(s.T * s.k, s.E) / 4), status, st)) != MOP_OK) return r;
+        if ((r = tn_up_swiglu(p, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else {   // F1: [G|U] = Xp [W_gate | W_up], SwiGLU epilogue
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
@@ -100,7 +95,7 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     }
     if (!with_down) return MOP_OK;
     if (tn_f2) {
-        if ((r = tn_down_gate(p, a, tiles + 2 * (tc_tile_table_bytes(s.T * s.k, s.E) / 4), status, st)) != MOP_OK) return r;
+        if ((r = tn_down_gate(p, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else {   // F2: Yp = gate * (H W_down)
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
@@ -132,29 +127,28 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
         if ((r = tc_build_row_tiles(p, a.offsets, tiles, st)) != MOP_OK) return r;
         ++*launches;
     }
-    CUtensorMap mWdKp, mWgKp, mWuKp;   // K-major weight maps boxed for a pair CTA (128 N rows)
-    if (!tc_map_3d(p, &mWdKp, a.W_down, s.E, s.f, s.d, 128) || !tc_map_3d(p, &mWgKp, a.W_gate, s.E, s.d, s.f, 128) ||
-        !tc_map_3d(p, &mWuKp, a.W_up, s.E, s.d, s.f, 128))
-        return MOP_ERR_CUDA;
-    CUtensorMap mdYpA, mWdK, mdG, mdU, mWgK, mWuK, mgH, mdYpB, mXpA, mdGB, mdUB, moWd, moWg, moWu;
+    CUtensorMap mgH, mdYpB, mXpA, mdGB, mdUB, moWd, moWg, moWu;   // weight gradients
     if (!tc_map_out_f32(p, &moWd, a.dW_down, s.E, s.f, s.d) || !tc_map_out_f32(p, &moWg, a.dW_gate, s.E, s.d, s.f) ||
-        !tc_map_out_f32(p, &moWu, a.dW_up, s.E, s.d, s.f))
+        !tc_map_out_f32(p, &moWu, a.dW_up, s.E, s.d, s.f) || !tc_map_chunked_2d(p, &mgH, a.gH, M, s.f, 2) ||
+        !tc_map_chunked_2d(p, &mdYpB, a.dYp, M, s.d, 4) || !tc_map_chunked_2d(p, &mXpA, a.Xp, M, s.d, 2) ||
+        !tc_map_chunked_2d(p, &mdGB, a.dG, M, s.f, 4) || !tc_map_chunked_2d(p, &mdUB, a.dU, M, s.f, 4))
         return MOP_ERR_CUDA;
-    if (!tc_map_2d(p, &mdYpA, a.dYp, M, s.d, 128) || !tc_map_3d(p, &mWdK, a.W_down, s.E, s.f, s.d, 256) ||
-        !tc_map_2d(p, &mdG, a.dG, M, s.f, 128) || !tc_map_2d(p, &mdU, a.dU, M, s.f, 128) ||
-        !tc_map_3d(p, &mWgK, a.W_gate, s.E, s.d, s.f, 256) || !tc_map_3d(p, &mWuK, a.W_up, s.E, s.d, s.f, 256) ||
-        !tc_map_chunked_2d(p, &mgH, a.gH, M, s.f, 2) || !tc_map_chunked_2d(p, &mdYpB, a.dYp, M, s.d, 4) ||
-        !tc_map_chunked_2d(p, &mXpA, a.Xp, M, s.d, 2) || !tc_map_chunked_2d(p, &mdGB, a.dG, M, s.f, 4) ||
-        !tc_map_chunked_2d(p, &mdUB, a.dU, M, s.f, 4))
+    // tokens-on-M data gradients: K-major weight maps boxed for one CTA (256 N rows) and for a pair CTA (128)
+    CUtensorMap mdYpA, mWdK, mWdKp, mdG, mdU, mWgK, mWuK, mWgKp, mWuKp;
+    if (!(p->fwd_tn & 8) && (!tc_map_2d(p, &mdYpA, a.dYp, M, s.d, 128) || !tc_map_3d(p, &mWdK, a.W_down, s.E, s.f, s.d, 256) ||
+                             !tc_map_3d(p, &mWdKp, a.W_down, s.E, s.f, s.d, 128)))
         return MOP_ERR_CUDA;
-    int32_t* ttiles = tiles + 2 * (tc_tile_table_bytes(s.T * s.k, s.E) / 4);
+    if (!(p->fwd_tn & 4) && (!tc_map_2d(p, &mdG, a.dG, M, s.f, 128) || !tc_map_2d(p, &mdU, a.dU, M, s.f, 128) ||
+                             !tc_map_3d(p, &mWgK, a.W_gate, s.E, s.d, s.f, 256) || !tc_map_3d(p, &mWuK, a.W_up, s.E, s.d, s.f, 256) ||
+                             !tc_map_3d(p, &mWgKp, a.W_gate, s.E, s.d, s.f, 128) || !tc_map_3d(p, &mWuKp, a.W_up, s.E, s.d, s.f, 128)))
+        return MOP_ERR_CUDA;
     if (p->fwd_tn & 12) {
-        if ((r = tn_build_tiles(p, a.offsets, ttiles, st)) != MOP_OK) return r;
+        if ((r = tn_build_tiles(p, a.offsets, tiles, false, st)) != MOP_OK) return r;
         ++*launches;
     }
     if (p->fwd_tn & 8) {   // B2 on the tokens-on-N kernel: one dgate partial per 32 columns of f
         *ntile_part = ceil_div(s.f, 32);
-        if ((r = tn_dgrad_down(p, a, ttiles, status, st)) != MOP_OK) return r;
+        if ((r = tn_dgrad_down(p, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else {   // B2: dHu = dYp W_down^T, SwiGLU backward epilogue
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
@@ -166,7 +160,7 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
             return r;
     }
     if (p->fwd_tn & 4) {   // B4 on the tokens-on-N kernel
-        if ((r = tn_dgrad_gate_up(p, a, ttiles, status, st)) != MOP_OK) return r;
+        if ((r = tn_dgrad_gate_up(p, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else {   // B4: dXp = dG W_gate^T + dU W_up^T
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);

@@ -1,30 +1,34 @@
-// "Tokens on N" two-CTA grouped GEMMs for the forward pass: the MMA computes the TRANSPOSED product
+// "Tokens on N" two-CTA grouped GEMMs: the MMA computes the TRANSPOSED product
 //     D^T [weight rows (M = 256 across the CTA pair) x tokens (N <= 256)] = W^T-tile * Xp^T
 // so that the ragged dimension (an expert's token count) sits on the MMA's N, whose granularity is
 // 16, instead of on M, whose granularity is 128: an expert with 171 rows costs one N = 176 tile
-// instead of two 128-row tiles.  The weights are the "A" operand (each CTA of the pair holds its
-// own 128 weight rows), the tokens the "B" operand (each CTA loads half of the tile's token rows),
-// tcgen05.mma.cta_group::2 multiplies, and each CTA's TMEM receives [its 128 weight rows x N].
+// instead of two 128-row tiles (the tensor core takes N / 2 cycles per K = 16: 88 for N = 176, 128 for
+// N = 256, 56 at the least, whatever the majors of A and B).  The weights are the "A" operand (each CTA of
+// the pair holds its own 128 weight rows), the tokens the "B" operand (each CTA loads half of the tile's
+// token rows), tcgen05.mma.cta_group::2 multiplies, and each CTA's TMEM receives [its 128 weight rows x N].
 //
 //   TN_F1  G^T|U^T: a CTA's 128 weight rows are 64 gate columns followed by the 64 matching up
 //          columns of W_gate / W_up, so G and U of one (f, token) land in the same CTA (TMEM lanes
-//          l and l + 64); the epilogue exchanges U through shared memory, applies SwiGLU and
+//          l and l + 64); the epilogue exchanges halves through shared memory, applies SwiGLU and
 //          writes H (+ G, U stash) back in token-major layout.
 //   TN_F2  O^T = W_down^T-tile * H^T, gate applied per token column, Yp written token-major.
 //   TN_F1G as TN_F1, but the token operand is gathered straight from the unpermuted x [T, d]: every
 //          lane of the producer warp owns four token rows of the tile and fetches them per K block
 //          with one TMA gather4 copy, so the expert-contiguous copy Xp never exists (the
 //          single-GPU form of keeping only a fraction of the routed inputs live, Section 3.3).
-//          The TMA unit retires these 4-row copies far more slowly than one 128-row box (about
+//          The TMA unit retires these 4-row copies far more slowly than one box (about
 //          60 ns each on B200), so this form trades time for memory and is opt-in.
 //   TN_B4  dXp^T = W_gate[e] dG^T + W_up[e] dU^T: the weights are read K-major ([E, d, f] as it
 //          lies in memory, rows of d on M), two K phases into one accumulator, dXp token-major.
-//   TN_B2  dHu^T = W_down[e] dYp^T (weights K-major, rows of f on M); the epilogue turns each
-//          32 x 32 block token-major through shared memory and then runs the SwiGLU backward on
-//          16-byte runs of the stash: dG, dU, gate*H out, and one dgate partial per 32 columns of f.
+//   TN_B2  dHu^T = W_down[e] dYp^T (weights K-major, rows of f on M); the epilogue runs the SwiGLU
+//          backward in the accumulator's layout: dG, dU, gate*H out, and one dgate partial per 32 columns of f.
 //
-// The epilogue transposes 32 x 32 blocks through shared memory so that global stores are 64-byte
-// row segments.  Barrier protocol, bounded waits and teardown as in the pair kernel.
+// Epilogues: the accumulator is read with tcgen05.ld.16x256b, whose layout is that of an mma fragment (a thread holds two
+// neighbouring tokens of a feature), packed to bf16 pairs and turned token-major by stmatrix.trans: a block of 32 features x 32
+// tokens costs 4 stmatrix, 4 16-byte shared loads and 4 16-byte global stores per lane where element-wise transposition took
+// 32 two-byte stores and as many conversions.  Eight warps: four per accumulator, so that both drain at the same time.
+//
+// Barrier protocol, bounded waits and teardown as in the pair kernel (gemm_tc2.cuh).
 #pragma once
 #include "gemm_tc2.cuh"
 
@@ -32,30 +36,40 @@ namespace mop {
 
 enum : int { TN_F1 = 0, TN_F2 = 1, TN_F1G = 2, TN_B4 = 3, TN_B2 = 4 };
 
-constexpr int TN_STAGES = 3;
-constexpr int TN_BK = 128;                           // K per pipeline stage: two 64-wide swizzle spans
-constexpr int TN_SUB_BYTES = 128 * 64 * 2;           // 16 KiB: 128 rows x 64 K (or one 64-wide MN chunk x 128 K)
-constexpr int TN_A_BYTES = 2 * TN_SUB_BYTES;         // 32 KiB: this CTA's 128 weight rows x 128 K
-constexpr int TN_B_BYTES = 2 * TN_SUB_BYTES;         // up to 128 token rows (half of N = 256) x 128 K
-constexpr int TN_STAGE_BYTES = TN_A_BYTES + TN_B_BYTES;
-constexpr int TN_EPI_BYTES = 4 * 8192;               // per epilogue warp: transposition buffers
-constexpr int TN_SMEM_BYTES = TN_STAGES * TN_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + TN_EPI_BYTES;
-constexpr int TN_THREADS = 192;
-constexpr int TN_BOX_ROWS = 128;                     // token rows per TMA box (one box per stage)
+constexpr int TN_STAGES = 6;
+constexpr int TN_BK = 64;                            // K per stage
+constexpr int TN_SUB_BYTES = 128 * TN_BK * 2;        // 16 KiB: this CTA's 128 weight rows, or up to 128 token rows
+constexpr int TN_CHUNK_BYTES = 64 * TN_BK * 2;       // one 64-wide chunk of an M-major operand
+constexpr int TN_STAGE_BYTES = 2 * TN_SUB_BYTES;
+constexpr int TN_EPI_WARPS = 8;
+constexpr int TN_EPI_BYTES = 4096;                   // per epilogue warp
+constexpr int TN_SMEM_BYTES = TN_STAGES * TN_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + TN_EPI_WARPS * TN_EPI_BYTES;
+constexpr int TN_THREADS = 64 + 32 * TN_EPI_WARPS;
+constexpr int TN_RING = 16;                          // work items announced to the roles of a cluster
+constexpr int TN_SIGNALS = 4;                        // requests for further items
+constexpr int TN_BOXES = 8;                          // token boxes of 16, 32, .. 128 rows
+
+struct TnMaps {
+    CUtensorMap a0, a1;                // weights (F1: gate, up; B4: gate, up)
+    CUtensorMap b[TN_BOXES];           // token rows, box of 16 (i + 1) rows
+    CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows
+};
 
 struct TnArgs {
-    const int4* ttiles;       // {expert, first row, rows (1..256), 0} per token tile
+    const int4* ttiles;       // {expert, first row, rows (1..256), position | number of tiles << 16} per token tile
     const int32_t* n_ttiles;  // device scalar
     int tiles_m;              // weight-row tiles per token tile (each 256 rows; F1: 128 columns of f)
-    int kblocks;              // K / 128 rounded up
+    int kblocks;              // K / 64 rounded up
     int Mw;                   // weight rows in total (F1: f; F2: d)
+    int a_split;              // F2: the two 64-wide weight chunks as one copy each (columns not a multiple of 64)
     const int32_t* row_src;   // F1G: assignment index t*k + j of every expert-contiguous row
     int topk;                 // F1G: k (token of a row = row_src / k)
+    int32_t* next;            // work items handed out so far (zero when the kernel starts)
     int32_t* status;
     EpiArgs ep;
 };
 
-// Token tiles: an expert's rows are cut into ceil(rows/256) nearly equal tiles.
+// Token tiles: an expert's rows are cut into ceil(rows / 256) nearly equal tiles.
 __device__ __forceinline__ void tn_build_ttiles_body(const int32_t* __restrict__ offsets, int E,
                                                      int4* __restrict__ tiles, int32_t* __restrict__ n_tiles,
                                                      int32_t* scan) {
@@ -76,20 +90,15 @@ __device__ __forceinline__ void tn_build_ttiles_body(const int32_t* __restrict__
     // .w = position of the tile within its expert | number of tiles of the expert << 16
     for (int i = 0; i < nt; ++i) tiles[first + i] = make_int4(e, off + i * sz, min(sz, cnt - i * sz), i | (nt << 16));
     if (e == 1023) *n_tiles = scan[1023];
+    if (e < 8) n_tiles[16 + e] = 0;      // the kinds' counters of work items handed out
 }
-__global__ void __launch_bounds__(1024) tn_build_ttiles_kernel(const int32_t* __restrict__ offsets, int E,
-                                                               int4* __restrict__ tiles,
-                                                               int32_t* __restrict__ n_tiles) {
+// The tile tables of the token-row GEMMs in one launch: block 0 the token tiles, block 1 the 128-row tiles of the
+// tokens-on-M kernels (where a forward or backward uses both).
+__global__ void __launch_bounds__(1024) tn_build_ttiles_kernel(const int32_t* __restrict__ offsets, int E, int32_t* __restrict__ ttiles,
+                                                               int32_t* __restrict__ mtiles) {
     __shared__ int32_t scan[1025];
-    tn_build_ttiles_body(offsets, E, tiles, n_tiles, scan);
-}
-// Both tables in one launch (block 0: 128-row tiles of the tokens-on-M kernels, block 1: token tiles).
-__global__ void __launch_bounds__(1024) build_both_tiles_kernel(const int32_t* __restrict__ offsets, int E,
-                                                                int4* __restrict__ mtiles, int32_t* __restrict__ n_mtiles,
-                                                                int4* __restrict__ ttiles, int32_t* __restrict__ n_ttiles) {
-    __shared__ int32_t scan[1025];
-    if (blockIdx.x == 0) tc_build_mtiles_body(offsets, E, mtiles, n_mtiles, scan);
-    else tn_build_ttiles_body(offsets, E, ttiles, n_ttiles, scan);
+    if (blockIdx.x == 0) tn_build_ttiles_body(offsets, E, reinterpret_cast<int4*>(ttiles + 64), ttiles, scan);
+    else tc_build_mtiles_body(offsets, E, reinterpret_cast<int4*>(mtiles + 64), mtiles, scan);
 }
 
 // Four rows of a [rows, cols] bf16 tensor (map box {64, 1}) -> 4 x 128 bytes at dst, swizzled like a tile box.
@@ -103,90 +112,209 @@ __device__ __forceinline__ void tma2_gather4(uint32_t dst, const CUtensorMap* ma
 
 __device__ __forceinline__ void bar_pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
-// 32 tokens x 32 features staged as bf16 [token][feature] -> 64-byte row segments in global memory
-__device__ __forceinline__ void tn_write_rows(bf16* __restrict__ dst, int ldo, const uint16_t* st, int row0,
-                                              int rows_left, int col0, int lane) {
+// ------------------------------------------------------------------------------------------ fragments
+// 16 TMEM lanes x 8 R fp32 columns as an mma fragment: v[4 j + 0, 1] = lane t / 4, columns 8 j + 2 (t % 4), + 1; v[4 j + 2, 3] =
+// lane t / 4 + 8, the same columns (t = the thread's lane).  The 16 lanes start at the lane field of taddr.  No wait.
+__device__ __forceinline__ void tmem_frag4(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int tok = 8 * i + (lane >> 2), part = lane & 3;
-        const uint4 v = *reinterpret_cast<const uint4*>(st + tok * 32 + part * 8);
-        if (tok < rows_left) *reinterpret_cast<uint4*>(dst + (size_t)(row0 + tok) * ldo + col0 + part * 8) = v;
-    }
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_frag2(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+template <int N>
+__device__ __forceinline__ void tmem_frag_wait(float (&a)[N], float (&b)[N]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(a[i]), "+f"(b[i]));
+}
+__device__ __forceinline__ void stmatrix4_trans(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1),
+                 "r"(r2), "r"(r3)
+                 : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ float2 lds64f(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
 }
 
-__device__ __forceinline__ uint16_t bf16_bits(float v) {
-    return __bfloat16_as_ushort(__float2bfloat16_rn(v));
+// Bounded wait on a barrier that another CTA of the cluster signals after writing into this CTA's shared memory.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t ok;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "r"(20000u)
+            : "memory");
+        if (ok) return true;
+        if (*abort_flag) return false;
+        if (clock64() - t0 > TC_WAIT_CYCLES) {
+            *abort_flag = 1;
+            atomicCAS(status, 0, code);
+            return false;
+        }
+    }
+}
+// 16 bytes into the shared memory of CTA `rank` of the cluster (at this CTA's address `addr`), then one arrival on its barrier
+__device__ __forceinline__ void publish16(uint32_t addr, uint32_t bar, uint32_t rank, int4 v) {
+    asm volatile(
+        "{\n.reg .b32 a, b;\nmapa.shared::cluster.u32 a, %0, %2;\nmapa.shared::cluster.u32 b, %1, %2;\n"
+        "st.shared::cluster.v4.b32 [a], {%3, %4, %5, %6};\n"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [b];\n}" ::"r"(addr),
+        "r"(bar), "r"(rank), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+        : "memory");
+}
+
+// Staging of a block token-major: 64-byte rows of 32 features, the four 16-byte pieces of a row XOR-swizzled by bits 1..2 of
+// the token, so that the eight rows of a matrix and the 32 pieces of a row-wise access each touch every bank once.
+// frag_off: this lane's row address for stmatrix / ldmatrix .x4 (matrix m = lane / 8 holds features 8 m .. 8 m + 7 of tokens
+// 8 j + lane % 8; + 512 j).  piece_off: token lane / 4, features 8 (lane % 4) .. + 7 (+ 512 i for token 8 i + lane / 4).
+__device__ __forceinline__ uint32_t frag_off(int lane) {
+    return (uint32_t)((lane & 7) * 64 + ((((lane >> 3) ^ (lane >> 1)) & 3) << 4));
+}
+__device__ __forceinline__ uint32_t piece_off(int lane) {
+    return (uint32_t)((lane >> 2) * 64 + (((lane ^ (lane >> 3)) & 3) << 4));
+}
+
+// 8 J tokens x 32 features staged at `st` -> global rows (16-byte pieces); features at and past Mw are not stored.
+template <int J>
+__device__ __forceinline__ void tn_write_rows(bf16* __restrict__ dst, int ldo, uint32_t st, int row0, int rows_left,
+                                              int col0, int Mw, int lane) {
+    const int col = col0 + (lane & 3) * 8;
+#pragma unroll
+    for (int i = 0; i < J; ++i) {
+        const int tok = 8 * i + (lane >> 2);
+        const uint4 v = lds128(st + 512 * i + piece_off(lane));
+        if (tok < rows_left && col < Mw) *reinterpret_cast<uint4*>(dst + (size_t)(row0 + tok) * ldo + col) = v;
+    }
 }
 
 template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TN_THREADS, 1)
-tn_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
-               const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB1, const TnArgs args) {
-    constexpr int S = TN_STAGES;
+tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
+    constexpr int S = TN_STAGES, STAGE_BYTES = TN_STAGE_BYTES;
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * TN_STAGE_BYTES);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * STAGE_BYTES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4 + TN_RING + TN_SIGNALS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    uint8_t* epi_smem = smem + S * TN_STAGE_BYTES + TC_BAR_BYTES;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_index(), lane = threadIdx.x % 32;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t bar_base = smem_u32(bars);
+    const uint32_t epi_base = bar_base + TC_BAR_BYTES;
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (S + s); };
     auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * S + b); };
     auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * S + 2 + b); };
+    // announced item n = 1, 2, .. is entry n - 1 of the ring (item 0 is never announced)
+    auto item_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + ((n - 1) & (TN_RING - 1))); };
+    auto item_slot = [&](int n) { return bar_base + 512u + 16u * ((n - 1) & (TN_RING - 1)); };
+    auto signal_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + TN_RING + (n & (TN_SIGNALS - 1))); };
+    static_assert(8 * (2 * S + 4 + TN_RING + TN_SIGNALS) + 8 <= 512 && 512 + 16 * TN_RING <= TC_BAR_BYTES, "barrier block");
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
+        for (int n = 0; n < TN_RING; ++n) mbar_init(item_bar(n), 1);
+        for (int n = 0; n < TN_SIGNALS; ++n) mbar_init(signal_bar(n), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_prefetch_desc(&tmA0); tma_prefetch_desc(&tmB);
-        if (KIND != TN_F2) tma_prefetch_desc(&tmA1);
-        if (KIND == TN_B4) tma_prefetch_desc(&tmB1);
+        tma_prefetch_desc(&maps.a0);
+        if (KIND != TN_F2 && KIND != TN_B2) tma_prefetch_desc(&maps.a1);
     }
     if (warp == 1) tmem2_alloc(smem_u32(tmem_slot), 512);
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int total_tiles = (*args.n_ttiles) * args.tiles_m;
     const int nkb = (KIND == TN_B4 ? 2 : 1) * args.kblocks;   // K blocks per tile (B4: two phases)
     const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-    // work tile t -> token tile t / tiles_m (its expert, first row, rows) and weight-row tile t % tiles_m
-    struct Tile { int e, row0, rows, nmma, mt; };
-    // Within an expert the token tiles vary fastest: the clusters that run at the same time on
-    // neighbouring work tiles then share one weight tile (the large operand) through L2.
+    // Work items are handed out in order as the clusters go along (one atomic addition per item): the items of one expert that
+    // share a weight tile start together and read it from L2 together, whatever the sizes of the items before them, and the
+    // last items spread evenly.  With a fixed round-robin the clusters drifted apart by whole items and the weights were fetched
+    // again: at d = 7168, f = 2048, 256 experts of 512 rows the up-projection took 7.3 ms under the power cap, 6.2 this way.
+    // Item t -> token tile t / tiles_m (its expert, first row, rows) and weight-row tile t % tiles_m.
+    // Item 0 of a cluster is its own number; the others are taken, decoded and written into the rings of both CTAs by the
+    // second CTA's MMA warp, which has nothing else to do, when the second CTA's producer asks (`ahead` items early where K is
+    // short: taking and announcing one takes about 2000 cycles).  No slot is written before it was read: the MMA is at most S
+    // K blocks behind the producer and the epilogue two items behind the MMA; TN_RING is more than S + 2 + ahead + 1.
+    struct Tile { int e, row0, rows, mt; };
+    const bool handout = total_tiles > n_clusters;
+    const int ahead = nkb >= 24 ? 0 : nkb >= 8 ? 1 : 3;
+    const int ask_at = ahead ? 0 : nkb - 10;
+    static_assert(TN_RING > S + 2 + 3 + 1 && TN_SIGNALS >= 3 + 1, "see above");
+    // Within an expert the token tiles vary fastest.  e < 0: no item left.
     auto decode = [&](int t) {
+        if (t >= total_tiles) return make_int4(-1, 0, 0, 0);
         const int q = t / args.tiles_m;
         int4 m = __ldg(args.ttiles + q);
         const int nt = m.w >> 16;
-        Tile ti;
-        ti.mt = t % args.tiles_m;
+        int mt = t - q * args.tiles_m;
         if (nt > 1) {
             const int first = q - (m.w & 0xffff);                 // first token tile of this expert
-            const int l = t - first * args.tiles_m;               // position among the expert's work tiles
-            ti.mt = l / nt;
-            m = __ldg(args.ttiles + first + l % nt);
+            const int l = t - first * args.tiles_m;               // position among the expert's work items
+            mt = l / nt;
+            m = __ldg(args.ttiles + first + (l - mt * nt));
         }
-        ti.e = m.x; ti.row0 = m.y; ti.rows = m.z; ti.nmma = (m.z + 15) & ~15;
-        return ti;
+        return make_int4(m.x, m.y, m.z, mt);
     };
+    // The n-th item of this cluster; false: none left (or the CTA is giving up).
+    auto next_item = [&](int n, Tile& ti) {
+        int4 v;
+        if (n == 0) v = decode(cluster_id);
+        else {
+            if (!handout) return false;
+            if (!mbar_wait_cluster(item_bar(n), (uint32_t)((n - 1) / TN_RING) & 1u, abort_flag, args.status, STATUS_WAIT_FULL)) return false;
+            const uint4 u = lds128(item_slot(n));
+            v = make_int4((int)u.x, (int)u.y, (int)u.z, (int)u.w);
+        }
+        ti.e = v.x; ti.row0 = v.y; ti.rows = v.z; ti.mt = v.w;
+        return ti.e >= 0;
+    };
+    auto nmma_of = [](int rows) { return (rows + 15) & ~15; };
 
     if (warp == 0 && KIND == TN_F1G) {
         // ============================================ TMA producer with row gather (both CTAs, whole warp)
         int stage = 0; uint32_t phase = 0; bool alive = true;
-        Tile nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
-        for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
-            const Tile ti = nxt;
-            if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
-            const int half = ti.nmma >> 1;                             // token rows per CTA (multiple of 8)
+        Tile ti;
+        for (int n = 0; alive && __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
+            const int half = nmma_of(ti.rows) >> 1;                    // token rows per CTA (multiple of 8)
             const int ngroups = half >> 2;                             // gather4 copies per K block (<= 32)
             const int brow0 = ti.row0 + (int)rank * half;
             const int last = ti.row0 + ti.rows - 1;                    // padding rows repeat the last valid one
@@ -195,151 +323,150 @@ tn_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 4; ++j) tok[j] = __ldg(args.row_src + min(brow0 + 4 * lane + j, last)) / args.topk;
             }
-            const uint32_t tx = 2u * (TN_A_BYTES + 2u * (uint32_t)half * 128u);
+            const uint32_t tx = 2u * (TN_SUB_BYTES + (uint32_t)half * 128u);
             for (int kb = 0; kb < args.kblocks; ++kb) {
                 if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY, lane)) {
                     alive = false; break;
                 }
                 const uint32_t fb = full_bar(stage) & T2_PEER_MASK;
-                const uint32_t sA = smem_base + stage * TN_STAGE_BYTES;
-                const uint32_t sB = sA + TN_A_BYTES;
+                const uint32_t sA = smem_base + stage * STAGE_BYTES;
+                const uint32_t sB = sA + TN_SUB_BYTES;
                 const int k0 = kb * TN_BK;
                 if (lane == 0) {
+                    if (!leader && handout && kb == ask_at) mbar_arrive(signal_bar(n));
                     if (leader) mbar_expect_tx(full_bar(stage), tx);
                     const int f0 = ti.mt * 128 + 64 * (int)rank;
-                    tma2_load_4d(sA, &tmA0, fb, 0, k0, f0 >> 6, ti.e);
-                    tma2_load_4d(sA + TN_SUB_BYTES, &tmA1, fb, 0, k0, f0 >> 6, ti.e);
+                    tma2_load_3d(sA, &maps.a0, fb, f0, k0, ti.e);
+                    tma2_load_3d(sA + TN_CHUNK_BYTES, &maps.a1, fb, f0, k0, ti.e);
                 }
-                if (lane < ngroups) {
-                    tma2_gather4(sB + lane * 512, &tmB, fb, k0, tok[0], tok[1], tok[2], tok[3]);
-                    tma2_gather4(sB + TN_SUB_BYTES + lane * 512, &tmB, fb, k0 + 64, tok[0], tok[1], tok[2], tok[3]);
-                }
+                if (lane < ngroups) tma2_gather4(sB + lane * 512, &maps.b[0], fb, k0, tok[0], tok[1], tok[2], tok[3]);
                 __syncwarp();
                 if (++stage == S) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 0) {
         // ===================================================================== TMA producer (both CTAs)
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0; bool alive = true;
-            const uint64_t pol_w = l2_policy_evict_last();
-            Tile nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
-            for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
-                const Tile ti = nxt;
-                if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
-                const int half = ti.nmma >> 1;                         // token rows per CTA
-                const int nbox = (half + TN_BOX_ROWS - 1) / TN_BOX_ROWS;
-                const int brow0 = ti.row0 + (int)rank * half;
-                const uint32_t tx = 2u * (TN_A_BYTES + 2u * (uint32_t)nbox * TN_BOX_ROWS * 128u);
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
-                        alive = false; break;
-                    }
-                    const uint32_t fb = full_bar(stage) & T2_PEER_MASK;
-                    if (leader) mbar_expect_tx(full_bar(stage), tx);
-                    const uint32_t sA = smem_base + stage * TN_STAGE_BYTES;
-                    const uint32_t sB = sA + TN_A_BYTES;
-                    const int ph = (KIND == TN_B4 && kb >= args.kblocks) ? 1 : 0;   // B4: gate phase, then up phase
-                    const int k0 = (kb - ph * args.kblocks) * TN_BK;
-                    if constexpr (KIND == TN_B4 || KIND == TN_B2) {
-                        // K-major weights: this CTA's 128 weight rows, two boxes of 64 columns of K
-                        const int m0 = ti.mt * 256 + 128 * (int)rank;
-                        tma2_load_3d(sA, ph ? &tmA1 : &tmA0, fb, k0, m0, ti.e);
-                        tma2_load_3d(sA + TN_SUB_BYTES, ph ? &tmA1 : &tmA0, fb, k0 + 64, m0, ti.e);
-                        tma2_load_2d(sB, ph ? &tmB1 : &tmB, fb, k0, brow0);
-                        tma2_load_2d(sB + TN_SUB_BYTES, ph ? &tmB1 : &tmB, fb, k0 + 64, brow0);
-                        if (++stage == S) { stage = 0; phase ^= 1u; }
-                        continue;
-                    }
-                    if constexpr (KIND != TN_F2) {
-                        // 64 gate columns, then the 64 matching up columns (N-major weights [E, d, f])
-                        const int f0 = ti.mt * 128 + 64 * (int)rank;
-                        tma2_load_4d_hint(sA, &tmA0, fb, 0, k0, f0 >> 6, ti.e, pol_w);
-                        tma2_load_4d_hint(sA + TN_SUB_BYTES, &tmA1, fb, 0, k0, f0 >> 6, ti.e, pol_w);
-                    } else {
-                        const int m0 = ti.mt * 256 + 128 * (int)rank;
-                        tma2_load_4d_hint(sA, &tmA0, fb, 0, k0, m0 >> 6, ti.e, pol_w);   // two chunks in one copy
-                    }
-                    tma2_load_2d(sB, &tmB, fb, k0, brow0);
-                    tma2_load_2d(sB + TN_SUB_BYTES, &tmB, fb, k0 + 64, brow0);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
+        const bool el = elect_one();
+        int stage = 0; uint32_t phase = 0; bool alive = true;
+        Tile ti;
+        for (int n = 0; alive && next_item(n, ti); ++n) {
+            // this CTA's half of the token rows, in the smallest box that holds it (what a box fetches past the half belongs
+            // to nobody: the MMA reads the half only)
+            const int half = nmma_of(ti.rows) >> 1, box = (half + 15) >> 4;
+            const int brow0 = ti.row0 + (int)rank * half;
+            const uint32_t tx = 2u * (TN_SUB_BYTES + (uint32_t)box * 2048u);
+            const CUtensorMap* mb = &maps.b[box - 1];
+            // first weight row of this CTA (F1: 64 gate columns, then the 64 matching up columns)
+            const int m0 = KIND == TN_F1 ? ti.mt * 128 + 64 * (int)rank : ti.mt * 256 + 128 * (int)rank;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                    alive = false; break;
                 }
+                const uint32_t fb = full_bar(stage) & T2_PEER_MASK;
+                const uint32_t sA = smem_base + stage * STAGE_BYTES;
+                const uint32_t sB = sA + TN_SUB_BYTES;
+                const int ph = (KIND == TN_B4 && kb >= args.kblocks) ? 1 : 0;   // B4: gate phase, then up phase
+                const int k0 = (kb - ph * args.kblocks) * TN_BK;
+                if (KIND == TN_B4 && kb == args.kblocks) mb = &maps.b1[box - 1];
+                if (el) {
+                    if (!leader && handout && kb == ask_at) mbar_arrive(signal_bar(n));
+                    if (leader) mbar_expect_tx(full_bar(stage), tx);
+                    if constexpr (KIND == TN_B4 || KIND == TN_B2) {
+                        tma2_load_3d(sA, ph ? &maps.a1 : &maps.a0, fb, k0, m0, ti.e);   // K-major weights
+                    } else if constexpr (KIND == TN_F1) {                               // N-major weights [E, d, f]
+                        tma2_load_3d(sA, &maps.a0, fb, m0, k0, ti.e);
+                        tma2_load_3d(sA + TN_CHUNK_BYTES, &maps.a1, fb, m0, k0, ti.e);
+                    } else if (args.a_split) {
+                        tma2_load_3d(sA, &maps.a0, fb, m0, k0, ti.e);
+                        tma2_load_3d(sA + TN_CHUNK_BYTES, &maps.a0, fb, m0 + 64, k0, ti.e);
+                    } else {
+                        tma2_load_4d(sA, &maps.a0, fb, 0, k0, m0 >> 6, ti.e);           // two chunks in one copy
+                    }
+                    tma2_load_2d(sB, mb, fb, k0, brow0);
+                }
+                if (++stage == S) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
         // ===================================================================== MMA issuer (leader CTA)
-        // One thread runs the whole loop (wait, fence, four MMAs, commit): per K block nothing but
-        // these instructions stands between two groups of MMAs, so the tensor pipe's queue stays fed.
-        if (leader && lane == 0) {
+        if (leader) {
+            const bool el = elect_one();
             constexpr bool A_KMAJOR = (KIND == TN_B4 || KIND == TN_B2);
-            // descriptors without the start address: A is M-major (N-major weights) or K-major, B is K-major
-            // A M-major: the two 64-wide chunks are TN_SUB_BYTES apart and hold 128 K rows each (2 KiB per
-            // K = 16); K-major operands: two 64-K sub-tiles TN_SUB_BYTES apart, 32 bytes per K = 16 inside one
-            const uint64_t desc_a = smem_desc(0, A_KMAJOR ? 0 : TN_SUB_BYTES, 1024);
+            // descriptors without the start address: A is M-major (N-major weights) or K-major, B is K-major.
+            // A M-major: the two 64-wide chunks are TN_CHUNK_BYTES apart, 2 KiB per K = 16; K-major: 32 bytes per K = 16
+            const uint64_t desc_a = smem_desc(0, A_KMAJOR ? 0 : TN_CHUNK_BYTES, 1024);
             const uint64_t desc_b = smem_desc(0, 0, 1024);
+            // M = 256 over the pair, N = the tile's tokens
+            constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((A_KMAJOR ? 0u : 1u) << 15) | ((uint32_t)(256 >> 4) << 24);
             int stage = 0; uint32_t phase = 0; int it = 0; bool alive = true;
-            Tile nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
-            for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
-                const Tile ti = nxt;
-                if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
-                // M = 256 over the pair, N = this tile's tokens
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_KMAJOR ? 0u : 1u) << 15) |
-                                       ((uint32_t)(ti.nmma >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+            Tile ti;
+            for (int n = 0; alive && next_item(n, ti); ++n) {
+                const uint32_t idesc = idesc0 | ((uint32_t)(nmma_of(ti.rows) >> 3) << 17);
                 const int buf = it & 1;
-                const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
-                if (!mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
-                tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * 256;
+                if (!mbar_wait(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
+                tc_fence_after();
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) {
-                        alive = false; break;
-                    }
+                    if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
                     tc_fence_after();
-                    const uint32_t sA = smem_base + stage * TN_STAGE_BYTES;
+                    const uint32_t sA = smem_base + stage * STAGE_BYTES;
                     const uint64_t da = desc_a | (uint64_t)((sA & 0x3ffffu) >> 4);
-                    const uint64_t db = desc_b | (uint64_t)(((sA + TN_A_BYTES) & 0x3ffffu) >> 4);
+                    const uint64_t db = desc_b | (uint64_t)(((sA + TN_SUB_BYTES) & 0x3ffffu) >> 4);
+                    if (el) {
 #pragma unroll
-                    for (int k8 = 0; k8 < TN_BK / 16; ++k8) {
-                        const uint32_t kmaj = (uint32_t)((k8 >> 2) * (TN_SUB_BYTES >> 4) + (k8 & 3) * 2);
-                        umma2_bf16(d_tmem, da + (A_KMAJOR ? kmaj : (uint32_t)(k8 * (2048 >> 4))), db + kmaj, idesc,
-                                   (kb | k8) != 0 ? 1u : 0u);
+                        for (int k4 = 0; k4 < TN_BK / 16; ++k4)
+                            umma2_bf16(d_tmem, da + k4 * (A_KMAJOR ? 2 : 2048 >> 4), db + k4 * 2, idesc, (kb | k4) != 0 ? 1u : 0u);
+                        umma2_commit_both(empty_bar(stage));
                     }
-                    umma2_commit_both(empty_bar(stage));
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
                 if (!alive) break;
-                umma2_commit_both(tfull_bar(buf));
+                if (el) umma2_commit_both(tfull_bar(buf));
                 ++it;
+            }
+        } else if (handout && lane == 0) {
+            // ================================================================= hands out work items (second CTA)
+            for (int m = 1;; ++m) {
+                const int r = m - 1 - ahead;             // announced when item r asks
+                if (r >= 0 && !mbar_wait(signal_bar(r), (uint32_t)(r / TN_SIGNALS) & 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) break;
+                const int4 v = decode(n_clusters + atomicAdd(args.next, 1));
+                publish16(item_slot(m), item_bar(m), 0, v);
+                publish16(item_slot(m), item_bar(m), 1, v);
+                if (v.x < 0) break;
             }
         }
     } else {
-        // ===================================================================== epilogue (4 warps, both CTAs)
+        // ===================================================================== epilogue (8 warps, both CTAs)
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31
-        uint8_t* wbuf = epi_smem + quarter * 8192;    // this warp's staging
-        int it = 0;
-        Tile nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
-        for (int t = cluster_id; t < total_tiles; t += n_clusters) {
-            const Tile ti = nxt;
-            if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
-            const int buf = it & 1;
-            const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
-            // F2: the gates of the tile's tokens (two dependent loads each) are fetched before the wait for the
-            // accumulator, so that their latency is hidden behind the main loop instead of paid per 32 tokens
-            float gpre[8];
-            if constexpr (KIND == TN_F2) {
+        const int group = (warp - 2) >> 2;            // the accumulator these four warps drain
+        const uint32_t wb = epi_base + (uint32_t)(warp - 2) * TN_EPI_BYTES;   // this warp's staging
+        const uint32_t fo = frag_off(lane);
+        const int tpair = 2 * (lane & 3);             // this thread's tokens within a run of 8: tpair, tpair + 1
+        Tile ti;
+        // (the lanes give up together: a lane that left alone would be missed at the shuffles below)
+        for (int n = 0; __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
+            if ((n & 1) != group) continue;
+            const int buf = group;
+            const int row0 = ti.row0, rows = ti.rows;
+            // F2, B2: the gates of the tile's tokens (two dependent loads each) are fetched before the wait for the
+            // accumulator, so that their latency is hidden behind the main loop
+            const uint32_t gbuf = wb + 3072;
+            if constexpr (KIND == TN_F2 || KIND == TN_B2) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int tk = 32 * j + lane;
-                    gpre[j] = tk < ti.rows ? args.ep.gate[args.ep.row_src[ti.row0 + tk]] : 0.0f;
+                    const float g = tk < rows ? args.ep.gate[args.ep.row_src[row0 + tk]] : 0.0f;
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(gbuf + 4u * tk), "f"(g) : "memory");
                 }
+                __syncwarp();
             }
-            bool ready = mbar_wait_warp(tfull_bar(buf), tphase, abort_flag, args.status, STATUS_WAIT_TMEM_FULL, lane);
+            bool ready = mbar_wait_warp(tfull_bar(buf), (uint32_t)(n >> 1) & 1u, abort_flag, args.status, STATUS_WAIT_TMEM_FULL, lane);
             // the gate warp and its up warp meet at a named barrier below: they give up together or not at all
-            if constexpr (KIND == TN_F1 || KIND == TN_F1G) ready = bar_vote_all(1 + (quarter & 1), 64, ready);
+            if constexpr (KIND == TN_F1 || KIND == TN_F1G) ready = bar_vote_all(1 + 2 * group + (quarter & 1), 64, ready);
             if (!ready) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * 256;
-            float v[32];
+            const int nmma = nmma_of(rows);
 
             if constexpr (KIND == TN_F1 || KIND == TN_F1G) {
                 // Lanes 0..63 of the CTA hold gate rows, lanes 64..127 the matching up rows: warp q (gate)
@@ -348,137 +475,176 @@ tn_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
                 // tokens 0..15), so each evaluates SwiGLU for 16 tokens and writes 16 rows of H.
                 const bool is_up = quarter >= 2;
                 const int fcol = ti.mt * 128 + 64 * (int)rank + 32 * (quarter & 1);   // first f of this warp
-                const bool f_ok = fcol < args.Mw;
-                float* my_x = reinterpret_cast<float*>(wbuf);                                  // 16 x 33 fp32
-                const float* peer_x = reinterpret_cast<const float*>(epi_smem + (quarter ^ 2) * 8192);
-                uint16_t* hb = reinterpret_cast<uint16_t*>(wbuf + 2176);                       // 16 x 32 bf16: H
-                uint16_t* sb = reinterpret_cast<uint16_t*>(wbuf + 3200);                       // 32 x 32 bf16: stash
+                const uint32_t peer = epi_base + (uint32_t)(((warp - 2) & 4) + (((warp - 2) ^ 2) & 3)) * TN_EPI_BYTES;
+                const uint32_t sb = wb + 2048;                                         // staged rows
                 bf16* stash_out = is_up ? args.ep.out2 : args.ep.out1;
                 const int t_own = is_up ? 16 : 0;
-                const int pair_bar = 1 + (quarter & 1);
+                const int pair_bar = 1 + 2 * group + (quarter & 1);
 #pragma unroll 1
-                for (int c = 0; c < ti.nmma; c += 32) {
-                    tmem_ld32(taddr + c, v);
-                    const int rows_left = ti.rows - c;
+                for (int c = 0; c < nmma; c += 32) {
+                    float v0[16], v1[16];
+                    tmem_frag4(taddr + c, v0);
+                    tmem_frag4(taddr + (16u << 16) + c, v1);
+                    tmem_frag_wait(v0, v1);
+                    const int rows_left = rows - c;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) my_x[i * 33 + lane] = is_up ? v[i] : v[16 + i];
-                    if (stash_out) {
+                    for (int q = 0; q < 4; ++q) {      // the partner's half: 16 fp32 values, 16 bytes per lane and store
+                        const int i = 4 * (q & 1);
+                        float x[4];
 #pragma unroll
-                        for (int tk = 0; tk < 32; ++tk) sb[tk * 32 + lane] = bf16_bits(v[tk]);
+                        for (int r = 0; r < 4; ++r)
+                            x[r] = q < 2 ? (is_up ? v0[i + r] : v0[8 + i + r]) : (is_up ? v1[i + r] : v1[8 + i + r]);
+                        sts128(wb + 512 * q + 16 * lane, make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]),
+                                                                    __float_as_uint(x[2]), __float_as_uint(x[3])));
+                    }
+                    if (stash_out) {                   // own 32 tokens of G or U, in two halves of 1 KiB
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int j = 2 * h; j < 2 * h + 2; ++j)
+                                stmatrix4_trans(sb + 512 * (j & 1) + fo, pack_bf16x2(v0[4 * j], v0[4 * j + 1]),
+                                                pack_bf16x2(v0[4 * j + 2], v0[4 * j + 3]), pack_bf16x2(v1[4 * j], v1[4 * j + 1]),
+                                                pack_bf16x2(v1[4 * j + 2], v1[4 * j + 3]));
+                            __syncwarp();
+                            tn_write_rows<2>(stash_out, args.ep.ldo, sb, row0 + c + 16 * h, rows_left - 16 * h, fcol, args.Mw, lane);
+                            __syncwarp();
+                        }
                     }
                     bar_pair_sync(pair_bar);     // both halves are in shared memory
+                    float h0[8], h1[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float other = peer_x[i * 33 + lane];
-                        const float mine = is_up ? v[16 + i] : v[i];
-                        const float g = is_up ? other : mine, u = is_up ? mine : other;
-                        hb[i * 32 + lane] = bf16_bits(g * sigmoidf_fast(g) * u);
-                    }
-                    __syncwarp();
-                    if (f_ok) {
+                    for (int q = 0; q < 4; ++q) {
+                        const uint4 o = lds128(peer + 512 * q + 16 * lane);
+                        const float other[4] = {__uint_as_float(o.x), __uint_as_float(o.y), __uint_as_float(o.z), __uint_as_float(o.w)};
+                        const int i = 4 * (q & 1);
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {     // 16 tokens x 32 features of H: 64-byte row segments
-                            const int tok = 8 * i + (lane >> 2), part = lane & 3;
-                            const uint4 hv = *reinterpret_cast<const uint4*>(hb + tok * 32 + part * 8);
-                            if (t_own + tok < rows_left)
-                                *reinterpret_cast<uint4*>(args.ep.out0 + (size_t)(ti.row0 + c + t_own + tok) * args.ep.ldo +
-                                                          fcol + part * 8) = hv;
+                        for (int r = 0; r < 4; ++r) {
+                            const float mine = q < 2 ? (is_up ? v0[8 + i + r] : v0[i + r]) : (is_up ? v1[8 + i + r] : v1[i + r]);
+                            const float g = is_up ? other[r] : mine, u = is_up ? mine : other[r];
+                            const float h = g * sigmoidf_fast(g) * u;
+                            if (q < 2) h0[i + r] = h; else h1[i + r] = h;
                         }
-                        if (stash_out) tn_write_rows(stash_out, args.ep.ldo, sb, ti.row0 + c, rows_left, fcol, lane);
                     }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        stmatrix4_trans(sb + 512 * j + fo, pack_bf16x2(h0[4 * j], h0[4 * j + 1]), pack_bf16x2(h0[4 * j + 2], h0[4 * j + 3]),
+                                        pack_bf16x2(h1[4 * j], h1[4 * j + 1]), pack_bf16x2(h1[4 * j + 2], h1[4 * j + 3]));
+                    __syncwarp();
+                    tn_write_rows<2>(args.ep.out0, args.ep.ldo, sb, row0 + c + t_own, rows_left - t_own, fcol, args.Mw, lane);
                     bar_pair_sync(pair_bar);     // the partner has read this warp's half
                 }
             } else if constexpr (KIND == TN_B2) {
+                // 16 tokens at a time: the stash (G, U, H) comes in as 16-byte pieces of token rows one step ahead, is staged and
+                // read back as fragments (ldmatrix.trans) that match the accumulator's; the results leave the same way.
                 const int fcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first f column of this warp
-                const bool f_ok = fcol < args.Mw;
-                float* fbuf = reinterpret_cast<float*>(wbuf);                       // 32 tokens x 33 fp32
-                const int part = lane & 3;
-#pragma unroll 1
-                for (int c = 0; c < ti.nmma; c += 32) {
-                    const int rows_left = ti.rows - c;
-                    // the stash (G, U, H: 16 bytes each per lane and sub-block) is requested first, so that its
-                    // latency overlaps the TMEM read and the transposition below
-                    uint4 gq[4], uq[4], hq[4];
-                    float gate[4];
-                    bool ok[4];
+                const int col = fcol + (lane & 3) * 8;
+                const bf16* const src[3] = {args.ep.in0, args.ep.in1, args.ep.in2};
+                bf16* const dst[3] = {args.ep.out0, args.ep.out1, args.ep.out2};
+                uint4 pre[3][2];
+                auto fetch = [&](int c) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int tok = 8 * i + (lane >> 2);
-                        ok[i] = f_ok && tok < rows_left;
-                        gate[i] = 0.0f;
-                        if (ok[i]) {
-                            const int row = ti.row0 + c + tok;
-                            const size_t o = (size_t)row * args.ep.ldo + fcol + part * 8;
-                            gq[i] = *reinterpret_cast<const uint4*>(args.ep.in0 + o);
-                            uq[i] = *reinterpret_cast<const uint4*>(args.ep.in1 + o);
-                            hq[i] = *reinterpret_cast<const uint4*>(args.ep.in2 + o);
-                            gate[i] = args.ep.gate[args.ep.row_src[row]];
+                    for (int i = 0; i < 2; ++i) {
+                        const int tok = c + 8 * i + (lane >> 2);
+                        const bool okk = tok < rows && col < args.Mw;
+                        const size_t o = (size_t)(row0 + tok) * args.ep.ldo + col;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+                            pre[a][i] = okk ? *reinterpret_cast<const uint4*>(src[a] + o) : make_uint4(0, 0, 0, 0);
+                    }
+                };
+                fetch(0);
+#pragma unroll 1
+                for (int c = 0; c < nmma; c += 16) {
+                    float v0[8], v1[8];
+                    tmem_frag2(taddr + c, v0);
+                    tmem_frag2(taddr + (16u << 16) + c, v1);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) sts128(wb + 1024 * a + 512 * i + piece_off(lane), pre[a][i]);
+                    __syncwarp();
+                    if (c + 16 < nmma) fetch(c + 16);
+                    uint32_t frag[3][2][4];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) ldmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j]);
+                    tmem_frag_wait(v0, v1);
+                    float dot[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float2 gt = lds64f(gbuf + 4u * (c + 8 * j + tpair));
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {          // features 8 m + lane / 4
+                            float dG[2], dU[2], gH[2];
+#pragma unroll
+                            for (int p = 0; p < 2; ++p) {      // tokens tpair, tpair + 1
+                                const float G = p ? bf16_hi(frag[0][j][m]) : bf16_lo(frag[0][j][m]);
+                                const float U = p ? bf16_hi(frag[1][j][m]) : bf16_lo(frag[1][j][m]);
+                                const float H = p ? bf16_hi(frag[2][j][m]) : bf16_lo(frag[2][j][m]);
+                                const float gate = p ? gt.y : gt.x;
+                                const float dhu = m < 2 ? v0[4 * j + 2 * m + p] : v1[4 * j + 2 * (m - 2) + p];
+                                dot[j][p] = fmaf(dhu, H, dot[j][p]);
+                                const float dh = gate * dhu;
+                                const float sg = sigmoidf_fast(G);
+                                dG[p] = dh * U * sg * (1.0f + G * (1.0f - sg));
+                                dU[p] = dh * (G * sg);
+                                gH[p] = gate * H;
+                            }
+                            frag[0][j][m] = pack_bf16x2(dG[0], dG[1]);
+                            frag[1][j][m] = pack_bf16x2(dU[0], dU[1]);
+                            frag[2][j][m] = pack_bf16x2(gH[0], gH[1]);
                         }
                     }
-                    tmem_ld32(taddr + c, v);
+                    __syncwarp();                              // every lane has its fragments of the stash
 #pragma unroll
-                    for (int tk = 0; tk < 32; ++tk) fbuf[tk * 33 + lane] = v[tk];
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            stmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j][0], frag[a][j][1], frag[a][j][2], frag[a][j][3]);
                     __syncwarp();
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int tok = 8 * i + (lane >> 2);
-                        float dot = 0.0f;
-                        if (ok[i]) {
-                            const uint32_t gw[4] = {gq[i].x, gq[i].y, gq[i].z, gq[i].w};
-                            const uint32_t uw[4] = {uq[i].x, uq[i].y, uq[i].z, uq[i].w};
-                            const uint32_t hw[4] = {hq[i].x, hq[i].y, hq[i].z, hq[i].w};
-                            float dG[8], dU[8], gH[8];
+                    for (int a = 0; a < 3; ++a)
+                        tn_write_rows<2>(dst[a], args.ep.ldo, wb + 1024 * a, row0 + c, rows - c, fcol, args.Mw, lane);
+                    // the 32 features' dot products: the 8 lanes with the same lane % 4 hold the shares of the same tokens
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const float G = (j & 1) ? bf16_hi(gw[j >> 1]) : bf16_lo(gw[j >> 1]);
-                                const float U = (j & 1) ? bf16_hi(uw[j >> 1]) : bf16_lo(uw[j >> 1]);
-                                const float H = (j & 1) ? bf16_hi(hw[j >> 1]) : bf16_lo(hw[j >> 1]);
-                                const float dhu = fbuf[tok * 33 + part * 8 + j];
-                                dot = fmaf(dhu, H, dot);
-                                const float dh = gate[i] * dhu;
-                                const float sg = sigmoidf_fast(G);
-                                dG[j] = dh * U * sg * (1.0f + G * (1.0f - sg));
-                                dU[j] = dh * (G * sg);
-                                gH[j] = gate[i] * H;
-                            }
-                            const size_t o = (size_t)(ti.row0 + c + tok) * args.ep.ldo + fcol + part * 8;
-                            store_bf16_run<8>(args.ep.out0 + o, dG);
-                            store_bf16_run<8>(args.ep.out1 + o, dU);
-                            store_bf16_run<8>(args.ep.out2 + o, gH);
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {
+#pragma unroll
+                            for (int off = 4; off < 32; off <<= 1) dot[j][p] += __shfl_xor_sync(0xffffffffu, dot[j][p], off);
+                            const int tok = c + 8 * j + tpair + p;
+                            if (lane < 4 && tok < rows && fcol < args.Mw)
+                                args.ep.part[(size_t)(fcol >> 5) * args.ep.M_total + row0 + tok] = dot[j][p];
                         }
-                        dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-                        dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                        if (ok[i] && part == 0)
-                            args.ep.part[(size_t)(fcol >> 5) * args.ep.M_total + ti.row0 + c + tok] = dot;
-                    }
                     __syncwarp();
                 }
             } else {
                 const int mcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first output column of this warp
-                const bool m_ok = mcol < args.Mw;
-                uint16_t* st0 = reinterpret_cast<uint16_t*>(wbuf);
+#pragma unroll 1
+                for (int c = 0; c < nmma; c += 32) {
+                    float v0[16], v1[16];
+                    tmem_frag4(taddr + c, v0);
+                    tmem_frag4(taddr + (16u << 16) + c, v1);
+                    tmem_frag_wait(v0, v1);
 #pragma unroll
-                for (int j8 = 0; j8 < 8; ++j8) {
-                    const int c = 32 * j8;
-                    if (c >= ti.nmma) break;
-                    tmem_ld32(taddr + c, v);
-                    const int rows_left = ti.rows - c;
-                    // gate of token (c + lane), handed round by shuffle
-                    const float gmine = (KIND == TN_F2) ? gpre[j8] : 1.0f;
-#pragma unroll
-                    for (int tk = 0; tk < 32; ++tk) {
-                        const float g = __shfl_sync(0xffffffffu, gmine, tk);
-                        st0[tk * 32 + lane] = bf16_bits(g * v[tk]);
+                    for (int j = 0; j < 4; ++j) {
+                        if constexpr (KIND == TN_F2) {
+                            const float2 g = lds64f(gbuf + 4u * (c + 8 * j + tpair));
+                            v0[4 * j] *= g.x; v0[4 * j + 1] *= g.y; v0[4 * j + 2] *= g.x; v0[4 * j + 3] *= g.y;
+                            v1[4 * j] *= g.x; v1[4 * j + 1] *= g.y; v1[4 * j + 2] *= g.x; v1[4 * j + 3] *= g.y;
+                        }
+                        stmatrix4_trans(wb + 512 * j + fo, pack_bf16x2(v0[4 * j], v0[4 * j + 1]), pack_bf16x2(v0[4 * j + 2], v0[4 * j + 3]),
+                                        pack_bf16x2(v1[4 * j], v1[4 * j + 1]), pack_bf16x2(v1[4 * j + 2], v1[4 * j + 3]));
                     }
                     __syncwarp();
-                    if (m_ok) tn_write_rows(args.ep.out0, args.ep.ldo, st0, ti.row0 + c, rows_left, mcol, lane);
+                    tn_write_rows<4>(args.ep.out0, args.ep.ldo, wb, row0 + c, rows - c, mcol, args.Mw, lane);
                     __syncwarp();
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_bar(buf) & T2_PEER_MASK);
-            ++it;
         }
     }
 
@@ -497,109 +663,110 @@ tn_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__
 }
 
 // ------------------------------------------------------------------------------------------ host
+template <int KIND>
+inline bool tn_set_smem() {
+    return cudaFuncSetAttribute(tn_gemm_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) == cudaSuccess;
+}
 inline mop_status tn_init() {
-    if (cudaFuncSetAttribute(tn_gemm_kernel<TN_F1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(tn_gemm_kernel<TN_F2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(tn_gemm_kernel<TN_F1G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(tn_gemm_kernel<TN_B4>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(tn_gemm_kernel<TN_B2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) !=
-            cudaSuccess)
-        return MOP_ERR_CUDA;
-    return MOP_OK;
+    return tn_set_smem<TN_F1>() && tn_set_smem<TN_F2>() && tn_set_smem<TN_F1G>() && tn_set_smem<TN_B4>() && tn_set_smem<TN_B2>()
+               ? MOP_OK : MOP_ERR_CUDA;
 }
 
-inline mop_status build_both_tiles(TcPlan* p, const int32_t* offsets, int32_t* mtiles, int32_t* ttiles, cudaStream_t st) {
-    p->prof->begin("build_tiles", st);
-    build_both_tiles_kernel<<<2, 1024, 0, st>>>(offsets, p->s.E, reinterpret_cast<int4*>(mtiles + 64), mtiles,
-                                                reinterpret_cast<int4*>(ttiles + 64), ttiles);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+// Tables behind `tiles`: 128-row tiles, (the mixed schedule's second list,) token tiles.
+inline int32_t* tn_table(const TcPlan* p, int32_t* tiles) {
+    return tiles + 2 * (tc_tile_table_bytes(p->s.T * p->s.k, p->s.E) / 4);
 }
-inline mop_status tn_build_tiles(TcPlan* p, const int32_t* offsets, int32_t* tiles, cudaStream_t st) {
+inline mop_status tn_build_tiles(TcPlan* p, const int32_t* offsets, int32_t* tiles, bool rows128, cudaStream_t st) {
     p->prof->begin("tn_build_ttiles", st);
-    tn_build_ttiles_kernel<<<1, 1024, 0, st>>>(offsets, p->s.E, reinterpret_cast<int4*>(tiles + 64), tiles);
+    tn_build_ttiles_kernel<<<rows128 ? 2 : 1, 1024, 0, st>>>(offsets, p->s.E, tn_table(p, tiles), tiles);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
 
-inline TnArgs tn_base_args(int32_t* tiles, int32_t* status) {
+inline TnArgs tn_base_args(const TcPlan* p, int32_t* tiles, int kind, int32_t* status) {
+    int32_t* table = tn_table(p, tiles);
     TnArgs g{};
-    g.ttiles = reinterpret_cast<const int4*>(tiles + 64);
-    g.n_ttiles = tiles;
+    g.next = table + 16 + kind;
+    g.ttiles = reinterpret_cast<const int4*>(table + 64);
+    g.n_ttiles = table;
     g.status = status;
     return g;
 }
 
-// Up-projection + SwiGLU on the tokens-on-N kernel (`tiles` holds the token-tile table).
+// Maps of a [rows, cols] bf16 token matrix with boxes of 16, 32, .. 128 rows, as far as a tile can need them: an expert gets a
+// token once, so its tiles have at most T rows, half of them (rounded up to 8) per CTA.
+inline bool tn_token_maps(const TcPlan* p, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
+    const int most = p->s.T < 256 ? p->s.T : 256;
+    const int boxes = (((most + 15) & ~15) / 2 + 15) >> 4;
+    for (int i = 0; i < boxes; ++i)
+        if (!tc_map_2d(p, &m[i], base, rows, cols, 16 * (i + 1))) return false;
+    return true;
+}
+
+template <int KIND>
+inline mop_status tn_launch(const TcPlan* p, const char* name, const TnMaps& m, const TnArgs& g, cudaStream_t st) {
+    p->prof->begin(name, st);
+    tn_gemm_kernel<KIND><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(m, g);
+    p->prof->end(st);
+    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+}
+
+// Up-projection + SwiGLU on the tokens-on-N kernel (`tiles`: the tables of tn_build_tiles).
 inline mop_status tn_up_swiglu(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st) {
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
-    CUtensorMap mXp, mWg, mWu;
-    if (!tc_map_2d(p, &mXp, a.Xp, M, s.d, TN_BOX_ROWS) || !tc_map_chunked_3d(p, &mWg, a.W_gate, s.E, s.d, s.f, 1, 128) ||
-        !tc_map_chunked_3d(p, &mWu, a.W_up, s.E, s.d, s.f, 1, 128))
+    TnMaps m;
+    if (!tc_map_3d(p, &m.a0, a.W_gate, s.E, s.d, s.f, TN_BK) || !tc_map_3d(p, &m.a1, a.W_up, s.E, s.d, s.f, TN_BK) ||
+        !tn_token_maps(p, m.b, a.Xp, M, s.d))
         return MOP_ERR_CUDA;
-    TnArgs g = tn_base_args(tiles, status);
+    TnArgs g = tn_base_args(p, tiles, TN_F1, status);
     g.tiles_m = ceil_div(s.f, 128); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.ep.out0 = a.H; g.ep.out1 = a.G_save; g.ep.out2 = a.U_save; g.ep.ldo = s.f; g.ep.M_total = (int)M;
-    p->prof->begin("gemm_up_swiglu", st);
-    tn_gemm_kernel<TN_F1><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(mWg, mWu, mXp, mXp, g);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+    return tn_launch<TN_F1>(p, "gemm_up_swiglu", m, g, st);
 }
 
 // Up-projection + SwiGLU reading its token rows straight from the unpermuted x (no Xp, no stash).
 inline mop_status tn_up_swiglu_gather(TcPlan* p, const bf16* x, const TcFwdArgs& a, int32_t* tiles, int32_t* status,
                                       cudaStream_t st) {
     const mop_moe_shape& s = p->s;
-    CUtensorMap mX, mWg, mWu;
-    if (!tc_map_2d(p, &mX, x, s.T, s.d, 1) || !tc_map_chunked_3d(p, &mWg, a.W_gate, s.E, s.d, s.f, 1, 128) ||
-        !tc_map_chunked_3d(p, &mWu, a.W_up, s.E, s.d, s.f, 1, 128))
+    TnMaps m;
+    if (!tc_map_2d(p, &m.b[0], x, s.T, s.d, 1) || !tc_map_3d(p, &m.a0, a.W_gate, s.E, s.d, s.f, TN_BK) ||
+        !tc_map_3d(p, &m.a1, a.W_up, s.E, s.d, s.f, TN_BK))
         return MOP_ERR_CUDA;
-    TnArgs g = tn_base_args(tiles, status);
+    TnArgs g = tn_base_args(p, tiles, TN_F1G, status);
     g.tiles_m = ceil_div(s.f, 128); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.row_src = a.row_src; g.topk = s.k;
     g.ep.out0 = a.H; g.ep.ldo = s.f; g.ep.M_total = s.T * s.k;
-    p->prof->begin("gemm_up_swiglu_gather", st);
-    tn_gemm_kernel<TN_F1G><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(mWg, mWu, mX, mX, g);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+    return tn_launch<TN_F1G>(p, "gemm_up_swiglu_gather", m, g, st);
 }
 
 // Down-projection + gate on the tokens-on-N kernel.
 inline mop_status tn_down_gate(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st) {
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
-    CUtensorMap mH, mWd;
-    if (!tc_map_2d(p, &mH, a.H, M, s.f, TN_BOX_ROWS) || !tc_map_chunked_3d(p, &mWd, a.W_down, s.E, s.f, s.d, 2, 128))
+    TnMaps m;
+    const bool split = s.d % 64 != 0;
+    if (!(split ? tc_map_3d(p, &m.a0, a.W_down, s.E, s.f, s.d, TN_BK) : tc_map_chunked_3d(p, &m.a0, a.W_down, s.E, s.f, s.d, 2, TN_BK)) ||
+        !tn_token_maps(p, m.b, a.H, M, s.f))
         return MOP_ERR_CUDA;
-    TnArgs g = tn_base_args(tiles, status);
-    g.tiles_m = ceil_div(s.d, 256); g.kblocks = ceil_div(s.f, TN_BK); g.Mw = s.d;
+    TnArgs g = tn_base_args(p, tiles, TN_F2, status);
+    g.tiles_m = ceil_div(s.d, 256); g.kblocks = ceil_div(s.f, TN_BK); g.Mw = s.d; g.a_split = split;
     g.ep.out0 = a.Yp; g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.ldo = s.d; g.ep.M_total = (int)M;
-    p->prof->begin("gemm_down_gate", st);
-    tn_gemm_kernel<TN_F2><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(mWd, mWd, mH, mH, g);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+    return tn_launch<TN_F2>(p, "gemm_down_gate", m, g, st);
 }
 
 // Data gradient of the up-projection on the tokens-on-N kernel: dXp = dG W_gate^T + dU W_up^T.
 inline mop_status tn_dgrad_gate_up(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st) {
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
-    CUtensorMap mWg, mWu, mdG, mdU;
-    if (!tc_map_3d(p, &mWg, a.W_gate, s.E, s.d, s.f, 128) || !tc_map_3d(p, &mWu, a.W_up, s.E, s.d, s.f, 128) ||
-        !tc_map_2d(p, &mdG, a.dG, M, s.f, TN_BOX_ROWS) || !tc_map_2d(p, &mdU, a.dU, M, s.f, TN_BOX_ROWS))
+    TnMaps m;
+    if (!tc_map_3d(p, &m.a0, a.W_gate, s.E, s.d, s.f, 128) || !tc_map_3d(p, &m.a1, a.W_up, s.E, s.d, s.f, 128) ||
+        !tn_token_maps(p, m.b, a.dG, M, s.f) || !tn_token_maps(p, m.b1, a.dU, M, s.f))
         return MOP_ERR_CUDA;
-    TnArgs g = tn_base_args(tiles, status);
+    TnArgs g = tn_base_args(p, tiles, TN_B4, status);
     g.tiles_m = ceil_div(s.d, 256); g.kblocks = ceil_div(s.f, TN_BK); g.Mw = s.d;
     g.ep.out0 = a.dXp; g.ep.ldo = s.d; g.ep.M_total = (int)M;
-    p->prof->begin("gemm_dgrad_gate_up", st);
-    tn_gemm_kernel<TN_B4><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(mWg, mWu, mdG, mdU, g);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+    return tn_launch<TN_B4>(p, "gemm_dgrad_gate_up", m, g, st);
 }
 
 // Data gradient of the down-projection with the SwiGLU backward on the tokens-on-N kernel.
@@ -607,17 +774,13 @@ inline mop_status tn_dgrad_gate_up(TcPlan* p, const TcBwdArgs& a, int32_t* tiles
 inline mop_status tn_dgrad_down(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st) {
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
-    CUtensorMap mWd, mdYp;
-    if (!tc_map_3d(p, &mWd, a.W_down, s.E, s.f, s.d, 128) || !tc_map_2d(p, &mdYp, a.dYp, M, s.d, TN_BOX_ROWS))
-        return MOP_ERR_CUDA;
-    TnArgs g = tn_base_args(tiles, status);
+    TnMaps m;
+    if (!tc_map_3d(p, &m.a0, a.W_down, s.E, s.f, s.d, 128) || !tn_token_maps(p, m.b, a.dYp, M, s.d)) return MOP_ERR_CUDA;
+    TnArgs g = tn_base_args(p, tiles, TN_B2, status);
     g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH; g.ep.in0 = a.G_save; g.ep.in1 = a.U_save; g.ep.in2 = a.H;
     g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
-    p->prof->begin("gemm_dgrad_down_dswiglu", st);
-    tn_gemm_kernel<TN_B2><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(mWd, mWd, mdYp, mdYp, g);
-    p->prof->end(st);
-    return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+    return tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
 }
 
 }  // namespace mop

@@ -414,15 +414,11 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         }
         c->plan.pairs = shape->gemm_path == MOP_GEMM_TENSOR_2CTA ? 1 : shape->gemm_path == MOP_GEMM_TENSOR_MIXED ? 2 : 0;
         if (c->sm_count < 2) c->plan.pairs = 0;
-        // Measured policy (B200): the tokens-on-N down-projection wins on every workload; the tokens-on-N
-        // up-projection wins when the K loop is long enough to hide its heavier epilogue (d >= 4096).
+        // The tokens-on-N kernels for all four token-row GEMMs (bits 0..3: up- and down-projection, their data gradients)
         c->plan.fwd_tn = 0;
-        if (c->sm_count >= 2) {
-            // bits 2, 3: the data gradients of the up- and down-projection on the same kernel
-            if (shape->gemm_path == MOP_GEMM_TENSOR_TN) c->plan.fwd_tn = 15;
-            else if (shape->gemm_path == MOP_GEMM_AUTO || shape->gemm_path == MOP_GEMM_TENSOR)
-                c->plan.fwd_tn = 8 | 4 | 2 | (shape->d >= 4096 ? 1 : 0);
-        }
+        if (c->sm_count >= 2 && (shape->gemm_path == MOP_GEMM_TENSOR_TN || shape->gemm_path == MOP_GEMM_AUTO ||
+                                 shape->gemm_path == MOP_GEMM_TENSOR))
+            c->plan.fwd_tn = 15;
     }
     *out = c;
     return MOP_OK;

@@ -152,6 +152,21 @@ def test_gathering_forward_refuses_the_scalar_path():
     assert e.value.code == 6
 
 
+@pytest.mark.parametrize("E,k,T,d,f", [(512, 8, 300, 64, 448),     # one K block per item, 27 items per cluster and more
+                                       (400, 4, 500, 640, 512),    # 10 K blocks: items announced one ahead
+                                       (160, 2, 700, 1600, 1088)],  # 25 K blocks: announced near the end of the one before
+                         ids=lambda v: str(v))
+def test_tokens_on_n_kernels_with_many_more_items_than_clusters(E, k, T, d, f):
+    """Work items are handed out through rings of 16 entries: more than 16 items per cluster wrap them."""
+    w = synth.small("c2_mid", T=T, d=d, E=E, k=k, f=f, backward=True, seed=46)
+    host = synth.make_inputs(w, "cuda")
+    _, _, _, buf = run(w, binding.GEMM_TENSOR_TN, host)
+    assert int((buf.counts > 0).sum()) * -(-f // 128) > 17 * 74
+    _, _, _, ref = run(w, binding.GEMM_TENSOR_1CTA, host)     # bit for bit the one-CTA kernel, which the cases above tie to the oracle
+    for n in ("H", "Yp", "Y", "dX", "dW_gate", "dW_up", "dW_down"):
+        assert torch.equal(getattr(buf, n), getattr(ref, n)), n
+
+
 def test_tokens_on_n_kernels_with_three_token_tiles_and_half_filled_k_stages():
     """700 rows per expert (three token tiles of 240) with d = 320 and f = 192: K is 2.5 and 1.5 pipeline
     stages of 128, so the last stage of every GEMM is half zero fill; all four token-row GEMMs forced
