@@ -15,8 +15,8 @@
  *   - Argument errors are detected on the host before any launch and reported by the return
  *     code; nothing is thrown, nothing aborts.  Kernels never trap: a wait that runs out of
  *     its poll budget records a code in the context's status word, which mop_poll() reads.
- *   - d and f must be multiples of 8 (16-byte rows); the tensor-core kernels further need
- *     d and f to be multiples of 64 and otherwise the call uses the scalar kernels.
+ *   - d and f must be multiples of 8 (16-byte rows).  gemm_path TENSOR and the forced schedules, the
+ *     gathering forward and the chunked layer further need multiples of 64.
  *   - No output is produced with atomics: results are bitwise reproducible run to run.
  *   - A context is bound to one device and one shape; calls on one context must not overlap
  *     on the GPU (they share its workspace).
@@ -51,10 +51,9 @@ typedef enum { MOP_SCORE_SOFTMAX = 0, MOP_SCORE_SIGMOID = 1 } mop_score_fn;
  * gate numerator in POST_SCORE mode. */
 typedef enum { MOP_BIAS_NONE = 0, MOP_BIAS_POST_SCORE = 1, MOP_BIAS_PRE_LOGIT = 2 } mop_bias_mode;
 
-/* AUTO: tensor cores when the shape allows, else scalar.  TENSOR: tensor cores or fail.  Both pick
- * per GEMM the schedule measured fastest: the forward down-projection, both data gradients (and the
- * up-projection when d >= 4096) on the two-CTA tokens-on-N kernel, the weight gradients (and the
- * up-projection otherwise) on the one-CTA kernel (128 x 256 tiles).
+/* AUTO: tensor cores at every supported shape.  TENSOR: the same, d and f multiples of 64 or fail.  Both run the
+ * four token-row GEMMs on the two-CTA tokens-on-N kernel and the weight gradients on the one-CTA
+ * kernel (128 x 256 tiles).
  * The remaining values force one schedule for testing and measurement: TENSOR_1CTA = one-CTA kernel
  * for all token-row GEMMs; TENSOR_2CTA = two-CTA kernel on 256-row pair tiles; TENSOR_MIXED = full
  * pairs on the two-CTA kernel, remaining rows on the one-CTA kernel; TENSOR_TN = all four token-row

@@ -129,9 +129,9 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
     }
     CUtensorMap mgH, mdYpB, mXpA, mdGB, mdUB, moWd, moWg, moWu;   // weight gradients
     if (!tc_map_out_f32(p, &moWd, a.dW_down, s.E, s.f, s.d) || !tc_map_out_f32(p, &moWg, a.dW_gate, s.E, s.d, s.f) ||
-        !tc_map_out_f32(p, &moWu, a.dW_up, s.E, s.d, s.f) || !tc_map_chunked_2d(p, &mgH, a.gH, M, s.f, 2) ||
-        !tc_map_chunked_2d(p, &mdYpB, a.dYp, M, s.d, 4) || !tc_map_chunked_2d(p, &mXpA, a.Xp, M, s.d, 2) ||
-        !tc_map_chunked_2d(p, &mdGB, a.dG, M, s.f, 4) || !tc_map_chunked_2d(p, &mdUB, a.dU, M, s.f, 4))
+        !tc_map_out_f32(p, &moWu, a.dW_up, s.E, s.d, s.f) || !tc_map_mn(p, &mgH, a.gH, M, s.f, 2) ||
+        !tc_map_mn(p, &mdYpB, a.dYp, M, s.d, 4) || !tc_map_mn(p, &mXpA, a.Xp, M, s.d, 2) ||
+        !tc_map_mn(p, &mdGB, a.dG, M, s.f, 4) || !tc_map_mn(p, &mdUB, a.dU, M, s.f, 4))
         return MOP_ERR_CUDA;
     // tokens-on-M data gradients: K-major weight maps boxed for one CTA (256 N rows) and for a pair CTA (128)
     CUtensorMap mdYpA, mWdK, mWdKp, mdG, mdU, mWgK, mWuK, mWgKp, mWuKp;
@@ -173,6 +173,7 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
     {   // WD: dW_down[e] = (gate H)_e^T dYp_e
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
         g.tiles_n = ceil_div(s.d, 256); g.tiles_m_fixed = ceil_div(s.f, TC_BM); g.Mfix = s.f; g.N = s.d;
+        g.a_split = s.f % 64 != 0; g.b_split = s.d % 64 != 0;
         g.ep.outf = a.dW_down; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
         if ((r = tc_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mgH, mdYpB, mdYpB, moWd, moWd, g, st)) != MOP_OK) return r;
         ++*launches;
@@ -180,6 +181,7 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
     {   // WGU: dW_gate[e] = Xp_e^T dG_e and dW_up[e] = Xp_e^T dU_e: per m-block the n-tiles of dW_gate, then those of dW_up
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
         g.tiles_n = 2 * ceil_div(s.f, 256); g.tiles_m_fixed = ceil_div(s.d, TC_BM); g.Mfix = s.d; g.N = s.f;
+        g.a_split = s.d % 64 != 0; g.b_split = s.f % 64 != 0;
         g.ep.outf = a.dW_gate; g.outf1 = a.dW_up; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
         if ((r = tc_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mXpA, mdGB, mdUB, moWg, moWu, g, st)) != MOP_OK) return r;
         ++*launches;

@@ -1,6 +1,4 @@
-// Scalar (CUDA-core) grouped GEMM: the generic path for shapes the tensor-core kernels do not
-// take (d or f not a multiple of 64) and the on-device cross-check used while bringing those
-// kernels up.  bf16 operands, fp32 accumulation, any operand strides, ragged M (rows of an
+// Scalar (CUDA-core) grouped GEMM: the on-device cross-check of the tensor-core kernels (gemm_path SCALAR).  bf16 operands, fp32 accumulation, any operand strides, ragged M (rows of an
 // expert) or ragged K (weight gradients), same epilogues as the tensor-core path.
 #pragma once
 #include "epilogue.cuh"

@@ -66,6 +66,8 @@ struct TcArgs {
     int tiles_n;             // n-tiles per row block
     int tiles_m_fixed;       // ragged K: m-tiles per expert
     int kblocks;             // ragged M: K / 64 (rounded up) per phase
+    int a_split, b_split;    // ragged K: that operand's columns are no multiple of 64: one copy per 64-wide chunk, the map's edge
+                             // zero-fills (a chunked view would run past the end of a row)
     int Mfix, N;             // ragged K: output rows per expert; N = columns per output tensor
     int m_fastest;           // tile order: 1 = consecutive tiles walk the row tiles of one column block
     const int32_t* targets;  // VL, VP: target column per row
@@ -188,6 +190,13 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
+}
+__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
+                                                 uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+        "{%3, %4}], [%2], %5;" ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(policy)
+        : "memory");
 }
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y,
                                                  int z, uint64_t policy) {
@@ -586,9 +595,13 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
                     mbar_expect_tx(fb, TC_STAGE_BYTES);
                     if constexpr (!Tr::A_MN) {
                         tma_load_2d(sA, (KIND == TC_B4 && ph) ? &tmA1 : &tmA0, fb, k0, ti.row0);
-                    } else {
+                    } else if (!args.a_split) {
                         // chunked map {64, rows, cols/64}: both 64-wide column chunks in one copy
                         tma_load_3d_hint(sA, &tmA0, fb, 0, ti.row0 + kb * TC_BK, ti.m0 >> 6, keep);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+                            tma_load_2d_hint(sA + q * TC_CHUNK_BYTES, &tmA0, fb, ti.m0 + 64 * q, ti.row0 + kb * TC_BK, keep);
                     }
                     if constexpr (!Tr::B_MN) {
                         tma_load_3d(sB, ph ? &tmB1 : &tmB0, fb, k0 + (KIND == TC_VX ? args.kb_base : 0), n0, ti.e);
@@ -600,7 +613,13 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
                             if constexpr (Tr::DUAL_B) tma_load_4d(sB + 2 * TC_CHUNK_BYTES, &tmB1, fb, 0, k0, n0 >> 6, ti.e);
                         } else {
                             const int krow = ti.row0 + kb * TC_BK;
-                            tma_load_3d_hint(sB, (Tr::SEL_B && ti.sel) ? &tmB1 : &tmB0, fb, 0, krow, n0 >> 6, keep);
+                            const CUtensorMap* mb = (Tr::SEL_B && ti.sel) ? &tmB1 : &tmB0;
+                            if (!args.b_split) tma_load_3d_hint(sB, mb, fb, 0, krow, n0 >> 6, keep);
+                            else {
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    tma_load_2d_hint(sB + q * TC_CHUNK_BYTES, mb, fb, n0 + 64 * q, krow, keep);
+                            }
                         }
                     }
                 }
@@ -868,6 +887,7 @@ struct TcBwdArgs {
     int keep_empty;   // experts without rows (in this call's offsets) keep their gradients: expert-chunked backward
 };
 
+// Shapes of the tokens-on-M, gathering and chunked forms; the tokens-on-N kernels and the weight gradients take any multiple of 8.
 inline bool tc_shape_supported(int d, int f) { return d % 64 == 0 && f % 64 == 0; }
 inline uint64_t tc_rows(const TcPlan* p) {
     return p->rows_override > 0 ? (uint64_t)p->rows_override : (uint64_t)p->s.T * p->s.k;
@@ -948,6 +968,10 @@ inline bool tc_map_chunked_2d(const TcPlan* p, CUtensorMap* m, const void* base,
                                                      dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// An MN-major operand of the weight gradients: the chunked view in one copy where the columns are a multiple of 64.
+inline bool tc_map_mn(const TcPlan* p, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t chunks) {
+    return cols % 64 ? tc_map_2d(p, m, base, rows, cols, TC_BK) : tc_map_chunked_2d(p, m, base, rows, cols, chunks);
 }
 inline bool tc_map_chunked_3d(const TcPlan* p, CUtensorMap* m, const void* base, uint64_t E, uint64_t rows,
                               uint64_t cols, uint32_t chunks, uint32_t box_rows = 64) {

@@ -23,7 +23,8 @@ struct mop_ctx {
     int device;
     int sm_count;
     int64_t launches;
-    bool tensor_ok;      // shape admits the tensor-core kernels
+    bool tensor_ok;      // shape admits every tensor-core kernel (d and f multiples of 64)
+    bool tensor_tn;      // the layer's GEMMs run on the tensor cores (tokens-on-N kernels and weight gradients: any multiple of 8)
     // workspace (one allocation)
     char* ws;
     size_t ws_bytes;
@@ -248,7 +249,7 @@ struct DeviceGuard {
     }
 };
 
-bool use_tensor(const mop_ctx* c) { return c->tensor_ok && c->s.gemm_path != MOP_GEMM_SCALAR; }
+bool use_tensor(const mop_ctx* c) { return c->tensor_tn; }
 
 // ---- scalar-path launches ---------------------------------------------------------------
 mop_status launch_scalar(mop_ctx* c, const char* name, const ScalarGemmArgs& g, cudaStream_t st) {
@@ -303,6 +304,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         delete c;
         return MOP_ERR_UNSUPPORTED;
     }
+    c->tensor_tn = shape->gemm_path != MOP_GEMM_SCALAR && (c->tensor_ok || (prop.major == 10 && c->sm_count >= 2));
     const Layout L = make_layout(*shape);
     c->ws_bytes = L.total;
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }
@@ -398,7 +400,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
             cudaFree(c->ws); delete c; return MOP_ERR_CUDA;
         }
     }
-    if (c->tensor_ok) {
+    if (c->tensor_ok || c->tensor_tn) {
         st = tc_plan_init(&c->plan, *shape, c->sm_count, &c->prof);
         if (st == MOP_OK) st = tc2_init();
         if (st == MOP_OK) st = tn_init();
@@ -735,7 +737,7 @@ mop_status mop_moe_expert_ffn_fwd_gather(mop_ctx* c, const void* x, const int32_
     if (!c) return MOP_ERR_INVALID_ARG;
     REQ_PTR_T(x); REQ_PTR(offsets); REQ_PTR_T(row_src); REQ_PTR_T(topk_gate); REQ_PTR(W_gate); REQ_PTR(W_up);
     REQ_PTR(W_down); REQ_PTR_T(H); REQ_PTR_T(Yp);
-    if (!use_tensor(c)) return MOP_ERR_UNSUPPORTED;   // the gather is a TMA feature of the tensor-core path
+    if (!use_tensor(c) || !c->tensor_ok) return MOP_ERR_UNSUPPORTED;   // the gather is a TMA feature of the tensor-core path
     const mop_moe_shape& s = c->s;
     if (s.T == 0) return MOP_OK;
     DeviceGuard guard(c->device);
@@ -881,7 +883,7 @@ mop_status chunk_check(mop_ctx* c, int32_t n_chunks, const void* workspace) {
     if (n_chunks < 1 || n_chunks > 64) return MOP_ERR_INVALID_ARG;
     if (!workspace) return MOP_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MOP_ERR_ALIGN;
-    if (!use_tensor(c)) return MOP_ERR_UNSUPPORTED;    // the chunked layer runs on the tensor-core kernels only
+    if (!use_tensor(c) || !c->tensor_ok) return MOP_ERR_UNSUPPORTED;    // the chunked layer runs on the tensor-core kernels only
     return MOP_OK;
 }
 // tables, gathered inputs of chunk i

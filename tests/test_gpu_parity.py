@@ -152,6 +152,22 @@ def test_gathering_forward_refuses_the_scalar_path():
     assert e.value.code == 6
 
 
+@pytest.mark.parametrize("T,d,E,k,f", [(40, 8, 3, 2, 8),            # narrower than one box
+                                       (700, 264, 5, 2, 392),       # one vector past tiles of 256 and of 128
+                                       (333, 200, 4, 1, 136),       # a weight tile whose second chunk is partly, or wholly, outside
+                                       (90, 1000, 7, 3, 1416)],     # the last K block of every GEMM is partly filled
+                         ids=lambda v: str(v))
+def test_widths_that_are_multiples_of_8_only_run_on_the_tensor_cores(T, d, E, k, f):
+    w = synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=f, backward=True, seed=47)
+    ctx, buf = check_layer(w, binding.GEMM_AUTO)
+    binding.mop_profile_enable(ctx)
+    host = synth.make_inputs(w, "cpu")
+    inp = to_dev(host)
+    binding.forward(ctx, inp, buf)
+    binding.backward(ctx, inp, buf)
+    assert not [n for n in binding.mop_profile_read(ctx) if n.startswith("scalar")]
+
+
 @pytest.mark.parametrize("E,k,T,d,f", [(512, 8, 300, 64, 448),     # one K block per item, 27 items per cluster and more
                                        (400, 4, 500, 640, 512),    # 10 K blocks: items announced one ahead
                                        (160, 2, 700, 1600, 1088)],  # 25 K blocks: announced near the end of the one before
