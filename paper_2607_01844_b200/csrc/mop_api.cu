@@ -1060,11 +1060,12 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
                                                                      s.bias_mode));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
-    dim3 gw(ceil_div(s.d, 1024), s.E);
+    dim3 gw(ceil_div(s.d, 256), s.E);
+    const int dwr_w = dwr_warps((long long)gw.x * gw.y, c->sm_count);
     float* db = (dbias_opt && s.bias_mode == MOP_BIAS_PRE_LOGIT) ? dbias_opt : nullptr;
     if (dbias_opt && !db) CUDA_OK(cudaMemsetAsync(dbias_opt, 0, (size_t)s.E * 4, st));
     LAUNCH(c, "route_bwd_dwr", st,
-           route_bwd_dwr_kernel<<<gw, 128, 0, st>>>(static_cast<const bf16*>(Xp), c->dz_row, offsets, dW_r, db, s.d, s.E));
+           route_bwd_dwr_kernel<<<gw, 32 * dwr_w, dwr_w * 1024, st>>>(static_cast<const bf16*>(Xp), c->dz_row, offsets, dW_r, db, s.d, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     if (s.T == 0) return MOP_OK;
     dim3 gt(ceil_div(s.E, 32), ceil_div(s.d, 32));

@@ -811,44 +811,59 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
     }
 }
 
-// dW_r[i,e] = sum over the rows p of expert e (ascending) of Xp[p,i] * dz_row[p].  Block (i-chunk, e):
-// 128 threads, eight columns i each (16-byte loads); Xp rows are read once, coalesced, two rows in
-// flight per thread.  Deterministic (no atomics).
-__global__ void __launch_bounds__(128) route_bwd_dwr_kernel(const bf16* __restrict__ Xp,
-                                                            const float* __restrict__ dz_row,
-                                                            const int32_t* __restrict__ offsets,
-                                                            float* __restrict__ dW_r, float* __restrict__ dbias,
-                                                            int d, int E) {
-    const int e = blockIdx.y;
-    const int i = (blockIdx.x * 128 + threadIdx.x) * 8;
+// dW_r[i,e] = sum over the rows p of expert e of Xp[p,i] * dz_row[p].  Block (256 columns i, e): warp w adds the rows w, w + W,
+// ... of the expert (eight columns per lane, four rows in flight), the W partial sums are added in order through shared memory.
+// Bound by reading Xp once.  With one thread per eight columns walking all rows two at a time (128 threads per 1024 columns)
+// there were too few bytes in flight: 141 us at T = 4096, d = 2048, E = 64, k = 6 and 292 us at T = 4096, d = 1024, E = 32,
+// k = 8; now 28 and 21.  Fixed order, no atomics.
+__global__ void __launch_bounds__(1024) route_bwd_dwr_kernel(const bf16* __restrict__ Xp, const float* __restrict__ dz_row,
+                                                             const int32_t* __restrict__ offsets, float* __restrict__ dW_r,
+                                                             float* __restrict__ dbias, int d, int E) {
+    extern __shared__ float dwr_smem[];                              // [W][256]
+    const int e = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32, W = blockDim.x / 32;
+    const int i = blockIdx.x * 256 + lane * 8;
     const int p0 = offsets[e], p1 = offsets[e + 1];
+    float a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = 0.0f;
     if (i < d) {
-        float a[8];
+        for (int p = p0 + warp; p < p1; p += 4 * W) {
+            uint4 v[4];
+            float w[4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = 0.0f;
-        auto add = [&](const uint4& v, float w) {
-            a[0] = fmaf(bf16_lo(v.x), w, a[0]); a[1] = fmaf(bf16_hi(v.x), w, a[1]);
-            a[2] = fmaf(bf16_lo(v.y), w, a[2]); a[3] = fmaf(bf16_hi(v.y), w, a[3]);
-            a[4] = fmaf(bf16_lo(v.z), w, a[4]); a[5] = fmaf(bf16_hi(v.z), w, a[5]);
-            a[6] = fmaf(bf16_lo(v.w), w, a[6]); a[7] = fmaf(bf16_hi(v.w), w, a[7]);
-        };
-        int p = p0;
-        for (; p + 1 < p1; p += 2) {
-            const uint4 v0 = __ldcs(reinterpret_cast<const uint4*>(Xp + (size_t)p * d + i));
-            const uint4 v1 = __ldcs(reinterpret_cast<const uint4*>(Xp + (size_t)(p + 1) * d + i));
-            add(v0, dz_row[p]);
-            add(v1, dz_row[p + 1]);
+            for (int r = 0; r < 4; ++r) {
+                const int pr = p + r * W;
+                w[r] = pr < p1 ? dz_row[pr] : 0.0f;
+                v[r] = pr < p1 ? __ldcs(reinterpret_cast<const uint4*>(Xp + (size_t)pr * d + i)) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                a[0] = fmaf(bf16_lo(v[r].x), w[r], a[0]); a[1] = fmaf(bf16_hi(v[r].x), w[r], a[1]);
+                a[2] = fmaf(bf16_lo(v[r].y), w[r], a[2]); a[3] = fmaf(bf16_hi(v[r].y), w[r], a[3]);
+                a[4] = fmaf(bf16_lo(v[r].z), w[r], a[4]); a[5] = fmaf(bf16_hi(v[r].z), w[r], a[5]);
+                a[6] = fmaf(bf16_lo(v[r].w), w[r], a[6]); a[7] = fmaf(bf16_hi(v[r].w), w[r], a[7]);
+            }
         }
-        if (p < p1) add(__ldcs(reinterpret_cast<const uint4*>(Xp + (size_t)p * d + i)), dz_row[p]);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) dW_r[(size_t)(i + q) * E + e] = a[q];
     }
-    if (dbias && blockIdx.x == 0 && threadIdx.x == 0) {
+    float* mine = dwr_smem + warp * 256 + lane * 8;
+    *reinterpret_cast<float4*>(mine) = make_float4(a[0], a[1], a[2], a[3]);
+    *reinterpret_cast<float4*>(mine + 4) = make_float4(a[4], a[5], a[6], a[7]);
+    __syncthreads();
+    if (threadIdx.x < 256 && blockIdx.x * 256 + (int)threadIdx.x < d) {
+        float s = 0.0f;
+        for (int w = 0; w < W; ++w) s += dwr_smem[w * 256 + threadIdx.x];
+        dW_r[(size_t)(blockIdx.x * 256 + threadIdx.x) * E + e] = s;
+    }
+    if (dbias && blockIdx.x == 0 && warp == 0) {
         float sb = 0.0f;
-        for (int p = p0; p < p1; ++p) sb += dz_row[p];
-        dbias[e] = sb;
+        for (int p = p0 + lane; p < p1; p += 32) sb += dz_row[p];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sb += __shfl_xor_sync(0xffffffffu, sb, off);
+        if (lane == 0) dbias[e] = sb;
     }
 }
+// Warps per block: enough to keep 16 warps and more on every SM (8 warps leave the other blocks room where there are many).
+inline int dwr_warps(long long blocks, int sm_count) { return blocks >= 4ll * sm_count ? 8 : blocks >= 2ll * sm_count ? 16 : 32; }
 
 // W_r^T [E,d] from W_r [d,E] (32 x 32 tiles through shared memory): gives the dX kernel contiguous rows.
 __global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, float* __restrict__ out,
