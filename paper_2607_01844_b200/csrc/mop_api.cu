@@ -305,6 +305,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         return MOP_ERR_UNSUPPORTED;
     }
     c->tensor_tn = shape->gemm_path != MOP_GEMM_SCALAR && (c->tensor_ok || (prop.major == 10 && c->sm_count >= 2));
+    if (!route_score_init()) { delete c; return MOP_ERR_CUDA; }
     const Layout L = make_layout(*shape);
     c->ws_bytes = L.total;
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }

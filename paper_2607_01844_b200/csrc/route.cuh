@@ -9,17 +9,20 @@ namespace mop {
 // Scoring.  z[t,e] = sum_i x[t,i] * W_r[i,e] as ONE chain of fused multiply-adds per (t,e), i
 // ascending, each step rounded once to fp32.  The chain order is part of the routing contract
 // (it makes top-k indices reproducible bit for bit), so there is no split over i and no tensor
-// core here; parallelism comes from the T*E independent chains and the kernel is bound by the
-// fp32 pipes.  Each thread owns RT tokens x RE experts (RT*RE chains) and advances two chains
-// per instruction with the packed fma.rn.f32x2 of sm_100 (two independent IEEE fused
-// multiply-adds: the rounding of each chain is unchanged).  A 128-thread CTA covers
-// (16 RT) tokens x (8 RE) experts; operands are staged through shared memory in slabs of 16 or 32
-// along i, double-buffered, the next slab prefetched into registers while the current one is
-// multiplied.  <8,8> needs 4 shared loads per 64 FMAs; smaller tiles trade that for more CTAs
-// when T*E is small.  Both slabs are laid out so that every shared access of a warp is free of
-// bank conflicts (interleaved expert columns, XOR-swizzled token columns).
+// core here; parallelism comes from the T*E independent chains.  Each thread owns RT tokens x RE
+// experts; with several experts it advances two chains (experts e, e + 1) per instruction with the
+// packed fma.rn.f32x2 of sm_100 (two independent IEEE fused multiply-adds: the rounding of each chain is unchanged).
+//
+// What bounds it: the fp32 pipes and shared memory where there are many chains, the latency of a dependent multiply-add where
+// there are few.  Either way the operands must not be waited for: stages of 64 steps are copied by cp.async two or three
+// stages ahead (x as bf16, W_r as fp32).  With one slab of 32 steps ahead in registers every slab cost a trip to L2: 48
+// cycles a step at T = 4096, d = 2048, E = 64.
+// A warp covers LT RT tokens x (32 / LT) RE experts, a block of four warps four times the tokens; the shape is picked by
+// route_score() from the number of blocks per SM and the cycles of a step.
 // ---------------------------------------------------------------------------------------------
 constexpr int SC_THREADS = 128;
+constexpr int SC_TK = 64;          // steps per stage
+constexpr int SC_XPITCH = SC_TK + 8;   // bf16 elements: neighbouring tokens' rows 16 bytes apart in the banks
 
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
     unsigned long long r;
@@ -33,161 +36,202 @@ __device__ __forceinline__ void fma_f32x2(unsigned long long& acc, unsigned long
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-template <int RT, int RE, int SC_TK>
-__global__ void __launch_bounds__(SC_THREADS, 4) route_score_kernel(const bf16* __restrict__ x,
-                                                                 const float* __restrict__ W_r,
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+
+template <int RT, int RE, int LT>
+struct ScoreShape {
+    static constexpr int LE = 32 / LT;
+    static constexpr int TT = 4 * LT * RT, TE = LE * RE;
+    static constexpr int X_BYTES = TT * SC_XPITCH * 2, W_BYTES = SC_TK * TE * 4, STAGE = X_BYTES + W_BYTES;
+    static constexpr int STAGES = RT * RE >= 32 ? 3 : 4;
+    static constexpr int SMEM = STAGES * STAGE;
+};
+
+template <int RT, int RE, int LT>
+__global__ void __launch_bounds__(SC_THREADS) route_score_kernel(const bf16* __restrict__ x, const float* __restrict__ W_r,
                                                                  float* __restrict__ z, int T, int d, int E) {
-    constexpr int TT = 16 * RT, TE = 8 * RE;          // CTA tile
-    constexpr int LDX = TT + 4, LDW = TE + 4;
-    constexpr int XV = TT * SC_TK / 8 / SC_THREADS;   // 16-byte x vectors fetched per thread per slab
-    constexpr int WV = TE * SC_TK / 4 / SC_THREADS;   // float4 W vectors per thread per slab
-    static_assert(RT % 2 == 0 && RE % 4 == 0 && XV >= 1 && WV >= 1, "tile shape");
-    __shared__ __align__(16) float xs[2][SC_TK][LDX];
-    __shared__ __align__(16) float ws[2][SC_TK][LDW];
+    using Sh = ScoreShape<RT, RE, LT>;
+    constexpr int LE = Sh::LE, TT = Sh::TT, TE = Sh::TE, S = Sh::STAGES;
+    static_assert(RE == 1 || (RE % 4 == 0 && LE == 8), "expert columns of a thread: one, or groups of four 32 apart");
+    static_assert(Sh::X_BYTES % 16 == 0 && Sh::STAGE % 16 == 0, "16-byte copies");
+    extern __shared__ __align__(16) uint8_t sc_smem[];
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sc_smem);
     const int t0 = blockIdx.x * TT, e0 = blockIdx.y * TE;
-    const int tid = threadIdx.x;
-    // Expert columns of a thread: groups of 4 at te + 32 b, so that the 8 threads that differ in
-    // tid % 8 read 32 consecutive floats (one conflict-free wavefront) per group.
-    const int tt = (tid / 8) * RT, te = (tid % 8) * 4;
-    constexpr int EG = (RE > 4) ? 32 : 4;             // column pitch between a thread's groups of 4
-    // Token columns of the x slab are XOR-swizzled by the 8-row chunk of i they belong to: the
-    // threads of a warp that stash different chunks of the same tokens then hit different banks.
-    constexpr int CH = SC_TK / 8, SWZ = 32 / CH;
-    static_assert(TT >= 32 && (SWZ % 4) == 0, "swizzle keeps float4 groups intact and stays inside the tile");
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    // Tokens of a thread: tt, tt + LT, ..  Lanes of a quarter warp share few addresses of both operands: a vector load whose
+    // quarters each read the same 128 bytes costs four wavefronts, one whose quarters read different ones together costs one.
+    const int tt = warp * LT * RT + (RE == 1 ? lane / LE : lane % LT);
+    const int te = RE == 1 ? lane % LE : (lane / LT) * 4;           // first expert; further groups of four 32 apart
     const bool w_vec = (E % 4 == 0);
 
-    unsigned long long acc[RT / 2][RE];   // acc[a][b] = chains of tokens (2a, 2a+1) for expert b
+    auto load = [&](int s, int i0) {
+        const uint32_t xb = base + s * Sh::STAGE, wb = xb + Sh::X_BYTES;
 #pragma unroll
-    for (int a = 0; a < RT / 2; ++a)
-#pragma unroll
-        for (int b = 0; b < RE; ++b) acc[a][b] = 0ull;
-
-    uint4 xr[XV];
-    float4 wr[WV];
-    // x slab: TT tokens x SC_TK i, vector v of a thread = token lin / (SC_TK/8), i offset (lin % (SC_TK/8)) * 8
-    auto fetch = [&](int i0) {
-#pragma unroll
-        for (int v = 0; v < XV; ++v) {
-            const int lin = v * SC_THREADS + tid;
-            const int t = t0 + lin / (SC_TK / 8), i = i0 + (lin % (SC_TK / 8)) * 8;
-            xr[v] = (t < T && i < d) ? *reinterpret_cast<const uint4*>(x + (size_t)t * d + i) : make_uint4(0, 0, 0, 0);
+        for (int v = tid; v < TT * (SC_TK / 8); v += SC_THREADS) {  // 16 bytes = 8 steps of one token
+            const int t = v / (SC_TK / 8), c = (v % (SC_TK / 8)) * 8;
+            const bool ok = t0 + t < T && i0 + c < d;
+            cp_async16(xb + (t * SC_XPITCH + c) * 2, ok ? x + (size_t)(t0 + t) * d + i0 + c : x, ok);
         }
+        if (w_vec) {
 #pragma unroll
-        for (int v = 0; v < WV; ++v) {
-            const int lin = v * SC_THREADS + tid;
-            const int i = i0 + lin / (TE / 4), e = e0 + (lin % (TE / 4)) * 4;
-            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i < d) {
-                const float* src = W_r + (size_t)i * E + e;
-                if (w_vec && e + 3 < E) q = *reinterpret_cast<const float4*>(src);
-                else {
-                    if (e < E) q.x = src[0];
-                    if (e + 1 < E) q.y = src[1];
-                    if (e + 2 < E) q.z = src[2];
-                    if (e + 3 < E) q.w = src[3];
+            for (int v = tid; v < SC_TK * TE / 4; v += SC_THREADS) {
+                const int i = v / (TE / 4), e = (v % (TE / 4)) * 4;
+                const bool ok = i0 + i < d && e0 + e < E;
+                cp_async16(wb + (i * TE + e) * 4, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
+            }
+        } else if (E % 2 == 0) {
+#pragma unroll 4
+            for (int v = tid; v < SC_TK * TE / 2; v += SC_THREADS) {
+                const int i = v / (TE / 2), e = (v % (TE / 2)) * 2;
+                const bool ok = i0 + i < d && e0 + e < E;
+                cp_async8(wb + v * 8, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
+            }
+        } else {
+#pragma unroll 4
+            for (int v = tid; v < SC_TK * TE; v += SC_THREADS) {
+                const int i = v / TE, e = v % TE;
+                const bool ok = i0 + i < d && e0 + e < E;
+                cp_async4(wb + v * 4, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int stages = (d + SC_TK - 1) / SC_TK;
+#pragma unroll
+    for (int s = 0; s < S - 1; ++s) {
+        if (s < stages) load(s, s * SC_TK);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    constexpr int G = RT * RE >= 32 ? 4 : 8;                        // steps whose operands are in registers
+    constexpr int NP = RE == 1 ? 1 : RE / 2;                        // pairs of experts (RE = 1: a plain chain)
+    unsigned long long acc[RT][NP];
+    float acc1[RT];
+#pragma unroll
+    for (int a = 0; a < RT; ++a) {
+        acc1[a] = 0.0f;
+#pragma unroll
+        for (int b = 0; b < NP; ++b) acc[a][b] = 0ull;
+    }
+    for (int st = 0; st < stages; ++st) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+        __syncthreads();          // stage st has arrived for every thread, and stage st - 1 has been read by every thread
+        if (st + S - 1 < stages) load((st + S - 1) % S, (st + S - 1) * SC_TK);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        const uint8_t* sx = sc_smem + (st % S) * Sh::STAGE;
+        const bf16* xs = reinterpret_cast<const bf16*>(sx) + tt * SC_XPITCH;
+        const float* ws = reinterpret_cast<const float*>(sx + Sh::X_BYTES) + te;
+        // Steps past d (d not a multiple of a stage) multiply zeros: fma(0, 0, acc) = acc, exact.  Operands of the next G steps
+        // are read while the current ones are multiplied.
+        uint32_t xv[2][RT][G / 2];
+        float wv[2][G][RE];
+        auto fetch = [&](int buf, int k) {
+#pragma unroll
+            for (int a = 0; a < RT; ++a) {
+                if constexpr (G == 8) {
+                    const uint4 q = *reinterpret_cast<const uint4*>(xs + a * LT * SC_XPITCH + k);
+                    xv[buf][a][0] = q.x; xv[buf][a][1] = q.y; xv[buf][a][2] = q.z; xv[buf][a][3] = q.w;
+                } else {
+                    const uint2 q = *reinterpret_cast<const uint2*>(xs + a * LT * SC_XPITCH + k);
+                    xv[buf][a][0] = q.x; xv[buf][a][1] = q.y;
                 }
             }
-            wr[v] = q;
-        }
-    };
-    auto stash = [&](int buf) {
 #pragma unroll
-        for (int v = 0; v < XV; ++v) {
-            const int lin = v * SC_THREADS + tid;
-            const int tok = lin / (SC_TK / 8), ii = (lin % (SC_TK / 8)) * 8;
-            const uint32_t w4[4] = {xr[v].x, xr[v].y, xr[v].z, xr[v].w};
+            for (int j = 0; j < G; ++j) {
+                if constexpr (RE == 1) wv[buf][j][0] = ws[(k + j) * TE];
+                else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                xs[buf][ii + 2 * q][tok ^ ((ii / 8) * SWZ)] = bf16_lo(w4[q]);
-                xs[buf][ii + 2 * q + 1][tok ^ ((ii / 8) * SWZ)] = bf16_hi(w4[q]);
+                    for (int b = 0; b < RE / 4; ++b) {
+                        const float4 v = *reinterpret_cast<const float4*>(ws + (k + j) * TE + 32 * b);
+                        wv[buf][j][4 * b] = v.x; wv[buf][j][4 * b + 1] = v.y; wv[buf][j][4 * b + 2] = v.z; wv[buf][j][4 * b + 3] = v.w;
+                    }
+                }
             }
+        };
+        fetch(0, 0);
+#pragma unroll
+        for (int k = 0; k < SC_TK; k += G) {
+            const int cur = (k / G) & 1;
+            if (k + G < SC_TK) fetch(cur ^ 1, k + G);
+#pragma unroll
+            for (int j = 0; j < G; ++j)
+#pragma unroll
+                for (int a = 0; a < RT; ++a) {
+                    const float x1 = (j & 1) ? bf16_hi(xv[cur][a][j >> 1]) : bf16_lo(xv[cur][a][j >> 1]);
+                    if constexpr (RE == 1) acc1[a] = __fmaf_rn(x1, wv[cur][j][0], acc1[a]);
+                    else {
+                        const unsigned long long xp = pack_f32x2(x1, x1);
+#pragma unroll
+                        for (int b = 0; b < NP; ++b) fma_f32x2(acc[a][b], xp, pack_f32x2(wv[cur][j][2 * b], wv[cur][j][2 * b + 1]));
+                    }
+                }
         }
+    }
 #pragma unroll
-        for (int v = 0; v < WV; ++v) {
-            const int lin = v * SC_THREADS + tid;
-            *reinterpret_cast<float4*>(&ws[buf][lin / (TE / 4)][(lin % (TE / 4)) * 4]) = wr[v];
-        }
-    };
-
-    fetch(0);
-    stash(0);
-    __syncthreads();
-    int buf = 0;
-    for (int i0 = 0; i0 < d; i0 += SC_TK) {
-        const bool more = i0 + SC_TK < d;
-        if (more) fetch(i0 + SC_TK);
-        // Past-the-end i (d not a multiple of the slab) multiplies zeros: fma(0, 0, acc) = acc, exact.
-#pragma unroll
-        for (int kk = 0; kk < SC_TK; ++kk) {
-            unsigned long long xp[RT / 2], wp[RE];
-#pragma unroll
-            for (int a = 0; a < RT / 4; ++a) {
-                const float4 v = *reinterpret_cast<const float4*>(&xs[buf][kk][(tt + 4 * a) ^ ((kk / 8) * SWZ)]);
-                xp[2 * a] = pack_f32x2(v.x, v.y);
-                xp[2 * a + 1] = pack_f32x2(v.z, v.w);
-            }
-            if constexpr (RT % 4 == 2) {
-                const float2 v = *reinterpret_cast<const float2*>(&xs[buf][kk][(tt + RT - 2) ^ ((kk / 8) * SWZ)]);
-                xp[RT / 2 - 1] = pack_f32x2(v.x, v.y);
-            }
+    for (int a = 0; a < RT; ++a) {
+        const int t = t0 + tt + LT * a;
+        if (t >= T) continue;
+        if constexpr (RE == 1) {
+            if (e0 + te < E) z[(size_t)t * E + e0 + te] = acc1[a];
+        } else {
 #pragma unroll
             for (int b = 0; b < RE / 4; ++b) {
-                const float4 v = *reinterpret_cast<const float4*>(&ws[buf][kk][te + EG * b]);
-                wp[4 * b] = pack_f32x2(v.x, v.x);
-                wp[4 * b + 1] = pack_f32x2(v.y, v.y);
-                wp[4 * b + 2] = pack_f32x2(v.z, v.z);
-                wp[4 * b + 3] = pack_f32x2(v.w, v.w);
-            }
-#pragma unroll
-            for (int a = 0; a < RT / 2; ++a)
-#pragma unroll
-                for (int b = 0; b < RE; ++b) fma_f32x2(acc[a][b], xp[a], wp[b]);
-        }
-        if (more) stash(buf ^ 1);
-        __syncthreads();
-        buf ^= 1;
-    }
-#pragma unroll
-    for (int a = 0; a < RT / 2; ++a) {
-        float lo[RE], hi[RE];
-#pragma unroll
-        for (int b = 0; b < RE; ++b) unpack_f32x2(acc[a][b], lo[b], hi[b]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int t = t0 + tt + 2 * a + h;
-            if (t >= T) continue;
-#pragma unroll
-            for (int b = 0; b < RE; b += 4) {
-                const float v0 = h ? hi[b] : lo[b], v1 = h ? hi[b + 1] : lo[b + 1];
-                const float v2 = h ? hi[b + 2] : lo[b + 2], v3 = h ? hi[b + 3] : lo[b + 3];
-                const int e = e0 + te + EG * (b / 4);
+                float v[4];
+                unpack_f32x2(acc[a][2 * b], v[0], v[1]);
+                unpack_f32x2(acc[a][2 * b + 1], v[2], v[3]);
+                const int e = e0 + te + 32 * b;
                 float* dst = z + (size_t)t * E + e;
                 if (w_vec && e + 3 < E) {
-                    *reinterpret_cast<float4*>(dst) = make_float4(v0, v1, v2, v3);
+                    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
-                    if (e < E) dst[0] = v0;
-                    if (e + 1 < E) dst[1] = v1;
-                    if (e + 2 < E) dst[2] = v2;
-                    if (e + 3 < E) dst[3] = v3;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (e + q < E) dst[q] = v[q];
                 }
             }
         }
     }
 }
 
-// Tile choice: the largest tile that still gives every SM a few CTAs.
-template <int RT, int RE, int TK>
-inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, cudaStream_t st) {
-    dim3 grid(ceil_div(T, 16 * RT), ceil_div(E, 8 * RE));
-    route_score_kernel<RT, RE, TK><<<grid, SC_THREADS, 0, st>>>(x, W_r, z, T, d, E);
+template <int RT, int RE, int LT>
+inline bool route_score_attr() {
+    return cudaFuncSetAttribute(route_score_kernel<RT, RE, LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                ScoreShape<RT, RE, LT>::SMEM) == cudaSuccess;
 }
-inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int sm_count,
-                        cudaStream_t st) {
-    const long long big = (long long)ceil_div(T, 128) * ceil_div(E, 64);
-    const long long mid = (long long)ceil_div(T, 64) * ceil_div(E, 32);
-    if (big >= 2ll * sm_count) launch_route_score<8, 8, 16>(x, W_r, z, T, d, E, st);
-    else if (2 * mid >= sm_count) launch_route_score<4, 4, 32>(x, W_r, z, T, d, E, st);
-    else launch_route_score<2, 4, 32>(x, W_r, z, T, d, E, st);
+inline bool route_score_init() {
+    return route_score_attr<1, 1, 4>() && route_score_attr<2, 4, 4>() && route_score_attr<4, 4, 4>() &&
+           route_score_attr<4, 8, 4>();
+}
+template <int RT, int RE, int LT>
+inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, cudaStream_t st) {
+    using Sh = ScoreShape<RT, RE, LT>;
+    dim3 grid(ceil_div(T, Sh::TT), ceil_div(E, Sh::TE));
+    route_score_kernel<RT, RE, LT><<<grid, SC_THREADS, Sh::SMEM, st>>>(x, W_r, z, T, d, E);
+}
+// Shape choice: the least estimated cycles per step on the fullest SM, first + more * (blocks on it - 1), as measured at
+// d = 7168 (one block alone on an SM; each further one).  Decoding (T = 64, E = 256) takes one chain per thread: 130 us with the
+// former slabs, 46 now, 136 with 4 x 4; T = 4096, d = 2048, E = 64 takes 4 x 4: 50 -> 44 us, 97 with one chain per thread;
+// T = 8192, d = 7168, E = 128 takes 4 x 8: 472 -> 370 us, 415 with 4 x 4.
+inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int sm_count, cudaStream_t st) {
+    const struct { int tt, te; float first, more; } shape[4] = {{16, 8, 12.f, 6.f}, {32, 32, 28.f, 15.f}, {64, 32, 36.5f, 26.f}, {64, 64, 55.5f, 45.f}};
+    int pick = 0;
+    float best = 0.0f;
+    for (int i = 0; i < 4; ++i) {
+        const long long blocks = (long long)ceil_div(T, shape[i].tt) * ceil_div(E, shape[i].te);
+        const float cost = shape[i].first + shape[i].more * (float)((blocks + sm_count - 1) / sm_count - 1);
+        if (i == 0 || cost <= best) { best = cost; pick = i; }
+    }
+    if (pick == 0) launch_route_score<1, 1, 4>(x, W_r, z, T, d, E, st);
+    else if (pick == 1) launch_route_score<2, 4, 4>(x, W_r, z, T, d, E, st);
+    else if (pick == 2) launch_route_score<4, 4, 4>(x, W_r, z, T, d, E, st);
+    else launch_route_score<4, 8, 4>(x, W_r, z, T, d, E, st);
 }
 
 // Sigmoid of the routing contract: a fixed sequence of fp32 operations, each rounded once

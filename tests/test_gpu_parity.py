@@ -523,6 +523,26 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     check_integers(w, host, buf)
 
 
+@pytest.mark.parametrize("T,d,E", [(17, 72, 9), (16, 64, 8),          # one chain per thread, tile edges of 16 x 8
+                                   (4100, 136, 33), (4096, 64, 64),    # 32 x 32 and 64 x 32 tiles, W rows at every alignment
+                                   (9000, 200, 34), (12000, 72, 127), (8200, 64, 260)])   # 64 x 64 tiles
+def test_exact_scoring_shapes_give_the_contract_chains(T, d, E):
+    w = synth.small("c2_mid", T=T, d=d, E=E, k=2, f=64, seed=48)
+    inp = synth.make_inputs(w, "cuda")
+    ctx = binding.context_for(w, route_path=binding.ROUTE_EXACT)
+    buf = binding.LayerBuffers(w)
+    z = torch.empty((T, E), dtype=torch.float32, device="cuda")
+    binding.mop_moe_route(ctx, inp["x"], inp["W_r"], None, buf.idx, buf.gate, z)
+    acc = torch.zeros((T, E), dtype=torch.float64, device="cuda")
+    for i in range(d):     # one fp32 rounding per step: the product of a bf16 and an fp32 number and the sum are exact enough in fp64
+        acc = (acc + inp["x"][:, i:i + 1].double() * inp["W_r"][i].double()).float().double()
+    # (a sum that fp64 rounds onto an fp32 tie is the only way to differ: at most a handful of last bits)
+    differ = z.double() != acc
+    assert int(differ.sum()) <= 1e-6 * z.numel() + 1 and torch.allclose(z.double(), acc, rtol=1e-6, atol=1e-6)
+    idx, _ = oracle.route(synth.bits(inp["x"][:300]), inp["W_r"].cpu().numpy(), None, 2, w.score_fn, w.bias_mode)
+    assert np.array_equal(buf.idx[:300].cpu().numpy(), idx[:300])
+
+
 FAST_ROUTE = [
     synth.small("c3_trillion", T=1000, d=512, E=256, k=8, f=64, seed=60),                  # sigmoid + post-score bias
     synth.small("c3_trillion", T=777, d=320, E=64, k=3, f=64, bias_mode=2, seed=61),        # sigmoid, bias before the score
