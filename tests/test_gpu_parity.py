@@ -460,6 +460,14 @@ def test_router_backward_matches_oracle(w):
     assert rel_fro(got, want) < 4e-3
 
 
+@pytest.mark.parametrize("T,d,E,k", [(100, 328, 160, 4),      # 16 warps per block of dW_r, the last block of columns partly filled
+                                     (150, 264, 300, 3),      # 8 warps, experts with fewer rows than warps
+                                     (900, 264, 300, 7)],     # 8 warps, more rows than four per warp
+                         ids=lambda v: str(v))
+def test_router_backward_with_many_blocks_matches_oracle(T, d, E, k):
+    test_router_backward_matches_oracle(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=64, bias_mode=2, backward=True, seed=34))
+
+
 def test_backward_with_recomputation_equals_backward_with_stash():
     """Activation checkpointing: forward without the G, U stash, backward recomputes them from Xp."""
     w = synth.small("c2_mid", T=700, d=256, E=10, k=3, f=192, backward=True, seed=40)
