@@ -198,6 +198,13 @@ mop_status mop_moe_expert_ffn_bwd(mop_ctx* ctx, const void* dY, const void* Xp, 
                                   const void* W_up, const void* W_down, void* dX, float* dW_gate, float* dW_up,
                                   float* dW_down, float* dgate, void* stream);
 
+/* One forward of the layer: mop_moe_route, mop_moe_permute, mop_moe_expert_ffn_fwd and mop_moe_combine on the same
+ * arguments, in one call (a small layer is bound by the caller's side of its launches).  logits are not returned. */
+mop_status mop_moe_layer_fwd(mop_ctx* ctx, const void* x, const float* W_r, const float* bias, const void* W_gate,
+                             const void* W_up, const void* W_down, int32_t* topk_idx, float* topk_gate, int32_t* counts,
+                             int32_t* offsets, int32_t* perm_row, int32_t* row_src, void* Xp, void* G_save, void* U_save,
+                             void* H, void* Yp, void* Y, void* stream);
+
 /* Expert-chunked layer: the memory-lean form of Section 3.3, where only a fraction of the routed buffers is
  * resident at any instant (the O(N k H + N_r I) activation term of Eq. 4 shrinks to one chunk of it).  The
  * experts are cut into n_chunks groups of about T k / n_chunks rows each (a group ends at an expert boundary, so

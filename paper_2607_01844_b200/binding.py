@@ -63,6 +63,7 @@ def lib() -> ctypes.CDLL:
         L.mop_moe_expert_ffn_fwd.argtypes = [_P] * 13
         L.mop_moe_expert_ffn_fwd_gather.argtypes = [_P] * 11
         L.mop_moe_combine.argtypes = [_P] * 5
+        L.mop_moe_layer_fwd.argtypes = [_P] * 20
         L.mop_moe_expert_ffn_bwd.argtypes = [_P] * 19
         L.mop_moe_forward_host.argtypes = [_P] * 11
         L.mop_moe_forward_host_async.argtypes = [_P] * 11
@@ -102,7 +103,8 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle without building a Stream object around it (3 us of a small layer's 50)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -200,6 +202,16 @@ def mop_moe_expert_ffn_fwd_gather(ctx, x, offsets, row_src, topk_gate, W_gate, W
 
 def mop_moe_combine(ctx, Yp, perm_row, Y, stream=None):
     _check("mop_moe_combine", lib().mop_moe_combine(ctx.handle, _ptr(Yp), _ptr(perm_row), _ptr(Y), _stream(stream)))
+
+
+def mop_moe_layer_fwd(ctx, x, W_r, bias, W_gate, W_up, W_down, topk_idx, topk_gate, counts, offsets, perm_row, row_src, Xp,
+                      G_save, U_save, H, Yp, Y, stream=None):
+    """route, permute, expert_ffn_fwd and combine in one call."""
+    _check("mop_moe_layer_fwd",
+           lib().mop_moe_layer_fwd(ctx.handle, _ptr(x), _ptr(W_r), _ptr(bias), _ptr(W_gate), _ptr(W_up), _ptr(W_down),
+                                   _ptr(topk_idx), _ptr(topk_gate), _ptr(counts), _ptr(offsets), _ptr(perm_row),
+                                   _ptr(row_src), _ptr(Xp), _ptr(G_save), _ptr(U_save), _ptr(H), _ptr(Yp), _ptr(Y),
+                                   _stream(stream)))
 
 
 def mop_moe_expert_ffn_bwd(ctx, dY, Xp, G_save, U_save, H, offsets, perm_row, row_src, topk_gate, W_gate, W_up,
@@ -378,18 +390,16 @@ class LayerBuffers:
 
 def forward(ctx, inp, buf, stream=None, gather=False):
     """route -> permute -> expert_ffn_fwd -> combine on device tensors (one pass of the forward path)."""
-    mop_moe_route(ctx, inp["x"], inp["W_r"], inp["bias"], buf.idx, buf.gate, None, stream)
     if gather:
+        mop_moe_route(ctx, inp["x"], inp["W_r"], inp["bias"], buf.idx, buf.gate, None, stream)
         # inference form: no expert-contiguous copy of x, no stash
         mop_moe_permute(ctx, None, buf.idx, buf.counts, buf.offsets, buf.perm_row, buf.row_src, None, stream)
         mop_moe_expert_ffn_fwd_gather(ctx, inp["x"], buf.offsets, buf.row_src, buf.gate, inp["W_gate"], inp["W_up"],
                                       inp["W_down"], buf.H, buf.Yp, stream)
         mop_moe_combine(ctx, buf.Yp, buf.perm_row, buf.Y, stream)
         return
-    mop_moe_permute(ctx, inp["x"], buf.idx, buf.counts, buf.offsets, buf.perm_row, buf.row_src, buf.Xp, stream)
-    mop_moe_expert_ffn_fwd(ctx, buf.Xp, buf.offsets, buf.row_src, buf.gate, inp["W_gate"], inp["W_up"], inp["W_down"],
-                           buf.G, buf.U, buf.H, buf.Yp, stream)
-    mop_moe_combine(ctx, buf.Yp, buf.perm_row, buf.Y, stream)
+    mop_moe_layer_fwd(ctx, inp["x"], inp["W_r"], inp["bias"], inp["W_gate"], inp["W_up"], inp["W_down"], buf.idx, buf.gate,
+                      buf.counts, buf.offsets, buf.perm_row, buf.row_src, buf.Xp, buf.G, buf.U, buf.H, buf.Yp, buf.Y, stream)
 
 
 def backward(ctx, inp, buf, stream=None):

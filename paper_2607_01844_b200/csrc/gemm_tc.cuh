@@ -407,6 +407,7 @@ __device__ __forceinline__ void tc_build_mtiles_body(const int32_t* __restrict__
 __global__ void __launch_bounds__(1024) tc_build_mtiles_kernel(const int32_t* __restrict__ offsets, int E,
                                                                int4* __restrict__ mtiles,
                                                                int32_t* __restrict__ n_mtiles) {
+    pdl_begin();
     __shared__ int32_t scan[1025];
     tc_build_mtiles_body(offsets, E, mtiles, n_mtiles, scan);
 }
@@ -563,6 +564,7 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    pdl_begin();
 
     int total_tiles;
     if constexpr (Tr::RAGGED_K) total_tiles = args.E * args.tiles_m_fixed * args.tiles_n;
@@ -1039,8 +1041,7 @@ inline mop_status tc_launch(const TcPlan* p, const char* name, const CUtensorMap
                             const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& o0, const CUtensorMap& o1,
                             const TcArgs& args, cudaStream_t st) {
     p->prof->begin(name, st);
-    tc_grouped_gemm_kernel<KIND><<<p->sm_count, TcTraits<KIND>::THREADS, TcTraits<KIND>::SMEM_BYTES, st>>>(
-        a0, a1, b0, b1, o0, o1, args);
+    pdl_launch(tc_grouped_gemm_kernel<KIND>, p->sm_count, TcTraits<KIND>::THREADS, TcTraits<KIND>::SMEM_BYTES, st, a0, a1, b0, b1, o0, o1, args);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
@@ -1057,7 +1058,7 @@ inline TcArgs tc_base_args(const TcPlan* p, const int32_t* offsets, int32_t* til
 
 inline mop_status tc_build_tiles(const TcPlan* p, const int32_t* offsets, int32_t* tiles, cudaStream_t st) {
     p->prof->begin("tc_build_mtiles", st);
-    tc_build_mtiles_kernel<<<1, 1024, 0, st>>>(offsets, p->s.E, reinterpret_cast<int4*>(tiles + 64), tiles);
+    pdl_launch(tc_build_mtiles_kernel, 1, 1024, 0, st, offsets, p->s.E, reinterpret_cast<int4*>(tiles + 64), tiles);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

@@ -96,6 +96,7 @@ __device__ __forceinline__ void tn_build_ttiles_body(const int32_t* __restrict__
 // tokens-on-M kernels (where a forward or backward uses both).
 __global__ void __launch_bounds__(1024) tn_build_ttiles_kernel(const int32_t* __restrict__ offsets, int E, int32_t* __restrict__ ttiles,
                                                                int32_t* __restrict__ mtiles) {
+    pdl_begin();
     __shared__ int32_t scan[1025];
     if (blockIdx.x == 0) tn_build_ttiles_body(offsets, E, reinterpret_cast<int4*>(ttiles + 64), ttiles, scan);
     else tc_build_mtiles_body(offsets, E, reinterpret_cast<int4*>(mtiles + 64), mtiles, scan);
@@ -261,6 +262,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    pdl_begin();
 
     const int total_tiles = (*args.n_ttiles) * args.tiles_m;
     const int nkb = (KIND == TN_B4 ? 2 : 1) * args.kblocks;   // K blocks per tile (B4: two phases)
@@ -678,7 +680,7 @@ inline int32_t* tn_table(const TcPlan* p, int32_t* tiles) {
 }
 inline mop_status tn_build_tiles(TcPlan* p, const int32_t* offsets, int32_t* tiles, bool rows128, cudaStream_t st) {
     p->prof->begin("tn_build_ttiles", st);
-    tn_build_ttiles_kernel<<<rows128 ? 2 : 1, 1024, 0, st>>>(offsets, p->s.E, tn_table(p, tiles), tiles);
+    pdl_launch(tn_build_ttiles_kernel, rows128 ? 2 : 1, 1024, 0, st, offsets, p->s.E, tn_table(p, tiles), tiles);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
@@ -706,7 +708,7 @@ inline bool tn_token_maps(const TcPlan* p, CUtensorMap* m, const void* base, uin
 template <int KIND>
 inline mop_status tn_launch(const TcPlan* p, const char* name, const TnMaps& m, const TnArgs& g, cudaStream_t st) {
     p->prof->begin(name, st);
-    tn_gemm_kernel<KIND><<<p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st>>>(m, g);
+    pdl_launch(tn_gemm_kernel<KIND>, p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st, m, g);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

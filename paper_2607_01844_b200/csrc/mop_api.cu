@@ -578,8 +578,7 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
     if (r != MOP_OK) return r;
     const size_t smem = (size_t)SEL_WARPS * 2 * s.E * sizeof(float);
     LAUNCH(c, "route_select", st,
-           route_select_kernel<<<ceil_div(s.T, SEL_WARPS), SEL_WARPS * 32, smem, st>>>(
-               z, bias, topk_idx, topk_gate, s.T, s.E, s.k, s.score_fn, s.bias_mode));
+           pdl_launch(route_select_kernel, ceil_div(s.T, SEL_WARPS), SEL_WARPS * 32, smem, st, z, bias, topk_idx, topk_gate, s.T, s.E, s.k, s.score_fn, s.bias_mode));
     return after_launch(c);
 }
 
@@ -617,27 +616,25 @@ mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, i
     mop_status r;
     if (perm_small_fits(units, s.E)) {   // a few units: one block does histogram, scan and rank
         LAUNCH(c, "perm_small", st,
-               perm_small_kernel<<<1, 1024, ((size_t)units * s.E + s.E + 1) * sizeof(int32_t), st>>>(
-                   topk_idx, counts, offsets, perm_row, row_src, M, s.E, units));
+               pdl_launch(perm_small_kernel, 1, 1024, ((size_t)units * s.E + s.E + 1) * sizeof(int32_t), st, topk_idx, counts, offsets, perm_row, row_src, M, s.E, units));
         if ((r = after_launch(c)) != MOP_OK) return r;
     } else {
     if (units > 0) {
         LAUNCH(c, "perm_hist", st,
-               perm_hist_kernel<<<ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st>>>(topk_idx, c->partial, M,
+               pdl_launch(perm_hist_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st, topk_idx, c->partial, M,
                                                                                             s.E));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     if (units == 0) {   // nothing to permute: counts and offsets are all zero
         LAUNCH(c, "perm_scan", st,
-               perm_scan_kernel<<<1, 1024, (s.E + 1) * sizeof(int32_t), st>>>(c->partial, counts, offsets, units, s.E));
+               pdl_launch(perm_scan_kernel, 1, 1024, (s.E + 1) * sizeof(int32_t), st, c->partial, counts, offsets, units, s.E));
         return after_launch(c);
     }
     LAUNCH(c, "perm_scan", st,
-           perm_scan_cols_kernel<<<ceil_div(s.E, 32), PSCAN_WARPS * 32, 0, st>>>(c->partial, counts, units, s.E));
+           pdl_launch(perm_scan_cols_kernel, ceil_div(s.E, 32), PSCAN_WARPS * 32, 0, st, c->partial, counts, units, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     LAUNCH(c, "perm_rank", st,
-           perm_rank_kernel<<<ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st>>>(
-               topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
+           pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st, topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     }
     if (!Xp) return MOP_OK;
@@ -834,9 +831,21 @@ mop_status mop_moe_expert_ffn_bwd(mop_ctx* c, const void* dY, const void* Xp, co
     }
     if (s.T == 0) return MOP_OK;
     LAUNCH(c, "dgate_reduce", st,
-           dgate_reduce_kernel<<<ceil_div(M, 256), 256, 0, st>>>(c->part, perm_row, dgate, M, ntile_part));
+           pdl_launch(dgate_reduce_kernel, ceil_div(M, 256), 256, 0, st, c->part, perm_row, dgate, M, ntile_part));
     if ((r = after_launch(c)) != MOP_OK) return r;
     return mop_moe_combine(c, c->dXp, perm_row, dX, stream);
+}
+
+mop_status mop_moe_layer_fwd(mop_ctx* c, const void* x, const float* W_r, const float* bias, const void* W_gate,
+                             const void* W_up, const void* W_down, int32_t* topk_idx, float* topk_gate, int32_t* counts,
+                             int32_t* offsets, int32_t* perm_row, int32_t* row_src, void* Xp, void* G_save, void* U_save,
+                             void* H, void* Yp, void* Y, void* stream) {
+    mop_status r;
+    if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
+    if ((r = mop_moe_permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, stream)) != MOP_OK) return r;
+    if ((r = mop_moe_expert_ffn_fwd(c, Xp, offsets, row_src, topk_gate, W_gate, W_up, W_down, G_save, U_save, H, Yp, stream)) != MOP_OK)
+        return r;
+    return mop_moe_combine(c, Yp, perm_row, Y, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -900,12 +909,11 @@ mop_status chunk_begin(mop_ctx* c, const ChunkLayout& L, char* w, int i, int C, 
     mop_status r;
     if (tables) {
         LAUNCH(c, "chunk_tables", st,
-               chunk_tables_kernel<<<min(ceil_div(M, 256), c->sm_count * 4), 256, 0, st>>>(
-                   offsets, row_src, perm_row, off_c, row_src_c, perm_c, bounds, s.E, M, i, C));
+               pdl_launch(chunk_tables_kernel, min(ceil_div(M, 256), c->sm_count * 4), 256, 0, st, offsets, row_src, perm_row, off_c, row_src_c, perm_c, bounds, s.E, M, i, C));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     LAUNCH(c, "chunk_gather_rows", st,
-           gather_rows_kernel<<<c->sm_count * 8, 256, 0, st>>>(static_cast<const uint4*>(src),
+           pdl_launch(gather_rows_kernel, c->sm_count * 8, 256, 0, st, static_cast<const uint4*>(src),
                                                                reinterpret_cast<uint4*>(w + dst_off), row_src_c, bounds,
                                                                s.k, s.d / 8));
     return after_launch(c);
@@ -949,7 +957,7 @@ mop_status mop_moe_layer_fwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         c->launches += n;
         if (r != MOP_OK) break;
         LAUNCH(c, "chunk_combine_acc", st,
-               combine_acc_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(w + L.Yp),
+               pdl_launch(combine_acc_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(w + L.Yp),
                                                          reinterpret_cast<const int32_t*>(w + L.perm_c),
                                                          reinterpret_cast<float4*>(w + L.acc), static_cast<uint4*>(Y), s.T,
                                                          s.k, s.d / 8, i == 0, i == n_chunks - 1));
@@ -1016,11 +1024,11 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         c->launches += n;
         if (r != MOP_OK) break;
         LAUNCH(c, "chunk_dgate_reduce", st,
-               dgate_reduce_chunk_kernel<<<ceil_div(M, 256), 256, 0, st>>>(a.part, reinterpret_cast<const int32_t*>(w + L.perm_c),
+               pdl_launch(dgate_reduce_chunk_kernel, ceil_div(M, 256), 256, 0, st, a.part, reinterpret_cast<const int32_t*>(w + L.perm_c),
                                                                            dgate, M, (int)L.cap, ntile_part));
         if ((r = after_launch(c)) != MOP_OK) break;
         LAUNCH(c, "chunk_combine_acc", st,
-               combine_acc_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(w + L.dXp),
+               pdl_launch(combine_acc_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(w + L.dXp),
                                                          reinterpret_cast<const int32_t*>(w + L.perm_c),
                                                          reinterpret_cast<float4*>(w + L.acc), static_cast<uint4*>(dX), s.T,
                                                          s.k, s.d / 8, i == 0, i == n_chunks - 1));
@@ -1031,7 +1039,7 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
     if (!s.dw_accumulate) {   // experts that received no row: zero gradients
         dim3 gz((unsigned)min((size_t)64, (wvec + 255) / 256), s.E);
         LAUNCH(c, "chunk_zero_empty_experts", st,
-               zero_empty_experts_kernel<<<gz, 256, 0, st>>>(offsets, reinterpret_cast<float4*>(dW_gate),
+               pdl_launch(zero_empty_experts_kernel, gz, 256, 0, st, offsets, reinterpret_cast<float4*>(dW_gate),
                                                              reinterpret_cast<float4*>(dW_up),
                                                              reinterpret_cast<float4*>(dW_down), wvec));
         r = after_launch(c);
@@ -1056,7 +1064,7 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     mop_status r;
     if (s.T > 0) {
         LAUNCH(c, "route_bwd_dz", st,
-               route_bwd_dz_kernel<<<ceil_div(s.T, 8), 256, 0, st>>>(logits, bias, topk_idx, topk_gate, dgate, perm_row,
+               pdl_launch(route_bwd_dz_kernel, ceil_div(s.T, 8), 256, 0, st, logits, bias, topk_idx, topk_gate, dgate, perm_row,
                                                                      c->dz_sel, c->dz_row, s.T, s.E, s.k, s.score_fn,
                                                                      s.bias_mode));
         if ((r = after_launch(c)) != MOP_OK) return r;
@@ -1066,14 +1074,14 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     float* db = (dbias_opt && s.bias_mode == MOP_BIAS_PRE_LOGIT) ? dbias_opt : nullptr;
     if (dbias_opt && !db) CUDA_OK(cudaMemsetAsync(dbias_opt, 0, (size_t)s.E * 4, st));
     LAUNCH(c, "route_bwd_dwr", st,
-           route_bwd_dwr_kernel<<<gw, 32 * dwr_w, dwr_w * 1024, st>>>(static_cast<const bf16*>(Xp), c->dz_row, offsets, dW_r, db, s.d, s.E));
+           pdl_launch(route_bwd_dwr_kernel, gw, 32 * dwr_w, dwr_w * 1024, st, static_cast<const bf16*>(Xp), c->dz_row, offsets, dW_r, db, s.d, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     if (s.T == 0) return MOP_OK;
     dim3 gt(ceil_div(s.E, 32), ceil_div(s.d, 32));
-    LAUNCH(c, "route_bwd_wrT", st, transpose_f32_kernel<<<gt, 256, 0, st>>>(W_r, c->wrT, s.d, s.E));
+    LAUNCH(c, "route_bwd_wrT", st, pdl_launch(transpose_f32_kernel, gt, 256, 0, st, W_r, c->wrT, s.d, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     LAUNCH(c, "route_bwd_dx", st,
-           route_bwd_dx_kernel<<<s.T, 256, 0, st>>>(c->wrT, topk_idx, c->dz_sel, static_cast<bf16*>(dX), s.T, s.d, s.E,
+           pdl_launch(route_bwd_dx_kernel, s.T, 256, 0, st, c->wrT, topk_idx, c->dz_sel, static_cast<bf16*>(dX), s.T, s.d, s.E,
                                                     s.k));
     return after_launch(c);
 }
@@ -1363,17 +1371,16 @@ mop_status mop_moe_permute_static(int device, int32_t T, int32_t d, int32_t E, i
     // Nothing in the scratch has to start at zero: the histogram kernel writes every entry
     // [unit][expert] that the scan and rank kernels read, so a previous call's contents are dead.
     if (units > 0) {
-        perm_hist_kernel<<<ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st>>>(topk_idx, su.scratch, M, E);
+        pdl_launch(perm_hist_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st, topk_idx, su.scratch, M, E);
         if (cudaGetLastError() != cudaSuccess) return MOP_ERR_CUDA;
     }
     if (units == 0) {
-        perm_scan_kernel<<<1, 1024, (E + 1) * sizeof(int32_t), st>>>(su.scratch, counts, offsets, units, E);
+        pdl_launch(perm_scan_kernel, 1, 1024, (E + 1) * sizeof(int32_t), st, su.scratch, counts, offsets, units, E);
         return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
     }
-    perm_scan_cols_kernel<<<ceil_div(E, 32), PSCAN_WARPS * 32, 0, st>>>(su.scratch, counts, units, E);
+    pdl_launch(perm_scan_cols_kernel, ceil_div(E, 32), PSCAN_WARPS * 32, 0, st, su.scratch, counts, units, E);
     if (cudaGetLastError() != cudaSuccess) return MOP_ERR_CUDA;
-    perm_rank_kernel<<<ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (E + 1) * sizeof(int32_t), st>>>(
-        topk_idx, su.scratch, counts, offsets, perm_row, row_src, M, E);
+    pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (E + 1) * sizeof(int32_t), st, topk_idx, su.scratch, counts, offsets, perm_row, row_src, M, E);
     if (cudaGetLastError() != cudaSuccess) return MOP_ERR_CUDA;
     if (!Xp) return MOP_OK;
     launch_scatter_rows(static_cast<const uint4*>(x), static_cast<uint4*>(Xp), perm_row, T, k, d / 8, su.sm_count, st);
@@ -1455,7 +1462,7 @@ mop_status mop_vocab_loss_fwd(int device, int32_t N, int32_t H, int32_t V, const
     CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
     const bool pair = false;                // measured: the one-CTA kernel is as fast here (online log-sum-exp epilogue)
     if (pair) tc_build_pairtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
-    else tc_build_mtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
+    else pdl_launch(tc_build_mtiles_kernel, 1, 1024, 0, st, off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
     CUtensorMap mX, mW;
     if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_3d(p, &mW, W_voc, 1, H, V, pair ? 2 : 4)) return MOP_ERR_CUDA;
     TcArgs g{};
@@ -1562,7 +1569,7 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
     CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
     const bool pair = p->sm_count >= 2;     // dY and dX products on the two-CTA kernel (256-row pair tiles)
     if (pair) tc_build_pairtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
-    else tc_build_mtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
+    else pdl_launch(tc_build_mtiles_kernel, 1, 1024, 0, st, off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
     CUtensorMap mX, mXT, mWn, mWk;
     if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_2d(p, &mXT, X, N, H, 2) ||
         !tc_map_chunked_3d(p, &mWn, W_voc, 1, H, V, pair ? 2 : 4) || !tc_map_3d(p, &mWk, W_voc, 1, H, V, pair ? 128 : 256))

@@ -12,6 +12,7 @@ constexpr int PERM_WARPS = 4;    // warps per block in the histogram / rank kern
 // Histogram per unit: partial[u][e] = number of assignments of unit u that go to expert e.
 __global__ void __launch_bounds__(PERM_WARPS * 32) perm_hist_kernel(const int32_t* __restrict__ idx,
                                                                     int32_t* __restrict__ partial, int M, int E) {
+    pdl_begin();
     extern __shared__ int32_t perm_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     int32_t* cnt = perm_smem + (size_t)warp * E;
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(PERM_WARPS * 32) perm_hist_kernel(const int32_
 // to permute (it still writes counts and offsets); otherwise perm_scan_cols_kernel + perm_rank_kernel do this.
 __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ partial, int32_t* __restrict__ counts,
                                                          int32_t* __restrict__ offsets, int units, int E) {
+    pdl_begin();
     extern __shared__ int32_t scan_smem[];  // E + 1
     for (int e = threadIdx.x; e < E; e += blockDim.x) {
         int32_t run = 0;
@@ -80,6 +82,7 @@ constexpr int PSCAN_WARPS = 8;
 __global__ void __launch_bounds__(PSCAN_WARPS * 32) perm_scan_cols_kernel(int32_t* __restrict__ partial,
                                                                           int32_t* __restrict__ counts, int units,
                                                                           int E) {
+    pdl_begin();
     __shared__ int32_t tot[PSCAN_WARPS][32];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int e = blockIdx.x * 32 + lane;
@@ -116,6 +119,7 @@ __global__ void __launch_bounds__(PERM_WARPS * 32) perm_rank_kernel(const int32_
                                                                     int32_t* __restrict__ offsets,
                                                                     int32_t* __restrict__ perm_row,
                                                                     int32_t* __restrict__ row_src, int M, int E) {
+    pdl_begin();
     extern __shared__ int32_t perm_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     int32_t* off = perm_smem + (size_t)PERM_WARPS * E;   // E + 1 words
@@ -173,6 +177,7 @@ constexpr int PERM_SMALL_MAX_WORDS = 10240;     // units * E words of shared mem
 __global__ void __launch_bounds__(1024) perm_small_kernel(const int32_t* __restrict__ idx, int32_t* __restrict__ counts,
                                                           int32_t* __restrict__ offsets, int32_t* __restrict__ perm_row,
                                                           int32_t* __restrict__ row_src, int M, int E, int units) {
+    pdl_begin();
     extern __shared__ int32_t perm_smem[];
     int32_t* cnt = perm_smem;                      // [units][E]
     int32_t* off = perm_smem + (size_t)units * E;  // [E + 1]
@@ -251,6 +256,7 @@ inline bool perm_small_fits(int units, int E) {
 __global__ void __launch_bounds__(256) scatter_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                            const int32_t* __restrict__ perm_row, int T, int k,
                                                            int vec_per_row) {
+    pdl_begin();
     const int warps_per_block = blockDim.x / 32;
     const int lane = threadIdx.x % 32;
     for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
@@ -283,6 +289,7 @@ __global__ void __launch_bounds__(256) scatter_rows_kernel(const uint4* __restri
 __global__ void __launch_bounds__(256) combine_rows_kernel(const uint4* __restrict__ Yp,
                                                            const int32_t* __restrict__ perm_row,
                                                            uint4* __restrict__ Y, int T, int k, int vec_per_row) {
+    pdl_begin();
     const int warps_per_block = blockDim.x / 32;
     const int lane = threadIdx.x % 32;
     for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
@@ -333,6 +340,7 @@ template <int VPL>
 __global__ void __launch_bounds__(256) scatter_rows_reg_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                                const int32_t* __restrict__ perm_row, int T, int k,
                                                                int vec_per_row) {
+    pdl_begin();
     const int warps_per_block = blockDim.x / 32;
     const int lane = threadIdx.x % 32;
     for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
@@ -365,6 +373,7 @@ template <int SEG>
 __global__ void __launch_bounds__(256) combine_rows_seg_kernel(const uint4* __restrict__ Yp,
                                                                const int32_t* __restrict__ perm_row,
                                                                uint4* __restrict__ Y, int T, int k, int vec_per_row) {
+    pdl_begin();
     const int warps_per_block = blockDim.x / 32;
     const int lane = threadIdx.x % 32;
     for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
@@ -426,11 +435,11 @@ inline void launch_scatter_rows(const uint4* src, uint4* dst, const int32_t* per
                                 int sm_count, cudaStream_t st) {
     const int blocks = min(ceil_div(T, 8), sm_count * 8);
     if (blocks <= 0) return;
-    if (vec_per_row <= 32 * 8) scatter_rows_reg_kernel<8><<<blocks, 256, 0, st>>>(src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 16) scatter_rows_reg_kernel<16><<<blocks, 256, 0, st>>>(src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 28) scatter_rows_reg_kernel<28><<<blocks, 256, 0, st>>>(src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 32) scatter_rows_reg_kernel<32><<<blocks, 256, 0, st>>>(src, dst, perm_row, T, k, vec_per_row);
-    else scatter_rows_kernel<<<blocks, 256, 0, st>>>(src, dst, perm_row, T, k, vec_per_row);
+    if (vec_per_row <= 32 * 8) pdl_launch(scatter_rows_reg_kernel<8>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
+    else if (vec_per_row <= 32 * 16) pdl_launch(scatter_rows_reg_kernel<16>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
+    else if (vec_per_row <= 32 * 28) pdl_launch(scatter_rows_reg_kernel<28>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
+    else if (vec_per_row <= 32 * 32) pdl_launch(scatter_rows_reg_kernel<32>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
+    else pdl_launch(scatter_rows_kernel, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
 }
 inline void launch_combine_rows(const uint4* Yp, const int32_t* perm_row, uint4* Y, int T, int k, int vec_per_row,
                                 int sm_count, cudaStream_t st) {
@@ -438,15 +447,16 @@ inline void launch_combine_rows(const uint4* Yp, const int32_t* perm_row, uint4*
     if (blocks <= 0) return;
     // short rows (d < 4096) keep the chunked kernel: measured faster there (more warps per SM)
     if (vec_per_row >= 32 * 16 && vec_per_row % (32 * 7) == 0)
-        combine_rows_seg_kernel<7><<<blocks, 256, 0, st>>>(Yp, perm_row, Y, T, k, vec_per_row);
-    else if (vec_per_row >= 32 * 16) combine_rows_seg_kernel<8><<<blocks, 256, 0, st>>>(Yp, perm_row, Y, T, k, vec_per_row);
-    else combine_rows_kernel<<<blocks, 256, 0, st>>>(Yp, perm_row, Y, T, k, vec_per_row);
+        pdl_launch(combine_rows_seg_kernel<7>, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
+    else if (vec_per_row >= 32 * 16) pdl_launch(combine_rows_seg_kernel<8>, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
+    else pdl_launch(combine_rows_kernel, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
 }
 
 // dgate[a] = sum over n-tiles of the partial dot products written by the dgrad-down epilogue
 // (row p = perm_row[a]; fixed order, so the result is reproducible).
 __global__ void dgate_reduce_kernel(const float* __restrict__ part, const int32_t* __restrict__ perm_row,
                                     float* __restrict__ dgate, int M, int ntiles) {
+    pdl_begin();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= M) return;
     const int32_t p = perm_row[a];
@@ -471,6 +481,7 @@ __global__ void __launch_bounds__(256) chunk_tables_kernel(const int32_t* __rest
                                                            int32_t* __restrict__ off_c, int32_t* __restrict__ row_src_c,
                                                            int32_t* __restrict__ perm_c, int32_t* __restrict__ bounds,
                                                            int E, int M, int chunk, int n_chunks) {
+    pdl_begin();
     __shared__ int32_t s_lo, s_hi;
     if (threadIdx.x == 0) {
         const long long t0 = ((long long)chunk * M + n_chunks - 1) / n_chunks;
@@ -499,6 +510,7 @@ __global__ void __launch_bounds__(256) chunk_tables_kernel(const int32_t* __rest
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                           const int32_t* __restrict__ row_src_c,
                                                           const int32_t* __restrict__ bounds, int k, int vec_per_row) {
+    pdl_begin();
     const int rows = bounds[1];
     const int lane = threadIdx.x % 32, wpb = blockDim.x / 32;
     for (int r = blockIdx.x * wpb + threadIdx.x / 32; r < rows; r += gridDim.x * wpb) {
@@ -515,6 +527,7 @@ __global__ void __launch_bounds__(256) combine_acc_kernel(const uint4* __restric
                                                           const int32_t* __restrict__ perm_c, float4* __restrict__ acc,
                                                           uint4* __restrict__ out, int T, int k, int vec_per_row,
                                                           int first, int last) {
+    pdl_begin();
     const int wpb = blockDim.x / 32, lane = threadIdx.x % 32;
     for (int t = blockIdx.x * wpb + threadIdx.x / 32; t < T; t += gridDim.x * wpb) {
         int32_t myrow = -1;
@@ -554,6 +567,7 @@ __global__ void __launch_bounds__(256) combine_acc_kernel(const uint4* __restric
 // dgate of the assignments that lie inside the chunk (others are left alone).
 __global__ void dgate_reduce_chunk_kernel(const float* __restrict__ part, const int32_t* __restrict__ perm_c,
                                           float* __restrict__ dgate, int M, int rows_pitch, int ntiles) {
+    pdl_begin();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= M) return;
     const int32_t p = perm_c[a];
@@ -567,6 +581,7 @@ __global__ void dgate_reduce_chunk_kernel(const float* __restrict__ part, const 
 __global__ void __launch_bounds__(256) zero_empty_experts_kernel(const int32_t* __restrict__ offsets,
                                                                 float4* __restrict__ dWg, float4* __restrict__ dWu,
                                                                 float4* __restrict__ dWd, size_t vec_per_expert) {
+    pdl_begin();
     const int e = blockIdx.y;
     if (offsets[e + 1] > offsets[e]) return;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -58,6 +58,7 @@ struct ScoreShape {
 template <int RT, int RE, int LT>
 __global__ void __launch_bounds__(SC_THREADS) route_score_kernel(const bf16* __restrict__ x, const float* __restrict__ W_r,
                                                                  float* __restrict__ z, int T, int d, int E) {
+    pdl_begin();
     using Sh = ScoreShape<RT, RE, LT>;
     constexpr int LE = Sh::LE, TT = Sh::TT, TE = Sh::TE, S = Sh::STAGES;
     static_assert(RE == 1 || (RE % 4 == 0 && LE == 8), "expert columns of a thread: one, or groups of four 32 apart");
@@ -213,7 +214,7 @@ template <int RT, int RE, int LT>
 inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, cudaStream_t st) {
     using Sh = ScoreShape<RT, RE, LT>;
     dim3 grid(ceil_div(T, Sh::TT), ceil_div(E, Sh::TE));
-    route_score_kernel<RT, RE, LT><<<grid, SC_THREADS, Sh::SMEM, st>>>(x, W_r, z, T, d, E);
+    pdl_launch(route_score_kernel<RT, RE, LT>, grid, SC_THREADS, Sh::SMEM, st, x, W_r, z, T, d, E);
 }
 // Shape choice: the least estimated cycles per step on the fullest SM, first + more * (blocks on it - 1), as measured at
 // d = 7168 (one block alone on an SM; each further one).  Decoding (T = 64, E = 256) takes one chain per thread: 130 us with the
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) route_select_kernel(const floa
                                                                       int32_t* __restrict__ idx,
                                                                       float* __restrict__ gate, int T, int E, int k,
                                                                       int score_fn, int bias_mode) {
+    pdl_begin();
     extern __shared__ float sel_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     float* key = sel_smem + (size_t)warp * 2 * E;  // keys
@@ -822,6 +824,7 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
                                                            const int32_t* __restrict__ perm_row,
                                                            float* __restrict__ dz_sel, float* __restrict__ dz_row,
                                                            int T, int E, int k, int score_fn, int bias_mode) {
+    pdl_begin();
     const int lane = threadIdx.x % 32;
     const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     if (t >= T) return;
@@ -863,6 +866,7 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
 __global__ void __launch_bounds__(1024) route_bwd_dwr_kernel(const bf16* __restrict__ Xp, const float* __restrict__ dz_row,
                                                              const int32_t* __restrict__ offsets, float* __restrict__ dW_r,
                                                              float* __restrict__ dbias, int d, int E) {
+    pdl_begin();
     extern __shared__ float dwr_smem[];                              // [W][256]
     const int e = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32, W = blockDim.x / 32;
     const int i = blockIdx.x * 256 + lane * 8;
@@ -912,6 +916,7 @@ inline int dwr_warps(long long blocks, int sm_count) { return blocks >= 4ll * sm
 // W_r^T [E,d] from W_r [d,E] (32 x 32 tiles through shared memory): gives the dX kernel contiguous rows.
 __global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, float* __restrict__ out,
                                                             int rows, int cols) {
+    pdl_begin();
     __shared__ float tile[32][33];
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
@@ -929,6 +934,7 @@ __global__ void __launch_bounds__(256) route_bwd_dx_kernel(const float* __restri
                                                            const int32_t* __restrict__ idx,
                                                            const float* __restrict__ dz_sel, bf16* __restrict__ dX,
                                                            int T, int d, int E, int k) {
+    pdl_begin();
     __shared__ int32_t es[32];
     __shared__ float dzs[32];
     const int t = blockIdx.x;
