@@ -90,8 +90,8 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
 }
 
 // Instruction descriptor of the pair: M = 256 across the two CTAs, N = 256.
-__host__ __device__ constexpr uint32_t make_idesc2(bool b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(256 >> 3) << 17) |
+__host__ __device__ constexpr uint32_t make_idesc2(bool a_mn, bool b_mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(256 >> 3) << 17) |
            ((uint32_t)(256 >> 4) << 24);
 }
 
@@ -188,15 +188,25 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    pdl_begin();
 
-    const int total_tiles = (*args.n_mtiles) * args.tiles_n;
+    const int row_tiles = KIND == TC_VW ? args.tiles_m_fixed : *args.n_mtiles;
+    const int total_tiles = row_tiles * args.tiles_n;
     const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
     auto decode = [&](int t) {
         TileInfo ti;
         int mt, nt;
-        if (args.m_fastest) { const int nm = __ldg(args.n_mtiles); nt = t / nm; mt = t - nt * nm; }
-        else { mt = t / args.tiles_n; nt = t - mt * args.tiles_n; }
-        const int4 m = __ldg(args.mtiles + mt);
+        if (args.n_group) {
+            // blocks of n_group n-tiles: the clusters that run at the same time cover a nearly square patch of the output, so that
+            // a K slab of either operand is fetched few times (74 clusters: 9 row tiles x 8 n-tiles; with one row of tiles after
+            // the other one operand is read whole for every two or three tiles of the other)
+            const int nm = row_tiles, per = args.n_group * nm, g = t / per, r = t - g * per;
+            const int w = min(args.n_group, args.tiles_n - g * args.n_group);
+            mt = r / w; nt = g * args.n_group + r - mt * w;
+        } else { mt = t / args.tiles_n; nt = t - mt * args.tiles_n; }
+        int4 m;
+        if constexpr (KIND == TC_VW) m = make_int4(0, 256 * mt, min(256, args.Mfix - 256 * mt), 0);
+        else m = __ldg(args.mtiles + mt);
         ti.e = m.x; ti.row0 = m.y + 128 * (int)rank; ti.rows = min(128, max(0, m.z - 128 * (int)rank));
         ti.m0 = 0; ti.nt = nt; ti.skip = false;
         return ti;
@@ -223,8 +233,14 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                 const int k0 = (kb - ph * args.kblocks) * TC_BK;
                 if (el) {
                     if (leader) mbar_expect_tx(full_bar(stage), 2 * T2_STAGE_BYTES);
+                    if constexpr (KIND == TC_VW) {
+                        // both operands as chunked 2-D views: two 64-wide column chunks of 64 rows of K each
+                        tma2_load_3d(sA, &tmA0, fb, 0, k0, ti.row0 >> 6);
+                        tma2_load_3d(sB, &tmB0, fb, 0, k0, (n0 + 128 * (int)rank) >> 6);
+                    } else
                     tma2_load_2d(sA, ph ? &tmA1 : &tmA0, fb, k0, ti.row0);
-                    if constexpr (!Tr::B_MN) {
+                    if constexpr (KIND == TC_VW) {
+                    } else if constexpr (!Tr::B_MN) {
                         // K-major weights: this CTA's 128 output columns are 128 rows of the [E, N, K] tensor
                         tma2_load_3d(sB, ph ? &tmB1 : &tmB0, fb, k0 + (KIND == TC_VX ? args.kb_base : 0), n0 + 128 * (int)rank,
                                      ti.e);
@@ -243,10 +259,10 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
         // ===================================================================== MMA issuer (leader CTA)
         if (leader) {
             const bool el = elect_one();
-            constexpr uint32_t idesc = make_idesc2(Tr::B_MN);
-            const uint64_t desc_a = smem_desc(0, 0, 1024);
+            constexpr uint32_t idesc = make_idesc2(Tr::A_MN, Tr::B_MN);
+            const uint64_t desc_a = Tr::A_MN ? smem_desc(0, TC_CHUNK_BYTES, 1024) : smem_desc(0, 0, 1024);
             const uint64_t desc_b = Tr::B_MN ? smem_desc(0, TC_CHUNK_BYTES, 1024) : smem_desc(0, 0, 1024);
-            constexpr uint32_t b_step = (Tr::B_MN ? 2048 : 32) >> 4;
+            constexpr uint32_t a_step = (Tr::A_MN ? 2048 : 32) >> 4, b_step = (Tr::B_MN ? 2048 : 32) >> 4;
             int stage = 0; uint32_t phase = 0; int it = 0; bool alive = true;
             const int nkb = Tr::PHASES * args.kblocks;
             for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
@@ -266,7 +282,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                     if (el) {
 #pragma unroll
                         for (int k4 = 0; k4 < TC_BK / 16; ++k4)
-                            umma2_bf16(d_tmem, da + k4 * 2, db + k4 * b_step, idesc, (kb | k4) != 0 ? 1u : 0u);
+                            umma2_bf16(d_tmem, da + k4 * a_step, db + k4 * b_step, idesc, (kb | k4) != 0 ? 1u : 0u);
                         umma2_commit_both(empty_bar(stage));
                     }
                     if (++stage == S) { stage = 0; phase ^= 1u; }
@@ -330,6 +346,7 @@ inline mop_status tc2_init() {
     if ((r = tc2_set_smem<TC_VL>()) != MOP_OK) return r;
     if ((r = tc2_set_smem<TC_VP>()) != MOP_OK) return r;
     if ((r = tc2_set_smem<TC_VX>()) != MOP_OK) return r;
+    if ((r = tc2_set_smem<TC_VW>()) != MOP_OK) return r;
     return MOP_OK;
 }
 
@@ -338,7 +355,7 @@ inline mop_status tc2_launch(const TcPlan* p, const char* name, const CUtensorMa
                              const CUtensorMap& b0, const CUtensorMap& b1, const TcArgs& args, cudaStream_t st) {
     p->prof->begin(name, st);
     const int grid = p->sm_count & ~1;   // whole pairs
-    tc_gemm2_kernel<KIND><<<grid, T2_THREADS, T2_SMEM_BYTES, st>>>(a0, a1, b0, b1, args);
+    pdl_launch(tc_gemm2_kernel<KIND>, grid, T2_THREADS, T2_SMEM_BYTES, st, a0, a1, b0, b1, args);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

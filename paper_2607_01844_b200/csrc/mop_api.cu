@@ -1391,19 +1391,21 @@ mop_status mop_moe_permute_static(int device, int32_t T, int32_t d, int32_t E, i
 // Vocabulary projection + online log-likelihood (no context: the caller owns the workspace)
 // ---------------------------------------------------------------------------------------------
 namespace {
-struct VocabLayout { size_t off, tiles, status, ylab, part, total; };
+struct VocabLayout { size_t tiles, status, ylab, part, total; };
 VocabLayout vocab_layout(int N, int V) {
     VocabLayout L{};
     size_t o = 0;
     auto take = [&](size_t b) { size_t r = o; o += align_up(b); return r; };
     L.status = take(256);                 // first: mop_vocab_poll reads it without knowing the shape
-    L.off = take(16);
     L.tiles = take(tc_tile_table_bytes(N, 1));
     L.ylab = take((size_t)N * 4);
     L.part = take((size_t)ceil_div(V, 256) * N * 8);
     L.total = o;
     return L;
 }
+// n-tiles per block of the tile order (see tc_gemm2_kernel).  N = 8192, H = 7168, V = 131072 forward and backward: 51.3 ms with 1
+// (row tiles fastest), 50.6 with 4, 48.5 with 8, 49.4 with 16; 55.0 before, with the weight gradient and the forward on one CTA.
+constexpr int VOCAB_N_GROUP = 8;
 std::mutex g_vocab_mutex;
 TcPlan g_vocab_plan[kMaxDevices];
 Profiler g_vocab_prof;           // never enabled: the plan needs one
@@ -1452,42 +1454,34 @@ mop_status mop_vocab_loss_fwd(int device, int32_t N, int32_t H, int32_t V, const
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const VocabLayout L = vocab_layout(N, V);
     char* w = static_cast<char*>(workspace);
-    int32_t* off = reinterpret_cast<int32_t*>(w + L.off);
     int32_t* tiles = reinterpret_cast<int32_t*>(w + L.tiles);
     int32_t* status = reinterpret_cast<int32_t*>(w + L.status);
     float* ylab = reinterpret_cast<float*>(w + L.ylab);
     float* part = reinterpret_cast<float*>(w + L.part);
-    const int32_t host_off[2] = {0, N};
-    CUDA_OK(cudaMemcpyAsync(off, host_off, sizeof(host_off), cudaMemcpyHostToDevice, st));
-    CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
-    const bool pair = false;                // measured: the one-CTA kernel is as fast here (online log-sum-exp epilogue)
-    if (pair) tc_build_pairtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
-    else pdl_launch(tc_build_mtiles_kernel, 1, 1024, 0, st, off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
+    pdl_launch(vocab_setup_kernel, 1, 256, 0, st, N, reinterpret_cast<int4*>(tiles + 64), tiles, status);
     CUtensorMap mX, mW;
-    if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_3d(p, &mW, W_voc, 1, H, V, pair ? 2 : 4)) return MOP_ERR_CUDA;
+    if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_3d(p, &mW, W_voc, 1, H, V, 2)) return MOP_ERR_CUDA;
     TcArgs g{};
-    g.offsets = off; g.n_mtiles = tiles; g.mtiles = reinterpret_cast<const int4*>(tiles + 64);
+    g.n_mtiles = tiles; g.mtiles = reinterpret_cast<const int4*>(tiles + 64);
     g.E = 1; g.status = status;
-    g.tiles_n = ceil_div(V, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.m_fastest = 1;
+    g.tiles_n = ceil_div(V, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.n_group = VOCAB_N_GROUP;
     g.targets = targets; g.ylab = ylab; g.ep.part = part; g.ep.M_total = N;
-    mop_status r = pair ? tc2_launch<TC_VL>(p, "vocab_logits_lse", mX, mX, mW, mW, g, st)
-                        : tc_launch<TC_VL>(p, "vocab_logits_lse", mX, mX, mW, mW, mX, mX, g, st);
+    const mop_status r = tc2_launch<TC_VL>(p, "vocab_logits_lse", mX, mX, mW, mW, g, st);
     if (r != MOP_OK) return r;
-    vocab_lse_merge_kernel<<<ceil_div(N, 256), 256, 0, st>>>(reinterpret_cast<const float2*>(part), ylab, loss,
-                                                            lse_opt, N, g.tiles_n);
+    pdl_launch(vocab_lse_merge_kernel, ceil_div(N, 32), 32 * LSE_WARPS, 0, st, reinterpret_cast<const float2*>(part), ylab, loss,
+               lse_opt, N, g.tiles_n);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
 
 namespace {
 constexpr int kVocabBlock = 8192;   // vocabulary columns whose logit gradients are live at a time
-struct VocabBwdLayout { size_t off, tiles, status, dy, dx32, total; int vc; };
+struct VocabBwdLayout { size_t tiles, status, dy, dx32, total; int vc; };
 VocabBwdLayout vocab_bwd_layout(int N, int H, int V) {
     VocabBwdLayout L{};
     size_t o = 0;
     auto take = [&](size_t b) { size_t r = o; o += align_up(b); return r; };
     L.vc = V < kVocabBlock ? V : kVocabBlock;
     L.status = take(256);                 // first, as in the forward's workspace
-    L.off = take(16);
     L.tiles = take(tc_tile_table_bytes(N, 1));
     L.dy = take((size_t)N * L.vc * 2);
     L.dx32 = take((size_t)N * H * 4);
@@ -1559,57 +1553,45 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
     if (r != MOP_OK) return r;
     const VocabBwdLayout L = vocab_bwd_layout(N, H, V);
     char* w = static_cast<char*>(workspace);
-    int32_t* off = reinterpret_cast<int32_t*>(w + L.off);
     int32_t* tiles = reinterpret_cast<int32_t*>(w + L.tiles);
     int32_t* status = reinterpret_cast<int32_t*>(w + L.status);
     bf16* dY = reinterpret_cast<bf16*>(w + L.dy);
     float* dx32 = reinterpret_cast<float*>(w + L.dx32);
-    const int32_t host_off[2] = {0, N};
-    CUDA_OK(cudaMemcpyAsync(off, host_off, sizeof(host_off), cudaMemcpyHostToDevice, st));
-    CUDA_OK(cudaMemsetAsync(status, 0, 4, st));
-    const bool pair = p->sm_count >= 2;     // dY and dX products on the two-CTA kernel (256-row pair tiles)
-    if (pair) tc_build_pairtiles_kernel<<<1, 1024, 0, st>>>(off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
-    else pdl_launch(tc_build_mtiles_kernel, 1, 1024, 0, st, off, 1, reinterpret_cast<int4*>(tiles + 64), tiles);
+    pdl_launch(vocab_setup_kernel, 1, 256, 0, st, N, reinterpret_cast<int4*>(tiles + 64), tiles, status);
     CUtensorMap mX, mXT, mWn, mWk;
     if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_2d(p, &mXT, X, N, H, 2) ||
-        !tc_map_chunked_3d(p, &mWn, W_voc, 1, H, V, pair ? 2 : 4) || !tc_map_3d(p, &mWk, W_voc, 1, H, V, pair ? 128 : 256))
+        !tc_map_chunked_3d(p, &mWn, W_voc, 1, H, V, 2) || !tc_map_3d(p, &mWk, W_voc, 1, H, V, 128))
         return MOP_ERR_CUDA;
     for (int c0 = 0; c0 < V; c0 += L.vc) {
         const int cw = V - c0 < L.vc ? V - c0 : L.vc;
-        CUtensorMap mdYk, mdYn, mOut;
-        if (!tc_map_2d_pitch(p, &mdYk, dY, N, cw, L.vc, 128) || !tc_map_chunked_2d_pitch(p, &mdYn, dY, N, cw, L.vc, 4) ||
-            !tc_map_out_f32_pitch(p, &mOut, dW_voc + c0, H, cw, V))
+        CUtensorMap mdYk, mdYn;
+        if (!tc_map_2d_pitch(p, &mdYk, dY, N, cw, L.vc, 128) || !tc_map_chunked_2d_pitch(p, &mdYn, dY, N, cw, L.vc, 2))
             return MOP_ERR_CUDA;
         TcArgs base{};
-        base.offsets = off; base.n_mtiles = tiles; base.mtiles = reinterpret_cast<const int4*>(tiles + 64);
+        base.n_mtiles = tiles; base.n_group = VOCAB_N_GROUP; base.mtiles = reinterpret_cast<const int4*>(tiles + 64);
         base.E = 1; base.status = status; base.ep.M_total = N;
         {   // dY block = g ([v = t] - exp(X W - lse)), logits recomputed on the tensor cores
             TcArgs g = base;
-            g.tiles_n = ceil_div(cw, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.m_fastest = 1; g.n_base = c0;
+            g.tiles_n = ceil_div(cw, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.n_base = c0;
             g.targets = targets; g.row_lse = lse; g.row_g = dloss; g.ep.out0 = dY; g.ep.ldo = L.vc;
-            r = pair ? tc2_launch<TC_VP>(p, "vocab_dlogits", mX, mX, mWn, mWn, g, st)
-                     : tc_launch<TC_VP>(p, "vocab_dlogits", mX, mX, mWn, mWn, mX, mX, g, st);
-            if (r != MOP_OK) return r;
+            if ((r = tc2_launch<TC_VP>(p, "vocab_dlogits", mX, mX, mWn, mWn, g, st)) != MOP_OK) return r;
         }
         {   // dW[:, block] = X^T dY (K = the N tokens), written once
             TcArgs g = base;
-            g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, TC_BM); g.Mfix = H; g.N = cw;
-            g.ep.outf = dW_voc + c0; g.ep.accumulate = 0;
-            if ((r = tc_launch<TC_WD>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, mOut, mOut, g, st)) != MOP_OK) return r;
+            g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, 256); g.Mfix = H; g.N = cw; g.kblocks = ceil_div(N, TC_BK);
+            g.ep.outf = dW_voc + c0; g.ep.ldo = V;
+            if ((r = tc2_launch<TC_VW>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, g, st)) != MOP_OK) return r;
         }
         {   // dX += dY W[:, block]^T in fp32 across the blocks
             TcArgs g = base;
             g.tiles_n = ceil_div(H, 256); g.kblocks = ceil_div(cw, TC_BK); g.N = H; g.kb_base = c0;
             g.ep.outf = dx32; g.ep.accumulate = c0 > 0 ? 1 : 0;
-            r = pair ? tc2_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, g, st)
-                     : tc_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, mX, mX, g, st);
-            if (r != MOP_OK) return r;
+            if ((r = tc2_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, g, st)) != MOP_OK) return r;
         }
     }
     const size_t n8 = (size_t)N * H / 8;
     const size_t cap = (size_t)p->sm_count * 16;
-    f32_to_bf16_kernel<<<(unsigned)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap), 256, 0, st>>>(
-        reinterpret_cast<const float4*>(dx32), static_cast<uint4*>(dX), n8);
+    pdl_launch(f32_to_bf16_kernel, (unsigned)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap), 256, 0, st, reinterpret_cast<const float4*>(dx32), static_cast<uint4*>(dX), n8);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
 

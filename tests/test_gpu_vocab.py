@@ -113,6 +113,30 @@ def test_vocab_loss_backward_matches_oracle(N, H, V, std):
     assert torch.equal(dX, dX2) and torch.equal(dW, dW2)
 
 
+@pytest.mark.parametrize("N,H,V", [(1500, 2368, 2624),       # 6 and 10 row tiles, blocks of 8 n-tiles and a last one of 3 or 2
+                                   (2304, 128, 8192 + 2112)],  # 9 row tiles, one row tile of X^T that is half empty, two blocks
+                         ids=lambda v: str(v))
+def test_vocab_tile_order_covers_every_tile_once(N, H, V):
+    """Against fp64 on the same device: fp32 sums over H or N, dY rounded once to bf16."""
+    X, W, t = _inputs(N, H, V, seed=N + 9, std=0.05)
+    g = torch.randn((N,), device="cuda") * 0.5 - 1.0
+    loss, lse = torch.full((N,), 7.0, device="cuda"), torch.full((N,), 7.0, device="cuda")
+    binding.mop_vocab_loss_fwd(0, X, W, t, loss, lse)
+    dX = torch.full((N, H), 3.0, device="cuda", dtype=torch.bfloat16)
+    dW = torch.full((H, V), 3.0, device="cuda")
+    binding.mop_vocab_loss_bwd(0, X, W, t, lse, g, dX, dW)
+    z = X.double() @ W.double()
+    ref = torch.logsumexp(z, 1)
+    assert float((lse.double() - ref).abs().max()) < 1e-4 and float((loss.double() - (z.gather(1, t.long()[:, None])[:, 0] - ref)).abs().max()) < 1e-4
+    p = -(z - ref[:, None]).exp()
+    p.scatter_add_(1, t.long()[:, None], torch.ones((N, 1), device="cuda", dtype=torch.float64))
+    p = (p * g.double()[:, None]).to(torch.bfloat16).double()
+    for got, want in ((dX, p @ W.double().T), (dW, X.double().T @ p)):
+        # one bf16 rounding of dX (2^-9 relative per element); a dY that flips its rounding moves single elements by 2^-8 of one term
+        assert float((got.double() - want).norm() / want.norm()) < 4e-3
+        assert float((got.double() - want).abs().max()) < 0.02 * float(want.abs().max())
+
+
 def test_vocab_loss_backward_without_tokens_zeroes_the_weight_gradient():
     X, W, t = _inputs(0, 64, 128, seed=3)
     dW = torch.full((64, 128), 3.0, device="cuda")
