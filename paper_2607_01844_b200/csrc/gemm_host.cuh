@@ -3,6 +3,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_tc2.cuh"
 #include "gemm_tn.cuh"
+#include "gemm_tw.cuh"
 
 namespace mop {
 
@@ -107,6 +108,11 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     return MOP_OK;
 }
 
+// Weight gradients on CTA pairs from 448 rows per expert on (average).  d = 7168, f = 2048, 512 rows: 757 + 1508 us on single
+// CTAs, 682 + 1346 on pairs; d = 2048, f = 1408: 246 + 492 and 258 + 496 at 384 rows, 207 + 397 and 194 + 353 at 2048 (16
+// experts); at 171 rows and d = 7168 1340 + 2660 and 1538 + 3087.
+inline bool tw_wanted(const TcPlan* p) { return p->fwd_tn == 15 && (uint64_t)p->s.T * p->s.k >= 448ull * p->s.E; }
+
 inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st,
                              int* launches, int* ntile_part) {
     const mop_moe_shape& s = p->s;
@@ -127,11 +133,13 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
         if ((r = tc_build_row_tiles(p, a.offsets, tiles, st)) != MOP_OK) return r;
         ++*launches;
     }
+    const bool wpair = tw_wanted(p);
+    const int bch = wpair ? 2 : 4;     // 64-wide chunks of B per copy: half of a tile per CTA of a pair
     CUtensorMap mgH, mdYpB, mXpA, mdGB, mdUB, moWd, moWg, moWu;   // weight gradients
     if (!tc_map_out_f32(p, &moWd, a.dW_down, s.E, s.f, s.d) || !tc_map_out_f32(p, &moWg, a.dW_gate, s.E, s.d, s.f) ||
         !tc_map_out_f32(p, &moWu, a.dW_up, s.E, s.d, s.f) || !tc_map_mn(p, &mgH, a.gH, M, s.f, 2) ||
-        !tc_map_mn(p, &mdYpB, a.dYp, M, s.d, 4) || !tc_map_mn(p, &mXpA, a.Xp, M, s.d, 2) ||
-        !tc_map_mn(p, &mdGB, a.dG, M, s.f, 4) || !tc_map_mn(p, &mdUB, a.dU, M, s.f, 4))
+        !tc_map_mn(p, &mdYpB, a.dYp, M, s.d, bch) || !tc_map_mn(p, &mXpA, a.Xp, M, s.d, 2) ||
+        !tc_map_mn(p, &mdGB, a.dG, M, s.f, bch) || !tc_map_mn(p, &mdUB, a.dU, M, s.f, bch))
         return MOP_ERR_CUDA;
     // tokens-on-M data gradients: K-major weight maps boxed for one CTA (256 N rows) and for a pair CTA (128)
     CUtensorMap mdYpA, mWdK, mWdKp, mdG, mdU, mWgK, mWuK, mWgKp, mWuKp;
@@ -172,18 +180,22 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
     }
     {   // WD: dW_down[e] = (gate H)_e^T dYp_e
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
-        g.tiles_n = ceil_div(s.d, 256); g.tiles_m_fixed = ceil_div(s.f, TC_BM); g.Mfix = s.f; g.N = s.d;
+        g.tiles_n = ceil_div(s.d, 256); g.tiles_m_fixed = ceil_div(s.f, wpair ? 256 : TC_BM); g.Mfix = s.f; g.N = s.d;
         g.a_split = s.f % 64 != 0; g.b_split = s.d % 64 != 0;
         g.ep.outf = a.dW_down; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
-        if ((r = tc_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mgH, mdYpB, mdYpB, moWd, moWd, g, st)) != MOP_OK) return r;
+        r = wpair ? tw_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mdYpB, mdYpB, moWd, moWd, g, st)
+                  : tc_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mgH, mdYpB, mdYpB, moWd, moWd, g, st);
+        if (r != MOP_OK) return r;
         ++*launches;
     }
     {   // WGU: dW_gate[e] = Xp_e^T dG_e and dW_up[e] = Xp_e^T dU_e: per m-block the n-tiles of dW_gate, then those of dW_up
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
-        g.tiles_n = 2 * ceil_div(s.f, 256); g.tiles_m_fixed = ceil_div(s.d, TC_BM); g.Mfix = s.d; g.N = s.f;
+        g.tiles_n = 2 * ceil_div(s.f, 256); g.tiles_m_fixed = ceil_div(s.d, wpair ? 256 : TC_BM); g.Mfix = s.d; g.N = s.f;
         g.a_split = s.d % 64 != 0; g.b_split = s.f % 64 != 0;
         g.ep.outf = a.dW_gate; g.outf1 = a.dW_up; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
-        if ((r = tc_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mXpA, mdGB, mdUB, moWg, moWu, g, st)) != MOP_OK) return r;
+        r = wpair ? tw_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mdGB, mdUB, moWg, moWu, g, st)
+                  : tc_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mXpA, mdGB, mdUB, moWg, moWu, g, st);
+        if (r != MOP_OK) return r;
         ++*launches;
     }
     return MOP_OK;

@@ -167,25 +167,6 @@ __device__ __forceinline__ float2 lds64f(uint32_t addr) {
     return v;
 }
 
-// Bounded wait on a barrier that another CTA of the cluster signals after writing into this CTA's shared memory.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity), "r"(20000u)
-            : "memory");
-        if (ok) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > TC_WAIT_CYCLES) {
-            *abort_flag = 1;
-            atomicCAS(status, 0, code);
-            return false;
-        }
-    }
-}
 // 16 bytes into the shared memory of CTA `rank` of the cluster (at this CTA's address `addr`), then one arrival on its barrier
 __device__ __forceinline__ void publish16(uint32_t addr, uint32_t bar, uint32_t rank, int4 v) {
     asm volatile(

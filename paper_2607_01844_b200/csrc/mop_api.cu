@@ -405,6 +405,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         st = tc_plan_init(&c->plan, *shape, c->sm_count, &c->prof);
         if (st == MOP_OK) st = tc2_init();
         if (st == MOP_OK) st = tn_init();
+        if (st == MOP_OK) st = tw_init();
         if (st == MOP_OK) st = rs_init();
         if (st != MOP_OK) { cudaFree(c->ws); delete c; return st; }
         if (c->fast_route) {

@@ -168,6 +168,35 @@ def test_widths_that_are_multiples_of_8_only_run_on_the_tensor_cores(T, d, E, k,
     assert not [n for n in binding.mop_profile_read(ctx) if n.startswith("scalar")]
 
 
+@pytest.mark.parametrize("T,d,E,k,f", [(1500, 256, 3, 1, 320),      # 500 rows: a tile of 256 whose second CTA is half outside
+                                       (1121, 200, 4, 2, 136),      # widths at every edge of a pair's halves, K tails of any length
+                                       (1344, 64, 3, 1, 64),        # 448 rows, one tile, the second CTA wholly outside
+                                       (1350, 320, 40, 16, 64)],    # many tiles per pair: both accumulators and the stage ring wrap
+                         ids=lambda v: str(v))
+@pytest.mark.parametrize("accumulate", [False, True], ids=["write", "add"])
+def test_weight_gradients_on_cta_pairs(T, d, E, k, f, accumulate):
+    w = synth.small("c4_skew", T=T, d=d, E=E, k=k, f=f, backward=True, skew=E > 4, seed=49)
+    assert w.M >= 448 * E
+    host = synth.make_inputs(w, "cuda")
+    out = []
+    # SCALAR: no tensor core at all, other sums (odd widths); 1CTA: the same sums in the same order
+    for path in (binding.GEMM_AUTO, binding.GEMM_SCALAR if d % 64 or f % 64 else binding.GEMM_TENSOR_1CTA):
+        ctx = binding.context_for(w, gemm_path=path, dw_accumulate=accumulate)
+        buf = binding.LayerBuffers(w)
+        for g in (buf.dW_gate, buf.dW_up, buf.dW_down):
+            g.fill_(0.5)
+        binding.forward(ctx, host, buf)
+        binding.backward(ctx, host, buf)
+        binding.mop_poll(ctx)
+        out.append(buf)
+    for n in ("dW_gate", "dW_up", "dW_down"):
+        a, b = getattr(out[0], n), getattr(out[1], n)
+        if d % 64 or f % 64:    # fp32 sums in another order of bf16 intermediates that may flip their rounding
+            assert rel_fro(a.cpu().numpy(), b.cpu().numpy()) < 1e-3
+        else:
+            assert torch.equal(a, b), n
+
+
 @pytest.mark.parametrize("E,k,T,d,f", [(512, 8, 300, 64, 448),     # one K block per item, 27 items per cluster and more
                                        (400, 4, 500, 640, 512),    # 10 K blocks: items announced one ahead
                                        (160, 2, 700, 1600, 1088)],  # 25 K blocks: announced near the end of the one before
