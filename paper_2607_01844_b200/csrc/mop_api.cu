@@ -43,7 +43,8 @@ struct mop_ctx {
     cudaEvent_t fr_fork, fr_join;
     bf16* fr_pieces;
     float *fr_wrT, *fr_colsq, *fr_xnorm, *fr_scal, *fr_wsq, *fr_z1;
-    int32_t* fr_todo;
+    int32_t *fr_todo, *fr_cnt, *fr_list;
+    uint32_t* fr_pre;
     int fr_rblocks;          // resident blocks of the resolving pass
     // host-buffer entry point scratch
     bf16 *hx, *hXp, *hH, *hYp, *hY, *hG, *hU, *hdY, *hdX;
@@ -78,7 +79,7 @@ constexpr uint32_t GUARD_PATTERN = 0xA5C3A5C3u;
 
 struct Layout {
     size_t z, partial, tiles, status, part, dYp, dG, dU, gH, dXp, dz_sel, dz_row, wrT, rG, rU, rH;
-    size_t fr_pieces, fr_wrT, fr_colsq, fr_xnorm, fr_scal, fr_wsq, fr_todo, fr_z1;
+    size_t fr_pieces, fr_wrT, fr_colsq, fr_xnorm, fr_scal, fr_wsq, fr_todo, fr_cnt, fr_list, fr_pre, fr_z1;
     size_t hx, hXp, hH, hYp, hY, hidx, hcounts, hoffsets, hperm, hsrc, hgate;
     size_t hG, hU, hdY, hdX, hdgate;
     size_t qx, qY, qidx, qgate, qdY, qdX, qdgate;   // second slot of the pipelined host entry points
@@ -135,6 +136,9 @@ Layout make_layout(const mop_moe_shape& s) {
         L.fr_scal = take(256);
         L.fr_wsq = take(E * 4);
         L.fr_todo = take(T * 4 + 16);
+        L.fr_cnt = take((E + 1) * 4);
+        L.fr_list = take(T * E * 4);
+        L.fr_pre = take(T * 32 * 4);
         L.fr_z1 = take(T * E * 4);
     }
     if (s.with_backward) {
@@ -305,7 +309,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         return MOP_ERR_UNSUPPORTED;
     }
     c->tensor_tn = shape->gemm_path != MOP_GEMM_SCALAR && (c->tensor_ok || (prop.major == 10 && c->sm_count >= 2));
-    if (!route_score_init()) { delete c; return MOP_ERR_CUDA; }
+    if (!route_score_init() || !route_chain_init()) { delete c; return MOP_ERR_CUDA; }
     const Layout L = make_layout(*shape);
     c->ws_bytes = L.total;
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }
@@ -323,6 +327,9 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         c->fr_scal = reinterpret_cast<float*>(w + L.fr_scal);
         c->fr_wsq = reinterpret_cast<float*>(w + L.fr_wsq);
         c->fr_todo = reinterpret_cast<int32_t*>(w + L.fr_todo);
+        c->fr_cnt = reinterpret_cast<int32_t*>(w + L.fr_cnt);
+        c->fr_list = reinterpret_cast<int32_t*>(w + L.fr_list);
+        c->fr_pre = reinterpret_cast<uint32_t*>(w + L.fr_pre);
         c->fr_z1 = reinterpret_cast<float*>(w + L.fr_z1);
         c->fast_route = route_fast_wanted(*shape);
     } else if (shape->route_path == MOP_ROUTE_TENSOR) {
@@ -560,18 +567,20 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
         c->launches += 1;
         CUDA_OK(cudaStreamWaitEvent(st, c->fr_join, 0));
         int32_t* stats = reinterpret_cast<int32_t*>(c->fr_scal) + 8;
-        int32_t* n_todo = reinterpret_cast<int32_t*>(c->fr_scal) + 16;
-        CUDA_OK(cudaMemsetAsync(n_todo, 0, 4, st));
+        const RouteLists lists = {c->fr_todo, c->fr_cnt, c->fr_list, c->fr_pre, stats, CHAIN_MIN_PER_SM * c->sm_count};
+        CUDA_OK(cudaMemsetAsync(c->fr_cnt, 0, (s.E + 1) * 4, st));
         const int rblocks = min(ceil_div(s.T, SELF_WARPS), c->fr_rblocks);
         LAUNCH(c, "route_select_screen", st,
                route_select_fast(z, z1, bias, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, topk_idx,
-                                 topk_gate, c->fr_todo, n_todo, stats, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 0,
-                                 rblocks, st));
+                                 topk_gate, lists, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 0, rblocks, st));
+        if ((r = after_launch(c)) != MOP_OK) return r;
+        LAUNCH(c, "route_chain", st,
+               route_chain_kernel<<<c->sm_count * CHAIN_BLOCKS, CHAIN_WARPS * 32, CHAIN_SMEM_BYTES, st>>>(
+                   z, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, c->fr_cnt, c->fr_list, stats, lists.min_listed, s.T, s.d, s.E));
         if ((r = after_launch(c)) != MOP_OK) return r;
         LAUNCH(c, "route_select_resolve", st,
                route_select_fast(z, nullptr, bias, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, topk_idx,
-                                 topk_gate, c->fr_todo, n_todo, stats, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 1,
-                                 rblocks, st));
+                                 topk_gate, lists, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 1, rblocks, st));
         return after_launch(c);
     }
     LAUNCH(c, "route_score", st, route_score(static_cast<const bf16*>(x), W_r, z, s.T, s.d, s.E, c->sm_count, st));

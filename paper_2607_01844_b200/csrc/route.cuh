@@ -349,10 +349,12 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) route_select_kernel(const floa
 // 2. Screening pass, one warp per token: the k largest approximate keys, every key with the interval that
 //    holds its exact value.  If the intervals of adjacent picks are disjoint and no other expert's
 //    interval reaches the weakest pick, the exact keys have the same order and the token is done
-//    (more than nine tenths of the tokens).  The others are listed.  Resolving pass, one warp per listed
-//    token: it evaluates the contract's chain (__fmaf_rn, i ascending, W_r read through its transposed
-//    copy) for the experts in doubt, whose intervals become points and whose keys are the contract's,
-//    writes those logits over z~, and selects again, until nothing that matters overlaps.  Indices and
+//    (more than nine tenths of the tokens when the router is fresh; none of them with the biases of a
+//    heavily skewed one).  The others are listed, and the experts in doubt of each go to that expert's list.
+//    Chain pass: the contract's chain (__fmaf_rn, i ascending, W_r read through its transposed copy) for
+//    every listed pair, 32 tokens of one expert per warp; the exact logits go over z~.  Resolving pass, one
+//    warp per listed token: the evaluated intervals are points now and their keys the contract's; it selects
+//    again, evaluates what is still in doubt, and so on until nothing that matters overlaps.  Indices and
 //    their order are then those of the exact path.
 // 3. Gates are ratios of scores, not an order: a pick keeps its approximate logit unless that could move
 //    its gate by more than 5e-6 relative (score far from saturation), in which case its chain is
@@ -493,21 +495,26 @@ __device__ __forceinline__ float key_error(float zz, float ez, int score_fn, int
     return 1.001f * (s * (1.0f - s) + 0.125f * ez) * ez + 4e-7f + ROUTE_FAST_KEY_ERR;   // |s''| <= 0.1
 }
 
-// One token, one warp.  RESOLVE = false: the screening pass; it returns false, writing nothing, as soon as some
-// order or gate is in doubt.  RESOLVE = true: evaluates the chains in doubt until everything is settled.
+// One token, one warp.  RESOLVE = false: the screening pass; if some order or gate is in doubt it lists the experts
+// whose chains are needed and returns false.  RESOLVE = true: starts with those logits exact, and evaluates the chains
+// still in doubt until everything is settled.
 // Lane l holds the keys of the experts l + 32 q in registers (Q = ceil(E / 32) rounded up to a supported size).
 // zg: E floats (logits); clist: E ints, xs, ws: staging of the chains (RESOLVE only).
+// pair_cnt [E], pair_list [E][T]: tokens listed per expert; pre [T][32]: bit q of word l: expert l + 32 q was listed.
 template <bool RESOLVE, int Q>
 __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t* clist, float* xs, float* ws,
                                             float* __restrict__ z, const float* __restrict__ z1,
                                             const float* __restrict__ bias,
                                             const bf16* __restrict__ x, const float* __restrict__ W_rT,
                                             const float* __restrict__ xnorm, float wmax, int32_t* __restrict__ idx,
-                                            float* __restrict__ gate, int32_t* __restrict__ stats, int d, int E, int k,
-                                            int score_fn, int bias_mode) {
+                                            float* __restrict__ gate, int32_t* __restrict__ stats,
+                                            int32_t* __restrict__ pair_cnt, int32_t* __restrict__ pair_list,
+                                            uint32_t* __restrict__ pre, int T, int d, int E, int k, int score_fn,
+                                            int bias_mode) {
     float* zrow = z + (size_t)t * E;
     float kv[Q];
     uint32_t invalid = 0;                            // slots q of this lane beyond E
+    uint32_t exact = RESOLVE && pre ? pre[(size_t)t * 32 + lane] : 0;       // this lane's experts that carry the chain's logit
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int e = lane + 32 * q;
@@ -520,7 +527,8 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
             }
             const float b = bias_mode ? bias[e] : 0.0f;
             if (bias_mode == 2) zz = __fadd_rn(zz, b);
-            kv[q] = route_key_approx(zz, b, score_fn, bias_mode);
+            kv[q] = RESOLVE && ((exact >> q) & 1u) ? route_key(zz, b, score_fn, bias_mode)
+                                                   : route_key_approx(zz, b, score_fn, bias_mode);
             zg[e] = zz;
         } else {
             invalid |= 1u << q;
@@ -530,7 +538,6 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
     // Bound of this token's logit error (see above).
     const float scale = 5.9604645e-8f * xnorm[t] * wmax;
     const float ez = ROUTE_EPS_C * scale, ez_gate = ROUTE_EPS_GATE_C * scale;
-    uint32_t exact = 0;                              // this lane's experts that carry the chain's logit
     int my_e; float my_key, my_z; uint32_t taken;
     int n_chains = 0, n_bad = 0;
     for (int iter = 0; iter <= k + 1; ++iter) {
@@ -553,7 +560,7 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
                                   ? 1.001f * (0.25f + 0.125f * ez) * ez + 4e-7f + ROUTE_FAST_KEY_ERR : ez;
         float out_hi = -INFINITY;
         int n_c = 0;
-        bool any_cand = false;
+        uint32_t cands = 0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int e = lane + 32 * q;
@@ -570,11 +577,8 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
                     n_c += __popc(m);
                 }
             } else {
-                any_cand |= cand;
+                if (cand) cands |= 1u << q;
             }
-        }
-        if constexpr (!RESOLVE) {
-            if (__any_sync(0xffffffffu, any_cand)) return false;
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) out_hi = fmaxf(out_hi, __shfl_xor_sync(0xffffffffu, out_hi, off));
@@ -588,8 +592,17 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
         const bool need = doubt && !pick_exact;
         const uint32_t m = __ballot_sync(0xffffffffu, need);
         if constexpr (!RESOLVE) {
-            if (m) return false;
-            break;
+            if (!m && !__any_sync(0xffffffffu, cands != 0)) break;
+            for (uint32_t r = m; r; r &= r - 1) {
+                const int e = __shfl_sync(0xffffffffu, my_e, __ffs(r) - 1);
+                if ((e & 31) == lane) cands |= 1u << (e >> 5);
+            }
+            pre[(size_t)t * 32 + lane] = cands;
+            for (uint32_t r = cands; r; r &= r - 1) {
+                const int e = lane + 32 * (__ffs(r) - 1);
+                pair_list[(size_t)e * T + atomicAdd(pair_cnt + e, 1)] = t;
+            }
+            return false;
         }
         if (need) clist[n_c + __popc(m & ((1u << lane) - 1u))] = my_e;
         n_c += __popc(m);
@@ -679,9 +692,9 @@ __device__ __forceinline__ bool route_token(int t, int lane, float* zg, int32_t*
         n_chains += n_c;
         __syncwarp();
     }
-    if (RESOLVE && stats && n_chains > 0) {          // statistics only: no result depends on them
+    if (RESOLVE && stats && n_chains > 0) {
         n_bad = __reduce_add_sync(0xffffffffu, n_bad);
-        if (lane == 0) { atomicAdd(stats, 1); atomicAdd(stats + 1, n_chains); if (n_bad) atomicAdd(stats + 2, n_bad); }
+        if (lane == 0) { atomicAdd(stats + 1, n_chains); if (n_bad) atomicAdd(stats + 2, n_bad); }
     }
     const bool act = lane < k;
     float s;
@@ -720,15 +733,142 @@ template <int Q>
 __global__ void __launch_bounds__(SCREEN_WARPS * 32) route_screen_kernel(
     float* __restrict__ z, const float* __restrict__ z1, const float* __restrict__ bias,
     const float* __restrict__ xnorm, const float* __restrict__ wsq, int32_t* __restrict__ idx, float* __restrict__ gate,
-    int32_t* __restrict__ todo, int32_t* __restrict__ n_todo, int T, int d, int E, int k, int score_fn, int bias_mode) {
+    int32_t* __restrict__ todo, int32_t* __restrict__ n_todo, int32_t* __restrict__ pair_cnt,
+    int32_t* __restrict__ pair_list, uint32_t* __restrict__ pre, int T, int d, int E, int k, int score_fn, int bias_mode) {
     extern __shared__ float sel_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int t = blockIdx.x * SCREEN_WARPS + warp;
     if (t >= T) return;
     const float wmax = route_wmax(wsq, E, lane);
     const bool done = route_token<false, Q>(t, lane, sel_smem + (size_t)warp * E, nullptr, nullptr, nullptr, z, z1, bias,
-                                            nullptr, nullptr, xnorm, wmax, idx, gate, nullptr, d, E, k, score_fn, bias_mode);
+                                            nullptr, nullptr, xnorm, wmax, idx, gate, nullptr, pair_cnt, pair_list, pre, T,
+                                            d, E, k, score_fn, bias_mode);
     if (!done && lane == 0) todo[atomicAdd(n_todo, 1)] = t;
+}
+
+// Chain pass: the listed (token, expert) pairs, 32 tokens of one expert per warp and one chain per lane, so that every
+// element of the expert's row of W_r^T is read once for 32 chains and a step of 8 elements costs 3 shared-memory loads
+// for all of them (evaluating a token's 1 to 4 chains in a warp of its own spends the same loads and steps on 4 lanes,
+// and fetches 28 KB of W_r^T per chain).  Bounded by the rows of x, which come from L2 once per chain.
+// d = 7168, E = 256, 16384 tokens with a skewed router (61 thousand chains, 0.88 GB of rows): 191 us, and 93 for the resolving
+// pass, which took 873 by itself.  Stages of 128 elements: 252; three stages instead of five: 221.
+//
+// From 6 listed tokens per SM on: below that the resolving pass evaluates the chains itself.  d = 7168, E = 256, chain pass +
+// resolving pass against the resolving pass alone, us: 512 tokens 59 + 14 and 72, 1023 tokens 60 + 14 and 96, 4092 tokens
+// 82 + 31 and 278 (d = 2048, E = 64: 24 + 10 and 28, 24 + 10 and 31, 26 + 17 and 68).
+constexpr int CHAIN_MIN_PER_SM = 6;
+constexpr int CHAIN_WARPS = 4;
+constexpr int CHAIN_STAGES = 5;
+constexpr int CHAIN_K = 64;                             // elements per stage
+constexpr int CHAIN_XPITCH = CHAIN_K * 2 + 16;          // bytes per row of x: eight lanes' 16-byte loads meet different banks
+constexpr int CHAIN_STAGE_BYTES = 32 * CHAIN_XPITCH + CHAIN_K * 4;
+constexpr int CHAIN_SMEM_BYTES = CHAIN_WARPS * CHAIN_STAGES * CHAIN_STAGE_BYTES;
+constexpr int CHAIN_BLOCKS = 227 * 1024 / (CHAIN_SMEM_BYTES + 6144);     // resident per SM
+__global__ void __launch_bounds__(CHAIN_WARPS * 32) route_chain_kernel(
+    float* __restrict__ z, const bf16* __restrict__ x, const float* __restrict__ W_rT, const float* __restrict__ xnorm,
+    const float* __restrict__ wsq, const int32_t* __restrict__ pair_cnt, const int32_t* __restrict__ pair_list,
+    int32_t* __restrict__ stats, int min_listed, int T, int d, int E) {
+    extern __shared__ __align__(16) char chain_smem[];
+    __shared__ int32_t first[1025];                      // first tile of 32 pairs of each expert
+    __shared__ int32_t part[CHAIN_WARPS];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (pair_cnt[E] < min_listed) return;                // the resolving pass takes all of them
+    const int per = (E + CHAIN_WARPS * 32 - 1) / (CHAIN_WARPS * 32), e0 = threadIdx.x * per;
+    int tiles = 0, pairs = 0;
+    for (int e = e0; e < min(e0 + per, E); ++e) {
+        const int c = pair_cnt[e];
+        tiles += (c + 31) / 32;
+        pairs += c;
+    }
+    if (stats && blockIdx.x == 0 && pairs > 0) atomicAdd(stats + 1, pairs);
+    int incl = tiles;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    int start = incl - tiles;
+    for (int w = 0; w < warp; ++w) start += part[w];
+    for (int e = e0; e < min(e0 + per, E); ++e) {
+        first[e] = start;
+        start += (pair_cnt[e] + 31) / 32;
+        if (e == E - 1) first[E] = start;
+    }
+    __syncthreads();
+    const int n_tiles = first[E];
+    const float wmax = route_wmax(wsq, E, lane);
+    char* stages = chain_smem + (size_t)warp * CHAIN_STAGES * CHAIN_STAGE_BYTES;
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(stages);
+    const int n_chunks = d / CHAIN_K;                    // d is a multiple of 64 on this path
+    constexpr int PIECES = CHAIN_K / 8, RSTEP = 32 / PIECES;         // 16-byte pieces of a row; rows per copy of the warp
+    const int piece = lane % PIECES;                     // this lane's piece of the rows lane / PIECES + RSTEP u
+    int n_bad = 0;
+    for (int tile = blockIdx.x * CHAIN_WARPS + warp; tile < n_tiles; tile += gridDim.x * CHAIN_WARPS) {
+        int lo = 0, hi = E;                              // the last expert whose first tile is at or before this one
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (first[mid] <= tile) lo = mid; else hi = mid;
+        }
+        const int e = lo, n_e = pair_cnt[e], i = (tile - first[e]) * 32 + lane;
+        const int rows = n_e - (i - lane);               // of this tile; the lanes past them repeat the last one's logit
+        const int t = pair_list[(size_t)e * T + min(i, n_e - 1)];
+        const float* wrow = W_rT + (size_t)e * d;
+        const bf16* xrow[PIECES];
+#pragma unroll
+        for (int u = 0; u < PIECES; ++u)
+            xrow[u] = x + (size_t)__shfl_sync(0xffffffffu, t, lane / PIECES + RSTEP * u) * d + piece * 8;
+        auto fetch = [&](int c) {
+            if (c < n_chunks) {
+                const int i0 = c * CHAIN_K;
+                const uint32_t st = sbase + (c % CHAIN_STAGES) * CHAIN_STAGE_BYTES;
+#pragma unroll
+                for (int u = 0; u < PIECES; ++u)
+                    if (lane / PIECES + RSTEP * u < rows)
+                        cp_async16(st + (lane / PIECES + RSTEP * u) * CHAIN_XPITCH + piece * 16, xrow[u] + i0, true);
+                if (lane < CHAIN_K / 4) cp_async16(st + 32 * CHAIN_XPITCH + lane * 16, wrow + i0 + lane * 4, true);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+#pragma unroll
+        for (int c = 0; c < CHAIN_STAGES - 1; ++c) fetch(c);
+        float acc = 0.0f;
+        for (int c = 0; c < n_chunks; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(CHAIN_STAGES - 2) : "memory");
+            __syncwarp();
+            fetch(c + CHAIN_STAGES - 1);                 // into the stage that was read last time round
+            const char* st = stages + (c % CHAIN_STAGES) * CHAIN_STAGE_BYTES;
+            const uint4* xs = reinterpret_cast<const uint4*>(st + min(lane, rows - 1) * CHAIN_XPITCH);
+            const float4* ws = reinterpret_cast<const float4*>(st + 32 * CHAIN_XPITCH);
+            // the contract's chain: one fused multiply-add per i, i ascending
+            auto step = [&](int j) {
+                const uint4 xv = xs[j];
+                const float4 w0 = ws[2 * j], w1 = ws[2 * j + 1];
+                acc = __fmaf_rn(bf16_lo(xv.x), w0.x, acc);
+                acc = __fmaf_rn(bf16_hi(xv.x), w0.y, acc);
+                acc = __fmaf_rn(bf16_lo(xv.y), w0.z, acc);
+                acc = __fmaf_rn(bf16_hi(xv.y), w0.w, acc);
+                acc = __fmaf_rn(bf16_lo(xv.z), w1.x, acc);
+                acc = __fmaf_rn(bf16_hi(xv.z), w1.y, acc);
+                acc = __fmaf_rn(bf16_lo(xv.w), w1.z, acc);
+                acc = __fmaf_rn(bf16_hi(xv.w), w1.w, acc);
+            };
+#pragma unroll
+            for (int j = 0; j < CHAIN_K / 8; ++j) step(j);
+        }
+        __syncwarp();                                    // the next tile's fetches overwrite the stages
+        if (i < n_e) {
+            float* zp = z + (size_t)t * E + e;
+            if (fabsf(*zp - acc) > 0.5f * ROUTE_EPS_C * (5.9604645e-8f * xnorm[t] * wmax)) ++n_bad;   // the model of the error is checked as we go
+            *zp = acc;
+        }
+    }
+    n_bad = __reduce_add_sync(0xffffffffu, n_bad);
+    if (stats && lane == 0 && n_bad) atomicAdd(stats + 2, n_bad);
+}
+inline bool route_chain_init() {
+    return cudaFuncSetAttribute(route_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CHAIN_SMEM_BYTES) == cudaSuccess;
 }
 
 // Resolving pass: the listed tokens, one warp each, with the staging memory of the chains.
@@ -737,10 +877,11 @@ __global__ void __launch_bounds__(SELF_WARPS * 32) route_resolve_kernel(
     float* __restrict__ z, const float* __restrict__ bias, const bf16* __restrict__ x, const float* __restrict__ W_rT,
     const float* __restrict__ xnorm, const float* __restrict__ wsq, int32_t* __restrict__ idx,
     float* __restrict__ gate, const int32_t* __restrict__ todo, const int32_t* __restrict__ n_todo,
-    int32_t* __restrict__ stats, int d, int E, int k, int score_fn, int bias_mode) {
+    int32_t* __restrict__ stats, uint32_t* __restrict__ pre, int min_listed, int d, int E, int k, int score_fn, int bias_mode) {
     extern __shared__ float sel_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int n = *n_todo;
+    if (stats && n > 0 && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(stats, n);   // statistics only: no result depends on them
     if ((int)blockIdx.x * SELF_WARPS >= n) return;
     float* zg = sel_smem + (size_t)warp * (2 * E + SELF_SMEM_FLOATS);
     int32_t* clist = reinterpret_cast<int32_t*>(zg + E);   // experts whose exact logit is needed
@@ -748,25 +889,36 @@ __global__ void __launch_bounds__(SELF_WARPS * 32) route_resolve_kernel(
     float* ws = xs + SELF_XCHUNK;                           // the same chunk of up to SELF_CAND rows of W_r^T
     const float wmax = route_wmax(wsq, E, lane);
     for (int i = blockIdx.x * SELF_WARPS + warp; i < n; i += gridDim.x * SELF_WARPS) {
-        route_token<true, Q>(todo[i], lane, zg, clist, xs, ws, z, nullptr, bias, x, W_rT, xnorm, wmax, idx, gate, stats, d,
-                             E, k, score_fn, bias_mode);
+        route_token<true, Q>(todo[i], lane, zg, clist, xs, ws, z, nullptr, bias, x, W_rT, xnorm, wmax, idx, gate, stats,
+                             nullptr, nullptr, n < min_listed ? nullptr : pre, 0, d, E, k, score_fn, bias_mode);
         __syncwarp();
     }
 }
 
-// The two passes for the smallest supported Q >= ceil(E / 32).
+// Buffers of the selection that its passes share.
+struct RouteLists {
+    int32_t* todo;           // [T] listed tokens
+    int32_t* pair_cnt;       // [E] listed tokens per expert, then the number of listed tokens: zeroed before the screening
+    int32_t* pair_list;      // [E][T]
+    uint32_t* pre;           // [T][32]
+    int32_t* stats;
+    int min_listed;          // the chain pass runs from this number of listed tokens on
+};
+
+// The screening and the resolving pass for the smallest supported Q >= ceil(E / 32).
 template <int Q>
 inline void route_select_fast_q(float* z, const float* z1, const float* bias, const bf16* x, const float* W_rT, const float* xnorm,
-                                const float* wsq, int32_t* idx, float* gate, int32_t* todo, int32_t* n_todo,
-                                int32_t* stats, int T, int d, int E, int k, int score_fn, int bias_mode, int pass,
-                                int resolve_blocks, cudaStream_t st) {
+                                const float* wsq, int32_t* idx, float* gate, const RouteLists& l, int T, int d, int E, int k,
+                                int score_fn, int bias_mode, int pass, int resolve_blocks, cudaStream_t st) {
     if (pass == 0) {
         route_screen_kernel<Q><<<ceil_div(T, SCREEN_WARPS), SCREEN_WARPS * 32, (size_t)SCREEN_WARPS * E * sizeof(float), st>>>(
-            z, z1, bias, xnorm, wsq, idx, gate, todo, n_todo, T, d, E, k, score_fn, bias_mode);
+            z, z1, bias, xnorm, wsq, idx, gate, l.todo, l.pair_cnt + E, l.pair_cnt, l.pair_list, l.pre, T, d, E, k, score_fn,
+            bias_mode);
     } else {
         const size_t smem = (size_t)SELF_WARPS * (2 * E + SELF_SMEM_FLOATS) * sizeof(float);
-        route_resolve_kernel<Q><<<resolve_blocks, SELF_WARPS * 32, smem, st>>>(z, bias, x, W_rT, xnorm, wsq, idx, gate, todo,
-                                                                                n_todo, stats, d, E, k, score_fn, bias_mode);
+        route_resolve_kernel<Q><<<resolve_blocks, SELF_WARPS * 32, smem, st>>>(z, bias, x, W_rT, xnorm, wsq, idx, gate, l.todo,
+                                                                                l.pair_cnt + E, l.stats, l.pre, l.min_listed, d, E, k, score_fn,
+                                                                                bias_mode);
     }
 }
 // Blocks of the resolving pass that are resident at once: its grid.  Every warp then walks its share of the list;
@@ -789,13 +941,12 @@ inline int route_resolve_resident(int E, int sm_count) {
     return route_resolve_resident_q<32>(E, sm_count);
 }
 inline void route_select_fast(float* z, const float* z1, const float* bias, const bf16* x, const float* W_rT, const float* xnorm,
-                              const float* wsq, int32_t* idx, float* gate, int32_t* todo, int32_t* n_todo, int32_t* stats,
-                              int T, int d, int E, int k, int score_fn, int bias_mode, int pass, int resolve_blocks,
+                              const float* wsq, int32_t* idx, float* gate, const RouteLists& l, int T, int d, int E, int k, int score_fn, int bias_mode, int pass, int resolve_blocks,
                               cudaStream_t st) {
     const int q = ceil_div(E, 32);
 #define MOP_ROUTE_Q(QQ)                                                                                                 \
-    route_select_fast_q<QQ>(z, z1, bias, x, W_rT, xnorm, wsq, idx, gate, todo, n_todo, stats, T, d, E, k, score_fn, bias_mode, \
-                            pass, resolve_blocks, st)
+    route_select_fast_q<QQ>(z, z1, bias, x, W_rT, xnorm, wsq, idx, gate, l, T, d, E, k, score_fn, bias_mode, pass,             \
+                            resolve_blocks, st)
     if (q <= 2) MOP_ROUTE_Q(2);
     else if (q <= 4) MOP_ROUTE_Q(4);
     else if (q <= 8) MOP_ROUTE_Q(8);

@@ -630,6 +630,36 @@ def test_tensor_core_scoring_gives_the_indices_of_the_exact_chains(w):
     assert float((err / eps).max()) < 0.5
 
 
+@pytest.mark.parametrize("w", [
+    synth.small("c4_skew", T=1501, d=64, E=64, k=4, f=64, skew=True, seed=71),              # one stage of the row, experts without pairs
+    synth.small("c4_skew", T=1300, d=448, E=320, k=16, f=64, skew=True, seed=72),           # many experts with a few pairs past a tile
+    synth.small("c2_mid", T=900, d=320, E=1024, k=8, f=64, seed=73),                        # softmax: picks' gates only, E at its largest
+], ids=lambda w: f"T{w.T}d{w.d}E{w.E}k{w.k}s{w.score_fn}")
+def test_tensor_core_scoring_with_most_tokens_in_doubt(w):
+    """Enough listed tokens for the chains to be evaluated expert by expert (one long column of W_r widens the error bound
+    of them all); every pair of a router without weights."""
+    inp = synth.make_inputs(w, "cuda")
+    inp["W_r"][:, 5] *= 64.0
+    for Wr in (inp["W_r"], torch.zeros_like(inp["W_r"])):
+        ctx = binding.context_for(w, route_path=binding.ROUTE_TENSOR)
+        exact = binding.context_for(w, route_path=binding.ROUTE_EXACT)
+        out = []
+        for c in (ctx, exact):
+            idx = torch.empty((w.T, w.k), dtype=torch.int32, device="cuda")
+            gate = torch.empty((w.T, w.k), dtype=torch.float32, device="cuda")
+            binding.mop_moe_route(c, inp["x"], Wr, inp["bias"], idx, gate)
+            binding.mop_poll(c)
+            out.append((idx, gate))
+        assert torch.equal(out[0][0], out[1][0])
+        assert torch.all((out[0][1] - out[1][1]).abs() <= 1e-6 + 1e-5 * out[1][1].abs())
+        tokens, chains, beyond = binding.mop_route_stats(ctx)
+        assert beyond == 0 and chains >= tokens
+        if Wr is inp["W_r"]:
+            assert tokens >= 6 * 148
+        elif not w.bias_mode:
+            assert (tokens, chains) == (w.T, w.T * w.E)
+
+
 def test_tensor_core_scoring_with_equal_and_duplicate_keys():
     """W_r = 0 makes all keys of a token equal (every expert is re-evaluated and the lower ids win); two equal
     columns of W_r make one exact tie per token that only the chain can order."""
