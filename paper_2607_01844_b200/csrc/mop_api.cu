@@ -952,7 +952,7 @@ mop_status mop_moe_layer_fwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const ChunkLayout L = chunk_layout(s, n_chunks, 0);
     char* w = static_cast<char*>(workspace);
-    const int blocks = min(ceil_div(s.T, 8), c->sm_count * 8);
+    const int blocks = min(s.T, c->sm_count * 8);
     c->plan.rows_override = L.cap;
     for (int i = 0; i < n_chunks && r == MOP_OK; ++i) {
         if ((r = chunk_begin(c, L, w, i, n_chunks, x, L.Xp, offsets, perm_row, row_src, true, st)) != MOP_OK) break;
@@ -1003,7 +1003,7 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
     const ChunkLayout L = chunk_layout(s, n_chunks, 1);
     char* w = static_cast<char*>(workspace);
     const int M = s.T * s.k;
-    const int blocks = min(ceil_div(s.T, 8), c->sm_count * 8);
+    const int blocks = min(s.T, c->sm_count * 8);
     c->plan.rows_override = L.cap;
     for (int i = 0; i < n_chunks && r == MOP_OK; ++i) {
         // the chunk's inputs again, and its up-projection recomputed (nothing of the forward was kept)

@@ -16,6 +16,7 @@ CASES = [
     synth.small("c3_trillion", T=600, d=192, E=40, k=8, f=128, backward=True, seed=71),     # sigmoid + bias, 120 rows each
     synth.small("c4_skew", T=1024, d=192, E=16, k=4, f=192, backward=True, seed=72),        # skewed: hot and empty experts
     synth.small("c1_tiny", T=3, d=64, E=5, k=1, f=64, backward=True, seed=73),              # fewer rows than experts
+    synth.small("c1_tiny", T=37, d=1344, E=7, k=3, f=64, backward=True, seed=74),           # rows of one whole segment and a part of one
 ]
 
 
