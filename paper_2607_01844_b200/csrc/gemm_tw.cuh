@@ -116,10 +116,13 @@ tw_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         int stage = 0; uint32_t phase = 0; bool alive = true;
         const uint64_t keep = l2_policy_evict_last();
         TileInfo nxt = decode(min(cluster_id, max(total_tiles - 1, 0)));
+        int expert = -1, ahead = 0;
+        const int rows_total = __ldg(args.offsets + args.E);
         for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
             const TileInfo ti = nxt;
             if (t + n_clusters < total_tiles) nxt = decode(t + n_clusters);
             if (ti.skip) continue;
+            if (ti.e != expert) { expert = ti.e; wgrad_prefetch(args, ti.row0 + ti.rows, rows_total, ahead); }
             const int nb = ti.nt * 256 + 128 * (int)rank;
             const int nkb = (ti.rows + TC_BK - 1) / TC_BK;
             const CUtensorMap* mb = (SEL_B && ti.sel) ? &tmB1 : &tmB0;

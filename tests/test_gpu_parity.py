@@ -171,12 +171,13 @@ def test_widths_that_are_multiples_of_8_only_run_on_the_tensor_cores(T, d, E, k,
 @pytest.mark.parametrize("T,d,E,k,f", [(1500, 256, 3, 1, 320),      # 500 rows: a tile of 256 whose second CTA is half outside
                                        (1121, 200, 4, 2, 136),      # widths at every edge of a pair's halves, K tails of any length
                                        (1344, 64, 3, 1, 64),        # 448 rows, one tile, the second CTA wholly outside
+                                       (1024, 192, 9, 2, 128),      # 228 rows: single CTAs that prefetch, short last expert
                                        (1350, 320, 40, 16, 64)],    # many tiles per pair: both accumulators and the stage ring wrap
                          ids=lambda v: str(v))
 @pytest.mark.parametrize("accumulate", [False, True], ids=["write", "add"])
 def test_weight_gradients_on_cta_pairs(T, d, E, k, f, accumulate):
     w = synth.small("c4_skew", T=T, d=d, E=E, k=k, f=f, backward=True, skew=E > 4, seed=49)
-    assert w.M >= 448 * E
+    assert w.M >= (224 if E == 9 else 448) * E
     host = synth.make_inputs(w, "cuda")
     out = []
     # SCALAR: no tensor core at all, other sums (odd widths); 1CTA: the same sums in the same order
