@@ -201,7 +201,9 @@ __device__ __forceinline__ void tn_write_rows(bf16* __restrict__ dst, int ldo, u
     }
 }
 
-template <int KIND>
+// ONCE: weights pass through L2 as evict-first (tn_stream_weights); a kernel of its own, since copies with a policy, or a choice
+// at each, take 1 to 2 % more where the copies set the pace.
+template <int KIND, bool ONCE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TN_THREADS, 1)
 tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     constexpr int S = TN_STAGES, STAGE_BYTES = TN_STAGE_BYTES;
@@ -330,6 +332,12 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     } else if (warp == 0) {
         // ===================================================================== TMA producer (both CTAs)
         const bool el = elect_one();
+        const uint64_t once = ONCE ? l2_policy_evict_first() : 0;
+        (void)once;
+        auto load_w3 = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
+            if constexpr (ONCE) tma2_load_3d_hint(dst, map, bar, x, y, z, once);
+            else tma2_load_3d(dst, map, bar, x, y, z);
+        };
         int stage = 0; uint32_t phase = 0; bool alive = true;
         Tile ti;
         for (int n = 0; alive && next_item(n, ti); ++n) {
@@ -355,15 +363,17 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                     if (!leader && handout && kb == ask_at) mbar_arrive(signal_bar(n));
                     if (leader) mbar_expect_tx(full_bar(stage), tx);
                     if constexpr (KIND == TN_B4 || KIND == TN_B2) {
-                        tma2_load_3d(sA, ph ? &maps.a1 : &maps.a0, fb, k0, m0, ti.e);   // K-major weights
+                        load_w3(sA, ph ? &maps.a1 : &maps.a0, fb, k0, m0, ti.e);   // K-major weights
                     } else if constexpr (KIND == TN_F1) {                               // N-major weights [E, d, f]
-                        tma2_load_3d(sA, &maps.a0, fb, m0, k0, ti.e);
-                        tma2_load_3d(sA + TN_CHUNK_BYTES, &maps.a1, fb, m0, k0, ti.e);
+                        load_w3(sA, &maps.a0, fb, m0, k0, ti.e);
+                        load_w3(sA + TN_CHUNK_BYTES, &maps.a1, fb, m0, k0, ti.e);
                     } else if (args.a_split) {
-                        tma2_load_3d(sA, &maps.a0, fb, m0, k0, ti.e);
-                        tma2_load_3d(sA + TN_CHUNK_BYTES, &maps.a0, fb, m0 + 64, k0, ti.e);
+                        load_w3(sA, &maps.a0, fb, m0, k0, ti.e);
+                        load_w3(sA + TN_CHUNK_BYTES, &maps.a0, fb, m0 + 64, k0, ti.e);
+                    } else if constexpr (ONCE) {
+                        tma2_load_4d_hint(sA, &maps.a0, fb, 0, k0, m0 >> 6, ti.e, once);   // two chunks in one copy
                     } else {
-                        tma2_load_4d(sA, &maps.a0, fb, 0, k0, m0 >> 6, ti.e);           // two chunks in one copy
+                        tma2_load_4d(sA, &maps.a0, fb, 0, k0, m0 >> 6, ti.e);
                     }
                     tma2_load_2d(sB, mb, fb, k0, brow0);
                 }
@@ -648,7 +658,8 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
 // ------------------------------------------------------------------------------------------ host
 template <int KIND>
 inline bool tn_set_smem() {
-    return cudaFuncSetAttribute(tn_gemm_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) == cudaSuccess;
+    return cudaFuncSetAttribute(tn_gemm_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) == cudaSuccess &&
+           cudaFuncSetAttribute(tn_gemm_kernel<KIND, KIND != TN_F1G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) == cudaSuccess;
 }
 inline mop_status tn_init() {
     return tn_set_smem<TN_F1>() && tn_set_smem<TN_F2>() && tn_set_smem<TN_F1G>() && tn_set_smem<TN_B4>() && tn_set_smem<TN_B2>()
@@ -664,6 +675,16 @@ inline mop_status tn_build_tiles(TcPlan* p, const int32_t* offsets, int32_t* til
     pdl_launch(tn_build_ttiles_kernel, rows128 ? 2 : 1, 1024, 0, st, offsets, p->s.E, tn_table(p, tiles), tiles);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
+}
+
+// Weights that are read by one token tile only need no place in L2: as evict-first lines they leave the activations there, which
+// the next kernels of the layer read.  That is so up to about 256 rows per expert (a second tile reads its weight tile again, from
+// DRAM if it went: 384 rows, d = 2048, f = 1408: up-projection 230 us, evicted first 235; its backward 204 and 211), and pays
+// where the activations fit beside them (d = 7168, 16384 rows: 929 us and 935).  One layer, d = 2048, f = 1408, 64 experts, default
+// policy and evict-first: 6 rows per expert 216 and 206 us, 48 rows 245 and 235, 96 rows 264 and 257, 171 rows 290 and 285.
+inline bool tn_stream_weights(const mop_moe_shape& s) {
+    const uint64_t M = (uint64_t)s.T * s.k;
+    return M <= 240ull * s.E && M * (uint64_t)(s.d + s.f) * 2 <= (96ull << 20);
 }
 
 inline TnArgs tn_base_args(const TcPlan* p, int32_t* tiles, int kind, int32_t* status) {
@@ -689,7 +710,8 @@ inline bool tn_token_maps(const TcPlan* p, CUtensorMap* m, const void* base, uin
 template <int KIND>
 inline mop_status tn_launch(const TcPlan* p, const char* name, const TnMaps& m, const TnArgs& g, cudaStream_t st) {
     p->prof->begin(name, st);
-    pdl_launch(tn_gemm_kernel<KIND>, p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st, m, g);
+    const bool once = KIND != TN_F1G && tn_stream_weights(p->s);
+    pdl_launch(once ? tn_gemm_kernel<KIND, KIND != TN_F1G> : tn_gemm_kernel<KIND, false>, p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st, m, g);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

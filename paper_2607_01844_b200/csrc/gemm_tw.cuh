@@ -22,13 +22,6 @@ constexpr int TW_EPI_WARPS = 8;
 constexpr int TW_THREADS = 64 + 32 * TW_EPI_WARPS;
 constexpr int TW_SMEM_BYTES = TW_STAGES * TW_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + 4 * 16384;
 
-__device__ __forceinline__ void tma2_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
-                                                  uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
-        "[%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy)
-        : "memory");
-}
 __device__ __forceinline__ void tma2_load_2d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, uint64_t policy) {
     asm volatile(
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
