@@ -55,6 +55,10 @@ struct TnMaps {
     CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows
 };
 
+// A tile's columns of the MMA, and the box (index into TnMaps) that holds one CTA's half of them.
+__host__ __device__ constexpr int tn_nmma(int rows) { return (rows + 15) & ~15; }
+__host__ __device__ constexpr int tn_box(int rows) { return ((tn_nmma(rows) >> 1) + 15) / 16 - 1; }
+
 struct TnArgs {
     const int4* ttiles;       // {expert, first row, rows (1..256), position | number of tiles << 16} per token tile
     const int32_t* n_ttiles;  // device scalar
@@ -292,14 +296,13 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         ti.e = v.x; ti.row0 = v.y; ti.rows = v.z; ti.mt = v.w;
         return ti.e >= 0;
     };
-    auto nmma_of = [](int rows) { return (rows + 15) & ~15; };
 
     if (warp == 0 && KIND == TN_F1G) {
         // ============================================ TMA producer with row gather (both CTAs, whole warp)
         int stage = 0; uint32_t phase = 0; bool alive = true;
         Tile ti;
         for (int n = 0; alive && __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
-            const int half = nmma_of(ti.rows) >> 1;                    // token rows per CTA (multiple of 8)
+            const int half = tn_nmma(ti.rows) >> 1;                    // token rows per CTA (multiple of 8)
             const int ngroups = half >> 2;                             // gather4 copies per K block (<= 32)
             const int brow0 = ti.row0 + (int)rank * half;
             const int last = ti.row0 + ti.rows - 1;                    // padding rows repeat the last valid one
@@ -343,10 +346,10 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         for (int n = 0; alive && next_item(n, ti); ++n) {
             // this CTA's half of the token rows, in the smallest box that holds it (what a box fetches past the half belongs
             // to nobody: the MMA reads the half only)
-            const int half = nmma_of(ti.rows) >> 1, box = (half + 15) >> 4;
+            const int half = tn_nmma(ti.rows) >> 1, box = tn_box(ti.rows);
             const int brow0 = ti.row0 + (int)rank * half;
-            const uint32_t tx = 2u * (TN_SUB_BYTES + (uint32_t)box * 2048u);
-            const CUtensorMap* mb = &maps.b[box - 1];
+            const uint32_t tx = 2u * (TN_SUB_BYTES + (uint32_t)(box + 1) * 2048u);
+            const CUtensorMap* mb = &maps.b[box];
             // first weight row of this CTA (F1: 64 gate columns, then the 64 matching up columns)
             const int m0 = KIND == TN_F1 ? ti.mt * 128 + 64 * (int)rank : ti.mt * 256 + 128 * (int)rank;
             for (int kb = 0; kb < nkb; ++kb) {
@@ -358,7 +361,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                 const uint32_t sB = sA + TN_SUB_BYTES;
                 const int ph = (KIND == TN_B4 && kb >= args.kblocks) ? 1 : 0;   // B4: gate phase, then up phase
                 const int k0 = (kb - ph * args.kblocks) * TN_BK;
-                if (KIND == TN_B4 && kb == args.kblocks) mb = &maps.b1[box - 1];
+                if (KIND == TN_B4 && kb == args.kblocks) mb = &maps.b1[box];
                 if (el) {
                     if (!leader && handout && kb == ask_at) mbar_arrive(signal_bar(n));
                     if (leader) mbar_expect_tx(full_bar(stage), tx);
@@ -394,7 +397,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             int stage = 0; uint32_t phase = 0; int it = 0; bool alive = true;
             Tile ti;
             for (int n = 0; alive && next_item(n, ti); ++n) {
-                const uint32_t idesc = idesc0 | ((uint32_t)(nmma_of(ti.rows) >> 3) << 17);
+                const uint32_t idesc = idesc0 | ((uint32_t)(tn_nmma(ti.rows) >> 3) << 17);
                 const int buf = it & 1;
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * 256;
                 if (!mbar_wait(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
@@ -459,7 +462,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             if (!ready) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * 256;
-            const int nmma = nmma_of(rows);
+            const int nmma = tn_nmma(rows);
 
             if constexpr (KIND == TN_F1 || KIND == TN_F1G) {
                 // Lanes 0..63 of the CTA hold gate rows, lanes 64..127 the matching up rows: warp q (gate)
@@ -697,11 +700,12 @@ inline TnArgs tn_base_args(const TcPlan* p, int32_t* tiles, int kind, int32_t* s
     return g;
 }
 
-// Maps of a [rows, cols] bf16 token matrix with boxes of 16, 32, .. 128 rows, as far as a tile can need them: an expert gets a
-// token once, so its tiles have at most T rows, half of them (rounded up to 8) per CTA.
+// Maps of a [rows, cols] bf16 token matrix with boxes of 16, 32, .. 128 rows, as far as a tile can need them.  The caller's tables
+// may give one expert every row (indices that name it more than once for a token included): a tile has up to min(rows, 256) rows,
+// half of them (rounded up to 8) per CTA.
 inline bool tn_token_maps(const TcPlan* p, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
-    const int most = p->s.T < 256 ? p->s.T : 256;
-    const int boxes = (((most + 15) & ~15) / 2 + 15) >> 4;
+    const int most = rows < 256 ? (int)rows : 256;
+    const int boxes = tn_box(most) + 1;
     for (int i = 0; i < boxes; ++i)
         if (!tc_map_2d(p, &m[i], base, rows, cols, 16 * (i + 1))) return false;
     return true;

@@ -168,6 +168,44 @@ def test_widths_that_are_multiples_of_8_only_run_on_the_tensor_cores(T, d, E, k,
     assert not [n for n in binding.mop_profile_read(ctx) if n.startswith("scalar")]
 
 
+@pytest.mark.parametrize("d,f", [(128, 192), (72, 136)], ids=lambda v: str(v))
+@pytest.mark.parametrize("T,E,k,experts", [(16, 8, 8, 1),       # 128 rows of 16 tokens: one tile with a box of 64 rows
+                                           (16, 6, 6, 2),       # 48 rows each
+                                           (3, 32, 31, 1),      # 93 rows of 3 tokens
+                                           (37, 5, 4, 1),       # 148 rows, the last ones of the box past the end
+                                           (200, 4, 4, 1)],     # 800 rows: four tiles
+                         ids=lambda v: str(v))
+def test_experts_named_more_than_once_for_a_token(T, E, k, experts, d, f):
+    """A caller's own indices: an expert may get more rows than there are tokens."""
+    w = synth.small("c1_tiny", T=T, d=d, E=E, k=k, f=f, backward=True, seed=50)
+    host = synth.make_inputs(w, "cpu")
+    inp = to_dev(host)
+    idx = np.random.default_rng(51).integers(0, experts, (T, k)).astype(np.int32) + E - experts
+    gate = np.random.default_rng(52).uniform(0.1, 0.4, (T, k)).astype(np.float32)
+    ctx, b = binding.context_for(w), binding.LayerBuffers(w)
+    b.idx.copy_(torch.from_numpy(idx))
+    b.gate.copy_(torch.from_numpy(gate))
+    binding.mop_moe_permute(ctx, inp["x"], b.idx, b.counts, b.offsets, b.perm_row, b.row_src, b.Xp)
+    binding.mop_moe_expert_ffn_fwd(ctx, b.Xp, b.offsets, b.row_src, b.gate, inp["W_gate"], inp["W_up"], inp["W_down"], b.G, b.U,
+                                   b.H, b.Yp)
+    binding.mop_moe_combine(ctx, b.Yp, b.perm_row, b.Y)
+    binding.backward(ctx, inp, b)
+    binding.mop_poll(ctx)
+    for got, want in zip((b.counts, b.offsets, b.perm_row, b.row_src), oracle.permute(idx, E)):
+        assert np.array_equal(got.cpu().numpy(), want)
+    xb, Wg, Wu, Wd, dYb = (synth.bits(host[n]) for n in ("x", "W_gate", "W_up", "W_down", "dY"))
+    case = f"repeated-T{T}d{d}E{E}k{k}f{f}"
+    check_float("Y", b.Y.float().cpu().numpy(), oracle.ffn_fwd(xb, idx, gate, Wg, Wu, Wd),
+                oracle.ffn_fwd(xb, idx, gate, Wg, Wu, Wd, declared=True), case)
+    exact, declared = (oracle.ffn_bwd_tokens(xb, dYb, idx, gate, Wg, Wu, Wd, declared=v) for v in (False, True))
+    check_float("dX", b.dX.float().cpu().numpy(), exact[0], declared[0], case)
+    check_float("dgate", b.dgate.cpu().numpy(), exact[1], declared[1], case)
+    ex = np.arange(E, dtype=np.int32)
+    exact, declared = (oracle.ffn_bwd_experts(xb, dYb, idx, gate, Wg, Wu, Wd, ex, declared=v) for v in (False, True))
+    for n, e, dd in zip(("dW_gate", "dW_up", "dW_down"), exact, declared):
+        check_float(n, getattr(b, n).cpu().numpy(), e, dd, case)
+
+
 @pytest.mark.parametrize("T,d,E,k,f", [(1500, 256, 3, 1, 320),      # 500 rows: a tile of 256 whose second CTA is half outside
                                        (1121, 200, 4, 2, 136),      # widths at every edge of a pair's halves, K tails of any length
                                        (1344, 64, 3, 1, 64),        # 448 rows, one tile, the second CTA wholly outside
