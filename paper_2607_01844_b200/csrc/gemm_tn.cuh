@@ -205,6 +205,27 @@ __device__ __forceinline__ void tn_write_rows(bf16* __restrict__ dst, int ldo, u
     }
 }
 
+// An epilogue warp's walk over the cluster's items: items n with n % 2 == group are drained, the others passed over.
+// next(n): item n is there; false: none is left, or the wait for it gave up.  wait(n): its accumulator is ready, or the wait gave up.
+// PAIRED: drain(n) meets a partner warp at barriers.  Two warps may see the CTA give up at different items, or one of them while
+// the other sees the end, so neither leaves by itself: vote(ok), a barrier of the two that ANDs their outcomes, is taken once per
+// drained item and once on leaving, and a warp that finds its partner leaving leaves too.
+#pragma nv_exec_check_disable
+template <bool PAIRED, class Next, class Wait, class Vote, class Drain>
+__host__ __device__ __forceinline__ void tn_walk_items(int group, Next next, Wait wait, Vote vote, Drain drain) {
+    for (int n = 0;; ++n) {
+        if (!next(n)) {
+            if constexpr (PAIRED) vote(false);
+            return;
+        }
+        if ((n & 1) != group) continue;
+        bool ready = wait(n);
+        if constexpr (PAIRED) ready = vote(ready);
+        if (!ready) return;
+        drain(n);
+    }
+}
+
 // ONCE: weights pass through L2 as evict-first (tn_stream_weights); a kernel of its own, since copies with a policy, or a choice
 // at each, take 1 to 2 % more where the copies set the pace.
 template <int KIND, bool ONCE>
@@ -438,28 +459,30 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         const uint32_t wb = epi_base + (uint32_t)(warp - 2) * TN_EPI_BYTES;   // this warp's staging
         const uint32_t fo = frag_off(lane);
         const int tpair = 2 * (lane & 3);             // this thread's tokens within a run of 8: tpair, tpair + 1
+        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G;   // a gate warp and its up warp
+        const int pair_bar = 1 + 2 * group + (quarter & 1);
+        const int buf = group;
+        const uint32_t gbuf = wb + 3072;
         Tile ti;
         // (the lanes give up together: a lane that left alone would be missed at the shuffles below)
-        for (int n = 0; __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
-            if ((n & 1) != group) continue;
-            const int buf = group;
-            const int row0 = ti.row0, rows = ti.rows;
+        auto next = [&](int n) { return __all_sync(0xffffffffu, next_item(n, ti)) != 0; };
+        auto wait = [&](int n) {
             // F2, B2: the gates of the tile's tokens (two dependent loads each) are fetched before the wait for the
             // accumulator, so that their latency is hidden behind the main loop
-            const uint32_t gbuf = wb + 3072;
             if constexpr (KIND == TN_F2 || KIND == TN_B2) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int tk = 32 * j + lane;
-                    const float g = tk < rows ? args.ep.gate[args.ep.row_src[row0 + tk]] : 0.0f;
+                    const float g = tk < ti.rows ? args.ep.gate[args.ep.row_src[ti.row0 + tk]] : 0.0f;
                     asm volatile("st.shared.f32 [%0], %1;" ::"r"(gbuf + 4u * tk), "f"(g) : "memory");
                 }
                 __syncwarp();
             }
-            bool ready = mbar_wait_warp(tfull_bar(buf), (uint32_t)(n >> 1) & 1u, abort_flag, args.status, STATUS_WAIT_TMEM_FULL, lane);
-            // the gate warp and its up warp meet at a named barrier below: they give up together or not at all
-            if constexpr (KIND == TN_F1 || KIND == TN_F1G) ready = bar_vote_all(1 + 2 * group + (quarter & 1), 64, ready);
-            if (!ready) break;
+            return mbar_wait_warp(tfull_bar(buf), (uint32_t)(n >> 1) & 1u, abort_flag, args.status, STATUS_WAIT_TMEM_FULL, lane);
+        };
+        auto vote = [&](bool ok) { return bar_vote_all(pair_bar, 64, ok); };
+        tn_walk_items<PAIRED>(group, next, wait, vote, [&](int) {
+            const int row0 = ti.row0, rows = ti.rows;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * 256;
             const int nmma = tn_nmma(rows);
@@ -475,7 +498,6 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                 const uint32_t sb = wb + 2048;                                         // staged rows
                 bf16* stash_out = is_up ? args.ep.out2 : args.ep.out1;
                 const int t_own = is_up ? 16 : 0;
-                const int pair_bar = 1 + 2 * group + (quarter & 1);
 #pragma unroll 1
                 for (int c = 0; c < nmma; c += 32) {
                     float v0[16], v1[16];
@@ -641,7 +663,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_bar(buf) & T2_PEER_MASK);
-        }
+        });
     }
 
     tc_fence_before();

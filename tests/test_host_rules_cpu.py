@@ -49,3 +49,56 @@ int main() {
     return bad != 0;
 }
 """)
+
+
+def test_the_two_warps_of_an_epilogue_pair_leave_together(tmp_path):
+    """The walk over the work items with every pair of points at which the two warps may see the CTA give up (or not at all):
+    neither is ever left waiting at the vote, and both drain the same items."""
+    run_host_program(tmp_path, r"""
+#include "gemm_tn.cuh"
+#include <chrono>
+#include <condition_variable>
+#include <cstdio>
+#include <mutex>
+#include <thread>
+#include <vector>
+using namespace mop;
+struct Vote {                         // a barrier of two that ANDs their outcomes
+    std::mutex m;
+    std::condition_variable cv;
+    int here = 0, round = 0;
+    bool all = true, result[64], hung = false;
+    bool operator()(bool ok) {
+        std::unique_lock<std::mutex> l(m);
+        all = all && ok;
+        const int r = round;
+        if (++here == 2) { here = 0; result[r % 64] = all; all = true; ++round; cv.notify_all(); return result[r % 64]; }
+        if (!cv.wait_for(l, std::chrono::seconds(2), [&] { return round != r || hung; }) || hung) { hung = true; cv.notify_all(); return false; }
+        return result[r % 64];
+    }
+};
+int main() {
+    const int items = 5;              // 0 .. 4, then none left
+    for (int group = 0; group < 2; ++group)
+        for (int a = 0; a <= 9; ++a)
+            for (int b = 0; b <= 9; ++b) {        // the step (waits for items and for accumulators) from which a warp gives up
+                Vote vote;
+                std::vector<int> drained[2];
+                auto warp = [&](int who, int give_up) {
+                    int step = 0;
+                    tn_walk_items<true>(group, [&](int n) { return step++ < give_up && n < items; },
+                                        [&](int) { return step++ < give_up; }, [&](bool ok) { return vote(ok); },
+                                        [&](int n) { drained[who].push_back(n); });
+                };
+                std::thread gate(warp, 0, a), up(warp, 1, b);
+                gate.join();
+                up.join();
+                if (vote.hung || vote.here || drained[0] != drained[1]) {
+                    std::printf("group %d: give-up at steps %d and %d leaves a warp behind\n", group, a, b);
+                    return 1;
+                }
+                if (a == 9 && b == 9 && (int)drained[0].size() != (items + 1 - group) / 2) { std::printf("not drained\n"); return 1; }
+            }
+    return 0;
+}
+""")
