@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(32 * LSE_WARPS) vocab_lse_merge_kernel(const f
     float t = 0.0f;
 #pragma unroll
     for (int w = 0; w < LSE_WARPS; ++w)
-        if (sh[w][lane].y > 0.0f) t += sh[w][lane].y * expf(sh[w][lane].x - m);   // (a warp without tiles holds (-inf, 0))
+        if (w < ntiles) t += sh[w][lane].y * expf(sh[w][lane].x - m);   // (the others hold no tile; a NaN sum has to come through)
     const float l = m + logf(t);
     if (lse) lse[n] = l;
     loss[n] = ylab[n] - l;

@@ -137,6 +137,27 @@ def test_vocab_tile_order_covers_every_tile_once(N, H, V):
         assert float((got.double() - want).abs().max()) < 0.02 * float(want.abs().max())
 
 
+@pytest.mark.parametrize("V,column", [(192, 40),            # one tile: seven of the merging warps hold nothing
+                                      (2624, 300),          # eleven tiles, in the second warp's share
+                                      (2624, 2600)],        # the last tile
+                         ids=lambda v: str(v))
+@pytest.mark.parametrize("value", [float("nan"), float("inf")], ids=["nan", "inf"])
+def test_a_logit_that_is_not_finite_shows_in_the_loss(V, column, value):
+    N, H = 70, 128
+    X, W, t = _inputs(N, H, V, seed=21)
+    t[t == column] = 0
+    W[5, column] = value                       # logits of this column: x[5] times it, so NaN, or infinities of either sign
+    loss, lse = torch.full((N,), 7.0, device="cuda"), torch.full((N,), 7.0, device="cuda")
+    binding.mop_vocab_loss_fwd(0, X, W, t, loss, lse)
+    z = X.double() @ torch.nan_to_num(W.double(), posinf=0.0, nan=0.0)
+    z[:, column] = X[:, 5].double() * value    # (a sum with one term that is not finite is that term)
+    lost = ~(z[:, column] < float("inf"))
+    ref = torch.logsumexp(z, 1)
+    assert int(lost.sum()) > N // 4 and not torch.isfinite(loss[lost]).any() and not torch.isfinite(lse[lost]).any()
+    assert torch.allclose(lse[~lost].double(), ref[~lost], rtol=0, atol=1e-4)
+    assert torch.allclose(loss[~lost].double(), (z.gather(1, t.long()[:, None])[:, 0] - ref)[~lost], rtol=0, atol=1e-4)
+
+
 def test_vocab_loss_backward_without_tokens_zeroes_the_weight_gradient():
     X, W, t = _inputs(0, 64, 128, seed=3)
     dW = torch.full((64, 128), 3.0, device="cuda")
