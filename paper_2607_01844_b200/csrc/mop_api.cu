@@ -850,6 +850,14 @@ mop_status mop_moe_layer_fwd(mop_ctx* c, const void* x, const float* W_r, const 
                              const void* W_up, const void* W_down, int32_t* topk_idx, float* topk_gate, int32_t* counts,
                              int32_t* offsets, int32_t* perm_row, int32_t* row_src, void* Xp, void* G_save, void* U_save,
                              void* H, void* Yp, void* Y, void* stream) {
+    // the arguments of all four calls, before the first one launches
+    if (!c) return MOP_ERR_INVALID_ARG;
+    REQ_PTR_T(x); REQ_PTR(W_r); REQ_PTR_T(topk_idx); REQ_PTR_T(topk_gate);
+    if ((c->s.bias_mode != MOP_BIAS_NONE) != (bias != nullptr)) return MOP_ERR_INVALID_ARG;
+    REQ_PTR(counts); REQ_PTR(offsets); REQ_PTR_T(perm_row); REQ_PTR_T(row_src); REQ_PTR_T(Xp);
+    REQ_PTR(W_gate); REQ_PTR(W_up); REQ_PTR(W_down); REQ_PTR_T(H); REQ_PTR_T(Yp); REQ_PTR_T(Y);
+    if ((G_save == nullptr) != (U_save == nullptr)) return MOP_ERR_INVALID_ARG;
+    if (G_save && (!aligned16(G_save) || !aligned16(U_save))) return MOP_ERR_ALIGN;
     mop_status r;
     if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
     if ((r = mop_moe_permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, stream)) != MOP_OK) return r;

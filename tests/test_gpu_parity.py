@@ -377,6 +377,36 @@ def test_bad_arguments_return_codes():
     assert e.value.code == 1
 
 
+LAYER_OUT = ("idx", "gate", "counts", "offsets", "perm_row", "row_src", "Xp", "G", "U", "H", "Yp", "Y")
+
+
+@pytest.mark.parametrize("name", ("x", "W_r", "W_gate", "W_up", "W_down") + LAYER_OUT)
+def test_forward_in_one_call_checks_every_argument_before_it_launches(name):
+    w = synth.small("c1_tiny", T=24, d=64, E=4, k=2, f=64, backward=True, seed=31)
+    inp = synth.make_inputs(w, "cuda")
+    ctx, b = binding.context_for(w), binding.LayerBuffers(w)
+    tensors = {**{n: inp[n] for n in ("x", "W_r", "W_gate", "W_up", "W_down")}, **{n: getattr(b, n) for n in LAYER_OUT}}
+    for n in LAYER_OUT:
+        tensors[n].fill_(7)
+
+    def call(**changed):
+        a = {**{n: t.data_ptr() for n, t in tensors.items()}, "bias": None, **changed}
+        binding.mop_moe_layer_fwd(ctx, a["x"], a["W_r"], a["bias"], a["W_gate"], a["W_up"], a["W_down"], *(a[n] for n in LAYER_OUT))
+
+    launched = ctx.launch_count
+    for changed, code in (({name: None}, 1), ({name: tensors[name].data_ptr() + 4}, 3), ({"bias": inp["W_r"].data_ptr()}, 1)):
+        with pytest.raises(binding.MopError) as e:
+            call(**changed)
+        assert e.value.code == code
+    torch.cuda.synchronize()
+    assert ctx.launch_count == launched
+    for n in LAYER_OUT:
+        assert bool((tensors[n] == 7).all()), n
+    call(G=None, U=None)                       # no stash: accepted
+    call()
+    binding.mop_poll(ctx)
+
+
 def test_the_step_can_be_captured_into_a_cuda_graph_and_replayed():
     """The device entry points allocate nothing and never synchronise, so a whole step captures."""
     w = synth.small("c2_mid", T=512, d=256, E=16, k=4, f=192, backward=True, seed=29)
