@@ -123,14 +123,14 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                 const int chunk0 = (nt * 256 + (int)rank * half_cols) >> 6;
                 const CUtensorMap* mw = half_cols == 128 ? &tmW2 : &tmW1;
                 for (int kb = u.kb0; kb < u.kb1 && alive; ++kb) {
-                    if (!mbar_wait(emptyA(sa), pa ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
+                    if (!mbar_wait_all(emptyA(sa), pa ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
                     if (el) {
                         if (leader) mbar_expect_tx(fullA(sa), 2 * RS_SLOT);
                         tma2_load_2d(slotA(sa), &tmX, fullA(sa) & T2_PEER_MASK, kb * TC_BK, row0);
                     }
                     if (++sa == RS_SA) { sa = 0; pa ^= 1u; }
                     for (int ph = 0; ph < 3; ++ph) {
-                        if (!mbar_wait(emptyB(sb), pb ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
+                        if (!mbar_wait_all(emptyB(sb), pb ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) { alive = false; break; }
                         if (el) {
                             if (leader) mbar_expect_tx(fullB(sb), 2 * half_cols * TC_BK * 2);
                             // chunked map {64 columns, d rows, E/64 chunks, 3 pieces}
@@ -154,16 +154,16 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
             for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
                 const Unit u = decode(t);
                 const uint32_t idesc = idesc0 | ((uint32_t)(tile_cols(u.nt) >> 3) << 17);
-                if (!mbar_wait(tempty_bar(it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
+                if (!mbar_wait_all(tempty_bar(it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
                                STATUS_WAIT_TMEM_EMPTY)) break;
                 tc_fence_after();
                 uint32_t d_tmem = tmem_base + (uint32_t)(it & 1) * TC_BN;
                 int kseg = 0;                            // K block inside the segment
                 for (int kb = u.kb0; kb < u.kb1 && alive; ++kb) {
-                    if (!mbar_wait(fullA(sa), pa, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
+                    if (!mbar_wait_all(fullA(sa), pa, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
                     const uint64_t da = desc_a | (uint64_t)((slotA(sa) & 0x3ffffu) >> 4);
                     for (int ph = 0; ph < 3; ++ph) {
-                        if (!mbar_wait(fullB(sb), pb, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
+                        if (!mbar_wait_all(fullB(sb), pb, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
                         tc_fence_after();
                         const uint64_t db = desc_b | (uint64_t)((slotB(sb) & 0x3ffffu) >> 4);
                         if (el) {
@@ -182,7 +182,7 @@ route_score_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         if (el) umma2_commit_both(tfull_bar(it & 1));
                         ++it;
                         kseg = 0;
-                        if (!mbar_wait(tempty_bar(it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
+                        if (!mbar_wait_all(tempty_bar(it & 1), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
                                        STATUS_WAIT_TMEM_EMPTY)) { alive = false; break; }
                         tc_fence_after();
                         d_tmem = tmem_base + (uint32_t)(it & 1) * TC_BN;

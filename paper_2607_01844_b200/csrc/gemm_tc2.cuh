@@ -250,7 +250,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
             const int n0 = ti.nt * Tr::N_PER_TILE + (KIND == TC_VP ? args.n_base : 0);
             const int nkb = Tr::PHASES * args.kblocks;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                if (!mbar_wait_all(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
                     alive = false; break;
                 }
                 const uint32_t fb = full_bar(stage) & T2_PEER_MASK;    // the leader's barrier
@@ -295,11 +295,11 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
             for (int t = cluster_id; t < total_tiles && alive; t += n_clusters) {
                 const int buf = it & 1;
                 const uint32_t tphase = (uint32_t)(it >> 1) & 1u;
-                if (!mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
+                if (!mbar_wait_all(tempty_bar(buf), tphase ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * TC_BN;
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) {
+                    if (!mbar_wait_all(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) {
                         alive = false; break;
                     }
                     tc_fence_after();

@@ -364,7 +364,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         };
         int stage = 0; uint32_t phase = 0; bool alive = true;
         Tile ti;
-        for (int n = 0; alive && next_item(n, ti); ++n) {
+        for (int n = 0; alive && __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
             // this CTA's half of the token rows, in the smallest box that holds it (what a box fetches past the half belongs
             // to nobody: the MMA reads the half only)
             const int half = tn_nmma(ti.rows) >> 1, box = tn_box(ti.rows);
@@ -374,7 +374,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             // first weight row of this CTA (F1: 64 gate columns, then the 64 matching up columns)
             const int m0 = KIND == TN_F1 ? ti.mt * 128 + 64 * (int)rank : ti.mt * 256 + 128 * (int)rank;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                if (!mbar_wait_all(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
                     alive = false; break;
                 }
                 const uint32_t fb = full_bar(stage) & T2_PEER_MASK;
@@ -417,14 +417,14 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((A_KMAJOR ? 0u : 1u) << 15) | ((uint32_t)(256 >> 4) << 24);
             int stage = 0; uint32_t phase = 0; int it = 0; bool alive = true;
             Tile ti;
-            for (int n = 0; alive && next_item(n, ti); ++n) {
+            for (int n = 0; alive && __all_sync(0xffffffffu, next_item(n, ti)); ++n) {
                 const uint32_t idesc = idesc0 | ((uint32_t)(tn_nmma(ti.rows) >> 3) << 17);
                 const int buf = it & 1;
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * 256;
-                if (!mbar_wait(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
+                if (!mbar_wait_all(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status, STATUS_WAIT_TMEM_EMPTY)) break;
                 tc_fence_after();
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
+                    if (!mbar_wait_all(full_bar(stage), phase, abort_flag, args.status, STATUS_WAIT_FULL)) { alive = false; break; }
                     tc_fence_after();
                     const uint32_t sA = smem_base + stage * STAGE_BYTES;
                     const uint64_t da = desc_a | (uint64_t)((sA & 0x3ffffu) >> 4);

@@ -120,7 +120,7 @@ tw_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int nkb = (ti.rows + TC_BK - 1) / TC_BK;
             const CUtensorMap* mb = (SEL_B && ti.sel) ? &tmB1 : &tmB0;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
+                if (!mbar_wait_all(empty_bar(stage), phase ^ 1u, abort_flag, args.status, STATUS_WAIT_EMPTY)) {
                     alive = false; break;
                 }
                 const uint32_t sA = smem_base + stage * TW_STAGE_BYTES;
@@ -159,10 +159,9 @@ tw_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int nkb = (ti.rows + TC_BK - 1) / TC_BK;
             const int buf = it & 1;
             const uint32_t d_tmem = tmem_base + (uint32_t)buf * TC_BN;
-            // (the lanes meet again at a tail: they give up together or not at all)
             if (leader) {
-                if (!__all_sync(0xffffffffu, mbar_wait(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
-                                                       STATUS_WAIT_TMEM_EMPTY))) break;
+                if (!mbar_wait_all(tempty_bar(buf), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, args.status,
+                                   STATUS_WAIT_TMEM_EMPTY)) break;
                 tc_fence_after();
             }
             for (int kb = 0; kb < nkb; ++kb) {
@@ -171,8 +170,8 @@ tw_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (valid < TC_BK) {
                     n_k4 = (valid + 15) >> 4;
                     if (valid & 15) {
-                        if (!__all_sync(0xffffffffu, mbar_wait(tail_bar(stage), (tail_phase >> stage) & 1u, abort_flag, args.status,
-                                                               STATUS_WAIT_FULL))) { alive = false; break; }
+                        if (!mbar_wait_all(tail_bar(stage), (tail_phase >> stage) & 1u, abort_flag, args.status,
+                                           STATUS_WAIT_FULL)) { alive = false; break; }
                         tail_phase ^= 1u << stage;
                         clear_tail(stage, valid);
                         if (el) mbar_arrive_cluster(full_bar(stage) & T2_PEER_MASK);

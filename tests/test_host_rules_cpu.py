@@ -1,4 +1,5 @@
 """Host-side rules of the kernels' headers, compiled and run without a device."""
+import re
 import subprocess
 from pathlib import Path
 
@@ -102,3 +103,19 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_warps_that_wait_with_all_lanes_go_on_together():
+    """Rings and parities count warps: a wait that every lane of a warp takes ends in a vote (mbar_wait_all, or an __all_sync of
+    its outcome).  Single lanes wait for themselves in mbar_wait_warp, in the self-test and where one lane hands out the work items."""
+    alone = ("if (lane == 0) ok = mbar_wait(", "limit_cycles);", "if (r >= 0 && !mbar_wait(signal_bar(")
+    for path in sorted(CSRC.glob("*.cuh")):
+        text = path.read_text()
+        for call in re.finditer(r"\b(mbar_wait|mbar_wait_cluster|next_item)\(", text):
+            start, end = text.rfind("\n", 0, call.start()) + 1, text.find("\n", call.end())
+            line, before = text[start:end], text[start:call.start()]
+            if "__forceinline__ bool mbar_wait" in line or "if (!mbar_wait_cluster(item_bar(n)" in line or any(a in line for a in alone):
+                continue                                          # definitions (next_item itself included), single lanes
+            # voted on in place, or in the next statements
+            assert "__all_sync(0xffffffffu, " in before or "if (!__all_sync(0xffffffffu, ok))" in text[end:end + 250], \
+                f"{path.name}: {line.strip()}"
