@@ -105,15 +105,11 @@ __global__ void guard_check_kernel(const char* ws, GuardList g, unsigned long lo
 }
 
 int perm_units(const mop_moe_shape& s) { return ceil_div(s.T * s.k, PERM_SEG); }
-// The tensor-core scoring path needs 64-wide K blocks of x and 64-wide column chunks of W_r.
-bool route_fast_possible(const mop_moe_shape& s) {
-    return s.route_path != MOP_ROUTE_EXACT && s.T > 0 && s.d % 64 == 0 && s.E % 64 == 0 && tc_shape_supported(s.d, s.f);
-}
-// Measured policy: the three-piece GEMM plus the selection with re-evaluation beats the fp32 chains once
-// the scoring is large (configs 3-5: 45-60 GFLOP); small layers keep the chains.
-bool route_fast_wanted(const mop_moe_shape& s) {
-    if (s.route_path == MOP_ROUTE_TENSOR) return true;
-    return 2.0 * s.T * s.d * s.E >= 2e10;
+// The tensor-core scoring path needs 64-wide K blocks of x and 64-wide column chunks of W_r.  AUTO takes it once the scoring is
+// large: small layers keep the fp32 chains, and their contexts hold none of its buffers.
+bool route_fast(const mop_moe_shape& s) {
+    if (s.route_path == MOP_ROUTE_EXACT || s.T <= 0 || s.d % 64 || s.E % 64 || !tc_shape_supported(s.d, s.f)) return false;
+    return s.route_path == MOP_ROUTE_TENSOR || 2.0 * s.T * s.d * s.E >= 2e10;
 }
 int part_tiles(const mop_moe_shape& s) { return ceil_div(s.f, 32); }
 
@@ -128,7 +124,7 @@ Layout make_layout(const mop_moe_shape& s) {
     L.partial = take((size_t)perm_units(s) * E * 4 + 4);
     L.tiles = take(tc_tables_bytes(s.T * s.k, s.E));
     L.status = take(256);
-    if (route_fast_possible(s)) {
+    if (route_fast(s)) {
         L.fr_pieces = take(3 * d * E * 2);
         L.fr_wrT = take(d * E * 4);
         L.fr_colsq = take((size_t)ceil_div(s.d, 32) * E * 4);
@@ -319,7 +315,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
     c->tiles = reinterpret_cast<int32_t*>(w + L.tiles);
     c->status = reinterpret_cast<int32_t*>(w + L.status);
     c->fast_route = false;
-    if (route_fast_possible(*shape) && prop.major == 10) {
+    if (route_fast(*shape) && prop.major == 10) {
         c->fr_pieces = reinterpret_cast<bf16*>(w + L.fr_pieces);
         c->fr_wrT = reinterpret_cast<float*>(w + L.fr_wrT);
         c->fr_colsq = reinterpret_cast<float*>(w + L.fr_colsq);
@@ -331,7 +327,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         c->fr_list = reinterpret_cast<int32_t*>(w + L.fr_list);
         c->fr_pre = reinterpret_cast<uint32_t*>(w + L.fr_pre);
         c->fr_z1 = reinterpret_cast<float*>(w + L.fr_z1);
-        c->fast_route = route_fast_wanted(*shape);
+        c->fast_route = true;
     } else if (shape->route_path == MOP_ROUTE_TENSOR) {
         cudaFree(c->ws); delete c;
         return MOP_ERR_UNSUPPORTED;

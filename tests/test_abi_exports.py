@@ -52,3 +52,12 @@ def test_argument_checks_need_no_device(lib):
     assert lib.mop_status_string(7) == b"device-side wait ran out"
     assert lib.mop_moe_combine(None, None, None, None, None) == 1
     assert lib.mop_launch_count(None) == 0
+
+
+@pytest.mark.parametrize("T,d,E,k,f,tensor", [(256, 256, 64, 2, 512, False), (4096, 2048, 64, 6, 1408, False),
+                                              (16384, 7168, 256, 8, 2048, True)], ids=lambda v: str(v))
+def test_only_layers_that_score_on_the_tensor_cores_hold_its_buffers(lib, T, d, E, k, f, tensor):
+    from paper_2607_01844_b200.binding import ROUTE_AUTO, ROUTE_EXACT, ROUTE_TENSOR, MopShape
+    auto, exact, forced = (lib.mop_workspace_bytes(ctypes.byref(MopShape(T, d, E, k, f, 0, 0, 0, 0, 0, 0, path)))
+                           for path in (ROUTE_AUTO, ROUTE_EXACT, ROUTE_TENSOR))
+    assert exact < forced and auto == (forced if tensor else exact)
