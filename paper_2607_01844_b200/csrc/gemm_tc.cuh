@@ -12,7 +12,7 @@
 //   VP   dY = g ([v = t] - exp(X W_voc - lse))     bf16, one block of vocabulary columns dense M
 //   VX   dX += dY W_voc^T over that block          fp32 read-modify-write              dense M
 //   VW   dW_voc[:, block] = X^T dY                 fp32 store                          dense M
-// (the V kinds on the two-CTA kernel of gemm_tc2.cuh only)
+// (the V kinds on the two-CTA kernel of gemm_tc2.cuh only; with few tokens dW_voc is a WD of one expert)
 // CTA tile 128 x 256 (one tcgen05.mma.cta_group::1 of M=128, N=256, K=16 per 32 bytes of K),
 // K step 64 per pipeline stage, 4 stages, two 256-column accumulators in TMEM so that the
 // epilogue of tile i overlaps the main loop of tile i+1.
@@ -912,13 +912,14 @@ __global__ void __launch_bounds__(32 * LSE_WARPS) vocab_lse_merge_kernel(const f
     loss[n] = ylab[n] - l;
 }
 
-// Row tiles of the dense GEMMs (256 rows per CTA pair) and a clean status word, in one launch.
+// Row tiles of the dense GEMMs (256 rows per CTA pair), the row range {0, N} as the offsets of one expert (words 32 and 33 of the
+// table), and a clean status word, in one launch.
 __global__ void __launch_bounds__(256) vocab_setup_kernel(int N, int4* __restrict__ tiles, int32_t* __restrict__ n_tiles,
                                                           int32_t* __restrict__ status) {
     pdl_begin();
     const int nt = (N + 255) / 256;
     for (int i = threadIdx.x; i < nt; i += blockDim.x) tiles[i] = make_int4(0, 256 * i, min(256, N - 256 * i), 0);
-    if (threadIdx.x == 0) { *n_tiles = nt; *status = 0; }
+    if (threadIdx.x == 0) { *n_tiles = nt; n_tiles[32] = 0; n_tiles[33] = N; *status = 0; }
 }
 
 // fp32 -> bf16 of a dense array (8 elements per thread; n a multiple of 8)
@@ -1077,11 +1078,13 @@ inline bool tc_map_chunked_2d_pitch(const TcPlan* p, CUtensorMap* m, const void*
                                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 3-D map over a dense [E, rows, cols] fp32 tensor for stores; box = {32 cols, 128 rows, 1}.
+// 3-D map over a dense [E, rows, cols] fp32 tensor for stores, or over `cols` columns of one whose rows are `pitch` elements
+// apart; box = {32 cols, 128 rows, 1}.
 inline bool tc_map_out_f32(const TcPlan* p, CUtensorMap* m, const void* base, uint64_t E, uint64_t rows,
-                           uint64_t cols) {
+                           uint64_t cols, uint64_t pitch = 0) {
+    if (pitch == 0) pitch = cols;
     const cuuint64_t dims[3] = {cols, rows, E};
-    const cuuint64_t strides[2] = {cols * 4, rows * cols * 4};
+    const cuuint64_t strides[2] = {pitch * 4, rows * pitch * 4};
     const cuuint32_t box[3] = {32, 128, 1};
     const cuuint32_t es[3] = {1, 1, 1};
     return reinterpret_cast<tc_encode_fn>(p->encode)(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base),

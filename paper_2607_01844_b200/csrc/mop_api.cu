@@ -1419,7 +1419,14 @@ VocabLayout vocab_layout(int N, int V) {
 }
 // n-tiles per block of the tile order (see tc_gemm2_kernel).  N = 8192, H = 7168, V = 131072 forward and backward: 51.3 ms with 1
 // (row tiles fastest), 50.6 with 4, 48.5 with 8, 49.4 with 16; 55.0 before, with the weight gradient and the forward on one CTA.
+// Elsewhere the orders lie within the runs' spread (N 256 to 2048, H 1024 and 2048, V 32000 and 50304: 1 %), but for few row tiles
+// of a large matrix: N = 2048, H = 7168, V = 131072 takes 2.53 + 9.7 ms with 1 and 2.59 + 10.2 with 8.
 constexpr int VOCAB_N_GROUP = 8;
+// Weight gradient: up to this many tokens (its K) on single CTAs with TMA tile stores, on CTA pairs above.  With few tokens the
+// fp32 stores set the pace, and the pairs' epilogue writes rows by lane.  Whole backward, us, single CTAs and pairs: N 256, H 2048,
+// V 32000 357 and 458; 512, 4096, 65536 965 and 1255; 777, 1024, 50304 587 and 636; 1024, 7168, 131072 4880 to 5530 and 5510 to
+// 5540 (clocks differ from run to run under the power cap); 4096, 2048, 65536 2750 and 2500; 8192, 7168, 65536 20900 and 18900.
+constexpr int VOCAB_WGRAD_FEW = 1024;
 std::mutex g_vocab_mutex;
 TcPlan g_vocab_plan[kMaxDevices];
 Profiler g_vocab_prof;           // never enabled: the plan needs one
@@ -1576,10 +1583,12 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
     if (!tc_map_2d(p, &mX, X, N, H, 128) || !tc_map_chunked_2d(p, &mXT, X, N, H, 2) ||
         !tc_map_chunked_3d(p, &mWn, W_voc, 1, H, V, 2) || !tc_map_3d(p, &mWk, W_voc, 1, H, V, 128))
         return MOP_ERR_CUDA;
+    const bool few = N <= VOCAB_WGRAD_FEW;
     for (int c0 = 0; c0 < V; c0 += L.vc) {
         const int cw = V - c0 < L.vc ? V - c0 : L.vc;
-        CUtensorMap mdYk, mdYn;
-        if (!tc_map_2d_pitch(p, &mdYk, dY, N, cw, L.vc, 128) || !tc_map_chunked_2d_pitch(p, &mdYn, dY, N, cw, L.vc, 2))
+        CUtensorMap mdYk, mdYn, mOut;
+        if (!tc_map_2d_pitch(p, &mdYk, dY, N, cw, L.vc, 128) || !tc_map_chunked_2d_pitch(p, &mdYn, dY, N, cw, L.vc, few ? 4 : 2) ||
+            (few && !tc_map_out_f32(p, &mOut, dW_voc + c0, 1, H, cw, V)))
             return MOP_ERR_CUDA;
         TcArgs base{};
         base.n_mtiles = tiles; base.n_group = VOCAB_N_GROUP; base.mtiles = reinterpret_cast<const int4*>(tiles + 64);
@@ -1592,9 +1601,16 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
         }
         {   // dW[:, block] = X^T dY (K = the N tokens), written once
             TcArgs g = base;
-            g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, 256); g.Mfix = H; g.N = cw; g.kblocks = ceil_div(N, TC_BK);
-            g.ep.outf = dW_voc + c0; g.ep.ldo = V;
-            if ((r = tc2_launch<TC_VW>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, g, st)) != MOP_OK) return r;
+            g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, few ? TC_BM : 256); g.Mfix = H; g.N = cw;
+            g.ep.outf = dW_voc + c0;
+            if (few) {
+                g.offsets = tiles + 32;
+                r = tc_launch<TC_WD>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, mOut, mOut, g, st);
+            } else {
+                g.kblocks = ceil_div(N, TC_BK); g.ep.ldo = V;
+                r = tc2_launch<TC_VW>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, g, st);
+            }
+            if (r != MOP_OK) return r;
         }
         {   // dX += dY W[:, block]^T in fp32 across the blocks
             TcArgs g = base;

@@ -137,6 +137,14 @@ def test_vocab_tile_order_covers_every_tile_once(N, H, V):
         assert float((got.double() - want).abs().max()) < 0.02 * float(want.abs().max())
 
 
+@pytest.mark.parametrize("N,H,V", [(37, 320, 8192 + 64),        # a K tail, a row tile that is half empty, a last block of one chunk
+                                   (1024, 192, 8192 + 320),     # the most tokens of the one-CTA weight gradient
+                                   (1025, 192, 8192 + 320)],    # the fewest of the two-CTA one
+                         ids=lambda v: str(v))
+def test_vocab_weight_gradient_with_few_and_with_many_tokens(N, H, V):
+    test_vocab_tile_order_covers_every_tile_once(N, H, V)
+
+
 @pytest.mark.parametrize("V,column", [(192, 40),            # one tile: seven of the merging warps hold nothing
                                       (2624, 300),          # eleven tiles, in the second warp's share
                                       (2624, 2600)],        # the last tile
