@@ -548,10 +548,11 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
         LAUNCH(c, "route_prep", st,
                route_prep_kernel<<<gp, 256, 0, st>>>(W_r, c->fr_pieces, c->fr_wrT, c->fr_colsq, s.d, s.E));
         if ((r = after_launch(c)) != MOP_OK) return r;
-        // only the selection needs the norms of x's rows and of W_r's columns: they run on a side stream beside
-        // the logit GEMM (which leaves room on every SM for such blocks, and DRAM idle)
+        // only the selection needs the norms of x's rows and of W_r's columns, and empty lists: they run on a side stream
+        // beside the logit GEMM (which leaves room on every SM for such blocks, and DRAM idle)
         CUDA_OK(cudaEventRecord(c->fr_fork, st));
         CUDA_OK(cudaStreamWaitEvent(c->fr_stream, c->fr_fork, 0));
+        CUDA_OK(cudaMemsetAsync(c->fr_cnt, 0, (s.E + 1) * 4, c->fr_stream));
         route_wnorm_kernel<<<ceil_div(s.E, 8), 256, 0, c->fr_stream>>>(c->fr_colsq, c->fr_wsq, ceil_div(s.d, 32), s.E);
         route_xnorm_kernel<<<ceil_div(s.T, 8), 256, 0, c->fr_stream>>>(static_cast<const bf16*>(x), c->fr_xnorm, s.T, s.d);
         CUDA_OK(cudaEventRecord(c->fr_join, c->fr_stream));
@@ -564,15 +565,15 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
         CUDA_OK(cudaStreamWaitEvent(st, c->fr_join, 0));
         int32_t* stats = reinterpret_cast<int32_t*>(c->fr_scal) + 8;
         const RouteLists lists = {c->fr_todo, c->fr_cnt, c->fr_list, c->fr_pre, stats, CHAIN_MIN_PER_SM * c->sm_count};
-        CUDA_OK(cudaMemsetAsync(c->fr_cnt, 0, (s.E + 1) * 4, st));
         const int rblocks = min(ceil_div(s.T, SELF_WARPS), c->fr_rblocks);
         LAUNCH(c, "route_select_screen", st,
                route_select_fast(z, z1, bias, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, topk_idx,
                                  topk_gate, lists, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 0, rblocks, st));
         if ((r = after_launch(c)) != MOP_OK) return r;
         LAUNCH(c, "route_chain", st,
-               route_chain_kernel<<<c->sm_count * CHAIN_BLOCKS, CHAIN_WARPS * 32, CHAIN_SMEM_BYTES, st>>>(
-                   z, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, c->fr_cnt, c->fr_list, stats, lists.min_listed, s.T, s.d, s.E));
+               pdl_launch(route_chain_kernel, c->sm_count * CHAIN_BLOCKS, CHAIN_WARPS * 32, CHAIN_SMEM_BYTES, st, z,
+                          static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, c->fr_cnt, c->fr_list, stats,
+                          lists.min_listed, s.T, s.d, s.E));
         if ((r = after_launch(c)) != MOP_OK) return r;
         LAUNCH(c, "route_select_resolve", st,
                route_select_fast(z, nullptr, bias, static_cast<const bf16*>(x), c->fr_wrT, c->fr_xnorm, c->fr_wsq, topk_idx,

@@ -756,6 +756,9 @@ __global__ void __launch_bounds__(SCREEN_WARPS * 32) route_screen_kernel(
 // From 6 listed tokens per SM on: below that the resolving pass evaluates the chains itself.  d = 7168, E = 256, chain pass +
 // resolving pass against the resolving pass alone, us: 512 tokens 59 + 14 and 72, 1023 tokens 60 + 14 and 96, 4092 tokens
 // 82 + 31 and 278 (d = 2048, E = 64: 24 + 10 and 28, 24 + 10 and 31, 26 + 17 and 68).
+// With few listed tokens it is an empty launch more: the two passes are dependent launches, and the lists are emptied beside the
+// logit GEMM, so that the whole router costs no more than without it (T 3000, d 7168, E 512: 153 us without, 156 with plain
+// launches, 149 so; T 1024, E 1024: 180, 192 and 182; T 8192, E 192: 144, 143 and 136).
 constexpr int CHAIN_MIN_PER_SM = 6;
 constexpr int CHAIN_WARPS = 4;
 constexpr int CHAIN_STAGES = 5;
@@ -768,6 +771,7 @@ __global__ void __launch_bounds__(CHAIN_WARPS * 32) route_chain_kernel(
     float* __restrict__ z, const bf16* __restrict__ x, const float* __restrict__ W_rT, const float* __restrict__ xnorm,
     const float* __restrict__ wsq, const int32_t* __restrict__ pair_cnt, const int32_t* __restrict__ pair_list,
     int32_t* __restrict__ stats, int min_listed, int T, int d, int E) {
+    pdl_begin();
     extern __shared__ __align__(16) char chain_smem[];
     __shared__ int32_t first[1025];                      // first tile of 32 pairs of each expert
     __shared__ int32_t part[CHAIN_WARPS];
@@ -878,6 +882,7 @@ __global__ void __launch_bounds__(SELF_WARPS * 32) route_resolve_kernel(
     const float* __restrict__ xnorm, const float* __restrict__ wsq, int32_t* __restrict__ idx,
     float* __restrict__ gate, const int32_t* __restrict__ todo, const int32_t* __restrict__ n_todo,
     int32_t* __restrict__ stats, uint32_t* __restrict__ pre, int min_listed, int d, int E, int k, int score_fn, int bias_mode) {
+    pdl_begin();
     extern __shared__ float sel_smem[];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int n = *n_todo;
@@ -916,9 +921,8 @@ inline void route_select_fast_q(float* z, const float* z1, const float* bias, co
             bias_mode);
     } else {
         const size_t smem = (size_t)SELF_WARPS * (2 * E + SELF_SMEM_FLOATS) * sizeof(float);
-        route_resolve_kernel<Q><<<resolve_blocks, SELF_WARPS * 32, smem, st>>>(z, bias, x, W_rT, xnorm, wsq, idx, gate, l.todo,
-                                                                                l.pair_cnt + E, l.stats, l.pre, l.min_listed, d, E, k, score_fn,
-                                                                                bias_mode);
+        pdl_launch(route_resolve_kernel<Q>, resolve_blocks, SELF_WARPS * 32, smem, st, z, bias, x, W_rT, xnorm, wsq, idx, gate, l.todo,
+                   l.pair_cnt + E, l.stats, l.pre, l.min_listed, d, E, k, score_fn, bias_mode);
     }
 }
 // Blocks of the resolving pass that are resident at once: its grid.  Every warp then walks its share of the list;
