@@ -103,8 +103,9 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        # the current stream's handle without building a Stream object around it (3 us of a small layer's 50)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # the current stream's handle without building a Stream object around it (3 us of a small layer's 50), where torch has it
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

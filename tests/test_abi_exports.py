@@ -61,3 +61,15 @@ def test_only_layers_that_score_on_the_tensor_cores_hold_its_buffers(lib, T, d, 
     auto, exact, forced = (lib.mop_workspace_bytes(ctypes.byref(MopShape(T, d, E, k, f, 0, 0, 0, 0, 0, 0, path)))
                            for path in (ROUTE_AUTO, ROUTE_EXACT, ROUTE_TENSOR))
     assert exact < forced and auto == (forced if tensor else exact)
+
+
+def test_the_current_stream_without_torchs_private_accessor(monkeypatch):
+    import types
+
+    import torch
+
+    from paper_2607_01844_b200 import binding
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    assert binding._stream(None) == 77
