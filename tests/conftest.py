@@ -14,10 +14,11 @@ def pytest_configure(config):
 
 
 def pytest_terminal_summary(terminalreporter):
-    """Realised float errors of the GPU parity checks: written to parity_errors.json in the output folder and summarised."""
+    """Realised float errors of the GPU parity checks: written to parity_errors.json in the run's cache directory and summarised."""
     sys.path.insert(0, str(Path(__file__).resolve().parent))
     import parity_util
-    table = parity_util.dump()
+    cache = getattr(terminalreporter.config, "cache", None)
+    table = parity_util.dump(cache.mkdir("parity") / "parity_errors.json" if cache else None)
     if table:
         terminalreporter.write_sep("-", "realised parity errors (worst case per tensor)")
         terminalreporter.write_line(table)

@@ -165,7 +165,8 @@ def test_widths_that_are_multiples_of_8_only_run_on_the_tensor_cores(T, d, E, k,
     inp = to_dev(host)
     binding.forward(ctx, inp, buf)
     binding.backward(ctx, inp, buf)
-    assert not [n for n in binding.mop_profile_read(ctx) if n.startswith("scalar")]
+    names = binding.mop_profile_read(ctx)
+    assert {"gemm_up_swiglu", "gemm_wgrad_down"} <= set(names) and not [n for n in names if n.startswith("scalar")]
 
 
 @pytest.mark.parametrize("d,f", [(128, 192), (72, 136)], ids=lambda v: str(v))
@@ -560,7 +561,7 @@ def test_router_backward_matches_oracle(w):
 
 @pytest.mark.parametrize("T,d,E,k", [(100, 328, 160, 4),      # 16 warps per block of dW_r, the last block of columns partly filled
                                      (150, 264, 300, 3),      # 8 warps, experts with fewer rows than warps
-                                     (900, 264, 300, 7)],     # 8 warps, more rows than four per warp
+                                     (900, 264, 300, 7)],     # 8 warps, up to 40 rows per expert: more than four per warp for some
                          ids=lambda v: str(v))
 def test_router_backward_with_many_blocks_matches_oracle(T, d, E, k):
     test_router_backward_matches_oracle(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=64, bias_mode=2, backward=True, seed=34))
@@ -630,8 +631,9 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
 
 
 @pytest.mark.parametrize("T,d,E", [(17, 72, 9), (16, 64, 8),          # one chain per thread, tile edges of 16 x 8
-                                   (4100, 136, 33), (4096, 64, 64),    # 32 x 32 and 64 x 32 tiles, W rows at every alignment
-                                   (9000, 200, 34), (12000, 72, 127), (8200, 64, 260)])   # 64 x 64 tiles
+                                   (2001, 136, 33), (2001, 72, 62), (1984, 64, 64),       # 32 x 32 tiles, W rows at every alignment
+                                   (4100, 136, 33), (4096, 64, 64), (8200, 64, 260),       # 64 x 32 tiles
+                                   (9000, 200, 34), (12000, 72, 127)])                     # 64 x 64 tiles
 def test_exact_scoring_shapes_give_the_contract_chains(T, d, E):
     w = synth.small("c2_mid", T=T, d=d, E=E, k=2, f=64, seed=48)
     inp = synth.make_inputs(w, "cuda")
