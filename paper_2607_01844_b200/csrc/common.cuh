@@ -21,8 +21,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&p);
 }
 
-__device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-
 __device__ __forceinline__ float sigmoidf_acc(float v) { return 1.0f / (1.0f + expf(-v)); }
 // Sigmoid of the SwiGLU epilogues: fast exponential and division (about 2 ulp), far inside the bf16
 // rounding of every value it feeds; all GEMM schedules share it, so they stay bit-identical.  (The

@@ -163,8 +163,8 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
         g.tiles_n = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TC_BK); g.N = s.f;
         g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH; g.ep.in0 = a.G_save; g.ep.in1 = a.U_save; g.ep.in2 = a.H;
         g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
-        if ((r = tc_rows_gemm<TC_B2>(p, "gemm_dgrad_down_dswiglu", "gemm_dgrad_down_dswiglu_2cta", mdYpA, mdYpA, mWdK, mWdK, mWdKp, mWdKp, g, tiles, st,
-                                     launches)) != MOP_OK)
+        if ((r = tc_rows_gemm<TC_B2>(p, "gemm_dgrad_down_dswiglu", "gemm_dgrad_down_dswiglu_2cta", mdYpA, mdYpA, mWdK, mWdK, mWdKp,
+                                     mWdKp, g, tiles, st, launches)) != MOP_OK)
             return r;
     }
     if (p->fwd_tn & 4) {   // B4 on the tokens-on-N kernel
@@ -198,7 +198,10 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
         g.tiles_n = 2 * ceil_div(s.f, 256); g.tiles_m_fixed = ceil_div(s.d, wpair ? 256 : TC_BM); g.Mfix = s.d; g.N = s.f;
         g.a_split = s.d % 64 != 0; g.b_split = s.f % 64 != 0;
         g.ep.outf = a.dW_gate; g.outf1 = a.dW_up; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
-        if (prefetch) { g.pf[0] = a.Xp; g.pf_bytes[0] = s.d * 2; g.pf[1] = a.dG; g.pf[2] = a.dU; g.pf_bytes[1] = g.pf_bytes[2] = s.f * 2; }
+        if (prefetch) {
+            g.pf[0] = a.Xp; g.pf[1] = a.dG; g.pf[2] = a.dU;
+            g.pf_bytes[0] = s.d * 2; g.pf_bytes[1] = g.pf_bytes[2] = s.f * 2;
+        }
         r = wpair ? tw_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mdGB, mdUB, moWg, moWu, g, st)
                   : tc_launch<TC_WGU>(p, "gemm_wgrad_gate_up", mXpA, mXpA, mdGB, mdUB, moWg, moWu, g, st);
         if (r != MOP_OK) return r;

@@ -1,5 +1,6 @@
-// Scalar (CUDA-core) grouped GEMM: the on-device cross-check of the tensor-core kernels (gemm_path SCALAR).  bf16 operands, fp32 accumulation, any operand strides, ragged M (rows of an
-// expert) or ragged K (weight gradients), same epilogues as the tensor-core path.
+// Scalar (CUDA-core) grouped GEMM: the on-device cross-check of the tensor-core kernels (gemm_path SCALAR).  bf16 operands, fp32
+// accumulation, any operand strides, ragged M (rows of an expert) or ragged K (weight gradients), same epilogues as the
+// tensor-core path.
 #pragma once
 #include "epilogue.cuh"
 

@@ -245,12 +245,7 @@ __device__ __forceinline__ void wgrad_prefetch(const TcArgs& args, int row_end, 
             asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(base + o) : "memory");
     }
 }
-// shared -> global tile store (or fp32 add) of one box; completion is tracked by bulk groups
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(map),
-                 "r"(src), "r"(x), "r"(y), "r"(z)
-                 : "memory");
-}
+// fp32 add of one box into a global tile; completion is tracked by bulk groups, as of the store above
 __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
     asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
                      map),
@@ -939,7 +934,7 @@ struct TcPlan {
     void* encode;   // cuTensorMapEncodeTiled
     int pairs;      // schedule of the token-row kinds (see gemm_host.cuh)
     long long rows_override;   // > 0: the row buffers of this call hold this many rows (an expert chunk), not T*k
-    int fwd_tn;     // GEMMs on the tokens-on-N kernels: bit 0 up-projection, bit 1 down-projection, bit 2 dgrad of the up-projection, bit 3 dgrad of the down-projection
+    int fwd_tn;     // GEMMs on the tokens-on-N kernels: bit 0 up-projection, bit 1 down-projection, bits 2 and 3 their data gradients
     Profiler* prof;
 };
 
@@ -1098,7 +1093,8 @@ inline mop_status tc_launch(const TcPlan* p, const char* name, const CUtensorMap
                             const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& o0, const CUtensorMap& o1,
                             const TcArgs& args, cudaStream_t st) {
     p->prof->begin(name, st);
-    pdl_launch(tc_grouped_gemm_kernel<KIND>, p->sm_count, TcTraits<KIND>::THREADS, TcTraits<KIND>::SMEM_BYTES, st, a0, a1, b0, b1, o0, o1, args);
+    pdl_launch(tc_grouped_gemm_kernel<KIND>, p->sm_count, TcTraits<KIND>::THREADS, TcTraits<KIND>::SMEM_BYTES, st, a0, a1, b0, b1,
+               o0, o1, args);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

@@ -737,7 +737,8 @@ template <int KIND>
 inline mop_status tn_launch(const TcPlan* p, const char* name, const TnMaps& m, const TnArgs& g, cudaStream_t st) {
     p->prof->begin(name, st);
     const bool once = KIND != TN_F1G && tn_stream_weights(p->s);
-    pdl_launch(once ? tn_gemm_kernel<KIND, KIND != TN_F1G> : tn_gemm_kernel<KIND, false>, p->sm_count & ~1, TN_THREADS, TN_SMEM_BYTES, st, m, g);
+    pdl_launch(once ? tn_gemm_kernel<KIND, KIND != TN_F1G> : tn_gemm_kernel<KIND, false>, p->sm_count & ~1, TN_THREADS,
+               TN_SMEM_BYTES, st, m, g);
     p->prof->end(st);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }

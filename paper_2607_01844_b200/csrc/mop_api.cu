@@ -585,7 +585,8 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
     if (r != MOP_OK) return r;
     const size_t smem = (size_t)SEL_WARPS * 2 * s.E * sizeof(float);
     LAUNCH(c, "route_select", st,
-           pdl_launch(route_select_kernel, ceil_div(s.T, SEL_WARPS), SEL_WARPS * 32, smem, st, z, bias, topk_idx, topk_gate, s.T, s.E, s.k, s.score_fn, s.bias_mode));
+           pdl_launch(route_select_kernel, ceil_div(s.T, SEL_WARPS), SEL_WARPS * 32, smem, st, z, bias, topk_idx, topk_gate, s.T,
+                      s.E, s.k, s.score_fn, s.bias_mode));
     return after_launch(c);
 }
 
@@ -623,13 +624,14 @@ mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, i
     mop_status r;
     if (perm_small_fits(units, s.E)) {   // a few units: one block does histogram, scan and rank
         LAUNCH(c, "perm_small", st,
-               pdl_launch(perm_small_kernel, 1, 1024, ((size_t)units * s.E + s.E + 1) * sizeof(int32_t), st, topk_idx, counts, offsets, perm_row, row_src, M, s.E, units));
+               pdl_launch(perm_small_kernel, 1, 1024, ((size_t)units * s.E + s.E + 1) * sizeof(int32_t), st, topk_idx, counts,
+                          offsets, perm_row, row_src, M, s.E, units));
         if ((r = after_launch(c)) != MOP_OK) return r;
     } else {
     if (units > 0) {
         LAUNCH(c, "perm_hist", st,
                pdl_launch(perm_hist_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st, topk_idx, c->partial, M,
-                                                                                            s.E));
+                          s.E));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     if (units == 0) {   // nothing to permute: counts and offsets are all zero
@@ -641,7 +643,8 @@ mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, i
            pdl_launch(perm_scan_cols_kernel, ceil_div(s.E, 32), PSCAN_WARPS * 32, 0, st, c->partial, counts, units, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     LAUNCH(c, "perm_rank", st,
-           pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st, topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
+           pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st,
+                      topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     }
     if (!Xp) return MOP_OK;
@@ -924,13 +927,13 @@ mop_status chunk_begin(mop_ctx* c, const ChunkLayout& L, char* w, int i, int C, 
     mop_status r;
     if (tables) {
         LAUNCH(c, "chunk_tables", st,
-               pdl_launch(chunk_tables_kernel, min(ceil_div(M, 256), c->sm_count * 4), 256, 0, st, offsets, row_src, perm_row, off_c, row_src_c, perm_c, bounds, s.E, M, i, C));
+               pdl_launch(chunk_tables_kernel, min(ceil_div(M, 256), c->sm_count * 4), 256, 0, st, offsets, row_src, perm_row,
+                          off_c, row_src_c, perm_c, bounds, s.E, M, i, C));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     LAUNCH(c, "chunk_gather_rows", st,
            pdl_launch(gather_rows_kernel, c->sm_count * 8, 256, 0, st, static_cast<const uint4*>(src),
-                                                               reinterpret_cast<uint4*>(w + dst_off), row_src_c, bounds,
-                                                               s.k, s.d / 8));
+                      reinterpret_cast<uint4*>(w + dst_off), row_src_c, bounds, s.k, s.d / 8));
     return after_launch(c);
 }
 }  // namespace
@@ -973,9 +976,8 @@ mop_status mop_moe_layer_fwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         if (r != MOP_OK) break;
         LAUNCH(c, "chunk_combine_acc", st,
                pdl_launch(combine_acc_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(w + L.Yp),
-                                                         reinterpret_cast<const int32_t*>(w + L.perm_c),
-                                                         reinterpret_cast<float4*>(w + L.acc), static_cast<uint4*>(Y), s.T,
-                                                         s.k, s.d / 8, i == 0, i == n_chunks - 1));
+                          reinterpret_cast<const int32_t*>(w + L.perm_c), reinterpret_cast<float4*>(w + L.acc),
+                          static_cast<uint4*>(Y), s.T, s.k, s.d / 8, i == 0, i == n_chunks - 1));
         r = after_launch(c);
     }
     c->plan.rows_override = 0;
@@ -1039,14 +1041,13 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         c->launches += n;
         if (r != MOP_OK) break;
         LAUNCH(c, "chunk_dgate_reduce", st,
-               pdl_launch(dgate_reduce_chunk_kernel, ceil_div(M, 256), 256, 0, st, a.part, reinterpret_cast<const int32_t*>(w + L.perm_c),
-                                                                           dgate, M, (int)L.cap, ntile_part));
+               pdl_launch(dgate_reduce_chunk_kernel, ceil_div(M, 256), 256, 0, st, a.part,
+                          reinterpret_cast<const int32_t*>(w + L.perm_c), dgate, M, (int)L.cap, ntile_part));
         if ((r = after_launch(c)) != MOP_OK) break;
         LAUNCH(c, "chunk_combine_acc", st,
                pdl_launch(combine_acc_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(w + L.dXp),
-                                                         reinterpret_cast<const int32_t*>(w + L.perm_c),
-                                                         reinterpret_cast<float4*>(w + L.acc), static_cast<uint4*>(dX), s.T,
-                                                         s.k, s.d / 8, i == 0, i == n_chunks - 1));
+                          reinterpret_cast<const int32_t*>(w + L.perm_c), reinterpret_cast<float4*>(w + L.acc),
+                          static_cast<uint4*>(dX), s.T, s.k, s.d / 8, i == 0, i == n_chunks - 1));
         r = after_launch(c);
     }
     c->plan.rows_override = 0;
@@ -1055,8 +1056,7 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         dim3 gz((unsigned)min((size_t)64, (wvec + 255) / 256), s.E);
         LAUNCH(c, "chunk_zero_empty_experts", st,
                pdl_launch(zero_empty_experts_kernel, gz, 256, 0, st, offsets, reinterpret_cast<float4*>(dW_gate),
-                                                             reinterpret_cast<float4*>(dW_up),
-                                                             reinterpret_cast<float4*>(dW_down), wvec));
+                          reinterpret_cast<float4*>(dW_up), reinterpret_cast<float4*>(dW_down), wvec));
         r = after_launch(c);
     }
     return r;
@@ -1080,8 +1080,7 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     if (s.T > 0) {
         LAUNCH(c, "route_bwd_dz", st,
                pdl_launch(route_bwd_dz_kernel, ceil_div(s.T, 8), 256, 0, st, logits, bias, topk_idx, topk_gate, dgate, perm_row,
-                                                                     c->dz_sel, c->dz_row, s.T, s.E, s.k, s.score_fn,
-                                                                     s.bias_mode));
+                          c->dz_sel, c->dz_row, s.T, s.E, s.k, s.score_fn, s.bias_mode));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     dim3 gw(ceil_div(s.d, 256), s.E);
@@ -1089,7 +1088,8 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     float* db = (dbias_opt && s.bias_mode == MOP_BIAS_PRE_LOGIT) ? dbias_opt : nullptr;
     if (dbias_opt && !db) CUDA_OK(cudaMemsetAsync(dbias_opt, 0, (size_t)s.E * 4, st));
     LAUNCH(c, "route_bwd_dwr", st,
-           pdl_launch(route_bwd_dwr_kernel, gw, 32 * dwr_w, dwr_w * 1024, st, static_cast<const bf16*>(Xp), c->dz_row, offsets, dW_r, db, s.d, s.E));
+           pdl_launch(route_bwd_dwr_kernel, gw, 32 * dwr_w, dwr_w * 1024, st, static_cast<const bf16*>(Xp), c->dz_row, offsets,
+                      dW_r, db, s.d, s.E));
     if ((r = after_launch(c)) != MOP_OK) return r;
     if (s.T == 0) return MOP_OK;
     dim3 gt(ceil_div(s.E, 32), ceil_div(s.d, 32));
@@ -1097,7 +1097,7 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     if ((r = after_launch(c)) != MOP_OK) return r;
     LAUNCH(c, "route_bwd_dx", st,
            pdl_launch(route_bwd_dx_kernel, s.T, 256, 0, st, c->wrT, topk_idx, c->dz_sel, static_cast<bf16*>(dX), s.T, s.d, s.E,
-                                                    s.k));
+                      s.k));
     return after_launch(c);
 }
 
@@ -1395,7 +1395,8 @@ mop_status mop_moe_permute_static(int device, int32_t T, int32_t d, int32_t E, i
     }
     pdl_launch(perm_scan_cols_kernel, ceil_div(E, 32), PSCAN_WARPS * 32, 0, st, su.scratch, counts, units, E);
     if (cudaGetLastError() != cudaSuccess) return MOP_ERR_CUDA;
-    pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (E + 1) * sizeof(int32_t), st, topk_idx, su.scratch, counts, offsets, perm_row, row_src, M, E);
+    pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (E + 1) * sizeof(int32_t), st, topk_idx,
+               su.scratch, counts, offsets, perm_row, row_src, M, E);
     if (cudaGetLastError() != cudaSuccess) return MOP_ERR_CUDA;
     if (!Xp) return MOP_OK;
     launch_scatter_rows(static_cast<const uint4*>(x), static_cast<uint4*>(Xp), perm_row, T, k, d / 8, su.sm_count, st);
@@ -1622,7 +1623,8 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
     }
     const size_t n8 = (size_t)N * H / 8;
     const size_t cap = (size_t)p->sm_count * 16;
-    pdl_launch(f32_to_bf16_kernel, (unsigned)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap), 256, 0, st, reinterpret_cast<const float4*>(dx32), static_cast<uint4*>(dX), n8);
+    pdl_launch(f32_to_bf16_kernel, (unsigned)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap), 256, 0, st,
+               reinterpret_cast<const float4*>(dx32), static_cast<uint4*>(dX), n8);
     return cudaGetLastError() == cudaSuccess ? MOP_OK : MOP_ERR_CUDA;
 }
 

@@ -221,7 +221,8 @@ inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T,
 // former slabs, 46 now, 136 with 4 x 4; T = 4096, d = 2048, E = 64 takes 4 x 4: 50 -> 44 us, 97 with one chain per thread;
 // T = 8192, d = 7168, E = 128 takes 4 x 8: 472 -> 370 us, 415 with 4 x 4.
 inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int sm_count, cudaStream_t st) {
-    const struct { int tt, te; float first, more; } shape[4] = {{16, 8, 12.f, 6.f}, {32, 32, 28.f, 15.f}, {64, 32, 36.5f, 26.f}, {64, 64, 55.5f, 45.f}};
+    const struct { int tt, te; float first, more; } shape[4] = {
+        {16, 8, 12.f, 6.f}, {32, 32, 28.f, 15.f}, {64, 32, 36.5f, 26.f}, {64, 64, 55.5f, 45.f}};
     int pick = 0;
     float best = 0.0f;
     for (int i = 0; i < 4; ++i) {
@@ -864,7 +865,8 @@ __global__ void __launch_bounds__(CHAIN_WARPS * 32) route_chain_kernel(
         __syncwarp();                                    // the next tile's fetches overwrite the stages
         if (i < n_e) {
             float* zp = z + (size_t)t * E + e;
-            if (fabsf(*zp - acc) > 0.5f * ROUTE_EPS_C * (5.9604645e-8f * xnorm[t] * wmax)) ++n_bad;   // the model of the error is checked as we go
+            // the model of the error is checked as we go
+            if (fabsf(*zp - acc) > 0.5f * ROUTE_EPS_C * (5.9604645e-8f * xnorm[t] * wmax)) ++n_bad;
             *zp = acc;
         }
     }
@@ -945,8 +947,8 @@ inline int route_resolve_resident(int E, int sm_count) {
     return route_resolve_resident_q<32>(E, sm_count);
 }
 inline void route_select_fast(float* z, const float* z1, const float* bias, const bf16* x, const float* W_rT, const float* xnorm,
-                              const float* wsq, int32_t* idx, float* gate, const RouteLists& l, int T, int d, int E, int k, int score_fn, int bias_mode, int pass, int resolve_blocks,
-                              cudaStream_t st) {
+                              const float* wsq, int32_t* idx, float* gate, const RouteLists& l, int T, int d, int E, int k,
+                              int score_fn, int bias_mode, int pass, int resolve_blocks, cudaStream_t st) {
     const int q = ceil_div(E, 32);
 #define MOP_ROUTE_Q(QQ)                                                                                                 \
     route_select_fast_q<QQ>(z, z1, bias, x, W_rT, xnorm, wsq, idx, gate, l, T, d, E, k, score_fn, bias_mode, pass,             \
