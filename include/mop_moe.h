@@ -52,8 +52,8 @@ typedef enum { MOP_SCORE_SOFTMAX = 0, MOP_SCORE_SIGMOID = 1 } mop_score_fn;
 typedef enum { MOP_BIAS_NONE = 0, MOP_BIAS_POST_SCORE = 1, MOP_BIAS_PRE_LOGIT = 2 } mop_bias_mode;
 
 /* AUTO: tensor cores at every supported shape.  TENSOR: the same, d and f multiples of 64 or fail.  Both run the
- * four token-row GEMMs on the two-CTA tokens-on-N kernel and the weight gradients on the one-CTA
- * kernel (128 x 256 tiles).
+ * four token-row GEMMs on the two-CTA tokens-on-N kernel and the weight gradients on the one-CTA kernel (128 x 256
+ * tiles) below 448 rows per expert (T k / E), on the two-CTA one (256 x 256 tiles) from there on.
  * The remaining values force one schedule for testing and measurement: TENSOR_1CTA = one-CTA kernel
  * for all token-row GEMMs; TENSOR_2CTA = two-CTA kernel on 256-row pair tiles; TENSOR_MIXED = full
  * pairs on the two-CTA kernel, remaining rows on the one-CTA kernel; TENSOR_TN = all four token-row
@@ -75,7 +75,7 @@ typedef struct {
     int32_t with_backward; /* 1: the context also holds the backward's intermediates; 2: and buffers to
                               recompute G, U, H in the backward (activation checkpointing) */
     int32_t dw_accumulate; /* 0: dW is overwritten (empty experts get zeros); 1: dW += */
-    int32_t gemm_path;     /* mop_gemm_path; AUTO = tensor cores when the shape allows */
+    int32_t gemm_path;     /* mop_gemm_path */
     int32_t host_io;       /* 1: the context also holds the activations of the host-buffer entry points;
                               2: and a second slot of every buffer a copy touches, for the *_async forms */
     int32_t route_path;    /* mop_route_path */
@@ -143,7 +143,8 @@ mop_status mop_route_stats(mop_ctx* ctx, int64_t* tokens_reevaluated, int64_t* c
  *   row_src     = inverse of perm_row;   Xp[p,:] = x[row_src[p] / k, :]
  * x [T,d] bf16; topk_idx [T,k]; counts [E]; offsets [E+1]; perm_row, row_src [T*k] i32 out;
  * Xp [T*k,d] bf16 out, or NULL: only the tables are built (x is then not read), for
- * mop_moe_expert_ffn_fwd_gather.  Indices outside [0,E) are a caller error (rows are dropped). */
+ * mop_moe_expert_ffn_fwd_gather.  Indices outside [0,E) are a caller error (rows are dropped); an expert may be named
+ * more than once for a token (the chunked backward alone relies on the tables of mop_moe_route's distinct picks). */
 mop_status mop_moe_permute(mop_ctx* ctx, const void* x, const int32_t* topk_idx, int32_t* counts, int32_t* offsets,
                            int32_t* perm_row, int32_t* row_src, void* Xp, void* stream);
 

@@ -61,7 +61,7 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
     mop_status r;
-    // Tokens-on-N kernels: fwd_tn bit 0 = up-projection, bit 1 = down-projection (see tc_plan_policy)
+    // Tokens-on-N kernels: fwd_tn bit 0 = up-projection, bit 1 = down-projection (set in mop_create)
     const bool gather = a.x_gather != nullptr;
     const bool tn_f1 = gather || (p->fwd_tn & 1), tn_f2 = p->fwd_tn & 2;
     if (tn_f1 || tn_f2) {
@@ -108,9 +108,11 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     return MOP_OK;
 }
 
-// Weight gradients on CTA pairs from 448 rows per expert on (average).  d = 7168, f = 2048, 512 rows: 757 + 1508 us on single
-// CTAs, 682 + 1346 on pairs; d = 2048, f = 1408: 246 + 492 and 258 + 496 at 384 rows, 207 + 397 and 194 + 353 at 2048 (16
-// experts); at 171 rows and d = 7168 1340 + 2660 and 1538 + 3087.
+// Weight gradients on CTA pairs from 448 rows per expert on (average).  dW_down + (dW_gate, dW_up), us, single CTAs and pairs, both
+// with the operands brought to L2 ahead: d = 2048, f = 1408, 64 experts of 256 rows 160 + 328 and 200 + 355, 384 rows 217 + 392 and
+// 230 + 402, 448 rows 241 + 427 and 242 + 424, 512 rows 261 + 469 and 257 + 451, 1024 rows 408 + 770 and 400 + 725; d = 7168,
+// f = 2048, 16 experts of 256 rows 205 + 396 and 286 + 560, 384 rows 254 + 494 and 256 + 486, 448 rows 286 + 555 and 276 + 522,
+// 512 rows 312 + 608 and 294 + 562, 2048 rows 886 + 1695 and 802 + 1518.
 inline bool tw_wanted(const TcPlan* p) { return p->fwd_tn == 15 && (uint64_t)p->s.T * p->s.k >= 448ull * p->s.E; }
 
 inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st,

@@ -1,7 +1,9 @@
 // Tensor-core grouped GEMMs for sm_100a: tcgen05.mma with TMEM accumulators, operands staged by
 // TMA into 128-byte-swizzled shared memory, one persistent warp-specialised CTA per SM.
 //
-// Every GEMM of the layer is one instantiation of tc_grouped_gemm_kernel<KIND>:
+// Kinds of GEMM, instantiations of tc_grouped_gemm_kernel<KIND> (one CTA per tile) and of the pair kernels that share its
+// arguments and epilogues.  By default this kernel runs the weight gradients below 448 rows per expert and the vocabulary's with
+// up to 1024 tokens; F1, F2, B2 and B4 run on gemm_tn.cuh, and here and in gemm_tc2.cuh where a schedule is forced:
 //   F1   [G|U] = Xp W_gate[e] | Xp W_up[e]        SwiGLU epilogue -> H (+ stash)      ragged M
 //   F2   O     = H W_down[e]                      gate epilogue   -> Yp               ragged M
 //   B2   dHu   = dYp W_down[e]^T                  SwiGLU-backward epilogue            ragged M

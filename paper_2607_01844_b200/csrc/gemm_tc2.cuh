@@ -1,5 +1,5 @@
-// Two-CTA tensor-core grouped GEMMs (tcgen05.mma.cta_group::2) for the kinds whose rows are token
-// rows (F1, F2, B2, B4).  A cluster of two CTAs on neighbouring SMs computes a 256 x 256 tile: each
+// Two-CTA tensor-core GEMMs (tcgen05.mma.cta_group::2): the vocabulary projection's kinds (VL, VP, VX, VW), and the grouped kinds
+// whose rows are token rows (F1, F2, B2, B4) where that schedule is forced.  A cluster of two CTAs on neighbouring SMs computes a 256 x 256 tile: each
 // CTA loads its own 128 rows of A and HALF of the B tile (128 of the 256 N columns), the leader CTA
 // issues one MMA of M=256, N=256, K=16 that reads both CTAs' shared memory, and each CTA's TMEM
 // receives its own 128 x 256 accumulator.  Per output element this halves the B bytes that cross

@@ -106,7 +106,10 @@ __global__ void guard_check_kernel(const char* ws, GuardList g, unsigned long lo
 
 int perm_units(const mop_moe_shape& s) { return ceil_div(s.T * s.k, PERM_SEG); }
 // The tensor-core scoring path needs 64-wide K blocks of x and 64-wide column chunks of W_r.  AUTO takes it once the scoring is
-// large: small layers keep the fp32 chains, and their contexts hold none of its buffers.
+// large: small layers keep the fp32 chains, and their contexts hold none of its buffers.  The line is a safe one and not where the
+// two paths cross: router, us, exact and tensor, at T 4096, d 2048, E 64 (1.1 GFLOP) 52 and 57, T 512, d 7168, E 256 (1.9) 116 and
+// 129, T 4096, d 7168, E 64 (3.8) 144 and 113, T 16384, d 2048, E 64 (4.3) 136 and 82, T 2048, d 7168, E 256 (7.5) 220 and 135,
+// T 8192, d 7168, E 128 (15) 394 and 147, T 16384, d 7168, E 256 (60) 1271 and 221; the crossing is near 3 GFLOP.
 bool route_fast(const mop_moe_shape& s) {
     if (s.route_path == MOP_ROUTE_EXACT || s.T <= 0 || s.d % 64 || s.E % 64 || !tc_shape_supported(s.d, s.f)) return false;
     return s.route_path == MOP_ROUTE_TENSOR || 2.0 * s.T * s.d * s.E >= 2e10;
