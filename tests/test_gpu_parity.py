@@ -731,6 +731,33 @@ def test_tensor_core_scoring_with_most_tokens_in_doubt(w):
             assert (tokens, chains) == (w.T, w.T * w.E)
 
 
+def test_tensor_core_scoring_can_be_captured_behind_other_work():
+    """Side stream, emptied lists and dependent launches inside a graph, after a copy and a join of two streams."""
+    w = synth.small("c3_trillion", T=1000, d=512, E=256, k=8, f=64, seed=75)
+    inp = synth.make_inputs(w, "cuda")
+    ctx = binding.context_for(w, route_path=binding.ROUTE_TENSOR)
+    want, got = ((torch.empty((w.T, w.k), dtype=torch.int32, device="cuda"), torch.empty((w.T, w.k), device="cuda")) for _ in range(2))
+    binding.mop_moe_route(ctx, inp["x"], inp["W_r"], inp["bias"], *want)
+    torch.cuda.synchronize()
+    x, W_r = torch.zeros_like(inp["x"]), torch.zeros_like(inp["W_r"])
+    side, other, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            other.wait_stream(side)
+            with torch.cuda.stream(other):
+                W_r.copy_(inp["W_r"])
+            x.copy_(inp["x"])
+            side.wait_stream(other)
+            binding.mop_moe_route(ctx, x, W_r, inp["bias"], *got, stream=side)
+    for _ in range(3):
+        for t in (x, W_r, *got):
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    binding.mop_poll(ctx)
+
+
 def test_tensor_core_scoring_with_equal_and_duplicate_keys():
     """W_r = 0 makes all keys of a token equal (every expert is re-evaluated and the lower ids win); two equal
     columns of W_r make one exact tie per token that only the chain can order."""
