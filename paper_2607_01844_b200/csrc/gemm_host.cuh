@@ -43,6 +43,10 @@ inline mop_status tc_rows_gemm(const TcPlan* p, const char* name, const char* na
     return MOP_OK;
 }
 
+// The table of token tiles that an earlier kernel of a call may write for the GEMMs (tiles_ready); null: none that they would read,
+// or tiles of another kind are needed too.
+inline int32_t* tn_shared_table(const TcPlan* p, int32_t* tiles) { return p->fwd_tn == 15 ? tn_table(p, tiles) : nullptr; }
+
 inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st,
                                   int* launches, bool with_down);
 
@@ -64,7 +68,7 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
     // Tokens-on-N kernels: fwd_tn bit 0 = up-projection, bit 1 = down-projection (set in mop_create)
     const bool gather = a.x_gather != nullptr;
     const bool tn_f1 = gather || (p->fwd_tn & 1), tn_f2 = p->fwd_tn & 2;
-    if (tn_f1 || tn_f2) {
+    if ((tn_f1 || tn_f2) && !a.tiles_ready) {
         if ((r = tn_build_tiles(p, a.offsets, tiles, !(tn_f1 && tn_f2) && p->pairs == 0, st)) != MOP_OK) return r;
         ++*launches;
     }
@@ -152,7 +156,7 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
                              !tc_map_3d(p, &mWgK, a.W_gate, s.E, s.d, s.f, 256) || !tc_map_3d(p, &mWuK, a.W_up, s.E, s.d, s.f, 256) ||
                              !tc_map_3d(p, &mWgKp, a.W_gate, s.E, s.d, s.f, 128) || !tc_map_3d(p, &mWuKp, a.W_up, s.E, s.d, s.f, 128)))
         return MOP_ERR_CUDA;
-    if (p->fwd_tn & 12) {
+    if ((p->fwd_tn & 12) && !a.tiles_ready) {
         if ((r = tn_build_tiles(p, a.offsets, tiles, false, st)) != MOP_OK) return r;
         ++*launches;
     }

@@ -945,6 +945,7 @@ struct TcFwdArgs {
     const bf16 *W_gate, *W_up, *W_down;
     bf16 *G_save, *U_save, *H, *Yp;
     const bf16* x_gather;   // non-null: the up-projection gathers its rows from x [T, d] and Xp is unused
+    bool tiles_ready;       // an earlier kernel of this call has written the token tiles of these offsets
 };
 struct TcBwdArgs {
     const bf16 *dYp, *Xp, *G_save, *U_save, *H;
@@ -953,6 +954,7 @@ struct TcBwdArgs {
     bf16 *dG, *dU, *gH, *dXp; float* part;
     float *dW_gate, *dW_up, *dW_down; int accumulate;
     int keep_empty;   // experts without rows (in this call's offsets) keep their gradients: expert-chunked backward
+    bool tiles_ready; // as in TcFwdArgs
 };
 
 // Shapes of the tokens-on-M, gathering and chunked forms; the tokens-on-N kernels and the weight gradients take any multiple of 8.

@@ -31,6 +31,7 @@
 // Barrier protocol, bounded waits and teardown as in the pair kernel (gemm_tc2.cuh).
 #pragma once
 #include "gemm_tc2.cuh"
+#include "tiles.cuh"
 
 namespace mop {
 
@@ -73,36 +74,13 @@ struct TnArgs {
     EpiArgs ep;
 };
 
-// Token tiles: an expert's rows are cut into ceil(rows / 256) nearly equal tiles.
-__device__ __forceinline__ void tn_build_ttiles_body(const int32_t* __restrict__ offsets, int E,
-                                                     int4* __restrict__ tiles, int32_t* __restrict__ n_tiles,
-                                                     int32_t* scan) {
-    const int e = threadIdx.x;
-    int cnt = 0, off = 0;
-    if (e < E) { off = offsets[e]; cnt = offsets[e + 1] - off; }
-    const int nt = (cnt + 255) / 256;
-    scan[e] = nt;
-    __syncthreads();
-    for (int s = 1; s < 1024; s <<= 1) {
-        const int v = (e >= s) ? scan[e - s] : 0;
-        __syncthreads();
-        scan[e] += v;
-        __syncthreads();
-    }
-    const int first = scan[e] - nt;
-    const int sz = nt ? (((cnt + nt - 1) / nt + 15) & ~15) : 0;
-    // .w = position of the tile within its expert | number of tiles of the expert << 16
-    for (int i = 0; i < nt; ++i) tiles[first + i] = make_int4(e, off + i * sz, min(sz, cnt - i * sz), i | (nt << 16));
-    if (e == 1023) *n_tiles = scan[1023];
-    if (e < 8) n_tiles[16 + e] = 0;      // the kinds' counters of work items handed out
-}
 // The tile tables of the token-row GEMMs in one launch: block 0 the token tiles, block 1 the 128-row tiles of the
 // tokens-on-M kernels (where a forward or backward uses both).
 __global__ void __launch_bounds__(1024) tn_build_ttiles_kernel(const int32_t* __restrict__ offsets, int E, int32_t* __restrict__ ttiles,
                                                                int32_t* __restrict__ mtiles) {
     pdl_begin();
     __shared__ int32_t scan[1025];
-    if (blockIdx.x == 0) tn_build_ttiles_body(offsets, E, reinterpret_cast<int4*>(ttiles + 64), ttiles, scan);
+    if (blockIdx.x == 0) write_token_tiles<1024>(offsets, E, ttiles, scan);
     else tc_build_mtiles_body(offsets, E, reinterpret_cast<int4*>(mtiles + 64), mtiles, scan);
 }
 
@@ -715,8 +693,8 @@ inline bool tn_stream_weights(const mop_moe_shape& s) {
 inline TnArgs tn_base_args(const TcPlan* p, int32_t* tiles, int kind, int32_t* status) {
     int32_t* table = tn_table(p, tiles);
     TnArgs g{};
-    g.next = table + 16 + kind;
-    g.ttiles = reinterpret_cast<const int4*>(table + 64);
+    g.next = table + TT_NEXT + kind;
+    g.ttiles = reinterpret_cast<const int4*>(table + TT_TILES);
     g.n_ttiles = table;
     g.status = status;
     return g;

@@ -308,7 +308,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         return MOP_ERR_UNSUPPORTED;
     }
     c->tensor_tn = shape->gemm_path != MOP_GEMM_SCALAR && (c->tensor_ok || (prop.major == 10 && c->sm_count >= 2));
-    if (!route_score_init() || !route_chain_init()) { delete c; return MOP_ERR_CUDA; }
+    if (!route_score_init() || !route_chain_init() || !perm_cluster_init()) { delete c; return MOP_ERR_CUDA; }
     const Layout L = make_layout(*shape);
     c->ws_bytes = L.total;
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }
@@ -612,8 +612,37 @@ mop_status mop_route_stats(mop_ctx* c, int64_t* tokens_reevaluated, int64_t* cha
     return MOP_OK;
 }
 
-mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, int32_t* counts, int32_t* offsets,
-                           int32_t* perm_row, int32_t* row_src, void* Xp, void* stream) {
+namespace {
+// Where the kernels before the GEMMs may write their token tiles (null: the GEMMs build what they need).
+int32_t* shared_tiles(mop_ctx* c) { return use_tensor(c) ? tn_shared_table(&c->plan, c->tiles) : nullptr; }
+
+// counts, offsets, perm_row, row_src; with a tile table also the token tiles of the layer's GEMMs (the single-launch form only)
+mop_status permutation_tables(mop_ctx* c, const int32_t* topk_idx, int32_t* counts, int32_t* offsets, int32_t* perm_row,
+                              int32_t* row_src, int32_t* tile_table, cudaStream_t st) {
+    const mop_moe_shape& s = c->s;
+    const int M = s.T * s.k;
+    if (perm_cluster_fits(M)) {
+        LAUNCH(c, "permute_tables", st, launch_perm_cluster(topk_idx, counts, offsets, perm_row, row_src, M, s.E, tile_table, st));
+        return after_launch(c);
+    }
+    const int units = perm_units(s);
+    const size_t smem = (size_t)PERM_WARPS * s.E * sizeof(int32_t);
+    mop_status r;
+    LAUNCH(c, "perm_hist", st,
+           pdl_launch(perm_hist_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st, topk_idx, c->partial, M, s.E));
+    if ((r = after_launch(c)) != MOP_OK) return r;
+    LAUNCH(c, "perm_scan", st,
+           pdl_launch(perm_scan_cols_kernel, ceil_div(s.E, 32), PSCAN_WARPS * 32, 0, st, c->partial, counts, units, s.E));
+    if ((r = after_launch(c)) != MOP_OK) return r;
+    LAUNCH(c, "perm_rank", st,
+           pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st,
+                      topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
+    return after_launch(c);
+}
+
+// tile_table: the token tiles of the GEMMs too, by the permutation or, where that takes three kernels, beside the row copy (with Xp)
+mop_status permute(mop_ctx* c, const void* x, const int32_t* topk_idx, int32_t* counts, int32_t* offsets, int32_t* perm_row,
+                   int32_t* row_src, void* Xp, int32_t* tile_table, void* stream) {
     if (!c) return MOP_ERR_INVALID_ARG;
     REQ_PTR_T(topk_idx); REQ_PTR(counts); REQ_PTR(offsets); REQ_PTR_T(perm_row); REQ_PTR_T(row_src);
     if (Xp) { REQ_PTR_T(x); REQ_PTR_T(Xp); }   // Xp == NULL: tables only, for the gathering forward
@@ -621,40 +650,20 @@ mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, i
     DeviceGuard guard(c->device);
     if (!guard.ok) return MOP_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int M = s.T * s.k;
-    const int units = perm_units(s);
-    const size_t smem = (size_t)PERM_WARPS * s.E * sizeof(int32_t);
     mop_status r;
-    if (perm_small_fits(units, s.E)) {   // a few units: one block does histogram, scan and rank
-        LAUNCH(c, "perm_small", st,
-               pdl_launch(perm_small_kernel, 1, 1024, ((size_t)units * s.E + s.E + 1) * sizeof(int32_t), st, topk_idx, counts,
-                          offsets, perm_row, row_src, M, s.E, units));
-        if ((r = after_launch(c)) != MOP_OK) return r;
-    } else {
-    if (units > 0) {
-        LAUNCH(c, "perm_hist", st,
-               pdl_launch(perm_hist_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem, st, topk_idx, c->partial, M,
-                          s.E));
-        if ((r = after_launch(c)) != MOP_OK) return r;
-    }
-    if (units == 0) {   // nothing to permute: counts and offsets are all zero
-        LAUNCH(c, "perm_scan", st,
-               pdl_launch(perm_scan_kernel, 1, 1024, (s.E + 1) * sizeof(int32_t), st, c->partial, counts, offsets, units, s.E));
-        return after_launch(c);
-    }
-    LAUNCH(c, "perm_scan", st,
-           pdl_launch(perm_scan_cols_kernel, ceil_div(s.E, 32), PSCAN_WARPS * 32, 0, st, c->partial, counts, units, s.E));
-    if ((r = after_launch(c)) != MOP_OK) return r;
-    LAUNCH(c, "perm_rank", st,
-           pdl_launch(perm_rank_kernel, ceil_div(units, PERM_WARPS), PERM_WARPS * 32, smem + (s.E + 1) * sizeof(int32_t), st,
-                      topk_idx, c->partial, counts, offsets, perm_row, row_src, M, s.E));
-    if ((r = after_launch(c)) != MOP_OK) return r;
-    }
-    if (!Xp) return MOP_OK;
+    if ((r = permutation_tables(c, topk_idx, counts, offsets, perm_row, row_src, tile_table, st)) != MOP_OK) return r;
+    if (!Xp || s.T == 0) return MOP_OK;
+    const TileJob job = {offsets, s.E, perm_cluster_fits((long long)s.T * s.k) ? nullptr : tile_table};
     LAUNCH(c, "permute_scatter_rows", st,
            launch_scatter_rows(static_cast<const uint4*>(x), static_cast<uint4*>(Xp), perm_row, s.T, s.k, s.d / 8,
-                               c->sm_count, st));
+                               c->sm_count, st, job));
     return after_launch(c);
+}
+}  // namespace
+
+mop_status mop_moe_permute(mop_ctx* c, const void* x, const int32_t* topk_idx, int32_t* counts, int32_t* offsets,
+                           int32_t* perm_row, int32_t* row_src, void* Xp, void* stream) {
+    return permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, nullptr, stream);
 }
 
 mop_status mop_moe_combine(mop_ctx* c, const void* Yp, const int32_t* perm_row, void* Y, void* stream) {
@@ -699,9 +708,10 @@ mop_status up_projection(mop_ctx* c, const void* Xp, const int32_t* offsets, con
 }
 }  // namespace
 
-mop_status mop_moe_expert_ffn_fwd(mop_ctx* c, const void* Xp, const int32_t* offsets, const int32_t* row_src,
-                                  const float* topk_gate, const void* W_gate, const void* W_up, const void* W_down,
-                                  void* G_save, void* U_save, void* H, void* Yp, void* stream) {
+namespace {
+mop_status expert_ffn_fwd(mop_ctx* c, const void* Xp, const int32_t* offsets, const int32_t* row_src, const float* topk_gate,
+                          const void* W_gate, const void* W_up, const void* W_down, void* G_save, void* U_save, void* H, void* Yp,
+                          bool tiles_ready, void* stream) {
     if (!c) return MOP_ERR_INVALID_ARG;
     REQ_PTR_T(Xp); REQ_PTR(offsets); REQ_PTR_T(row_src); REQ_PTR_T(topk_gate); REQ_PTR(W_gate); REQ_PTR(W_up);
     REQ_PTR(W_down); REQ_PTR_T(H); REQ_PTR_T(Yp);
@@ -720,6 +730,7 @@ mop_status mop_moe_expert_ffn_fwd(mop_ctx* c, const void* Xp, const int32_t* off
         a.W_down = static_cast<const bf16*>(W_down);
         a.G_save = static_cast<bf16*>(G_save); a.U_save = static_cast<bf16*>(U_save);
         a.H = static_cast<bf16*>(H); a.Yp = static_cast<bf16*>(Yp);
+        a.tiles_ready = tiles_ready;
         int n = 0;
         mop_status r = tc_ffn_fwd(&c->plan, a, c->tiles, c->status, st, &n);
         c->launches += n;
@@ -740,6 +751,28 @@ mop_status mop_moe_expert_ffn_fwd(mop_ctx* c, const void* Xp, const int32_t* off
     h.offsets = offsets; h.ragged_k = 0; h.N = s.d; h.Kfix = s.f; h.npairs = 1; h.epi = EPI_GATE;
     h.ep.out0 = static_cast<bf16*>(Yp); h.ep.gate = topk_gate; h.ep.row_src = row_src; h.ep.ldo = s.d; h.ep.M_total = M;
     return launch_scalar(c, "scalar_down_gate", h, st);
+}
+
+// route -> permute -> expert FFN -> combine
+mop_status layer_forward(mop_ctx* c, const void* x, const float* W_r, const float* bias, const void* W_gate, const void* W_up,
+                         const void* W_down, int32_t* topk_idx, float* topk_gate, int32_t* counts, int32_t* offsets,
+                         int32_t* perm_row, int32_t* row_src, void* Xp, void* G_save, void* U_save, void* H, void* Yp, void* Y,
+                         void* stream) {
+    int32_t* table = shared_tiles(c);
+    mop_status r;
+    if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
+    if ((r = permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, table, stream)) != MOP_OK) return r;
+    if ((r = expert_ffn_fwd(c, Xp, offsets, row_src, topk_gate, W_gate, W_up, W_down, G_save, U_save, H, Yp, table != nullptr,
+                            stream)) != MOP_OK)
+        return r;
+    return mop_moe_combine(c, Yp, perm_row, Y, stream);
+}
+}  // namespace
+
+mop_status mop_moe_expert_ffn_fwd(mop_ctx* c, const void* Xp, const int32_t* offsets, const int32_t* row_src,
+                                  const float* topk_gate, const void* W_gate, const void* W_up, const void* W_down,
+                                  void* G_save, void* U_save, void* H, void* Yp, void* stream) {
+    return expert_ffn_fwd(c, Xp, offsets, row_src, topk_gate, W_gate, W_up, W_down, G_save, U_save, H, Yp, false, stream);
 }
 
 mop_status mop_moe_expert_ffn_fwd_gather(mop_ctx* c, const void* x, const int32_t* offsets, const int32_t* row_src,
@@ -789,11 +822,12 @@ mop_status mop_moe_expert_ffn_bwd(mop_ctx* c, const void* dY, const void* Xp, co
         if ((r = up_projection(c, Xp, offsets, W_gate, W_up, c->rG, c->rU, c->rH, st)) != MOP_OK) return r;
         G_save = c->rG; U_save = c->rU; H = c->rH;
     }
+    const TileJob job = {offsets, s.E, shared_tiles(c)};
     if (s.T > 0) {
         // dYp[p,:] = dY[t,:]  (unscaled; the gate enters through dH and gate*H)
         LAUNCH(c, "dy_scatter_rows", st,
                launch_scatter_rows(static_cast<const uint4*>(dY), reinterpret_cast<uint4*>(c->dYp), perm_row, s.T, s.k,
-                                   s.d / 8, c->sm_count, st));
+                                   s.d / 8, c->sm_count, st, job));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     int ntile_part = 0;
@@ -806,6 +840,7 @@ mop_status mop_moe_expert_ffn_bwd(mop_ctx* c, const void* dY, const void* Xp, co
         a.W_down = static_cast<const bf16*>(W_down);
         a.dG = c->dG; a.dU = c->dU; a.gH = c->gH; a.dXp = c->dXp; a.part = c->part;
         a.dW_gate = dW_gate; a.dW_up = dW_up; a.dW_down = dW_down; a.accumulate = s.dw_accumulate;
+        a.tiles_ready = job.table != nullptr;
         int n = 0;
         r = tc_ffn_bwd(&c->plan, a, c->tiles, c->status, st, &n, &ntile_part);
         c->launches += n;
@@ -861,12 +896,8 @@ mop_status mop_moe_layer_fwd(mop_ctx* c, const void* x, const float* W_r, const 
     REQ_PTR(W_gate); REQ_PTR(W_up); REQ_PTR(W_down); REQ_PTR_T(H); REQ_PTR_T(Yp); REQ_PTR_T(Y);
     if ((G_save == nullptr) != (U_save == nullptr)) return MOP_ERR_INVALID_ARG;
     if (G_save && (!aligned16(G_save) || !aligned16(U_save))) return MOP_ERR_ALIGN;
-    mop_status r;
-    if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
-    if ((r = mop_moe_permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, stream)) != MOP_OK) return r;
-    if ((r = mop_moe_expert_ffn_fwd(c, Xp, offsets, row_src, topk_gate, W_gate, W_up, W_down, G_save, U_save, H, Yp, stream)) != MOP_OK)
-        return r;
-    return mop_moe_combine(c, Yp, perm_row, Y, stream);
+    return layer_forward(c, x, W_r, bias, W_gate, W_up, W_down, topk_idx, topk_gate, counts, offsets, perm_row, row_src, Xp, G_save,
+                         U_save, H, Yp, Y, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -921,6 +952,7 @@ mop_status chunk_check(mop_ctx* c, int32_t n_chunks, const void* workspace) {
 mop_status chunk_begin(mop_ctx* c, const ChunkLayout& L, char* w, int i, int C, const void* src, size_t dst_off,
                        const int32_t* offsets, const int32_t* perm_row, const int32_t* row_src, bool tables,
                        cudaStream_t st) {
+    // the chunk's token tiles are written beside its first row copy: up-projection and backward read the same ones
     const mop_moe_shape& s = c->s;
     const int M = s.T * s.k;
     int32_t* off_c = reinterpret_cast<int32_t*>(w + L.off_c);
@@ -934,9 +966,10 @@ mop_status chunk_begin(mop_ctx* c, const ChunkLayout& L, char* w, int i, int C, 
                           off_c, row_src_c, perm_c, bounds, s.E, M, i, C));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
+    const TileJob job = {off_c, s.E, tables ? shared_tiles(c) : nullptr};
     LAUNCH(c, "chunk_gather_rows", st,
            pdl_launch(gather_rows_kernel, c->sm_count * 8, 256, 0, st, static_cast<const uint4*>(src),
-                      reinterpret_cast<uint4*>(w + dst_off), row_src_c, bounds, s.k, s.d / 8));
+                      reinterpret_cast<uint4*>(w + dst_off), row_src_c, bounds, s.k, s.d / 8, job));
     return after_launch(c);
 }
 }  // namespace
@@ -973,6 +1006,7 @@ mop_status mop_moe_layer_fwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         a.W_gate = static_cast<const bf16*>(W_gate); a.W_up = static_cast<const bf16*>(W_up);
         a.W_down = static_cast<const bf16*>(W_down);
         a.H = reinterpret_cast<bf16*>(w + L.H); a.Yp = reinterpret_cast<bf16*>(w + L.Yp);
+        a.tiles_ready = shared_tiles(c) != nullptr;
         int n = 0;
         r = tc_ffn_fwd(&c->plan, a, c->tiles, c->status, st, &n);
         c->launches += n;
@@ -1026,6 +1060,7 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         fa.W_gate = static_cast<const bf16*>(W_gate); fa.W_up = static_cast<const bf16*>(W_up);
         fa.G_save = reinterpret_cast<bf16*>(w + L.G); fa.U_save = reinterpret_cast<bf16*>(w + L.U);
         fa.H = reinterpret_cast<bf16*>(w + L.H);
+        fa.tiles_ready = shared_tiles(c) != nullptr;
         int n = 0;
         r = tc_up_only(&c->plan, fa, c->tiles, c->status, st, &n);
         c->launches += n;
@@ -1038,6 +1073,7 @@ mop_status mop_moe_layer_bwd_chunked(mop_ctx* c, int32_t n_chunks, const void* x
         a.gH = reinterpret_cast<bf16*>(w + L.gH); a.dXp = reinterpret_cast<bf16*>(w + L.dXp);
         a.part = reinterpret_cast<float*>(w + L.part);
         a.dW_gate = dW_gate; a.dW_up = dW_up; a.dW_down = dW_down; a.accumulate = s.dw_accumulate; a.keep_empty = 1;
+        a.tiles_ready = fa.tiles_ready;
         int ntile_part = 0;
         n = 0;
         r = tc_ffn_bwd(&c->plan, a, c->tiles, c->status, st, &n, &ntile_part);
@@ -1128,13 +1164,9 @@ mop_status step_host(mop_ctx* c, const void* x_host, const void* dY_host, const 
         }
     }
     mop_status r;
-    if ((r = mop_moe_route(c, c->hx, W_r, bias, c->hidx, c->hgate, nullptr, stream)) != MOP_OK) return r;
-    if ((r = mop_moe_permute(c, c->hx, c->hidx, c->hcounts, c->hoffsets, c->hperm, c->hsrc, c->hXp, stream)) != MOP_OK)
+    if ((r = layer_forward(c, c->hx, W_r, bias, W_gate, W_up, W_down, c->hidx, c->hgate, c->hcounts, c->hoffsets, c->hperm, c->hsrc,
+                           c->hXp, bwd ? c->hG : nullptr, bwd ? c->hU : nullptr, c->hH, c->hYp, c->hY, stream)) != MOP_OK)
         return r;
-    if ((r = mop_moe_expert_ffn_fwd(c, c->hXp, c->hoffsets, c->hsrc, c->hgate, W_gate, W_up, W_down,
-                                    bwd ? c->hG : nullptr, bwd ? c->hU : nullptr, c->hH, c->hYp, stream)) != MOP_OK)
-        return r;
-    if ((r = mop_moe_combine(c, c->hYp, c->hperm, c->hY, stream)) != MOP_OK) return r;
     if (s.T > 0) {
         cudaStream_t os = bwd ? cs : st;                       // forward only: nothing to overlap with
         if (bwd) {
@@ -1193,14 +1225,9 @@ mop_status step_host_pipelined(mop_ctx* c, const void* x_host, const void* dY_ho
         CUDA_OK(cudaStreamWaitEvent(st, c->ev_drained[q], 0));    // step i-2's results have left this slot
     }
     mop_status r;
-    if ((r = mop_moe_route(c, c->px[q], W_r, bias, c->pidx[q], c->pgate[q], nullptr, stream)) != MOP_OK) return r;
-    if ((r = mop_moe_permute(c, c->px[q], c->pidx[q], c->hcounts, c->hoffsets, c->hperm, c->hsrc, c->hXp, stream)) !=
-        MOP_OK)
+    if ((r = layer_forward(c, c->px[q], W_r, bias, W_gate, W_up, W_down, c->pidx[q], c->pgate[q], c->hcounts, c->hoffsets, c->hperm,
+                           c->hsrc, c->hXp, bwd ? c->hG : nullptr, bwd ? c->hU : nullptr, c->hH, c->hYp, c->pY[q], stream)) != MOP_OK)
         return r;
-    if ((r = mop_moe_expert_ffn_fwd(c, c->hXp, c->hoffsets, c->hsrc, c->pgate[q], W_gate, W_up, W_down,
-                                    bwd ? c->hG : nullptr, bwd ? c->hU : nullptr, c->hH, c->hYp, stream)) != MOP_OK)
-        return r;
-    if ((r = mop_moe_combine(c, c->hYp, c->hperm, c->pY[q], stream)) != MOP_OK) return r;
     if (s.T > 0) {
         CUDA_OK(cudaEventRecord(c->ev_fwd[q], st));
         CUDA_OK(cudaStreamWaitEvent(out, c->ev_fwd[q], 0));

@@ -2,7 +2,7 @@
 // row movers (scatter x -> Xp, k-row combine Yp -> Y).  No atomics anywhere: the order inside an
 // expert is the assignment id, fixed by a two-level (warp segment, expert) prefix sum.
 #pragma once
-#include "common.cuh"
+#include "tiles.cuh"
 
 namespace mop {
 
@@ -169,97 +169,147 @@ __global__ void __launch_bounds__(PERM_WARPS * 32) perm_rank_kernel(const int32_
     }
 }
 
-// Small layers: histogram, scan and rank in ONE block (the three launches above cost more than their work when
-// there are only a few units).  Warp w owns the units w, w + 32, ...; cnt[u][e] lives in shared memory, first as
-// the unit's histogram, then as the first row of unit u inside expert e.  Same tables as the three-kernel path.
-constexpr int PERM_SMALL_MAX_UNITS = 8;       // beyond that the three parallel kernels are faster (measured at 48 units)
-constexpr int PERM_SMALL_MAX_WORDS = 10240;     // units * E words of shared memory (40 KiB)
-__global__ void __launch_bounds__(1024) perm_small_kernel(const int32_t* __restrict__ idx, int32_t* __restrict__ counts,
-                                                          int32_t* __restrict__ offsets, int32_t* __restrict__ perm_row,
-                                                          int32_t* __restrict__ row_src, int M, int E, int units) {
-    pdl_begin();
+// The whole permutation in ONE launch: a cluster of up to eight CTAs of 32 warps, each warp with its run of `per_warp` assignments.
+// A warp counts its run (counts need no order: atomics on its own row of shared memory), a thread per expert scans the 32 rows of
+// its CTA, the CTAs read each other's totals through distributed shared memory, every CTA scans the experts for itself, and the
+// warps walk their runs again in order.  Same tables as the three kernels above.  tile_table: the token tiles of the GEMMs too.
+// Bounded by latency, and by the scattered row_src entries (a store of 32 of them takes 32 cycles of an SM, and there are eight SMs)
+// where there are many: us a call in a graph, three kernels (one block with a single cluster's work below 4097 assignments) and this
+// one: M 32, E 8 4.4 and 2.4; 512, 256 11.0 and 3.6; 4096, 64 11.4 and 4.8; 4611, 20 13.0 and 4.6; 24576, 64 15.7 and 6.9; 16384,
+// 1024 20.8 and 10.0; 131072, 256 21.9 and 24.0; 262144, 64 25.4 and 37.5.  Hence the line, PC_MAX_M.
+constexpr int PC_WARPS = 32;
+constexpr int PC_BATCH = 8;            // loads of a lane in flight
+constexpr long long PC_MAX_M = 98304;
+constexpr int PC_MAX_CTAS = 8;         // the portable cluster size
+__global__ void __launch_bounds__(PC_WARPS * 32) perm_cluster_kernel(const int32_t* __restrict__ idx, int32_t* __restrict__ counts,
+                                                                     int32_t* __restrict__ offsets, int32_t* __restrict__ perm_row,
+                                                                     int32_t* __restrict__ row_src, int M, int E, int per_warp,
+                                                                     int32_t* __restrict__ tile_table) {
     extern __shared__ int32_t perm_smem[];
-    int32_t* cnt = perm_smem;                      // [units][E]
-    int32_t* off = perm_smem + (size_t)units * E;  // [E + 1]
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int i = threadIdx.x; i < units * E; i += blockDim.x) cnt[i] = 0;
-    __syncthreads();
-    for (int u = warp; u < units; u += 32) {
-        int32_t* c = cnt + (size_t)u * E;
-        for (int it = 0; it < PERM_SEG / 32; ++it) {
-            const int a = u * PERM_SEG + it * 32 + lane;
-            int e = (a < M) ? idx[a] : -1;
-            if (e < 0 || e >= E) e = -1;
-            const uint32_t same = __match_any_sync(0xffffffffu, e);
-            if (e >= 0 && lane == __ffs(same) - 1) c[e] += __popc(same);
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-        int32_t run = 0;
-        for (int u = 0; u < units; ++u) {
-            const int32_t c = cnt[(size_t)u * E + e];
-            cnt[(size_t)u * E + e] = run;
-            run += c;
-        }
-        counts[e] = run;
-        off[e] = run;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        int32_t carry = 0;
-        for (int e0 = 0; e0 < E; e0 += 32) {
-            const int e = e0 + lane;
-            const int32_t c = (e < E) ? off[e] : 0;
-            int32_t inc = c;
+    int32_t* cnt = perm_smem;                          // [PC_WARPS][E]
+    int32_t* first = cnt + (size_t)PC_WARPS * E;       // [E] first row of this CTA's assignments of an expert
+    int32_t* off = first + E;                          // [E + 1]
+    int32_t* tot = off + E + 1;                        // [E] this CTA's totals, read by the others
+    int32_t* wsum = tot + E;                           // [32]
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tid = threadIdx.x;
+    const int n_ctas = gridDim.x, rank = blockIdx.x;   // the grid is one cluster
+    int32_t* mine = cnt + (size_t)warp * E;
+    for (int e = lane; e < E; e += 32) mine[e] = 0;
+    __syncwarp();
+    pdl_begin();
+    const long long a0 = (long long)(rank * PC_WARPS + warp) * per_warp;
+    const int n = (int)max(0ll, min((long long)per_warp, M - a0));       // assignments of this warp
+    const int32_t* run_idx = idx + a0;
+    auto load = [&](int b, int (&ev)[PC_BATCH]) {
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += v;
-            }
-            if (e < E) off[e] = carry + inc - c;
-            carry += __shfl_sync(0xffffffffu, inc, 31);
+        for (int i = 0; i < PC_BATCH; ++i) {
+            const int o = b + 32 * i + lane;
+            const int e = o < n ? run_idx[o] : -1;
+            ev[i] = e >= 0 && e < E ? e : -1;
         }
-        if (lane == 0) off[E] = carry;
+    };
+    for (int b = 0; b < n; b += 32 * PC_BATCH) {
+        int ev[PC_BATCH];
+        load(b, ev);
+#pragma unroll
+        for (int i = 0; i < PC_BATCH; ++i)
+            if (ev[i] >= 0) atomicAdd(&mine[ev[i]], 1);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e <= E; e += blockDim.x) offsets[e] = off[e];
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int u = warp; u < units; u += 32) {
-        int32_t* run = cnt + (size_t)u * E;
-        for (int e = lane; e < E; e += 32) run[e] += off[e];
+    int total = 0;
+    if (tid < E) {                                     // E <= 1024: a thread per expert
+#pragma unroll
+        for (int w0 = 0; w0 < PC_WARPS; w0 += 16) {
+            int c[16];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) c[w] = cnt[(w0 + w) * E + tid];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) { cnt[(w0 + w) * E + tid] = total; total += c[w]; }
+        }
+        tot[tid] = total;
+    }
+    int before = 0;
+    if (n_ctas > 1) {
+        cluster_sync_all();
+        if (tid < E) {
+            const uint32_t addr = (uint32_t)__cvta_generic_to_shared(tot + tid);
+            total = 0;
+            for (int r = 0; r < n_ctas; ++r) {
+                int v;
+                asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.s32 %0, [a];\n}"
+                             : "=r"(v) : "r"(addr), "r"(r) : "memory");
+                if (r < rank) before += v;
+                total += v;
+            }
+        }
         __syncwarp();
-        for (int it = 0; it < PERM_SEG / 32; ++it) {
-            const int a = u * PERM_SEG + it * 32 + lane;
-            int e = (a < M) ? idx[a] : -1;
-            if (e < 0 || e >= E) e = -1;
-            const uint32_t same = __match_any_sync(0xffffffffu, e);
-            int32_t p = -1;
-            if (e >= 0) p = run[e] + __popc(same & lt);
-            __syncwarp();
-            if (e >= 0 && lane == __ffs(same) - 1) run[e] += __popc(same);
-            __syncwarp();
-            if (a < M) {
-                perm_row[a] = p;
-                if (p >= 0) row_src[p] = a;
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");    // (waited for before this CTA leaves)
+    }
+    int rows;
+    const int base = block_exclusive_sum<PC_WARPS * 32>(total, wsum, rows);
+    if (tid < E) {
+        off[tid] = base;
+        first[tid] = base + before;
+        if (rank == 0) { counts[tid] = total; offsets[tid] = base; }
+    }
+    if (tid == 0) {
+        off[E] = rows;
+        if (rank == 0) offsets[E] = rows;
+    }
+    __syncthreads();
+    if (n > 0) {
+        for (int e = lane; e < E; e += 32) mine[e] += first[e];
+        __syncwarp();
+        const uint32_t lt = (1u << lane) - 1u;
+        for (int b = 0; b < n; b += 32 * PC_BATCH) {
+            int ev[PC_BATCH];
+            load(b, ev);
+#pragma unroll
+            for (int i = 0; i < PC_BATCH; ++i) {
+                if (b + 32 * i >= n) break;
+                const int e = ev[i];
+                const uint32_t same = __match_any_sync(0xffffffffu, e);
+                int32_t p = -1;
+                if (e >= 0) p = mine[e] + __popc(same & lt);
+                __syncwarp();
+                if (e >= 0 && (same & lt) == 0) mine[e] += __popc(same);
+                __syncwarp();
+                const int o = b + 32 * i + lane;
+                if (o < n) {
+                    perm_row[a0 + o] = p;
+                    if (p >= 0) row_src[p] = (int32_t)(a0 + o);
+                }
             }
         }
     }
+    if (tile_table && rank == n_ctas - 1) write_token_tiles<PC_WARPS * 32>(off, E, tile_table, wsum);
+    if (n_ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-inline bool perm_small_fits(int units, int E) {
-    return units > 0 && units <= PERM_SMALL_MAX_UNITS && (long long)units * E <= PERM_SMALL_MAX_WORDS;
+inline size_t perm_cluster_smem(int E) { return ((size_t)PC_WARPS * E + 3 * E + 1 + 32) * sizeof(int32_t); }
+inline bool perm_cluster_init() {
+    return cudaFuncSetAttribute(perm_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)perm_cluster_smem(TT_MAX_E)) ==
+           cudaSuccess;
+}
+inline bool perm_cluster_fits(long long M) { return M <= PC_MAX_M; }
+inline void launch_perm_cluster(const int32_t* idx, int32_t* counts, int32_t* offsets, int32_t* perm_row, int32_t* row_src, int M,
+                                int E, int32_t* tile_table, cudaStream_t st) {
+    int ctas = 1;
+    while (ctas < PC_MAX_CTAS && ctas * PC_WARPS * 32 < M) ctas *= 2;
+    const int per_warp = ceil_div(ceil_div(M, ctas * PC_WARPS), 32) * 32;
+    pdl_launch_clusters(perm_cluster_kernel, ctas, ctas, PC_WARPS * 32, perm_cluster_smem(E), st, idx, counts, offsets, perm_row,
+                        row_src, M, E, per_warp, tile_table);
 }
 
 // Scatter rows: one warp per token reads x[t,:] once (16-byte vectors, coalesced) and writes it to
 // its k destination rows.  Used for x -> Xp and for dY -> dYp.
 __global__ void __launch_bounds__(256) scatter_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                            const int32_t* __restrict__ perm_row, int T, int k,
-                                                           int vec_per_row) {
+                                                           int vec_per_row, TileJob job) {
     pdl_begin();
-    const int warps_per_block = blockDim.x / 32;
+    if (tile_block(job)) return;
+    const int warps_per_block = blockDim.x / 32, block = blockIdx.x - job.blocks(), blocks = gridDim.x - job.blocks();
     const int lane = threadIdx.x % 32;
-    for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
+    for (int t = block * warps_per_block + threadIdx.x / 32; t < T; t += blocks * warps_per_block) {
         int32_t myrow = -1;
         if (lane < k) myrow = perm_row[(size_t)t * k + lane];  // k <= 32 checked on the host
         const uint4* s = src + (size_t)t * vec_per_row;
@@ -339,11 +389,12 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(const uint4* __restri
 template <int VPL>
 __global__ void __launch_bounds__(256) scatter_rows_reg_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                                const int32_t* __restrict__ perm_row, int T, int k,
-                                                               int vec_per_row) {
+                                                               int vec_per_row, TileJob job) {
     pdl_begin();
-    const int warps_per_block = blockDim.x / 32;
+    if (tile_block(job)) return;
+    const int warps_per_block = blockDim.x / 32, block = blockIdx.x - job.blocks(), blocks = gridDim.x - job.blocks();
     const int lane = threadIdx.x % 32;
-    for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
+    for (int t = block * warps_per_block + threadIdx.x / 32; t < T; t += blocks * warps_per_block) {
         int32_t myrow = -1;
         if (lane < k) myrow = perm_row[(size_t)t * k + lane];  // k <= 32 checked on the host
         const uint4* s = src + (size_t)t * vec_per_row;
@@ -432,14 +483,14 @@ __global__ void __launch_bounds__(256) combine_rows_seg_kernel(const uint4* __re
 
 // Launchers: the register-row forms for rows of up to 16 KiB, the chunked kernels otherwise.
 inline void launch_scatter_rows(const uint4* src, uint4* dst, const int32_t* perm_row, int T, int k, int vec_per_row,
-                                int sm_count, cudaStream_t st) {
-    const int blocks = min(ceil_div(T, 8), sm_count * 8);
-    if (blocks <= 0) return;
-    if (vec_per_row <= 32 * 8) pdl_launch(scatter_rows_reg_kernel<8>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 16) pdl_launch(scatter_rows_reg_kernel<16>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 28) pdl_launch(scatter_rows_reg_kernel<28>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
-    else if (vec_per_row <= 32 * 32) pdl_launch(scatter_rows_reg_kernel<32>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
-    else pdl_launch(scatter_rows_kernel, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row);
+                                int sm_count, cudaStream_t st, const TileJob& job = TileJob{}) {
+    const int blocks = min(ceil_div(T, 8), sm_count * 8) + job.blocks();
+    if (T <= 0) return;
+    if (vec_per_row <= 32 * 8) pdl_launch(scatter_rows_reg_kernel<8>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row, job);
+    else if (vec_per_row <= 32 * 16) pdl_launch(scatter_rows_reg_kernel<16>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row, job);
+    else if (vec_per_row <= 32 * 28) pdl_launch(scatter_rows_reg_kernel<28>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row, job);
+    else if (vec_per_row <= 32 * 32) pdl_launch(scatter_rows_reg_kernel<32>, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row, job);
+    else pdl_launch(scatter_rows_kernel, blocks, 256, 0, st, src, dst, perm_row, T, k, vec_per_row, job);
 }
 inline void launch_combine_rows(const uint4* Yp, const int32_t* perm_row, uint4* Y, int T, int k, int vec_per_row,
                                 int sm_count, cudaStream_t st) {
@@ -513,12 +564,14 @@ constexpr int CHUNK_SEG = 4;
 // d = 7168, 4096 rows (117 MB): 25 us, 26 with a warp per row.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
                                                           const int32_t* __restrict__ row_src_c,
-                                                          const int32_t* __restrict__ bounds, int k, int vec_per_row) {
+                                                          const int32_t* __restrict__ bounds, int k, int vec_per_row,
+                                                          TileJob job) {
     pdl_begin();
-    const int lane = threadIdx.x % 32, wpb = blockDim.x / 32;
+    if (tile_block(job)) return;
+    const int lane = threadIdx.x % 32, wpb = blockDim.x / 32, block = blockIdx.x - job.blocks(), blocks = gridDim.x - job.blocks();
     const int segs = (vec_per_row + 32 * CHUNK_SEG - 1) / (32 * CHUNK_SEG);
     const long long items = (long long)bounds[1] * segs;
-    for (long long i = (long long)blockIdx.x * wpb + threadIdx.x / 32; i < items; i += (long long)gridDim.x * wpb) {
+    for (long long i = (long long)block * wpb + threadIdx.x / 32; i < items; i += (long long)blocks * wpb) {
         const int r = (int)(i / segs), c = (int)(i % segs) * 32 * CHUNK_SEG + lane;
         const uint4* s = src + (size_t)(row_src_c[r] / k) * vec_per_row;
         uint4* o = dst + (size_t)r * vec_per_row;

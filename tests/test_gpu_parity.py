@@ -330,6 +330,29 @@ def test_permutation_tables_on_both_sides_of_the_single_block_limit(T, k, E):
     assert torch.equal(Xp.cpu(), x.cpu()[torch.from_numpy(row_src // k).long()])
 
 
+@pytest.mark.parametrize("T,k,E", [(1, 1, 1), (11, 3, 5), (512, 2, 33), (1025, 1, 1024), (341, 12, 40),   # 1, 1, 1, 2, 4 blocks
+                                   (8192, 1, 2), (2731, 3, 257),                # eight: 32 assignments a warp, 64
+                                   (32768, 3, 31), (32769, 3, 31)])             # the longest runs, the three kernels
+def test_permutation_in_one_launch_with_indices_out_of_range(T, k, E):
+    """Assignments whose index names no expert get row -1 and are counted nowhere; the others keep their order."""
+    gen = torch.Generator().manual_seed(3 * T + E)
+    idx = torch.randint(-1, E + 1, (T, k), generator=gen, dtype=torch.int32)
+    flat = idx.numpy().reshape(-1)
+    ok = (flat >= 0) & (flat < E)
+    counts = np.bincount(flat[ok], minlength=E)
+    order = np.flatnonzero(ok)[np.argsort(flat[ok], kind="stable")]
+    perm_row = np.full(T * k, -1, dtype=np.int32)
+    perm_row[order] = np.arange(order.size)
+    ctx = binding.Context(T, 64, E, k, 64)
+    dev = {n: torch.full((s,), -7, dtype=torch.int32, device="cuda") for n, s in
+           (("counts", E), ("offsets", E + 1), ("perm_row", T * k), ("row_src", T * k))}
+    binding.mop_moe_permute(ctx, None, idx.cuda(), dev["counts"], dev["offsets"], dev["perm_row"], dev["row_src"], None)
+    got = {n: v.cpu().numpy() for n, v in dev.items()}
+    assert np.array_equal(got["counts"], counts) and np.array_equal(got["offsets"], np.concatenate(([0], np.cumsum(counts))))
+    assert np.array_equal(got["perm_row"], perm_row) and np.array_equal(got["row_src"][:order.size], order)
+    assert (got["row_src"][order.size:] == -7).all()
+
+
 def test_zero_tokens_is_a_no_op():
     w = synth.small("c1_tiny", T=0, d=64, E=4, k=2, f=64, backward=True)
     host, inp, ctx, buf = run(w)
