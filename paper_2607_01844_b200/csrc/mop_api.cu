@@ -583,7 +583,7 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
                                  topk_gate, lists, s.T, s.d, s.E, s.k, s.score_fn, s.bias_mode, 1, rblocks, st));
         return after_launch(c);
     }
-    LAUNCH(c, "route_score", st, route_score(static_cast<const bf16*>(x), W_r, z, s.T, s.d, s.E, c->sm_count, st));
+    LAUNCH(c, "route_score", st, route_score(static_cast<const bf16*>(x), W_r, z, s.T, s.d, s.E, c->sm_count, c->status, st));
     mop_status r = after_launch(c);
     if (r != MOP_OK) return r;
     const size_t smem = (size_t)SEL_WARPS * 2 * s.E * sizeof(float);

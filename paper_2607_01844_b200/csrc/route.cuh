@@ -1,240 +1,9 @@
-// Router kernels: exact fp32 scoring and warp-per-token top-k with gate renormalisation
+// Router kernels: warp-per-token top-k with gate renormalisation, the tensor-core scoring path, the router backward
 // (the router of the MoE block, Section 2.1 of the paper).
 #pragma once
-#include "common.cuh"
+#include "route_score.cuh"
 
 namespace mop {
-
-// ---------------------------------------------------------------------------------------------
-// Scoring.  z[t,e] = sum_i x[t,i] * W_r[i,e] as ONE chain of fused multiply-adds per (t,e), i
-// ascending, each step rounded once to fp32.  The chain order is part of the routing contract
-// (it makes top-k indices reproducible bit for bit), so there is no split over i and no tensor
-// core here; parallelism comes from the T*E independent chains.  Each thread owns RT tokens x RE
-// experts; with several experts it advances two chains (experts e, e + 1) per instruction with the
-// packed fma.rn.f32x2 of sm_100 (two independent IEEE fused multiply-adds: the rounding of each chain is unchanged).
-//
-// What bounds it: the fp32 pipes and shared memory where there are many chains, the latency of a dependent multiply-add where
-// there are few.  Either way the operands must not be waited for: stages of 64 steps are copied by cp.async two or three
-// stages ahead (x as bf16, W_r as fp32).  With one slab of 32 steps ahead in registers every slab cost a trip to L2: 48
-// cycles a step at T = 4096, d = 2048, E = 64.
-// A warp covers LT RT tokens x (32 / LT) RE experts, a block of four warps four times the tokens; the shape is picked by
-// route_score() from the number of blocks per SM and the cycles of a step.
-// ---------------------------------------------------------------------------------------------
-constexpr int SC_THREADS = 128;
-constexpr int SC_TK = 64;          // steps per stage
-constexpr int SC_XPITCH = SC_TK + 8;   // bf16 elements: neighbouring tokens' rows 16 bytes apart in the banks
-
-__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void fma_f32x2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool ok) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
-}
-
-template <int RT, int RE, int LT>
-struct ScoreShape {
-    static constexpr int LE = 32 / LT;
-    static constexpr int TT = 4 * LT * RT, TE = LE * RE;
-    static constexpr int X_BYTES = TT * SC_XPITCH * 2, W_BYTES = SC_TK * TE * 4, STAGE = X_BYTES + W_BYTES;
-    static constexpr int STAGES = RT * RE >= 32 ? 3 : 4;
-    static constexpr int SMEM = STAGES * STAGE;
-};
-
-template <int RT, int RE, int LT>
-__global__ void __launch_bounds__(SC_THREADS) route_score_kernel(const bf16* __restrict__ x, const float* __restrict__ W_r,
-                                                                 float* __restrict__ z, int T, int d, int E) {
-    pdl_begin();
-    using Sh = ScoreShape<RT, RE, LT>;
-    constexpr int LE = Sh::LE, TT = Sh::TT, TE = Sh::TE, S = Sh::STAGES;
-    static_assert(RE == 1 || (RE % 4 == 0 && LE == 8), "expert columns of a thread: one, or groups of four 32 apart");
-    static_assert(Sh::X_BYTES % 16 == 0 && Sh::STAGE % 16 == 0, "16-byte copies");
-    extern __shared__ __align__(16) uint8_t sc_smem[];
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sc_smem);
-    const int t0 = blockIdx.x * TT, e0 = blockIdx.y * TE;
-    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    // Tokens of a thread: tt, tt + LT, ..  Lanes of a quarter warp share few addresses of both operands: a vector load whose
-    // quarters each read the same 128 bytes costs four wavefronts, one whose quarters read different ones together costs one.
-    const int tt = warp * LT * RT + (RE == 1 ? lane / LE : lane % LT);
-    const int te = RE == 1 ? lane % LE : (lane / LT) * 4;           // first expert; further groups of four 32 apart
-    const bool w_vec = (E % 4 == 0);
-
-    auto load = [&](int s, int i0) {
-        const uint32_t xb = base + s * Sh::STAGE, wb = xb + Sh::X_BYTES;
-#pragma unroll
-        for (int v = tid; v < TT * (SC_TK / 8); v += SC_THREADS) {  // 16 bytes = 8 steps of one token
-            const int t = v / (SC_TK / 8), c = (v % (SC_TK / 8)) * 8;
-            const bool ok = t0 + t < T && i0 + c < d;
-            cp_async16(xb + (t * SC_XPITCH + c) * 2, ok ? x + (size_t)(t0 + t) * d + i0 + c : x, ok);
-        }
-        if (w_vec) {
-#pragma unroll
-            for (int v = tid; v < SC_TK * TE / 4; v += SC_THREADS) {
-                const int i = v / (TE / 4), e = (v % (TE / 4)) * 4;
-                const bool ok = i0 + i < d && e0 + e < E;
-                cp_async16(wb + (i * TE + e) * 4, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
-            }
-        } else if (E % 2 == 0) {
-#pragma unroll 4
-            for (int v = tid; v < SC_TK * TE / 2; v += SC_THREADS) {
-                const int i = v / (TE / 2), e = (v % (TE / 2)) * 2;
-                const bool ok = i0 + i < d && e0 + e < E;
-                cp_async8(wb + v * 8, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
-            }
-        } else {
-#pragma unroll 4
-            for (int v = tid; v < SC_TK * TE; v += SC_THREADS) {
-                const int i = v / TE, e = v % TE;
-                const bool ok = i0 + i < d && e0 + e < E;
-                cp_async4(wb + v * 4, ok ? W_r + (size_t)(i0 + i) * E + e0 + e : W_r, ok);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    const int stages = (d + SC_TK - 1) / SC_TK;
-#pragma unroll
-    for (int s = 0; s < S - 1; ++s) {
-        if (s < stages) load(s, s * SC_TK);
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    constexpr int G = RT * RE >= 32 ? 4 : 8;                        // steps whose operands are in registers
-    constexpr int NP = RE == 1 ? 1 : RE / 2;                        // pairs of experts (RE = 1: a plain chain)
-    unsigned long long acc[RT][NP];
-    float acc1[RT];
-#pragma unroll
-    for (int a = 0; a < RT; ++a) {
-        acc1[a] = 0.0f;
-#pragma unroll
-        for (int b = 0; b < NP; ++b) acc[a][b] = 0ull;
-    }
-    for (int st = 0; st < stages; ++st) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
-        __syncthreads();          // stage st has arrived for every thread, and stage st - 1 has been read by every thread
-        if (st + S - 1 < stages) load((st + S - 1) % S, (st + S - 1) * SC_TK);
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-        const uint8_t* sx = sc_smem + (st % S) * Sh::STAGE;
-        const bf16* xs = reinterpret_cast<const bf16*>(sx) + tt * SC_XPITCH;
-        const float* ws = reinterpret_cast<const float*>(sx + Sh::X_BYTES) + te;
-        // Steps past d (d not a multiple of a stage) multiply zeros: fma(0, 0, acc) = acc, exact.  Operands of the next G steps
-        // are read while the current ones are multiplied.
-        uint32_t xv[2][RT][G / 2];
-        float wv[2][G][RE];
-        auto fetch = [&](int buf, int k) {
-#pragma unroll
-            for (int a = 0; a < RT; ++a) {
-                if constexpr (G == 8) {
-                    const uint4 q = *reinterpret_cast<const uint4*>(xs + a * LT * SC_XPITCH + k);
-                    xv[buf][a][0] = q.x; xv[buf][a][1] = q.y; xv[buf][a][2] = q.z; xv[buf][a][3] = q.w;
-                } else {
-                    const uint2 q = *reinterpret_cast<const uint2*>(xs + a * LT * SC_XPITCH + k);
-                    xv[buf][a][0] = q.x; xv[buf][a][1] = q.y;
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < G; ++j) {
-                if constexpr (RE == 1) wv[buf][j][0] = ws[(k + j) * TE];
-                else {
-#pragma unroll
-                    for (int b = 0; b < RE / 4; ++b) {
-                        const float4 v = *reinterpret_cast<const float4*>(ws + (k + j) * TE + 32 * b);
-                        wv[buf][j][4 * b] = v.x; wv[buf][j][4 * b + 1] = v.y; wv[buf][j][4 * b + 2] = v.z; wv[buf][j][4 * b + 3] = v.w;
-                    }
-                }
-            }
-        };
-        fetch(0, 0);
-#pragma unroll
-        for (int k = 0; k < SC_TK; k += G) {
-            const int cur = (k / G) & 1;
-            if (k + G < SC_TK) fetch(cur ^ 1, k + G);
-#pragma unroll
-            for (int j = 0; j < G; ++j)
-#pragma unroll
-                for (int a = 0; a < RT; ++a) {
-                    const float x1 = (j & 1) ? bf16_hi(xv[cur][a][j >> 1]) : bf16_lo(xv[cur][a][j >> 1]);
-                    if constexpr (RE == 1) acc1[a] = __fmaf_rn(x1, wv[cur][j][0], acc1[a]);
-                    else {
-                        const unsigned long long xp = pack_f32x2(x1, x1);
-#pragma unroll
-                        for (int b = 0; b < NP; ++b) fma_f32x2(acc[a][b], xp, pack_f32x2(wv[cur][j][2 * b], wv[cur][j][2 * b + 1]));
-                    }
-                }
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < RT; ++a) {
-        const int t = t0 + tt + LT * a;
-        if (t >= T) continue;
-        if constexpr (RE == 1) {
-            if (e0 + te < E) z[(size_t)t * E + e0 + te] = acc1[a];
-        } else {
-#pragma unroll
-            for (int b = 0; b < RE / 4; ++b) {
-                float v[4];
-                unpack_f32x2(acc[a][2 * b], v[0], v[1]);
-                unpack_f32x2(acc[a][2 * b + 1], v[2], v[3]);
-                const int e = e0 + te + 32 * b;
-                float* dst = z + (size_t)t * E + e;
-                if (w_vec && e + 3 < E) {
-                    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (e + q < E) dst[q] = v[q];
-                }
-            }
-        }
-    }
-}
-
-template <int RT, int RE, int LT>
-inline bool route_score_attr() {
-    return cudaFuncSetAttribute(route_score_kernel<RT, RE, LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                ScoreShape<RT, RE, LT>::SMEM) == cudaSuccess;
-}
-inline bool route_score_init() {
-    return route_score_attr<1, 1, 4>() && route_score_attr<2, 4, 4>() && route_score_attr<4, 4, 4>() &&
-           route_score_attr<4, 8, 4>();
-}
-template <int RT, int RE, int LT>
-inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, cudaStream_t st) {
-    using Sh = ScoreShape<RT, RE, LT>;
-    dim3 grid(ceil_div(T, Sh::TT), ceil_div(E, Sh::TE));
-    pdl_launch(route_score_kernel<RT, RE, LT>, grid, SC_THREADS, Sh::SMEM, st, x, W_r, z, T, d, E);
-}
-// Shape choice: the least estimated cycles per step on the fullest SM, first + more * (blocks on it - 1), as measured at
-// d = 7168 (one block alone on an SM; each further one).  Decoding (T = 64, E = 256) takes one chain per thread: 130 us with the
-// former slabs, 46 now, 136 with 4 x 4; T = 4096, d = 2048, E = 64 takes 4 x 4: 50 -> 44 us, 97 with one chain per thread;
-// T = 8192, d = 7168, E = 128 takes 4 x 8: 472 -> 370 us, 415 with 4 x 4.
-inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int sm_count, cudaStream_t st) {
-    const struct { int tt, te; float first, more; } shape[4] = {
-        {16, 8, 12.f, 6.f}, {32, 32, 28.f, 15.f}, {64, 32, 36.5f, 26.f}, {64, 64, 55.5f, 45.f}};
-    int pick = 0;
-    float best = 0.0f;
-    for (int i = 0; i < 4; ++i) {
-        const long long blocks = (long long)ceil_div(T, shape[i].tt) * ceil_div(E, shape[i].te);
-        const float cost = shape[i].first + shape[i].more * (float)((blocks + sm_count - 1) / sm_count - 1);
-        if (i == 0 || cost <= best) { best = cost; pick = i; }
-    }
-    if (pick == 0) launch_route_score<1, 1, 4>(x, W_r, z, T, d, E, st);
-    else if (pick == 1) launch_route_score<2, 4, 4>(x, W_r, z, T, d, E, st);
-    else if (pick == 2) launch_route_score<4, 4, 4>(x, W_r, z, T, d, E, st);
-    else launch_route_score<4, 8, 4>(x, W_r, z, T, d, E, st);
-}
 
 // Sigmoid of the routing contract: a fixed sequence of fp32 operations, each rounded once
 // (explicit-rounding intrinsics so that no contraction or fast path can change a step).

@@ -674,6 +674,14 @@ def test_exact_scoring_shapes_give_the_contract_chains(T, d, E):
     assert np.array_equal(buf.idx[:300].cpu().numpy(), idx[:300])
 
 
+@pytest.mark.parametrize("T,d,E", [(40, 1000, 9),                        # 16 x 8: the ring of stages around, the last one partly filled
+                                   (1500, 776, 17), (4000, 8, 8),        # 32 x 8, and a single stage of 8 steps
+                                   (1300, 520, 40), (1300, 456, 41),     # 32 x 32
+                                   (4100, 392, 62), (8200, 328, 65)])    # 64 x 32 and 64 x 64
+def test_exact_scoring_with_more_steps_than_its_ring_holds(T, d, E):
+    test_exact_scoring_shapes_give_the_contract_chains(T, d, E)
+
+
 FAST_ROUTE = [
     synth.small("c3_trillion", T=1000, d=512, E=256, k=8, f=64, seed=60),                  # sigmoid + post-score bias
     synth.small("c3_trillion", T=777, d=320, E=64, k=3, f=64, bias_mode=2, seed=61),        # sigmoid, bias before the score
