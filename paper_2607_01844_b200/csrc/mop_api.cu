@@ -13,8 +13,7 @@
 #include "gemm_scalar.cuh"
 #include "gemm_host.cuh"
 #include "gemm_rs.cuh"
-#include "permute.cuh"
-#include "route.cuh"
+#include "route_permute.cuh"
 
 using namespace mop;
 
@@ -308,7 +307,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
         return MOP_ERR_UNSUPPORTED;
     }
     c->tensor_tn = shape->gemm_path != MOP_GEMM_SCALAR && (c->tensor_ok || (prop.major == 10 && c->sm_count >= 2));
-    if (!route_score_init() || !route_chain_init() || !perm_cluster_init()) { delete c; return MOP_ERR_CUDA; }
+    if (!route_score_init() || !route_chain_init() || !perm_cluster_init() || !route_permute_init()) { delete c; return MOP_ERR_CUDA; }
     const Layout L = make_layout(*shape);
     c->ws_bytes = L.total;
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }
@@ -586,10 +585,7 @@ mop_status mop_moe_route(mop_ctx* c, const void* x, const float* W_r, const floa
     LAUNCH(c, "route_score", st, route_score(static_cast<const bf16*>(x), W_r, z, s.T, s.d, s.E, c->sm_count, c->status, st));
     mop_status r = after_launch(c);
     if (r != MOP_OK) return r;
-    const size_t smem = (size_t)SEL_WARPS * 2 * s.E * sizeof(float);
-    LAUNCH(c, "route_select", st,
-           pdl_launch(route_select_kernel, ceil_div(s.T, SEL_WARPS), SEL_WARPS * 32, smem, st, z, bias, topk_idx, topk_gate, s.T,
-                      s.E, s.k, s.score_fn, s.bias_mode));
+    LAUNCH(c, "route_select", st, launch_route_select(z, bias, topk_idx, topk_gate, s.T, s.E, s.k, s.score_fn, s.bias_mode, st));
     return after_launch(c);
 }
 
@@ -758,10 +754,24 @@ mop_status layer_forward(mop_ctx* c, const void* x, const float* W_r, const floa
                          const void* W_down, int32_t* topk_idx, float* topk_gate, int32_t* counts, int32_t* offsets,
                          int32_t* perm_row, int32_t* row_src, void* Xp, void* G_save, void* U_save, void* H, void* Yp, void* Y,
                          void* stream) {
+    const mop_moe_shape& s = c->s;
     int32_t* table = shared_tiles(c);
     mop_status r;
-    if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
-    if ((r = permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, table, stream)) != MOP_OK) return r;
+    if (!c->fast_route && route_permute_fits(s.T, s.d, s.E, s.k)) {
+        DeviceGuard guard(c->device);
+        if (!guard.ok) return MOP_ERR_CUDA;
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        LAUNCH(c, "route_score", st,
+               route_score(static_cast<const bf16*>(x), W_r, c->z, s.T, s.d, s.E, c->sm_count, c->status, st));
+        if ((r = after_launch(c)) != MOP_OK) return r;
+        LAUNCH(c, "route_select_permute", st,
+               launch_route_permute(c->z, bias, topk_idx, topk_gate, counts, offsets, perm_row, row_src, s.T, s.d, s.E, s.k, s.score_fn,
+                                    s.bias_mode, table, static_cast<const uint4*>(x), static_cast<uint4*>(Xp), st));
+        if ((r = after_launch(c)) != MOP_OK) return r;
+    } else {
+        if ((r = mop_moe_route(c, x, W_r, bias, topk_idx, topk_gate, nullptr, stream)) != MOP_OK) return r;
+        if ((r = permute(c, x, topk_idx, counts, offsets, perm_row, row_src, Xp, table, stream)) != MOP_OK) return r;
+    }
     if ((r = expert_ffn_fwd(c, Xp, offsets, row_src, topk_gate, W_gate, W_up, W_down, G_save, U_save, H, Yp, table != nullptr,
                             stream)) != MOP_OK)
         return r;

@@ -181,19 +181,76 @@ constexpr int PC_WARPS = 32;
 constexpr int PC_BATCH = 8;            // loads of a lane in flight
 constexpr long long PC_MAX_M = 98304;
 constexpr int PC_MAX_CTAS = 8;         // the portable cluster size
+struct PermSmem {
+    int32_t *cnt, *first, *off, *tot, *wsum;
+    __device__ PermSmem(int32_t* base, int E) {
+        cnt = base;                                    // [PC_WARPS][E] counts of the warps, then the next rows of each
+        first = cnt + (size_t)PC_WARPS * E;            // [E] first row of this CTA's assignments of an expert
+        off = first + E;                               // [E + 1]
+        tot = off + E + 1;                             // [E] this CTA's totals, read by the others
+        wsum = tot + E;                                // [32]
+    }
+};
+inline size_t perm_cluster_smem(int E) { return ((size_t)PC_WARPS * E + 3 * E + 1 + 32) * sizeof(int32_t); }
+
+// From the warps' counts to their first rows (less sm.first, which the caller adds), counts, offsets and sm.off.  Every CTA of the
+// cluster calls it with all its threads, and waits for the cluster's barrier once more before it leaves (n_ctas > 1).
+__device__ __forceinline__ void perm_cluster_scan(const PermSmem& sm, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
+                                                  int E, int n_ctas, int rank) {
+    const int tid = threadIdx.x;
+    __syncthreads();
+    int total = 0;
+    if (tid < E) {                                     // E <= 1024: a thread per expert
+#pragma unroll
+        for (int w0 = 0; w0 < PC_WARPS; w0 += 16) {
+            int c[16];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) c[w] = sm.cnt[(w0 + w) * E + tid];
+#pragma unroll
+            for (int w = 0; w < 16; ++w) { sm.cnt[(w0 + w) * E + tid] = total; total += c[w]; }
+        }
+        sm.tot[tid] = total;
+    }
+    int before = 0;
+    if (n_ctas > 1) {
+        cluster_sync_all();
+        if (tid < E) {
+            const uint32_t addr = (uint32_t)__cvta_generic_to_shared(sm.tot + tid);
+            total = 0;
+            for (int r = 0; r < n_ctas; ++r) {
+                int v;
+                asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.s32 %0, [a];\n}"
+                             : "=r"(v) : "r"(addr), "r"(r) : "memory");
+                if (r < rank) before += v;
+                total += v;
+            }
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
+    int rows;
+    const int base = block_exclusive_sum<PC_WARPS * 32>(total, sm.wsum, rows);
+    if (tid < E) {
+        sm.off[tid] = base;
+        sm.first[tid] = base + before;
+        if (rank == 0) { counts[tid] = total; offsets[tid] = base; }
+    }
+    if (tid == 0) {
+        sm.off[E] = rows;
+        if (rank == 0) offsets[E] = rows;
+    }
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(PC_WARPS * 32) perm_cluster_kernel(const int32_t* __restrict__ idx, int32_t* __restrict__ counts,
                                                                      int32_t* __restrict__ offsets, int32_t* __restrict__ perm_row,
                                                                      int32_t* __restrict__ row_src, int M, int E, int per_warp,
                                                                      int32_t* __restrict__ tile_table) {
     extern __shared__ int32_t perm_smem[];
-    int32_t* cnt = perm_smem;                          // [PC_WARPS][E]
-    int32_t* first = cnt + (size_t)PC_WARPS * E;       // [E] first row of this CTA's assignments of an expert
-    int32_t* off = first + E;                          // [E + 1]
-    int32_t* tot = off + E + 1;                        // [E] this CTA's totals, read by the others
-    int32_t* wsum = tot + E;                           // [32]
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, tid = threadIdx.x;
+    const PermSmem sm(perm_smem, E);
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int n_ctas = gridDim.x, rank = blockIdx.x;   // the grid is one cluster
-    int32_t* mine = cnt + (size_t)warp * E;
+    int32_t* mine = sm.cnt + (size_t)warp * E;
     for (int e = lane; e < E; e += 32) mine[e] = 0;
     __syncwarp();
     pdl_begin();
@@ -215,50 +272,9 @@ __global__ void __launch_bounds__(PC_WARPS * 32) perm_cluster_kernel(const int32
         for (int i = 0; i < PC_BATCH; ++i)
             if (ev[i] >= 0) atomicAdd(&mine[ev[i]], 1);
     }
-    __syncthreads();
-    int total = 0;
-    if (tid < E) {                                     // E <= 1024: a thread per expert
-#pragma unroll
-        for (int w0 = 0; w0 < PC_WARPS; w0 += 16) {
-            int c[16];
-#pragma unroll
-            for (int w = 0; w < 16; ++w) c[w] = cnt[(w0 + w) * E + tid];
-#pragma unroll
-            for (int w = 0; w < 16; ++w) { cnt[(w0 + w) * E + tid] = total; total += c[w]; }
-        }
-        tot[tid] = total;
-    }
-    int before = 0;
-    if (n_ctas > 1) {
-        cluster_sync_all();
-        if (tid < E) {
-            const uint32_t addr = (uint32_t)__cvta_generic_to_shared(tot + tid);
-            total = 0;
-            for (int r = 0; r < n_ctas; ++r) {
-                int v;
-                asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.s32 %0, [a];\n}"
-                             : "=r"(v) : "r"(addr), "r"(r) : "memory");
-                if (r < rank) before += v;
-                total += v;
-            }
-        }
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");    // (waited for before this CTA leaves)
-    }
-    int rows;
-    const int base = block_exclusive_sum<PC_WARPS * 32>(total, wsum, rows);
-    if (tid < E) {
-        off[tid] = base;
-        first[tid] = base + before;
-        if (rank == 0) { counts[tid] = total; offsets[tid] = base; }
-    }
-    if (tid == 0) {
-        off[E] = rows;
-        if (rank == 0) offsets[E] = rows;
-    }
-    __syncthreads();
+    perm_cluster_scan(sm, counts, offsets, E, n_ctas, rank);
     if (n > 0) {
-        for (int e = lane; e < E; e += 32) mine[e] += first[e];
+        for (int e = lane; e < E; e += 32) mine[e] += sm.first[e];
         __syncwarp();
         const uint32_t lt = (1u << lane) - 1u;
         for (int b = 0; b < n; b += 32 * PC_BATCH) {
@@ -282,10 +298,10 @@ __global__ void __launch_bounds__(PC_WARPS * 32) perm_cluster_kernel(const int32
             }
         }
     }
-    if (tile_table && rank == n_ctas - 1) write_token_tiles<PC_WARPS * 32>(off, E, tile_table, wsum);
+    if (tile_table && rank == n_ctas - 1) write_token_tiles<PC_WARPS * 32>(sm.off, E, tile_table, sm.wsum);
+    __syncwarp();
     if (n_ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-inline size_t perm_cluster_smem(int E) { return ((size_t)PC_WARPS * E + 3 * E + 1 + 32) * sizeof(int32_t); }
 inline bool perm_cluster_init() {
     return cudaFuncSetAttribute(perm_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)perm_cluster_smem(TT_MAX_E)) ==
            cudaSuccess;

@@ -353,6 +353,49 @@ def test_permutation_in_one_launch_with_indices_out_of_range(T, k, E):
     assert (got["row_src"][order.size:] == -7).all()
 
 
+@pytest.mark.parametrize("T,d,E,k,score,bias", [(1, 64, 256, 32, 1, 1), (7, 64, 3, 3, 0, 0), (9, 1032, 65, 4, 1, 2),     # one block, eight
+                                                (256, 64, 129, 8, 1, 1), (255, 520, 64, 4, 0, 0), (128, 1024, 40, 4, 1, 1),
+                                                (257, 64, 64, 4, 1, 1), (129, 1024, 40, 4, 0, 0), (60, 64, 257, 4, 1, 0)])   # in three
+def test_small_forward_in_one_call_equals_the_separate_calls(T, d, E, k, score, bias):
+    """Selection, permutation and row copy in one launch: the same bits as the separate entry points', on both sides of its limits."""
+    w = synth.Workload("one", T, d, E, k, 64, score, bias, 0.01 if bias else 0.0, seed=T + E)
+    inp = synth.make_inputs(w, "cuda")
+    ctx = binding.context_for(w, route_path=binding.ROUTE_EXACT)
+    one, sep = binding.LayerBuffers(w), binding.LayerBuffers(w)
+    binding.forward(ctx, inp, one)
+    binding.mop_moe_route(ctx, inp["x"], inp["W_r"], inp["bias"], sep.idx, sep.gate)
+    binding.mop_moe_permute(ctx, inp["x"], sep.idx, sep.counts, sep.offsets, sep.perm_row, sep.row_src, sep.Xp)
+    binding.mop_moe_expert_ffn_fwd(ctx, sep.Xp, sep.offsets, sep.row_src, sep.gate, inp["W_gate"], inp["W_up"], inp["W_down"],
+                                   None, None, sep.H, sep.Yp)
+    binding.mop_moe_combine(ctx, sep.Yp, sep.perm_row, sep.Y)
+    binding.mop_poll(ctx)
+    for name in ("idx", "gate", "counts", "offsets", "perm_row", "row_src", "Xp", "Y"):
+        assert torch.equal(getattr(one, name), getattr(sep, name)), name
+    x, W_r = synth.bits(inp["x"]), inp["W_r"].cpu().numpy()
+    idx, gate = oracle.route(x, W_r, None if not bias else inp["bias"].cpu().numpy(), k, score, bias)
+    assert np.array_equal(one.idx.cpu().numpy(), idx) and np.allclose(one.gate.cpu().numpy(), gate, rtol=1e-5, atol=1e-6)
+
+
+@pytest.mark.parametrize("E,k", [(31, 5), (200, 8), (500, 3), (1024, 32)])
+def test_selection_of_equal_signed_zero_and_infinite_logits(E, k):
+    """x = 1 everywhere and one row of W_r: the logits are that row.  Ties go to the lower id, -0 equals +0, infinities keep their place."""
+    d, T = 8, 5
+    gen = torch.Generator().manual_seed(E)
+    row = torch.randint(-2, 3, (E,), generator=gen).float()
+    row[::3] = torch.where(torch.arange(0, E, 3) % 2 == 0, 0.0, -0.0)
+    row[E // 2], row[E // 3] = float("inf"), float("-inf")
+    W_r = torch.zeros((d, E))
+    W_r[0] = row
+    order = np.lexsort((np.arange(E), -row.numpy().astype(np.float64)))[:k]
+    ctx = binding.Context(T, d, E, k, 64)
+    x = torch.zeros((T, d), dtype=torch.bfloat16)
+    x[:, 0] = 1.0
+    idx = torch.empty((T, k), dtype=torch.int32, device="cuda")
+    gate = torch.empty((T, k), dtype=torch.float32, device="cuda")
+    binding.mop_moe_route(ctx, x.cuda(), W_r.cuda(), None, idx, gate)
+    assert (idx.cpu().numpy() == order).all()
+
+
 def test_zero_tokens_is_a_no_op():
     w = synth.small("c1_tiny", T=0, d=64, E=4, k=2, f=64, backward=True)
     host, inp, ctx, buf = run(w)
