@@ -350,55 +350,6 @@ __global__ void __launch_bounds__(256) scatter_rows_kernel(const uint4* __restri
     }
 }
 
-// Combine: Y[t,:] = bf16(sum_j Yp[perm_row[t*k+j],:]) with the k-row sum kept in fp32 registers,
-// j ascending.  One warp per token, 16-byte vectors.
-__global__ void __launch_bounds__(256) combine_rows_kernel(const uint4* __restrict__ Yp,
-                                                           const int32_t* __restrict__ perm_row,
-                                                           uint4* __restrict__ Y, int T, int k, int vec_per_row) {
-    pdl_begin();
-    const int warps_per_block = blockDim.x / 32;
-    const int lane = threadIdx.x % 32;
-    for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
-        int32_t myrow = -1;
-        if (lane < k) myrow = perm_row[(size_t)t * k + lane];
-        for (int c0 = 0; c0 < vec_per_row; c0 += 64) {
-            float acc[2][8];
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc[q][i] = 0.0f;
-            for (int j = 0; j < k; ++j) {
-                const int32_t p = __shfl_sync(0xffffffffu, myrow, j);
-                if (p < 0) continue;
-                const uint4* r = Yp + (size_t)p * vec_per_row;
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int c = c0 + q * 32 + lane;
-                    if (c < vec_per_row) {
-                        const uint4 v = __ldcs(r + c);
-                        acc[q][0] += bf16_lo(v.x); acc[q][1] += bf16_hi(v.x);
-                        acc[q][2] += bf16_lo(v.y); acc[q][3] += bf16_hi(v.y);
-                        acc[q][4] += bf16_lo(v.z); acc[q][5] += bf16_hi(v.z);
-                        acc[q][6] += bf16_lo(v.w); acc[q][7] += bf16_hi(v.w);
-                    }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int c = c0 + q * 32 + lane;
-                if (c < vec_per_row) {
-                    uint4 o;
-                    o.x = pack_bf16x2(acc[q][0], acc[q][1]);
-                    o.y = pack_bf16x2(acc[q][2], acc[q][3]);
-                    o.z = pack_bf16x2(acc[q][4], acc[q][5]);
-                    o.w = pack_bf16x2(acc[q][6], acc[q][7]);
-                    Y[(size_t)t * vec_per_row + c] = o;
-                }
-            }
-        }
-    }
-}
-
 // Scatter rows with the whole source row in registers (VPL 16-byte vectors per lane, rows of up to 512 VPL
 // bytes): the row is read once and each of its k copies is written as one contiguous run, which DRAM takes
 // better than pieces of 2 KiB interleaved over k rows (random 2 KiB pieces: 4.4 TB/s at T = 16384, d = 7168).
@@ -433,67 +384,61 @@ __global__ void __launch_bounds__(256) scatter_rows_reg_kernel(const uint4* __re
     }
 }
 
-// Combine with longer runs per row: the row is walked in segments of 32 SEG vectors (3.5 or 4 KiB); for every
-// segment the k rows are read one after the other, the next row's vectors in flight while the current ones are
-// added.  Same sums in the same order as combine_rows_kernel (j ascending, fp32), so the same bits.
-template <int SEG>
-__global__ void __launch_bounds__(256) combine_rows_seg_kernel(const uint4* __restrict__ Yp,
-                                                               const int32_t* __restrict__ perm_row,
-                                                               uint4* __restrict__ Y, int T, int k, int vec_per_row) {
+// Combine: Y[t,:] = bf16(sum_j Yp[perm_row[t*k+j],:]) with the k-row sum kept in fp32 registers, j ascending.  A warp takes 32 SEG
+// vectors of a token's row, R rows' at a time.  HBM bound where there are many (T = 16384, d = 7168, k = 8: 338 us, 0.96 of the copy
+// rate), and there one row of 2 KiB at a time does best (T = 8192, d = 4096, k = 4: 55 us, 64 with two rows of 1 KiB, 78 with four,
+// 82 with a warp per token and rows of 4 KiB); latency bound where there are few, where a warp takes 512 bytes of all rows at once
+// (T = 16, d = 2048, k = 6 3.5 us, 12.9 with a warp per token; T = 64, d = 7168, k = 8 4.5 and 29.8).
+template <int SEG, int R>
+__global__ void __launch_bounds__(256) combine_rows_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ perm_row,
+                                                            uint4* __restrict__ Y, int T, int k, int vec_per_row) {
     pdl_begin();
-    const int warps_per_block = blockDim.x / 32;
-    const int lane = threadIdx.x % 32;
-    for (int t = blockIdx.x * warps_per_block + threadIdx.x / 32; t < T; t += gridDim.x * warps_per_block) {
+    const int lane = threadIdx.x % 32, wpb = blockDim.x / 32;
+    const int segs = (vec_per_row + 32 * SEG - 1) / (32 * SEG);
+    const long long items = (long long)T * segs;
+    for (long long i = (long long)blockIdx.x * wpb + threadIdx.x / 32; i < items; i += (long long)gridDim.x * wpb) {
+        const int t = (int)(i / segs), c = (int)(i - (long long)t * segs) * 32 * SEG + lane;
         int32_t myrow = -1;
         if (lane < k) myrow = perm_row[(size_t)t * k + lane];
-        for (int c0 = 0; c0 < vec_per_row; c0 += 32 * SEG) {
-            float acc[SEG][8];
+        float acc[SEG][8];
 #pragma unroll
-            for (int q = 0; q < SEG; ++q)
+        for (int q = 0; q < SEG; ++q)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[q][i] = 0.0f;
-            uint4 a[SEG], b[SEG];
-            auto load = [&](uint4 (&buf)[SEG], int j) -> bool {
-                const int32_t p = __shfl_sync(0xffffffffu, myrow, j);
-                if (p < 0) return false;
-                const uint4* r = Yp + (size_t)p * vec_per_row + c0 + lane;
+            for (int u = 0; u < 8; ++u) acc[q][u] = 0.0f;
+        for (int j0 = 0; j0 < k; j0 += R) {
+            uint4 v[R][SEG];
+            int32_t p[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                p[r] = __shfl_sync(0xffffffffu, myrow, (j0 + r) & 31);
+                if (j0 + r >= k) p[r] = -1;
+                const uint4* src = Yp + (size_t)max(p[r], 0) * vec_per_row + c;
 #pragma unroll
                 for (int q = 0; q < SEG; ++q)
-                    if (c0 + q * 32 + lane < vec_per_row) buf[q] = __ldcs(r + q * 32);
-                return true;
-            };
-            auto add = [&](const uint4 (&buf)[SEG]) {
-#pragma unroll
-                for (int q = 0; q < SEG; ++q) {
-                    if (c0 + q * 32 + lane < vec_per_row) {
-                        const uint4 v = buf[q];
-                        acc[q][0] += bf16_lo(v.x); acc[q][1] += bf16_hi(v.x);
-                        acc[q][2] += bf16_lo(v.y); acc[q][3] += bf16_hi(v.y);
-                        acc[q][4] += bf16_lo(v.z); acc[q][5] += bf16_hi(v.z);
-                        acc[q][6] += bf16_lo(v.w); acc[q][7] += bf16_hi(v.w);
-                    }
-                }
-            };
-            bool va = load(a, 0), vb = false;
-            for (int j = 0; j < k; j += 2) {
-                if (j + 1 < k) vb = load(b, j + 1);
-                if (va) add(a);
-                if (j + 2 < k) va = load(a, j + 2);
-                if (j + 1 < k && vb) add(b);
+                    if (p[r] >= 0 && c + 32 * q < vec_per_row) v[r][q] = __ldcs(src + 32 * q);
             }
 #pragma unroll
-            for (int q = 0; q < SEG; ++q) {
-                const int c = c0 + q * 32 + lane;
-                if (c < vec_per_row) {
-                    uint4 o;
-                    o.x = pack_bf16x2(acc[q][0], acc[q][1]);
-                    o.y = pack_bf16x2(acc[q][2], acc[q][3]);
-                    o.z = pack_bf16x2(acc[q][4], acc[q][5]);
-                    o.w = pack_bf16x2(acc[q][6], acc[q][7]);
-                    Y[(size_t)t * vec_per_row + c] = o;
+            for (int r = 0; r < R; ++r) {
+                if (p[r] < 0) continue;
+#pragma unroll
+                for (int q = 0; q < SEG; ++q) {
+                    acc[q][0] += bf16_lo(v[r][q].x); acc[q][1] += bf16_hi(v[r][q].x);
+                    acc[q][2] += bf16_lo(v[r][q].y); acc[q][3] += bf16_hi(v[r][q].y);
+                    acc[q][4] += bf16_lo(v[r][q].z); acc[q][5] += bf16_hi(v[r][q].z);
+                    acc[q][6] += bf16_lo(v[r][q].w); acc[q][7] += bf16_hi(v[r][q].w);
                 }
             }
         }
+#pragma unroll
+        for (int q = 0; q < SEG; ++q)
+            if (c + 32 * q < vec_per_row) {
+                uint4 o;
+                o.x = pack_bf16x2(acc[q][0], acc[q][1]);
+                o.y = pack_bf16x2(acc[q][2], acc[q][3]);
+                o.z = pack_bf16x2(acc[q][4], acc[q][5]);
+                o.w = pack_bf16x2(acc[q][6], acc[q][7]);
+                Y[(size_t)t * vec_per_row + c + 32 * q] = o;
+            }
     }
 }
 
@@ -510,13 +455,19 @@ inline void launch_scatter_rows(const uint4* src, uint4* dst, const int32_t* per
 }
 inline void launch_combine_rows(const uint4* Yp, const int32_t* perm_row, uint4* Y, int T, int k, int vec_per_row,
                                 int sm_count, cudaStream_t st) {
-    const int blocks = min(ceil_div(T, 8), sm_count * 8);
-    if (blocks <= 0) return;
-    // short rows (d < 4096) keep the chunked kernel: measured faster there (more warps per SM)
-    if (vec_per_row >= 32 * 16 && vec_per_row % (32 * 7) == 0)
-        pdl_launch(combine_rows_seg_kernel<7>, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
-    else if (vec_per_row >= 32 * 16) pdl_launch(combine_rows_seg_kernel<8>, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
-    else pdl_launch(combine_rows_kernel, blocks, 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
+    if (T <= 0) return;
+    auto go = [&](auto kernel, int seg, int threads) {
+        const long long items = (long long)T * ceil_div(vec_per_row, 32 * seg);
+        const long long most = (long long)sm_count * (2048 / threads);
+        const int blocks = (int)min((items + threads / 32 - 1) / (threads / 32), most);
+        pdl_launch(kernel, blocks, threads, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
+    };
+    // us: T 512, d 1024, k 4 (14 warps per SM of one vector each) 2.8 and 3.5 with four vectors; T 256, d 7168, k 8 (48) 10.1 and 8.2
+    if ((long long)T * ceil_div(vec_per_row, 32) <= 24ll * sm_count) go(combine_rows_kernel<1, 8>, 1, 128);
+    // rows shorter than four vectors a lane: T 16384, d 256, k 8 24.6 us, 32.8 with four; d 512, k 4 22.7 and 24.6
+    else if (vec_per_row <= 32) go(combine_rows_kernel<1, 2>, 1, 256);
+    else if (vec_per_row < 128) go(combine_rows_kernel<2, 2>, 2, 128);
+    else go(combine_rows_kernel<4, 1>, 4, 256);
 }
 
 // dgate[a] = sum over n-tiles of the partial dot products written by the dgrad-down epilogue

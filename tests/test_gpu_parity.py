@@ -396,6 +396,25 @@ def test_selection_of_equal_signed_zero_and_infinite_logits(E, k):
     assert (idx.cpu().numpy() == order).all()
 
 
+@pytest.mark.parametrize("T,d,k", [(1, 8, 1), (3, 264, 32), (130, 1032, 9),             # a vector a lane, rows in batches of 8
+                                   (3600, 256, 3), (3600, 264, 2), (1800, 1016, 5),      # one and two vectors, two rows at a time
+                                   (900, 1024, 4), (900, 1032, 3)])                      # four vectors, a row at a time
+def test_combine_sums_the_rows_in_order(T, d, k):
+    """Bit for bit the fp32 sum in ascending j, rounded once; rows of -1 are left out."""
+    gen = torch.Generator().manual_seed(T + d)
+    Yp = torch.randn((T * k, d), generator=gen).to(torch.bfloat16).cuda()
+    perm = torch.randperm(T * k, generator=gen).to(torch.int32).reshape(T, k)
+    perm[torch.rand((T, k), generator=gen) < 0.1] = -1
+    ctx = binding.Context(T, d, max(k, 4), k, 64)
+    Y = torch.empty((T, d), dtype=torch.bfloat16, device="cuda")
+    binding.mop_moe_combine(ctx, Yp, perm.cuda().reshape(-1), Y)
+    acc = torch.zeros((T, d), device="cuda")
+    for j in range(k):
+        rows = perm[:, j].cuda().long()
+        acc = torch.where(rows[:, None] >= 0, acc + Yp[rows.clamp(min=0)].float(), acc)
+    assert torch.equal(Y, acc.to(torch.bfloat16))
+
+
 def test_zero_tokens_is_a_no_op():
     w = synth.small("c1_tiny", T=0, d=64, E=4, k=2, f=64, backward=True)
     host, inp, ctx, buf = run(w)
