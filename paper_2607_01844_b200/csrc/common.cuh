@@ -37,6 +37,12 @@ __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (gridDim.x * gridDim.y <= 64) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// The exception: a GEMM followed by a GEMM.  Both take a whole SM per CTA, so the next one's CTAs can only come up where one of this
+// grid has left, one each, and find their barriers, tensor memory and descriptors ready when the last one leaves.
+__device__ __forceinline__ void pdl_begin_gemm(bool gemm_follows) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (gemm_follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 template <class... P, class... A>
 inline cudaError_t pdl_launch_clusters(void (*kernel)(P...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                        A... args) {

@@ -89,7 +89,7 @@ inline mop_status tc_ffn_fwd_impl(TcPlan* p, const TcFwdArgs& a, int32_t* tiles,
         if ((r = tn_up_swiglu_gather(p, a.x_gather, a, tiles, status, st)) != MOP_OK) return r;
         ++*launches;
     } else if (tn_f1) {
-        if ((r = tn_up_swiglu(p, a, tiles, status, st)) != MOP_OK) return r;
+        if ((r = tn_up_swiglu(p, a, tiles, status, with_down && tn_f2, st)) != MOP_OK) return r;
         ++*launches;
     } else {   // F1: [G|U] = Xp [W_gate | W_up], SwiGLU epilogue
         TcArgs g = tc_base_args(p, a.offsets, tiles, status);
@@ -193,6 +193,7 @@ inline mop_status tc_ffn_bwd(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, int3
         g.tiles_n = ceil_div(s.d, 256); g.tiles_m_fixed = ceil_div(s.f, wpair ? 256 : TC_BM); g.Mfix = s.f; g.N = s.d;
         g.a_split = s.f % 64 != 0; g.b_split = s.d % 64 != 0;
         g.ep.outf = a.dW_down; g.ep.accumulate = a.accumulate; g.keep_empty = a.keep_empty;
+        g.gemm_follows = true;
         if (prefetch) { g.pf[0] = a.gH; g.pf_bytes[0] = s.f * 2; g.pf[1] = a.dYp; g.pf_bytes[1] = s.d * 2; }
         r = wpair ? tw_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mdYpB, mdYpB, moWd, moWd, g, st)
                   : tc_launch<TC_WD>(p, "gemm_wgrad_down", mgH, mgH, mdYpB, mdYpB, moWd, moWd, g, st);

@@ -84,6 +84,7 @@ struct TcArgs {
     EpiArgs ep;
     float* outf1;            // WGU: second output tensor
     int keep_empty;          // weight gradients: leave the gradients of experts without rows untouched
+    bool gemm_follows;       // weight gradients: the next launch on the stream is a GEMM of this layer
     const void* pf[3];       // weight gradients: the operands (rows of all experts, dense) and the bytes of a row of each,
     int pf_bytes[3];         // which the producers bring to L2 an expert ahead (wgrad_prefetch); 0: they do not
 };
@@ -598,7 +599,7 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    pdl_begin();
+    pdl_begin_gemm(args.gemm_follows);
 
     int total_tiles;
     if constexpr (Tr::RAGGED_K) total_tiles = args.E * args.tiles_m_fixed * args.tiles_n;

@@ -72,6 +72,7 @@ struct TnArgs {
     int32_t* next;            // work items handed out so far (zero when the kernel starts)
     int32_t* status;
     EpiArgs ep;
+    bool gemm_follows;        // the next launch on the stream is a GEMM of this layer
 };
 
 // The tile tables of the token-row GEMMs in one launch: block 0 the token tiles, block 1 the 128-row tiles of the
@@ -248,7 +249,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    pdl_begin();
+    pdl_begin_gemm(args.gemm_follows);
 
     const int total_tiles = (*args.n_ttiles) * args.tiles_m;
     const int nkb = (KIND == TN_B4 ? 2 : 1) * args.kblocks;   // K blocks per tile (B4: two phases)
@@ -722,7 +723,7 @@ inline mop_status tn_launch(const TcPlan* p, const char* name, const TnMaps& m, 
 }
 
 // Up-projection + SwiGLU on the tokens-on-N kernel (`tiles`: the tables of tn_build_tiles).
-inline mop_status tn_up_swiglu(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, int32_t* status, cudaStream_t st) {
+inline mop_status tn_up_swiglu(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, int32_t* status, bool gemm_follows, cudaStream_t st) {
     const mop_moe_shape& s = p->s;
     const uint64_t M = tc_rows(p);
     TnMaps m;
@@ -732,6 +733,7 @@ inline mop_status tn_up_swiglu(TcPlan* p, const TcFwdArgs& a, int32_t* tiles, in
     TnArgs g = tn_base_args(p, tiles, TN_F1, status);
     g.tiles_m = ceil_div(s.f, 128); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.ep.out0 = a.H; g.ep.out1 = a.G_save; g.ep.out2 = a.U_save; g.ep.ldo = s.f; g.ep.M_total = (int)M;
+    g.gemm_follows = gemm_follows;
     return tn_launch<TN_F1>(p, "gemm_up_swiglu", m, g, st);
 }
 
@@ -776,6 +778,7 @@ inline mop_status tn_dgrad_gate_up(TcPlan* p, const TcBwdArgs& a, int32_t* tiles
     TnArgs g = tn_base_args(p, tiles, TN_B4, status);
     g.tiles_m = ceil_div(s.d, 256); g.kblocks = ceil_div(s.f, TN_BK); g.Mw = s.d;
     g.ep.out0 = a.dXp; g.ep.ldo = s.d; g.ep.M_total = (int)M;
+    g.gemm_follows = true;
     return tn_launch<TN_B4>(p, "gemm_dgrad_gate_up", m, g, st);
 }
 
@@ -790,6 +793,7 @@ inline mop_status tn_dgrad_down(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, i
     g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH; g.ep.in0 = a.G_save; g.ep.in1 = a.U_save; g.ep.in2 = a.H;
     g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
+    g.gemm_follows = true;
     return tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
 }
 
