@@ -230,6 +230,10 @@ __device__ __forceinline__ void tma_store_3d_hint(const CUtensorMap* map, uint32
         "r"(src), "r"(x), "r"(y), "r"(z), "l"(policy)
         : "memory");
 }
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src), "r"(x), "r"(y)
+                 : "memory");
+}
 // Weight gradients: when a CTA's tiles reach an expert, its share of the operand rows after that expert's goes to L2, up to 512
 // rows ahead.  All CTAs change experts at about the same time, and without this each change waits for DRAM, behind the
 // stores of the gradients, with less than a tile of loads in flight.  Plain prefetches, a line each: the bulk form goes

@@ -45,6 +45,13 @@ constexpr int TN_STAGE_BYTES = 2 * TN_SUB_BYTES;
 constexpr int TN_EPI_WARPS = 8;
 constexpr int TN_EPI_BYTES = 4096;                   // per epilogue warp
 constexpr int TN_SMEM_BYTES = TN_STAGES * TN_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + TN_EPI_WARPS * TN_EPI_BYTES;
+// The SwiGLU backward (TN_B2) has one stage less, and per pair of epilogue warps two buffers of the stash's three tensors (16 tokens x
+// 64 features) beside the gates of a tile.
+constexpr int TN_B2_STAGES = 5;
+constexpr int TN_STASH_BYTES = 16 * 128;             // of one tensor
+constexpr int TN_STASH_BUFS = 2;
+constexpr int TN_STASH_PAIR_BYTES = TN_STASH_BUFS * 3 * TN_STASH_BYTES;
+static_assert(TN_B2_STAGES * TN_STAGE_BYTES + 1024 + TC_BAR_BYTES + 4 * TN_STASH_PAIR_BYTES + TN_EPI_WARPS * 1024 <= TN_SMEM_BYTES, "shared memory");
 constexpr int TN_THREADS = 64 + 32 * TN_EPI_WARPS;
 constexpr int TN_RING = 16;                          // work items announced to the roles of a cluster
 constexpr int TN_SIGNALS = 4;                        // requests for further items
@@ -53,7 +60,7 @@ constexpr int TN_BOXES = 8;                          // token boxes of 16, 32, .
 struct TnMaps {
     CUtensorMap a0, a1;                // weights (F1: gate, up; B4: gate, up)
     CUtensorMap b[TN_BOXES];           // token rows, box of 16 (i + 1) rows
-    CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows
+    CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows; B2: [0..2] the stash G, U, H, [3..5] dG, dU, gH (16 rows)
 };
 
 // A tile's columns of the MMA, and the box (index into TnMaps) that holds one CTA's half of them.
@@ -210,11 +217,12 @@ __host__ __device__ __forceinline__ void tn_walk_items(int group, Next next, Wai
 template <int KIND, bool ONCE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TN_THREADS, 1)
 tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
-    constexpr int S = TN_STAGES, STAGE_BYTES = TN_STAGE_BYTES;
+    constexpr int S = KIND == TN_B2 ? TN_B2_STAGES : TN_STAGES, STAGE_BYTES = TN_STAGE_BYTES;
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * STAGE_BYTES);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4 + TN_RING + TN_SIGNALS);
+    constexpr int STASH_BARS = KIND == TN_B2 ? 4 * TN_STASH_BUFS : 0;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4 + TN_RING + TN_SIGNALS + STASH_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = warp_index(), lane = threadIdx.x % 32;
@@ -231,17 +239,22 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     auto item_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + ((n - 1) & (TN_RING - 1))); };
     auto item_slot = [&](int n) { return bar_base + 512u + 16u * ((n - 1) & (TN_RING - 1)); };
     auto signal_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + TN_RING + (n & (TN_SIGNALS - 1))); };
-    static_assert(8 * (2 * S + 4 + TN_RING + TN_SIGNALS) + 8 <= 512 && 512 + 16 * TN_RING <= TC_BAR_BYTES, "barrier block");
+    auto stash_bar = [&](int pair, int b) { return bar_base + 8u * (2 * S + 4 + TN_RING + TN_SIGNALS + pair * TN_STASH_BUFS + b); };
+    (void)stash_bar;
+    static_assert(8 * (2 * S + 4 + TN_RING + TN_SIGNALS + STASH_BARS) + 8 <= 512 && 512 + 16 * TN_RING <= TC_BAR_BYTES, "barrier block");
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
         for (int n = 0; n < TN_RING; ++n) mbar_init(item_bar(n), 1);
         for (int n = 0; n < TN_SIGNALS; ++n) mbar_init(signal_bar(n), 1);
+        for (int n = 0; n < STASH_BARS; ++n) mbar_init(stash_bar(n / TN_STASH_BUFS, n % TN_STASH_BUFS), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&maps.a0);
         if (KIND != TN_F2 && KIND != TN_B2) tma_prefetch_desc(&maps.a1);
+        if (KIND == TN_B2)
+            for (int i = 0; i < 6; ++i) tma_prefetch_desc(&maps.b1[i]);
     }
     if (warp == 1) tmem2_alloc(smem_u32(tmem_slot), 512);
     tc_fence_before();
@@ -438,14 +451,40 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         const uint32_t wb = epi_base + (uint32_t)(warp - 2) * TN_EPI_BYTES;   // this warp's staging
         const uint32_t fo = frag_off(lane);
         const int tpair = 2 * (lane & 3);             // this thread's tokens within a run of 8: tpair, tpair + 1
-        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G;   // a gate warp and its up warp
-        const int pair_bar = 1 + 2 * group + (quarter & 1);
+        // F1: a gate warp and its up warp; B2: two warps that share 128-byte lines of the stash
+        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G || KIND == TN_B2;
+        const int pair_bar = 1 + 2 * group + (KIND == TN_B2 ? quarter >> 1 : quarter & 1);
         const int buf = group;
-        const uint32_t gbuf = wb + 3072;
-        Tile ti;
+        const uint32_t gbuf = KIND == TN_B2 ? epi_base + 4 * TN_STASH_PAIR_BYTES + (uint32_t)(warp - 2) * 1024 : wb + 3072;
+        Tile ti = {0, 0, 0, 0};
+        // B2: the pair's buffers, its steps so far (16 tokens each; the buffers and their barriers' phases alternate) and the warp
+        // that copies for both
+        const int stash_pair = (warp - 2) >> 1;
+        const uint32_t stash = epi_base + (uint32_t)stash_pair * TN_STASH_PAIR_BYTES;
+        const bool el = elect_one();
+        const bool copies = (quarter & 1) == 0 && el;
+        int steps = 0;
+        bool gone = false;
+        (void)stash; (void)copies; (void)steps; (void)gone;
+        auto fetch_stash = [&](int step, int row) {
+            const int b = step % TN_STASH_BUFS;
+            const int f0 = ti.mt * 256 + 128 * (int)rank + 64 * (quarter >> 1);
+            mbar_expect_tx(stash_bar(stash_pair, b), 3 * TN_STASH_BYTES);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                tma_load_2d(stash + (b * 3 + a) * TN_STASH_BYTES, &maps.b1[a], stash_bar(stash_pair, b), f0, row);
+        };
         // (the lanes give up together: a lane that left alone would be missed at the shuffles below)
-        auto next = [&](int n) { return __all_sync(0xffffffffu, next_item(n, ti)) != 0; };
+        auto next = [&](int n) { return !gone && __all_sync(0xffffffffu, next_item(n, ti)) != 0; };
         auto wait = [&](int n) {
+            if constexpr (KIND == TN_B2) {       // the stash of the tile's first steps as well
+                if (copies) {
+                    tma_store_wait_read<0>();
+#pragma unroll
+                    for (int i = 0; i < TN_STASH_BUFS; ++i)
+                        if (16 * i < ti.rows) fetch_stash(steps + i, ti.row0 + 16 * i);
+                }
+            }
             // F2, B2: the gates of the tile's tokens (two dependent loads each) are fetched before the wait for the
             // accumulator, so that their latency is hidden behind the main loop
             if constexpr (KIND == TN_F2 || KIND == TN_B2) {
@@ -531,41 +570,34 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                     bar_pair_sync(pair_bar);     // the partner has read this warp's half
                 }
             } else if constexpr (KIND == TN_B2) {
-                // 16 tokens at a time: the stash (G, U, H) comes in as 16-byte pieces of token rows one step ahead, is staged and
-                // read back as fragments (ldmatrix.trans) that match the accumulator's; the results leave the same way.
+                // 16 tokens at a time.  The stash (G, U, H) and the results (dG, dU, gH) travel as boxes of 64 features, whole 128-byte
+                // lines, between global and shared memory, in the buffers' place; a warp works on its 32 of them in the layout of the
+                // accumulator's fragments (ldmatrix.trans, stmatrix.trans).  With 16-byte loads and stores of half lines, one step
+                // ahead, they were more than half of a tile's time (30 thousand cycles for 192 tokens, 12 without them; d = 2048,
+                // f = 1408, 64 experts of 384 rows 224 us, now 198).  Three buffers and a stage less: the epilogue waits no
+                // more, but the operands do, and nothing is gained.
                 const int fcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first f column of this warp
-                const int col = fcol + (lane & 3) * 8;
-                const bf16* const src[3] = {args.ep.in0, args.ep.in1, args.ep.in2};
+                const int sub = 4 * (quarter & 1);                                  // its first 16-byte piece of a line
+                const uint32_t fo2 = (uint32_t)((lane & 7) * 128 + (((sub + (lane >> 3)) ^ (lane & 7)) << 4));
                 bf16* const dst[3] = {args.ep.out0, args.ep.out1, args.ep.out2};
-                uint4 pre[3][2];
-                auto fetch = [&](int c) {
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int tok = c + 8 * i + (lane >> 2);
-                        const bool okk = tok < rows && col < args.Mw;
-                        const size_t o = (size_t)(row0 + tok) * args.ep.ldo + col;
-#pragma unroll
-                        for (int a = 0; a < 3; ++a)
-                            pre[a][i] = okk ? *reinterpret_cast<const uint4*>(src[a] + o) : make_uint4(0, 0, 0, 0);
-                    }
-                };
-                fetch(0);
 #pragma unroll 1
-                for (int c = 0; c < nmma; c += 16) {
+                for (int c = 0; c < nmma; c += 16, ++steps) {
+                    const int b = steps % TN_STASH_BUFS;
+                    const uint32_t st = stash + b * 3 * TN_STASH_BYTES;
                     float v0[8], v1[8];
                     tmem_frag2(taddr + c, v0);
                     tmem_frag2(taddr + (16u << 16) + c, v1);
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-#pragma unroll
-                        for (int i = 0; i < 2; ++i) sts128(wb + 1024 * a + 512 * i + piece_off(lane), pre[a][i]);
-                    __syncwarp();
-                    if (c + 16 < nmma) fetch(c + 16);
+                    bool ok = mbar_wait_warp(stash_bar(stash_pair, b), (uint32_t)(steps / TN_STASH_BUFS) & 1u, abort_flag, args.status, STATUS_WAIT_FULL, lane);
                     uint32_t frag[3][2][4];
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
 #pragma unroll
-                        for (int j = 0; j < 2; ++j) ldmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j]);
+                        for (int j = 0; j < 2; ++j) ldmatrix4_trans(st + a * TN_STASH_BYTES + 1024 * j + fo2, frag[a][j]);
+                    // the step before left its buffer to the store that reads it: once that is done, the step after this one
+                    if (copies && c > 0 && c + 16 * (TN_STASH_BUFS - 1) < nmma) {
+                        tma_store_wait_read<0>();
+                        fetch_stash(steps + TN_STASH_BUFS - 1, row0 + c + 16 * (TN_STASH_BUFS - 1));
+                    }
                     tmem_frag_wait(v0, v1);
                     float dot[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll
@@ -598,11 +630,29 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                     for (int a = 0; a < 3; ++a)
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
-                            stmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j][0], frag[a][j][1], frag[a][j][2], frag[a][j][3]);
-                    __syncwarp();
+                            stmatrix4_trans(st + a * TN_STASH_BYTES + 1024 * j + fo2, frag[a][j][0], frag[a][j][1], frag[a][j][2], frag[a][j][3]);
+                    const bool whole = c + 16 <= rows;
+                    if (whole) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    else {                                     // the rows after the tile's are another expert's: row by row
+                        __syncwarp();
+                        const int tok = lane >> 2, col = fcol + (lane & 3) * 8;
 #pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        tn_write_rows<2>(dst[a], args.ep.ldo, wb + 1024 * a, row0 + c, rows - c, fcol, args.Mw, lane);
+                        for (int a = 0; a < 3; ++a)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                const uint4 v = lds128(st + a * TN_STASH_BYTES + (8 * i + tok) * 128 + (((sub + (lane & 3)) ^ tok) << 4));
+                                if (c + 8 * i + tok < rows && col < args.Mw)
+                                    *reinterpret_cast<uint4*>(dst[a] + (size_t)(row0 + c + 8 * i + tok) * args.ep.ldo + col) = v;
+                            }
+                    }
+                    ok = bar_vote_all(pair_bar, 64, ok);       // both halves of the lines are there (or one of the two gives up)
+                    if (copies && ok && whole) {
+                        const int f0 = ti.mt * 256 + 128 * (int)rank + 64 * (quarter >> 1);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+                            if (f0 < args.Mw) tma_store_2d(&maps.b1[3 + a], st + a * TN_STASH_BYTES, f0, row0 + c);
+                        tma_store_commit();
+                    }
                     // the 32 features' dot products: the 8 lanes with the same lane % 4 hold the shares of the same tokens
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
@@ -614,7 +664,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                             if (lane < 4 && tok < rows && fcol < args.Mw)
                                 args.ep.part[(size_t)(fcol >> 5) * args.ep.M_total + row0 + tok] = dot[j][p];
                         }
-                    __syncwarp();
+                    if (!ok) { gone = true; break; }
                 }
             } else {
                 const int mcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first output column of this warp
@@ -643,6 +693,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_bar(buf) & T2_PEER_MASK);
         });
+        if (KIND == TN_B2 && copies) tma_store_wait_all();
     }
 
     tc_fence_before();
@@ -789,9 +840,12 @@ inline mop_status tn_dgrad_down(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, i
     const uint64_t M = tc_rows(p);
     TnMaps m;
     if (!tc_map_3d(p, &m.a0, a.W_down, s.E, s.f, s.d, 128) || !tn_token_maps(p, m.b, a.dYp, M, s.d)) return MOP_ERR_CUDA;
+    const void* const boxes[6] = {a.G_save, a.U_save, a.H, a.dG, a.dU, a.gH};
+    for (int i = 0; i < 6; ++i)
+        if (!tc_map_2d(p, &m.b1[i], boxes[i], M, s.f, 16)) return MOP_ERR_CUDA;
     TnArgs g = tn_base_args(p, tiles, TN_B2, status);
     g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
-    g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH; g.ep.in0 = a.G_save; g.ep.in1 = a.U_save; g.ep.in2 = a.H;
+    g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH;
     g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
     g.gemm_follows = true;
     return tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
