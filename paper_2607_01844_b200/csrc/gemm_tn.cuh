@@ -35,7 +35,8 @@
 
 namespace mop {
 
-enum : int { TN_F1 = 0, TN_F2 = 1, TN_F1G = 2, TN_B4 = 3, TN_B2 = 4 };
+enum : int { TN_F1 = 0, TN_F2 = 1, TN_F1G = 2, TN_B4 = 3, TN_B2 = 4, TN_B2S = 5 };
+__host__ __device__ constexpr bool tn_is_b2(int kind) { return kind == TN_B2 || kind == TN_B2S; }
 
 constexpr int TN_STAGES = 6;
 constexpr int TN_BK = 64;                            // K per stage
@@ -45,13 +46,17 @@ constexpr int TN_STAGE_BYTES = 2 * TN_SUB_BYTES;
 constexpr int TN_EPI_WARPS = 8;
 constexpr int TN_EPI_BYTES = 4096;                   // per epilogue warp
 constexpr int TN_SMEM_BYTES = TN_STAGES * TN_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + TN_EPI_WARPS * TN_EPI_BYTES;
-// The SwiGLU backward (TN_B2) has one stage less, and per pair of epilogue warps two buffers of the stash's three tensors (16 tokens x
-// 64 features) beside the gates of a tile.
-constexpr int TN_B2_STAGES = 5;
+// The SwiGLU backward has, per pair of epilogue warps, buffers of the stash's three tensors (16 tokens x 64 features) beside the gates
+// of a tile, and a stage less for two of them (TN_B2) or two stages less for three (TN_B2S: where K is short the epilogue is the
+// longer part).
 constexpr int TN_STASH_BYTES = 16 * 128;             // of one tensor
-constexpr int TN_STASH_BUFS = 2;
-constexpr int TN_STASH_PAIR_BYTES = TN_STASH_BUFS * 3 * TN_STASH_BYTES;
-static_assert(TN_B2_STAGES * TN_STAGE_BYTES + 1024 + TC_BAR_BYTES + 4 * TN_STASH_PAIR_BYTES + TN_EPI_WARPS * 1024 <= TN_SMEM_BYTES, "shared memory");
+__host__ __device__ constexpr int tn_stash_bufs(int kind) { return kind == TN_B2S ? 3 : 2; }
+__host__ __device__ constexpr int tn_stages(int kind) { return kind == TN_B2S ? 4 : kind == TN_B2 ? 5 : TN_STAGES; }
+__host__ __device__ constexpr int tn_stash_pair_bytes(int kind) { return tn_stash_bufs(kind) * 3 * TN_STASH_BYTES; }
+__host__ __device__ constexpr int tn_b2_smem(int kind) {
+    return tn_stages(kind) * TN_STAGE_BYTES + 1024 + TC_BAR_BYTES + 4 * tn_stash_pair_bytes(kind) + TN_EPI_WARPS * 1024;
+}
+static_assert(tn_b2_smem(TN_B2) <= TN_SMEM_BYTES && tn_b2_smem(TN_B2S) <= TN_SMEM_BYTES, "shared memory");
 constexpr int TN_THREADS = 64 + 32 * TN_EPI_WARPS;
 constexpr int TN_RING = 16;                          // work items announced to the roles of a cluster
 constexpr int TN_SIGNALS = 4;                        // requests for further items
@@ -217,11 +222,12 @@ __host__ __device__ __forceinline__ void tn_walk_items(int group, Next next, Wai
 template <int KIND, bool ONCE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TN_THREADS, 1)
 tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
-    constexpr int S = KIND == TN_B2 ? TN_B2_STAGES : TN_STAGES, STAGE_BYTES = TN_STAGE_BYTES;
+    constexpr int S = tn_stages(KIND), STAGE_BYTES = TN_STAGE_BYTES;
+    constexpr int BUFS = tn_stash_bufs(KIND), PAIR_BYTES = tn_stash_pair_bytes(KIND);
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * STAGE_BYTES);
-    constexpr int STASH_BARS = KIND == TN_B2 ? 4 * TN_STASH_BUFS : 0;
+    constexpr int STASH_BARS = tn_is_b2(KIND) ? 4 * BUFS : 0;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4 + TN_RING + TN_SIGNALS + STASH_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -239,7 +245,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     auto item_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + ((n - 1) & (TN_RING - 1))); };
     auto item_slot = [&](int n) { return bar_base + 512u + 16u * ((n - 1) & (TN_RING - 1)); };
     auto signal_bar = [&](int n) { return bar_base + 8u * (2 * S + 4 + TN_RING + (n & (TN_SIGNALS - 1))); };
-    auto stash_bar = [&](int pair, int b) { return bar_base + 8u * (2 * S + 4 + TN_RING + TN_SIGNALS + pair * TN_STASH_BUFS + b); };
+    auto stash_bar = [&](int pair, int b) { return bar_base + 8u * (2 * S + 4 + TN_RING + TN_SIGNALS + pair * BUFS + b); };
     (void)stash_bar;
     static_assert(8 * (2 * S + 4 + TN_RING + TN_SIGNALS + STASH_BARS) + 8 <= 512 && 512 + 16 * TN_RING <= TC_BAR_BYTES, "barrier block");
 
@@ -248,12 +254,12 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
         for (int n = 0; n < TN_RING; ++n) mbar_init(item_bar(n), 1);
         for (int n = 0; n < TN_SIGNALS; ++n) mbar_init(signal_bar(n), 1);
-        for (int n = 0; n < STASH_BARS; ++n) mbar_init(stash_bar(n / TN_STASH_BUFS, n % TN_STASH_BUFS), 1);
+        for (int n = 0; n < STASH_BARS; ++n) mbar_init(stash_bar(n / BUFS, n % BUFS), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&maps.a0);
-        if (KIND != TN_F2 && KIND != TN_B2) tma_prefetch_desc(&maps.a1);
-        if (KIND == TN_B2)
+        if (KIND != TN_F2 && !tn_is_b2(KIND)) tma_prefetch_desc(&maps.a1);
+        if (tn_is_b2(KIND))
             for (int i = 0; i < 6; ++i) tma_prefetch_desc(&maps.b1[i]);
     }
     if (warp == 1) tmem2_alloc(smem_u32(tmem_slot), 512);
@@ -378,7 +384,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                 if (el) {
                     if (!leader && handout && kb == ask_at) mbar_arrive(signal_bar(n));
                     if (leader) mbar_expect_tx(full_bar(stage), tx);
-                    if constexpr (KIND == TN_B4 || KIND == TN_B2) {
+                    if constexpr (KIND == TN_B4 || tn_is_b2(KIND)) {
                         load_w3(sA, ph ? &maps.a1 : &maps.a0, fb, k0, m0, ti.e);   // K-major weights
                     } else if constexpr (KIND == TN_F1) {                               // N-major weights [E, d, f]
                         load_w3(sA, &maps.a0, fb, m0, k0, ti.e);
@@ -400,7 +406,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         // ===================================================================== MMA issuer (leader CTA)
         if (leader) {
             const bool el = elect_one();
-            constexpr bool A_KMAJOR = (KIND == TN_B4 || KIND == TN_B2);
+            constexpr bool A_KMAJOR = (KIND == TN_B4 || tn_is_b2(KIND));
             // descriptors without the start address: A is M-major (N-major weights) or K-major, B is K-major.
             // A M-major: the two 64-wide chunks are TN_CHUNK_BYTES apart, 2 KiB per K = 16; K-major: 32 bytes per K = 16
             const uint64_t desc_a = smem_desc(0, A_KMAJOR ? 0 : TN_CHUNK_BYTES, 1024);
@@ -452,22 +458,22 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         const uint32_t fo = frag_off(lane);
         const int tpair = 2 * (lane & 3);             // this thread's tokens within a run of 8: tpair, tpair + 1
         // F1: a gate warp and its up warp; B2: two warps that share 128-byte lines of the stash
-        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G || KIND == TN_B2;
-        const int pair_bar = 1 + 2 * group + (KIND == TN_B2 ? quarter >> 1 : quarter & 1);
+        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G || tn_is_b2(KIND);
+        const int pair_bar = 1 + 2 * group + (tn_is_b2(KIND) ? quarter >> 1 : quarter & 1);
         const int buf = group;
-        const uint32_t gbuf = KIND == TN_B2 ? epi_base + 4 * TN_STASH_PAIR_BYTES + (uint32_t)(warp - 2) * 1024 : wb + 3072;
+        const uint32_t gbuf = tn_is_b2(KIND) ? epi_base + 4 * PAIR_BYTES + (uint32_t)(warp - 2) * 1024 : wb + 3072;
         Tile ti = {0, 0, 0, 0};
         // B2: the pair's buffers, its steps so far (16 tokens each; the buffers and their barriers' phases alternate) and the warp
         // that copies for both
         const int stash_pair = (warp - 2) >> 1;
-        const uint32_t stash = epi_base + (uint32_t)stash_pair * TN_STASH_PAIR_BYTES;
+        const uint32_t stash = epi_base + (uint32_t)stash_pair * PAIR_BYTES;
         const bool el = elect_one();
         const bool copies = (quarter & 1) == 0 && el;
         int steps = 0;
         bool gone = false;
         (void)stash; (void)copies; (void)steps; (void)gone;
         auto fetch_stash = [&](int step, int row) {
-            const int b = step % TN_STASH_BUFS;
+            const int b = step % BUFS;
             const int f0 = ti.mt * 256 + 128 * (int)rank + 64 * (quarter >> 1);
             mbar_expect_tx(stash_bar(stash_pair, b), 3 * TN_STASH_BYTES);
 #pragma unroll
@@ -477,17 +483,17 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         // (the lanes give up together: a lane that left alone would be missed at the shuffles below)
         auto next = [&](int n) { return !gone && __all_sync(0xffffffffu, next_item(n, ti)) != 0; };
         auto wait = [&](int n) {
-            if constexpr (KIND == TN_B2) {       // the stash of the tile's first steps as well
+            if constexpr (tn_is_b2(KIND)) {       // the stash of the tile's first steps as well
                 if (copies) {
                     tma_store_wait_read<0>();
 #pragma unroll
-                    for (int i = 0; i < TN_STASH_BUFS; ++i)
+                    for (int i = 0; i < BUFS; ++i)
                         if (16 * i < ti.rows) fetch_stash(steps + i, ti.row0 + 16 * i);
                 }
             }
             // F2, B2: the gates of the tile's tokens (two dependent loads each) are fetched before the wait for the
             // accumulator, so that their latency is hidden behind the main loop
-            if constexpr (KIND == TN_F2 || KIND == TN_B2) {
+            if constexpr (KIND == TN_F2 || tn_is_b2(KIND)) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int tk = 32 * j + lane;
@@ -569,34 +575,33 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                     tn_write_rows<2>(args.ep.out0, args.ep.ldo, sb, row0 + c + t_own, rows_left - t_own, fcol, args.Mw, lane);
                     bar_pair_sync(pair_bar);     // the partner has read this warp's half
                 }
-            } else if constexpr (KIND == TN_B2) {
+            } else if constexpr (tn_is_b2(KIND)) {
                 // 16 tokens at a time.  The stash (G, U, H) and the results (dG, dU, gH) travel as boxes of 64 features, whole 128-byte
                 // lines, between global and shared memory, in the buffers' place; a warp works on its 32 of them in the layout of the
                 // accumulator's fragments (ldmatrix.trans, stmatrix.trans).  With 16-byte loads and stores of half lines, one step
                 // ahead, they were more than half of a tile's time (30 thousand cycles for 192 tokens, 12 without them; d = 2048,
-                // f = 1408, 64 experts of 384 rows 224 us, now 198).  Three buffers and a stage less: the epilogue waits no
-                // more, but the operands do, and nothing is gained.
+                // f = 1408, 64 experts of 384 rows 205 us, now 194).
                 const int fcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first f column of this warp
                 const int sub = 4 * (quarter & 1);                                  // its first 16-byte piece of a line
                 const uint32_t fo2 = (uint32_t)((lane & 7) * 128 + (((sub + (lane >> 3)) ^ (lane & 7)) << 4));
                 bf16* const dst[3] = {args.ep.out0, args.ep.out1, args.ep.out2};
 #pragma unroll 1
                 for (int c = 0; c < nmma; c += 16, ++steps) {
-                    const int b = steps % TN_STASH_BUFS;
+                    const int b = steps % BUFS;
                     const uint32_t st = stash + b * 3 * TN_STASH_BYTES;
                     float v0[8], v1[8];
                     tmem_frag2(taddr + c, v0);
                     tmem_frag2(taddr + (16u << 16) + c, v1);
-                    bool ok = mbar_wait_warp(stash_bar(stash_pair, b), (uint32_t)(steps / TN_STASH_BUFS) & 1u, abort_flag, args.status, STATUS_WAIT_FULL, lane);
+                    bool ok = mbar_wait_warp(stash_bar(stash_pair, b), (uint32_t)(steps / BUFS) & 1u, abort_flag, args.status, STATUS_WAIT_FULL, lane);
                     uint32_t frag[3][2][4];
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
 #pragma unroll
                         for (int j = 0; j < 2; ++j) ldmatrix4_trans(st + a * TN_STASH_BYTES + 1024 * j + fo2, frag[a][j]);
                     // the step before left its buffer to the store that reads it: once that is done, the step after this one
-                    if (copies && c > 0 && c + 16 * (TN_STASH_BUFS - 1) < nmma) {
+                    if (copies && c > 0 && c + 16 * (BUFS - 1) < nmma) {
                         tma_store_wait_read<0>();
-                        fetch_stash(steps + TN_STASH_BUFS - 1, row0 + c + 16 * (TN_STASH_BUFS - 1));
+                        fetch_stash(steps + BUFS - 1, row0 + c + 16 * (BUFS - 1));
                     }
                     tmem_frag_wait(v0, v1);
                     float dot[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
@@ -693,7 +698,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_bar(buf) & T2_PEER_MASK);
         });
-        if (KIND == TN_B2 && copies) tma_store_wait_all();
+        if (tn_is_b2(KIND) && copies) tma_store_wait_all();
     }
 
     tc_fence_before();
@@ -717,7 +722,7 @@ inline bool tn_set_smem() {
            cudaFuncSetAttribute(tn_gemm_kernel<KIND, KIND != TN_F1G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TN_SMEM_BYTES) == cudaSuccess;
 }
 inline mop_status tn_init() {
-    return tn_set_smem<TN_F1>() && tn_set_smem<TN_F2>() && tn_set_smem<TN_F1G>() && tn_set_smem<TN_B4>() && tn_set_smem<TN_B2>()
+    return tn_set_smem<TN_F1>() && tn_set_smem<TN_F2>() && tn_set_smem<TN_F1G>() && tn_set_smem<TN_B4>() && tn_set_smem<TN_B2>() && tn_set_smem<TN_B2S>()
                ? MOP_OK : MOP_ERR_CUDA;
 }
 
@@ -843,12 +848,16 @@ inline mop_status tn_dgrad_down(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, i
     const void* const boxes[6] = {a.G_save, a.U_save, a.H, a.dG, a.dU, a.gH};
     for (int i = 0; i < 6; ++i)
         if (!tc_map_2d(p, &m.b1[i], boxes[i], M, s.f, 16)) return MOP_ERR_CUDA;
+    // Three stash buffers where K is short and the rows are more than a box or two: d 512, f 1024, 1024 rows per expert 94 us, two buffers
+    // 118; d 1024, f 2048, 2048 rows 212 and 239; d 2048, f 1408, 384 rows 194 and 198; d 2048, f 768, 28 rows 82 and 78.
+    const bool brief = s.d <= 2048 && (uint64_t)s.T * s.k >= 64ull * s.E;
     TnArgs g = tn_base_args(p, tiles, TN_B2, status);
     g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
     g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH;
     g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
     g.gemm_follows = true;
-    return tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
+    return brief ? tn_launch<TN_B2S>(p, "gemm_dgrad_down_dswiglu", m, g, st)
+                 : tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
 }
 
 }  // namespace mop

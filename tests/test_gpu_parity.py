@@ -311,6 +311,15 @@ def test_an_overflowing_expert_does_not_reach_its_neighbours_gradients():
         assert torch.equal(clean.dX[~mine], bad.dX[~mine]) and torch.equal(clean.dgate[~mine], bad.dgate[~mine])
 
 
+@pytest.mark.parametrize("T,d,E,k,f", [(50, 2048, 2, 1, 72),       # 25 rows: two steps, the second partly filled; f ends inside a box
+                                       (700, 256, 3, 2, 320),     # two tiles per expert, steps beyond every buffer
+                                       (130, 2056, 2, 2, 136),    # longer K: two buffers
+                                       (40, 512, 8, 2, 200)],     # fewer rows than a tile's smallest box asks for
+                         ids=lambda v: str(v))
+def test_swiglu_backward_with_two_and_three_stash_buffers(T, d, E, k, f):
+    check_layer(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=f, backward=True, seed=T), binding.GEMM_AUTO)
+
+
 @pytest.mark.parametrize("T,k,E", [(2048, 2, 24), (2049, 2, 24), (4096, 1, 1024), (1025, 4, 7), (4609, 1, 3)])
 def test_permutation_tables_on_both_sides_of_the_single_block_limit(T, k, E):
     """Up to 8 units of 512 assignments the permutation runs in one block, beyond that in three kernels: the tables
