@@ -1126,27 +1126,23 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
     if (!guard.ok) return MOP_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     mop_status r;
+    const int dwr_blocks = ceil_div(s.d, 256) * s.E;
     if (s.T > 0) {
+        const int dz_blocks = ceil_div(s.T, 8);
         LAUNCH(c, "route_bwd_dz", st,
-               pdl_launch(route_bwd_dz_kernel, ceil_div(s.T, 8), 256, 0, st, logits, bias, topk_idx, topk_gate, dgate, perm_row,
-                          c->dz_sel, c->dz_row, s.T, s.E, s.k, s.score_fn, s.bias_mode));
+               pdl_launch(route_bwd_dz_kernel, dz_blocks + ceil_div(s.E, 32) * ceil_div(s.d, 32), 256, 0, st, logits, bias, topk_idx,
+                          topk_gate, dgate, perm_row, c->dz_sel, c->dz_row, s.T, s.E, s.k, s.score_fn, s.bias_mode, dz_blocks, W_r,
+                          c->wrT, s.d));
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
-    dim3 gw(ceil_div(s.d, 256), s.E);
-    const int dwr_w = dwr_warps((long long)gw.x * gw.y, c->sm_count);
+    const int dwr_w = dwr_warps(dwr_blocks, c->sm_count);
+    const long long dx_items = (long long)s.T * ceil_div(s.d, 256);
+    const int dx_blocks = (int)min((dx_items + dwr_w - 1) / dwr_w, (long long)c->sm_count * (64 / dwr_w));
     float* db = (dbias_opt && s.bias_mode == MOP_BIAS_PRE_LOGIT) ? dbias_opt : nullptr;
     if (dbias_opt && !db) CUDA_OK(cudaMemsetAsync(dbias_opt, 0, (size_t)s.E * 4, st));
-    LAUNCH(c, "route_bwd_dwr", st,
-           pdl_launch(route_bwd_dwr_kernel, gw, 32 * dwr_w, dwr_w * 1024, st, static_cast<const bf16*>(Xp), c->dz_row, offsets,
-                      dW_r, db, s.d, s.E));
-    if ((r = after_launch(c)) != MOP_OK) return r;
-    if (s.T == 0) return MOP_OK;
-    dim3 gt(ceil_div(s.E, 32), ceil_div(s.d, 32));
-    LAUNCH(c, "route_bwd_wrT", st, pdl_launch(transpose_f32_kernel, gt, 256, 0, st, W_r, c->wrT, s.d, s.E));
-    if ((r = after_launch(c)) != MOP_OK) return r;
-    LAUNCH(c, "route_bwd_dx", st,
-           pdl_launch(route_bwd_dx_kernel, s.T, 256, 0, st, c->wrT, topk_idx, c->dz_sel, static_cast<bf16*>(dX), s.T, s.d, s.E,
-                      s.k));
+    LAUNCH(c, "route_bwd_dwr_dx", st,
+           pdl_launch(route_bwd_dwr_dx_kernel, dwr_blocks + dx_blocks, 32 * dwr_w, dwr_w * 1024, st, static_cast<const bf16*>(Xp),
+                      c->dz_row, offsets, dW_r, db, s.d, s.E, c->wrT, topk_idx, c->dz_sel, static_cast<bf16*>(dX), s.T, s.k));
     return after_launch(c);
 }
 

@@ -756,8 +756,22 @@ inline void route_select_fast(float* z, const float* z1, const float* bias, cons
 // bias added before the score, dbias = column sums of dz.
 // ---------------------------------------------------------------------------------------------
 
+// W_r^T [E,d] from W_r [d,E], a tile of 32 x 32 per block through shared memory: gives the dX kernel contiguous rows.
+__device__ __forceinline__ void transpose_tile(const float* __restrict__ in, float* __restrict__ out, int rows, int cols, int block) {
+    __shared__ float tile[32][33];
+    const int across = (cols + 31) / 32;
+    const int c0 = (block % across) * 32, r0 = (block / across) * 32;
+    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+    for (int r = ty; r < 32; r += 8)
+        if (r0 + r < rows && c0 + tx < cols) tile[r][tx] = in[(size_t)(r0 + r) * cols + c0 + tx];
+    __syncthreads();
+    for (int c = ty; c < 32; c += 8)
+        if (c0 + c < cols && r0 + tx < rows) out[(size_t)(c0 + c) * rows + r0 + tx] = tile[tx][c];
+}
+
 // One warp per token: lane j < k owns the j-th selected expert.  Writes dz per assignment and, in
 // expert-contiguous row order (row = perm_row[assignment]), the copy that the dW_r kernel reads.
+// The blocks behind the first dz_blocks transpose W_r, which the next kernel reads as well: a launch less.
 __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restrict__ logits,
                                                            const float* __restrict__ bias,
                                                            const int32_t* __restrict__ idx,
@@ -765,8 +779,10 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
                                                            const float* __restrict__ dgate,
                                                            const int32_t* __restrict__ perm_row,
                                                            float* __restrict__ dz_sel, float* __restrict__ dz_row,
-                                                           int T, int E, int k, int score_fn, int bias_mode) {
+                                                           int T, int E, int k, int score_fn, int bias_mode, int dz_blocks,
+                                                           const float* __restrict__ W_r, float* __restrict__ W_rT, int d) {
     pdl_begin();
+    if ((int)blockIdx.x >= dz_blocks) { transpose_tile(W_r, W_rT, d, E, blockIdx.x - dz_blocks); return; }
     const int lane = threadIdx.x % 32;
     const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     if (t >= T) return;
@@ -800,18 +816,64 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
     }
 }
 
+// dX[t,:] += dz[t,:] W_r^T = sum_j dz[t,j] * W_r^T[e_j,:]: a warp takes 256 columns of a token, eight a lane, and the k rows of W_r^T
+// (contiguous, L2-resident) four at a time; dX is read, updated in fp32 and rounded back to bf16.  d is a multiple of 8.
+__device__ __forceinline__ void route_bwd_dx(const float* __restrict__ W_rT, const int32_t* __restrict__ idx,
+                                             const float* __restrict__ dz_sel, bf16* __restrict__ dX, int T, int d, int k,
+                                             int warp, int warps) {
+    const int lane = threadIdx.x % 32, segs = (d + 255) / 256;
+    const long long items = (long long)T * segs;
+    for (long long it = warp; it < items; it += warps) {
+        const int t = (int)(it / segs), i = (int)(it - (long long)t * segs) * 256 + lane * 8;
+        int e = 0;
+        float dz = 0.0f;
+        if (lane < k) { e = idx[(size_t)t * k + lane]; dz = dz_sel[(size_t)t * k + lane]; }
+        uint4* px = reinterpret_cast<uint4*>(dX + (size_t)t * d + i);
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < d) v = *px;
+        float a[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a[q] = 0.0f;
+#pragma unroll 4
+        for (int j = 0; j < k; ++j) {
+            const float* w = W_rT + (size_t)__shfl_sync(0xffffffffu, e, j) * d + i;
+            const float s = __shfl_sync(0xffffffffu, dz, j);
+            if (i < d) {
+                const float4 w0 = *reinterpret_cast<const float4*>(w), w1 = *reinterpret_cast<const float4*>(w + 4);
+                a[0] = fmaf(s, w0.x, a[0]); a[1] = fmaf(s, w0.y, a[1]); a[2] = fmaf(s, w0.z, a[2]); a[3] = fmaf(s, w0.w, a[3]);
+                a[4] = fmaf(s, w1.x, a[4]); a[5] = fmaf(s, w1.y, a[5]); a[6] = fmaf(s, w1.z, a[6]); a[7] = fmaf(s, w1.w, a[7]);
+            }
+        }
+        if (i < d) {
+            v.x = pack_bf16x2(bf16_lo(v.x) + a[0], bf16_hi(v.x) + a[1]);
+            v.y = pack_bf16x2(bf16_lo(v.y) + a[2], bf16_hi(v.y) + a[3]);
+            v.z = pack_bf16x2(bf16_lo(v.z) + a[4], bf16_hi(v.z) + a[5]);
+            v.w = pack_bf16x2(bf16_lo(v.w) + a[6], bf16_hi(v.w) + a[7]);
+            *px = v;
+        }
+    }
+}
+
 // dW_r[i,e] = sum over the rows p of expert e of Xp[p,i] * dz_row[p].  Block (256 columns i, e): warp w adds the rows w, w + W,
 // ... of the expert (eight columns per lane, four rows in flight), the W partial sums are added in order through shared memory.
 // Bound by reading Xp once.  With one thread per eight columns walking all rows two at a time (128 threads per 1024 columns)
 // there were too few bytes in flight: 141 us at T = 4096, d = 2048, E = 64, k = 6 and 292 us at T = 4096, d = 1024, E = 32,
 // k = 8; now 28 and 21.  Fixed order, no atomics.
-__global__ void __launch_bounds__(1024) route_bwd_dwr_kernel(const bf16* __restrict__ Xp, const float* __restrict__ dz_row,
-                                                             const int32_t* __restrict__ offsets, float* __restrict__ dW_r,
-                                                             float* __restrict__ dbias, int d, int E) {
+// The blocks behind these, if any, add the router's share to dX: neither waits for the other.
+__global__ void __launch_bounds__(1024) route_bwd_dwr_dx_kernel(const bf16* __restrict__ Xp, const float* __restrict__ dz_row,
+                                                                const int32_t* __restrict__ offsets, float* __restrict__ dW_r,
+                                                                float* __restrict__ dbias, int d, int E, const float* __restrict__ W_rT,
+                                                                const int32_t* __restrict__ idx, const float* __restrict__ dz_sel,
+                                                                bf16* __restrict__ dX, int T, int k) {
     pdl_begin();
     extern __shared__ float dwr_smem[];                              // [W][256]
-    const int e = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32, W = blockDim.x / 32;
-    const int i = blockIdx.x * 256 + lane * 8;
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, W = blockDim.x / 32;
+    const int across = (d + 255) / 256, dwr_blocks = across * E;
+    if ((int)blockIdx.x >= dwr_blocks) {
+        route_bwd_dx(W_rT, idx, dz_sel, dX, T, d, k, ((int)blockIdx.x - dwr_blocks) * W + warp, ((int)gridDim.x - dwr_blocks) * W);
+        return;
+    }
+    const int e = blockIdx.x / across, c0 = (blockIdx.x - e * across) * 256, i = c0 + lane * 8;
     const int p0 = offsets[e], p1 = offsets[e + 1];
     float a[8];
 #pragma unroll
@@ -839,12 +901,12 @@ __global__ void __launch_bounds__(1024) route_bwd_dwr_kernel(const bf16* __restr
     *reinterpret_cast<float4*>(mine) = make_float4(a[0], a[1], a[2], a[3]);
     *reinterpret_cast<float4*>(mine + 4) = make_float4(a[4], a[5], a[6], a[7]);
     __syncthreads();
-    if (threadIdx.x < 256 && blockIdx.x * 256 + (int)threadIdx.x < d) {
+    if (threadIdx.x < 256 && c0 + (int)threadIdx.x < d) {
         float s = 0.0f;
         for (int w = 0; w < W; ++w) s += dwr_smem[w * 256 + threadIdx.x];
-        dW_r[(size_t)(blockIdx.x * 256 + threadIdx.x) * E + e] = s;
+        dW_r[(size_t)(c0 + threadIdx.x) * E + e] = s;
     }
-    if (dbias && blockIdx.x == 0 && warp == 0) {
+    if (dbias && c0 == 0 && warp == 0) {
         float sb = 0.0f;
         for (int p = p0 + lane; p < p1; p += 32) sb += dz_row[p];
 #pragma unroll
@@ -854,51 +916,5 @@ __global__ void __launch_bounds__(1024) route_bwd_dwr_kernel(const bf16* __restr
 }
 // Warps per block: enough to keep 16 warps and more on every SM (8 warps leave the other blocks room where there are many).
 inline int dwr_warps(long long blocks, int sm_count) { return blocks >= 4ll * sm_count ? 8 : blocks >= 2ll * sm_count ? 16 : 32; }
-
-// W_r^T [E,d] from W_r [d,E] (32 x 32 tiles through shared memory): gives the dX kernel contiguous rows.
-__global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restrict__ in, float* __restrict__ out,
-                                                            int rows, int cols) {
-    pdl_begin();
-    __shared__ float tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-    for (int r = ty; r < 32; r += 8)
-        if (r0 + r < rows && c0 + tx < cols) tile[r][tx] = in[(size_t)(r0 + r) * cols + c0 + tx];
-    __syncthreads();
-    for (int c = ty; c < 32; c += 8)
-        if (c0 + c < cols && r0 + tx < rows) out[(size_t)(c0 + c) * rows + r0 + tx] = tile[tx][c];
-}
-
-// dX[t,:] += dz[t,:] W_r^T = sum_j dz[t,j] * W_r^T[e_j,:]: one CTA per token walks its k selected rows
-// of W_r^T (contiguous, L2-resident) four columns per thread; dX is read, updated in fp32 and rounded
-// back to bf16.  d is a multiple of 8.
-__global__ void __launch_bounds__(256) route_bwd_dx_kernel(const float* __restrict__ W_rT,
-                                                           const int32_t* __restrict__ idx,
-                                                           const float* __restrict__ dz_sel, bf16* __restrict__ dX,
-                                                           int T, int d, int E, int k) {
-    pdl_begin();
-    __shared__ int32_t es[32];
-    __shared__ float dzs[32];
-    const int t = blockIdx.x;
-    if (threadIdx.x < k) {
-        es[threadIdx.x] = idx[(size_t)t * k + threadIdx.x];
-        dzs[threadIdx.x] = dz_sel[(size_t)t * k + threadIdx.x];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x * 4; i < d; i += 256 * 4) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int j = 0; j < k; ++j) {
-            const float4 w = *reinterpret_cast<const float4*>(W_rT + (size_t)es[j] * d + i);
-            const float s = dzs[j];
-            acc.x = fmaf(s, w.x, acc.x); acc.y = fmaf(s, w.y, acc.y);
-            acc.z = fmaf(s, w.z, acc.z); acc.w = fmaf(s, w.w, acc.w);
-        }
-        uint2* px = reinterpret_cast<uint2*>(dX + (size_t)t * d + i);
-        uint2 v = *px;
-        v.x = pack_bf16x2(bf16_lo(v.x) + acc.x, bf16_hi(v.x) + acc.y);
-        v.y = pack_bf16x2(bf16_lo(v.y) + acc.z, bf16_hi(v.y) + acc.w);
-        *px = v;
-    }
-}
 
 }  // namespace mop
