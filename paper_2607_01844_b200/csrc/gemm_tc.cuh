@@ -84,7 +84,8 @@ struct TcArgs {
     EpiArgs ep;
     float* outf1;            // WGU: second output tensor
     int keep_empty;          // weight gradients: leave the gradients of experts without rows untouched
-    bool gemm_follows;       // weight gradients: the next launch on the stream is a GEMM of this layer
+    bool gemm_follows;       // the next launch on the stream is a GEMM of this call (kernels that check it: see pdl_begin_gemm)
+    bool beside;             // VX: the launch before it on the stream is the weight gradient of the same block, which lets it start
     const void* pf[3];       // weight gradients: the operands (rows of all experts, dense) and the bytes of a row of each,
     int pf_bytes[3];         // which the producers bring to L2 an expert ahead (wgrad_prefetch); 0: they do not
 };

@@ -1635,12 +1635,14 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
             TcArgs g = base;
             g.tiles_n = ceil_div(cw, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.n_base = c0;
             g.targets = targets; g.row_lse = lse; g.row_g = dloss; g.ep.out0 = dY; g.ep.ldo = L.vc;
+            g.gemm_follows = true;
             if ((r = tc2_launch<TC_VP>(p, "vocab_dlogits", mX, mX, mWn, mWn, g, st)) != MOP_OK) return r;
         }
         {   // dW[:, block] = X^T dY (K = the N tokens), written once
             TcArgs g = base;
             g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, few ? TC_BM : 256); g.Mfix = H; g.N = cw;
             g.ep.outf = dW_voc + c0;
+            g.gemm_follows = true;
             if (few) {
                 g.offsets = tiles + 32;
                 r = tc_launch<TC_WD>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, mOut, mOut, g, st);
@@ -1650,8 +1652,10 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
             }
             if (r != MOP_OK) return r;
         }
-        {   // dX += dY W[:, block]^T in fp32 across the blocks
+        {   // dX += dY W[:, block]^T in fp32 across the blocks.  Its CTAs take over from those of the weight gradient: N = 8192, H = 7168
+            // makes 896 tiles of either, 12.1 for each of 74 pairs of CTAs, and 25 rounds of both together instead of 26.
             TcArgs g = base;
+            g.beside = true;
             g.tiles_n = ceil_div(H, 256); g.kblocks = ceil_div(cw, TC_BK); g.N = H; g.kb_base = c0;
             g.ep.outf = dx32; g.ep.accumulate = c0 > 0 ? 1 : 0;
             if ((r = tc2_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, g, st)) != MOP_OK) return r;
