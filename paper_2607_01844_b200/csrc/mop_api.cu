@@ -758,6 +758,9 @@ mop_status layer_forward(mop_ctx* c, const void* x, const float* W_r, const floa
     int32_t* table = shared_tiles(c);
     mop_status r;
     if (!c->fast_route && route_permute_fits(s.T, s.d, s.E, s.k)) {
+        // (mop_moe_route makes these checks; the host-buffer entry points come here without any of their own)
+        REQ_PTR(W_r);
+        if ((s.bias_mode != MOP_BIAS_NONE) != (bias != nullptr)) return MOP_ERR_INVALID_ARG;
         DeviceGuard guard(c->device);
         if (!guard.ok) return MOP_ERR_CUDA;
         cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -554,6 +554,27 @@ def test_forward_host_entry_point_matches_device_path():
     assert torch.equal(Yh, buf.Y.cpu()) and torch.equal(idxh, buf.idx.cpu()) and torch.equal(gh, buf.gate.cpu())
 
 
+@pytest.mark.parametrize("T,host_io", [(40, 1), (40, 2), (400, 1), (400, 2)])     # routed in one launch, and by the separate calls
+def test_host_entry_points_refuse_a_missing_router_or_bias(T, host_io):
+    w = synth.small("c3_trillion", T=T, d=128, E=8, k=2, f=64, seed=20)
+    inp = synth.make_inputs(w, "cuda")
+    ctx = binding.context_for(w, host_io=host_io)
+    xh = inp["x"].cpu().pin_memory()
+    Yh = torch.empty_like(xh).pin_memory()
+    call = binding.mop_moe_forward_host if host_io == 1 else binding.mop_moe_forward_host_async
+    assert inp["bias"] is not None
+    for W_r, bias in ((None, inp["bias"]), (inp["W_r"], None)):
+        with pytest.raises(binding.MopError) as e:
+            call(ctx, xh, W_r, bias, inp["W_gate"], inp["W_up"], inp["W_down"], Yh)
+        assert e.value.code == 1
+    call(ctx, xh, inp["W_r"], inp["bias"], inp["W_gate"], inp["W_up"], inp["W_down"], Yh)
+    if host_io == 2:
+        binding.mop_host_drain(ctx)
+    buf = binding.LayerBuffers(w)
+    binding.forward(binding.context_for(w), inp, buf)
+    assert torch.equal(Yh, buf.Y.cpu())
+
+
 @pytest.mark.parametrize("backward", [False, True], ids=["fwd", "train"])
 def test_pipelined_host_steps_match_the_device_path_step_by_step(backward):
     """Five steps with different inputs in flight through the two slots; every step's results are its own."""
