@@ -29,7 +29,7 @@ __device__ __forceinline__ float sigmoidf_fast(float v) { return __fdividef(1.0f
 
 // Programmatic dependent launch: a kernel started by pdl_launch() may be brought up before its predecessor in the stream has
 // drained; pdl_begin() waits until the predecessor has finished and its writes are visible.  Nothing may be read or written
-// before it, and every kernel started by pdl_launch() calls it in every thread.
+// before it, and every kernel started by pdl_launch() calls it, or one of its two forms below, in every thread.
 // A grid of few blocks also lets the next kernel come up while it runs (blocks resident, barriers and tensor memory set up).  A
 // grid that fills the SMs does not: the next kernel's blocks would pile up on the SMs that empty first (training step at
 // T 1537, d 1000, E 20: 346 us without any of this, 391 with every kernel letting its successor in at its start).
@@ -39,10 +39,37 @@ __device__ __forceinline__ void pdl_begin() {
 }
 // The exception: a GEMM followed by a GEMM.  Both take a whole SM per CTA, so the next one's CTAs can only come up where one of this
 // grid has left, one each, and find their barriers, tensor memory and descriptors ready when the last one leaves.
-__device__ __forceinline__ void pdl_begin_gemm(bool gemm_follows) {
+// `note`: the next kernel runs beside this one, and this one leaves word that everything before it is complete.
+struct PdlNote {
+    int32_t* word;           // null: no such kernel follows
+    int32_t value;           // another one for every pair of kernels since the word was cleared
+};
+__device__ __forceinline__ void pdl_begin_gemm(bool gemm_follows, const PdlNote& note) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (note.word) {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(note.word), "r"(note.value) : "memory");
+        __syncthreads();     // so that the word is on its way before this block lets the next kernel start
+    }
     if (gemm_follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// A kernel that runs beside the one before it (A), and reads and writes only what kernels before A have written and read.
+//  - A waits first (pdl_begin_gemm with the same note), so all grids before A are complete and visible to A when it writes the word;
+//    each of those has waited for the one before it in turn.
+//  - Only this kernel's own griddepcontrol.wait would make their writes visible to it, and that one waits for A as well.  So the
+//    ordering goes through the word: A's release, the acquire here, the barrier, and, because TMA reads through another proxy than
+//    the one those kernels wrote through, a proxy fence in every thread.  The word is not waited for: a block that does not find it
+//    takes the grid's wait.
+//  - What A reads may only be overwritten, and what A writes only be read, by kernels after this one: it waits for A before it
+//    leaves (pdl_end_beside), so that its end is the end of both.
+__device__ __forceinline__ void pdl_begin_beside(const PdlNote& note) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    int32_t v = note.value;
+    if (threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(note.word) : "memory");
+    if (!__syncthreads_and(v == note.value)) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_end_beside() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
 inline cudaError_t pdl_launch_clusters(void (*kernel)(P...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                        A... args) {

@@ -85,7 +85,7 @@ struct TcArgs {
     float* outf1;            // WGU: second output tensor
     int keep_empty;          // weight gradients: leave the gradients of experts without rows untouched
     bool gemm_follows;       // the next launch on the stream is a GEMM of this call (kernels that check it: see pdl_begin_gemm)
-    bool beside;             // VX: the launch before it on the stream is the weight gradient of the same block, which lets it start
+    PdlNote note;            // the vocabulary's weight gradient and the VX that runs beside it
     const void* pf[3];       // weight gradients: the operands (rows of all experts, dense) and the bytes of a row of each,
     int pf_bytes[3];         // which the producers bring to L2 an expert ahead (wgrad_prefetch); 0: they do not
 };
@@ -604,7 +604,7 @@ tc_grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    pdl_begin_gemm(args.gemm_follows);
+    pdl_begin_gemm(args.gemm_follows, args.note);
 
     int total_tiles;
     if constexpr (Tr::RAGGED_K) total_tiles = args.E * args.tiles_m_fixed * args.tiles_n;
@@ -916,13 +916,14 @@ __global__ void __launch_bounds__(32 * LSE_WARPS) vocab_lse_merge_kernel(const f
 }
 
 // Row tiles of the dense GEMMs (256 rows per CTA pair), the row range {0, N} as the offsets of one expert (words 32 and 33 of the
-// table), and a clean status word, in one launch.
+// table), a clean status word and a clean PdlNote in the same block, in one launch.
+constexpr int VOCAB_NOTE = 16;         // word of the status block
 __global__ void __launch_bounds__(256) vocab_setup_kernel(int N, int4* __restrict__ tiles, int32_t* __restrict__ n_tiles,
                                                           int32_t* __restrict__ status) {
     pdl_begin();
     const int nt = (N + 255) / 256;
     for (int i = threadIdx.x; i < nt; i += blockDim.x) tiles[i] = make_int4(0, 256 * i, min(256, N - 256 * i), 0);
-    if (threadIdx.x == 0) { *n_tiles = nt; n_tiles[32] = 0; n_tiles[33] = N; *status = 0; }
+    if (threadIdx.x == 0) { *n_tiles = nt; n_tiles[32] = 0; n_tiles[33] = N; *status = 0; status[VOCAB_NOTE] = 0; }
 }
 
 // fp32 -> bf16 of a dense array (8 elements per thread; n a multiple of 8)

@@ -206,11 +206,9 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     cluster_sync_all();          // the peer's barriers exist before anything signals them
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    // Beside the launch before: this one reads nothing that it writes (nor the other way round), and what both read was complete
-    // before that one let this one start.  Its last CTAs and this one's first run together; the end of this one is the end of both.
-    const bool beside = KIND == TC_VX && args.beside;
-    if (beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    else pdl_begin_gemm(args.gemm_follows);
+    // dX runs beside the weight gradient of its block: both read the logit gradients, neither what the other writes.
+    if constexpr (KIND == TC_VX) pdl_begin_beside(args.note);
+    else pdl_begin_gemm(args.gemm_follows, args.note);
 
     const int row_tiles = KIND == TC_VW ? args.tiles_m_fixed : *args.n_mtiles;
     const int total_tiles = row_tiles * args.tiles_n;
@@ -338,7 +336,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     }
 
     // ------------------------------------------------------------------------- teardown
-    if (beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (KIND == TC_VX) pdl_end_beside();
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {

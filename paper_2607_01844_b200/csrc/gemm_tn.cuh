@@ -268,7 +268,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    pdl_begin_gemm(args.gemm_follows);
+    pdl_begin_gemm(args.gemm_follows, PdlNote{});
 
     const int total_tiles = (*args.n_ttiles) * args.tiles_m;
     const int nkb = (KIND == TN_B4 ? 2 : 1) * args.kblocks;   // K blocks per tile (B4: two phases)

@@ -68,7 +68,7 @@ tw_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    pdl_begin_gemm(args.gemm_follows);
+    pdl_begin_gemm(args.gemm_follows, PdlNote{});
 
     const int per_e = args.tiles_m_fixed * args.tiles_n;      // tiles_m_fixed: 256-row blocks of the gradient
     const int total_tiles = args.E * per_e;

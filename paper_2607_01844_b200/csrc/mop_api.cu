@@ -1634,6 +1634,7 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
         TcArgs base{};
         base.n_mtiles = tiles; base.n_group = VOCAB_N_GROUP; base.mtiles = reinterpret_cast<const int4*>(tiles + 64);
         base.E = 1; base.status = status; base.ep.M_total = N;
+        const PdlNote note = {status + VOCAB_NOTE, c0 / L.vc + 1};
         {   // dY block = g ([v = t] - exp(X W - lse)), logits recomputed on the tensor cores
             TcArgs g = base;
             g.tiles_n = ceil_div(cw, 256); g.kblocks = ceil_div(H, TC_BK); g.N = V; g.n_base = c0;
@@ -1646,6 +1647,7 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
             g.tiles_n = ceil_div(cw, 256); g.tiles_m_fixed = ceil_div(H, few ? TC_BM : 256); g.Mfix = H; g.N = cw;
             g.ep.outf = dW_voc + c0;
             g.gemm_follows = true;
+            g.note = note;
             if (few) {
                 g.offsets = tiles + 32;
                 r = tc_launch<TC_WD>(p, "vocab_wgrad", mXT, mXT, mdYn, mdYn, mOut, mOut, g, st);
@@ -1658,7 +1660,7 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
         {   // dX += dY W[:, block]^T in fp32 across the blocks.  Its CTAs take over from those of the weight gradient: N = 8192, H = 7168
             // makes 896 tiles of either, 12.1 for each of 74 pairs of CTAs, and 25 rounds of both together instead of 26.
             TcArgs g = base;
-            g.beside = true;
+            g.note = note;
             g.tiles_n = ceil_div(H, 256); g.kblocks = ceil_div(cw, TC_BK); g.N = H; g.kb_base = c0;
             g.ep.outf = dx32; g.ep.accumulate = c0 > 0 ? 1 : 0;
             if ((r = tc2_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, g, st)) != MOP_OK) return r;

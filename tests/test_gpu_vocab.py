@@ -145,6 +145,34 @@ def test_vocab_weight_gradient_with_few_and_with_many_tokens(N, H, V):
     test_vocab_tile_order_covers_every_tile_once(N, H, V)
 
 
+@pytest.mark.parametrize("N", [200, 1100], ids=["few", "many"])     # either form of the weight gradient that dX runs beside
+def test_vocab_backward_takes_nothing_from_what_the_workspace_held(N):
+    """Three blocks of columns: the same bits whether the workspace holds NaN, small counts or the logit gradients and sums of
+    another call, calls back to back included."""
+    H, V = 256, 2 * 8192 + 64
+    g = torch.randn((N,), device="cuda") * 0.5 - 1.0
+    calls = []
+    for seed in (1, 2):
+        X, W, t = _inputs(N, H, V, seed=seed, std=0.05)
+        loss, lse = torch.empty((N,), device="cuda"), torch.empty((N,), device="cuda")
+        binding.mop_vocab_loss_fwd(0, X, W, t, loss, lse)
+        calls.append((X, W, t, lse))
+    ws = torch.empty(binding.mop_vocab_bwd_workspace_bytes(N, H, V), dtype=torch.uint8, device="cuda")
+    first = []
+    for fill in (0xFF, 1, 2, None, None):
+        if fill == 0xFF:
+            ws.fill_(fill)
+        elif fill:
+            ws.view(torch.int32).fill_(fill)
+        out = [(torch.empty((N, H), device="cuda", dtype=torch.bfloat16), torch.empty((H, V), device="cuda")) for _ in calls]
+        for (X, W, t, lse), (dX, dW) in zip(calls, out):
+            binding.mop_vocab_loss_bwd(0, X, W, t, lse, g, dX, dW, ws)
+        binding.mop_vocab_poll(0, ws)
+        first = first or out
+        for a, b in zip(first, out):
+            assert torch.isfinite(b[0].float()).all() and torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
 @pytest.mark.parametrize("V,column", [(192, 40),            # one tile: seven of the merging warps hold nothing
                                       (2624, 300),          # eleven tiles, in the second warp's share
                                       (2624, 2600)],        # the last tile

@@ -119,3 +119,28 @@ def test_warps_that_wait_with_all_lanes_go_on_together():
             # voted on in place, or in the next statements
             assert "__all_sync(0xffffffffu, " in before or "if (!__all_sync(0xffffffffu, ok))" in text[end:end + 250], \
                 f"{path.name}: {line.strip()}"
+
+
+def test_kernels_launched_beside_their_predecessor_wait_or_acquire_what_they_read():
+    """Every kernel that pdl_launch starts begins with one of the forms of pdl_begin.  They are all there is of griddepcontrol, and
+    the one that does not wait for its predecessor acquires a word that the predecessor releases after its own wait, waits all
+    the same where it does not find it, puts a proxy fence before what TMA reads, and waits at its end."""
+    texts = {p.name: p.read_text() for p in sorted(CSRC.glob("*.cu*"))}
+    for name, text in texts.items():
+        assert name == "common.cuh" or "griddepcontrol" not in text, name
+    every = "\n".join(texts.values())
+    started = set(re.findall(r"\bpdl_launch(?:_clusters)?\((\w+_kernel)\b", every)) | set(re.findall(r"\bgo\((\w+_kernel)<", every))
+    assert len(started) > 20
+    for kernel in sorted(started):
+        body = re.search(r"__global__[^;{]*?\b" + kernel + r"\((?:[^{;]*)\{(.*?)\n\}", every, re.S).group(1)
+        assert re.search(r"\bpdl_begin(_gemm|_beside)?\(", body), kernel
+
+    def function(name):
+        return re.search(r"void " + name + r"\(.*?\{\n(.*?)\n\}|void " + name + r"\(\) \{(.*?)\}\n", texts["common.cuh"], re.S).group(0)
+    order = lambda text, *parts: [text.index(p) for p in parts] == sorted(text.index(p) for p in parts)
+    assert order(function("pdl_begin"), "griddepcontrol.wait", "griddepcontrol.launch_dependents")
+    assert order(function("pdl_begin_gemm"), "griddepcontrol.wait", "st.release.gpu", "__syncthreads()", "griddepcontrol.launch_dependents")
+    assert order(function("pdl_begin_beside"), "ld.acquire.gpu", "__syncthreads_and", "griddepcontrol.wait", "fence.proxy.async.global")
+    assert "griddepcontrol.wait" in function("pdl_end_beside")
+    for name, text in texts.items():
+        assert text.count("pdl_begin_beside(") == text.count("pdl_end_beside("), name
