@@ -637,8 +637,9 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                         for (int j = 0; j < 2; ++j)
                             stmatrix4_trans(st + a * TN_STASH_BYTES + 1024 * j + fo2, frag[a][j][0], frag[a][j][1], frag[a][j][2], frag[a][j][3]);
                     const bool whole = c + 16 <= rows;
-                    if (whole) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    else {                                     // the rows after the tile's are another expert's: row by row
+                    // (in either case: TMA reads these bytes now, or writes the next tile's stash over them)
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    if (!whole) {                              // the rows after the tile's are another expert's: row by row
                         __syncwarp();
                         const int tok = lane >> 2, col = fcol + (lane & 3) * 8;
 #pragma unroll

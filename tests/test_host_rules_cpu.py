@@ -144,3 +144,13 @@ def test_kernels_launched_beside_their_predecessor_wait_or_acquire_what_they_rea
     assert "griddepcontrol.wait" in function("pdl_end_beside")
     for name, text in texts.items():
         assert text.count("pdl_begin_beside(") == text.count("pdl_end_beside("), name
+
+
+def test_what_is_written_to_a_buffer_that_tma_copies_is_fenced_in_every_case():
+    """SwiGLU backward: a step's results lie in a buffer that TMA then reads, or, where the rows leave one by one, writes over.
+    Both are another proxy's accesses, so the fence between them and the lanes' stores hangs on no condition."""
+    text = (CSRC / "gemm_tn.cuh").read_text()
+    start = text.index("stmatrix4_trans(st + a * TN_STASH_BYTES")
+    step = text[start:text.index("bar_vote_all(pair_bar", start)]
+    assert re.search(r'\n +asm volatile\("fence\.proxy\.async\.shared::cta;"', step)
+    assert step.index("fence.proxy.async") < step.index("if (")
