@@ -405,6 +405,20 @@ def test_selection_of_equal_signed_zero_and_infinite_logits(E, k):
     assert (idx.cpu().numpy() == order).all()
 
 
+@pytest.mark.parametrize("E,k", [(33, 3), (65, 8), (128, 1), (257, 8), (513, 32), (1024, 2)])     # every number of keys a lane holds
+@pytest.mark.parametrize("score,bias", [(0, 2), (1, 0), (1, 1), (1, 2)])
+def test_selection_with_every_form_of_key_matches_oracle(E, k, score, bias):
+    w = synth.Workload("keys", 70, 64, E, k, 64, score, bias, 0.05 if bias else 0.0, seed=E + score)
+    inp = synth.make_inputs(w, "cuda")
+    ctx = binding.context_for(w, route_path=binding.ROUTE_EXACT)
+    idx = torch.empty((w.T, k), dtype=torch.int32, device="cuda")
+    gate = torch.empty((w.T, k), dtype=torch.float32, device="cuda")
+    b = inp["bias"] if not bias or inp["bias"] is not None else torch.randn(E, device="cuda") * 0.05
+    binding.mop_moe_route(ctx, inp["x"], inp["W_r"], b, idx, gate)
+    want, g = oracle.route(synth.bits(inp["x"]), inp["W_r"].cpu().numpy(), None if b is None else b.cpu().numpy(), k, score, bias)
+    assert np.array_equal(idx.cpu().numpy(), want) and np.allclose(gate.cpu().numpy(), g, rtol=1e-5, atol=1e-6)
+
+
 @pytest.mark.parametrize("T,d,k", [(1, 8, 1), (3, 264, 32), (130, 1032, 9),             # a vector a lane, rows in batches of 8
                                    (3600, 256, 3), (3600, 264, 2), (1800, 1016, 5),      # one and two vectors, two rows at a time
                                    (900, 1024, 4), (900, 1032, 3)])                      # four vectors, a row at a time
