@@ -384,61 +384,74 @@ __global__ void __launch_bounds__(256) scatter_rows_reg_kernel(const uint4* __re
     }
 }
 
-// Combine: Y[t,:] = bf16(sum_j Yp[perm_row[t*k+j],:]) with the k-row sum kept in fp32 registers, j ascending.  A warp takes 32 SEG
-// vectors of a token's row, R rows' at a time.  HBM bound where there are many (T = 16384, d = 7168, k = 8: 338 us, 0.96 of the copy
-// rate), and there one row of 2 KiB at a time does best (T = 8192, d = 4096, k = 4: 55 us, 64 with two rows of 1 KiB, 78 with four,
-// 82 with a warp per token and rows of 4 KiB); latency bound where there are few, where a warp takes 512 bytes of all rows at once
-// (T = 16, d = 2048, k = 6 3.5 us, 12.9 with a warp per token; T = 64, d = 7168, k = 8 4.5 and 29.8).
-template <int SEG, int R>
+// Combine: Y[t,:] = bf16(sum_j Yp[perm_row[t*k+j],:]) with the k-row sum kept in fp32 registers, j ascending.  Rows of -1 are left out.
+__device__ __forceinline__ void add_bf16x8(float (&a)[8], const uint4& v) {
+    a[0] += bf16_lo(v.x); a[1] += bf16_hi(v.x); a[2] += bf16_lo(v.y); a[3] += bf16_hi(v.y);
+    a[4] += bf16_lo(v.z); a[5] += bf16_hi(v.z); a[6] += bf16_lo(v.w); a[7] += bf16_hi(v.w);
+}
+__device__ __forceinline__ uint4 pack_bf16x8(const float (&a)[8]) {
+    return make_uint4(pack_bf16x2(a[0], a[1]), pack_bf16x2(a[2], a[3]), pack_bf16x2(a[4], a[5]), pack_bf16x2(a[6], a[7]));
+}
+// Much to do: a warp takes 2 KiB of a token's row, one of the k rows at a time.  HBM bound (T = 16384, d = 7168, k = 8: 338 us, 0.96 of
+// the copy rate), and there one row of 2 KiB at a time does best (T = 8192, d = 4096, k = 4: 55 us, 64 with two rows of 1 KiB, 78 with
+// four, 82 with a warp per token and rows of 4 KiB).
+constexpr int COMB_SEG = 4;
 __global__ void __launch_bounds__(256) combine_rows_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ perm_row,
                                                             uint4* __restrict__ Y, int T, int k, int vec_per_row) {
     pdl_begin();
-    const int lane = threadIdx.x % 32, wpb = blockDim.x / 32;
-    const int segs = (vec_per_row + 32 * SEG - 1) / (32 * SEG);
-    const long long items = (long long)T * segs;
-    for (long long i = (long long)blockIdx.x * wpb + threadIdx.x / 32; i < items; i += (long long)gridDim.x * wpb) {
-        const int t = (int)(i / segs), c = (int)(i - (long long)t * segs) * 32 * SEG + lane;
+    const int lane = threadIdx.x % 32;
+    const uint32_t wpb = blockDim.x / 32, segs = (vec_per_row + 32 * COMB_SEG - 1) / (32 * COMB_SEG);
+    const uint32_t items = (uint32_t)T * segs;         // (32 bits: T < 2^31, and the rest of 16-byte vectors fits the device's memory)
+    for (uint32_t i = blockIdx.x * wpb + threadIdx.x / 32; i < items; i += gridDim.x * wpb) {
+        const int t = (int)(i / segs), c = (int)(i - t * segs) * 32 * COMB_SEG + lane;
         int32_t myrow = -1;
         if (lane < k) myrow = perm_row[(size_t)t * k + lane];
-        float acc[SEG][8];
+        float acc[COMB_SEG][8];
 #pragma unroll
-        for (int q = 0; q < SEG; ++q)
+        for (int q = 0; q < COMB_SEG; ++q)
 #pragma unroll
             for (int u = 0; u < 8; ++u) acc[q][u] = 0.0f;
-        for (int j0 = 0; j0 < k; j0 += R) {
-            uint4 v[R][SEG];
-            int32_t p[R];
+        for (int j = 0; j < k; ++j) {
+            const int32_t p = __shfl_sync(0xffffffffu, myrow, j);
+            if (p < 0) continue;
+            const uint4* src = Yp + (size_t)p * vec_per_row + c;
+            uint4 v[COMB_SEG];
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                p[r] = __shfl_sync(0xffffffffu, myrow, (j0 + r) & 31);
-                if (j0 + r >= k) p[r] = -1;
-                const uint4* src = Yp + (size_t)max(p[r], 0) * vec_per_row + c;
+            for (int q = 0; q < COMB_SEG; ++q)
+                if (c + 32 * q < vec_per_row) v[q] = __ldcs(src + 32 * q);
 #pragma unroll
-                for (int q = 0; q < SEG; ++q)
-                    if (p[r] >= 0 && c + 32 * q < vec_per_row) v[r][q] = __ldcs(src + 32 * q);
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (p[r] < 0) continue;
-#pragma unroll
-                for (int q = 0; q < SEG; ++q) {
-                    acc[q][0] += bf16_lo(v[r][q].x); acc[q][1] += bf16_hi(v[r][q].x);
-                    acc[q][2] += bf16_lo(v[r][q].y); acc[q][3] += bf16_hi(v[r][q].y);
-                    acc[q][4] += bf16_lo(v[r][q].z); acc[q][5] += bf16_hi(v[r][q].z);
-                    acc[q][6] += bf16_lo(v[r][q].w); acc[q][7] += bf16_hi(v[r][q].w);
-                }
-            }
+            for (int q = 0; q < COMB_SEG; ++q) add_bf16x8(acc[q], v[q]);
         }
 #pragma unroll
-        for (int q = 0; q < SEG; ++q)
-            if (c + 32 * q < vec_per_row) {
-                uint4 o;
-                o.x = pack_bf16x2(acc[q][0], acc[q][1]);
-                o.y = pack_bf16x2(acc[q][2], acc[q][3]);
-                o.z = pack_bf16x2(acc[q][4], acc[q][5]);
-                o.w = pack_bf16x2(acc[q][6], acc[q][7]);
-                Y[(size_t)t * vec_per_row + c + 32 * q] = o;
-            }
+        for (int q = 0; q < COMB_SEG; ++q)
+            if (c + 32 * q < vec_per_row) Y[(size_t)t * vec_per_row + c + 32 * q] = pack_bf16x8(acc[q]);
+    }
+}
+// Little to do, or rows too short for that: a thread per vector of Y, R of its rows in flight.  Nothing is left idle where a row is
+// no multiple of what a warp takes, and there is little to set up.
+template <int R>
+__global__ void __launch_bounds__(256) combine_vectors_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ perm_row,
+                                                              uint4* __restrict__ Y, uint32_t n, int k, uint32_t vec_per_row) {
+    pdl_begin();
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t t = i / vec_per_row, c = i - t * vec_per_row;
+        const int32_t* rows = perm_row + (size_t)t * k;
+        float acc[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
+        for (int j = 0; j < k; j += R) {
+            uint4 v[R];
+            int32_t p[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r] = j + r < k ? rows[j + r] : -1;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (p[r] >= 0) v[r] = __ldcs(Yp + (size_t)p[r] * vec_per_row + c);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (p[r] >= 0) add_bf16x8(acc, v[r]);
+        }
+        Y[i] = pack_bf16x8(acc);
     }
 }
 
@@ -456,18 +469,25 @@ inline void launch_scatter_rows(const uint4* src, uint4* dst, const int32_t* per
 inline void launch_combine_rows(const uint4* Yp, const int32_t* perm_row, uint4* Y, int T, int k, int vec_per_row,
                                 int sm_count, cudaStream_t st) {
     if (T <= 0) return;
-    auto go = [&](auto kernel, int seg, int threads) {
-        const long long items = (long long)T * ceil_div(vec_per_row, 32 * seg);
-        const long long most = (long long)sm_count * (2048 / threads);
-        const int blocks = (int)min((items + threads / 32 - 1) / (threads / 32), most);
-        pdl_launch(kernel, blocks, threads, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
-    };
-    // us: T 512, d 1024, k 4 (14 warps per SM of one vector each) 2.8 and 3.5 with four vectors; T 256, d 7168, k 8 (48) 10.1 and 8.2
-    if ((long long)T * ceil_div(vec_per_row, 32) <= 24ll * sm_count) go(combine_rows_kernel<1, 8>, 1, 128);
-    // rows shorter than four vectors a lane: T 16384, d 256, k 8 24.6 us, 32.8 with four; d 512, k 4 22.7 and 24.6
-    else if (vec_per_row <= 32) go(combine_rows_kernel<1, 2>, 1, 256);
-    else if (vec_per_row < 128) go(combine_rows_kernel<2, 2>, 2, 128);
-    else go(combine_rows_kernel<4, 1>, 4, 256);
+    // us, vectors and pieces of rows: T 1000, d 1024 (128 thousand vectors) k 1 1.8 and 1.8, k 8 2.8 and 4.0; d 2048 (256 thousand) k 1
+    // 2.3 and 2.2, k 8 4.4 and 4.6; T 4096, d 2048, k 1 4.9 and 4.5, k 4 9.4 and 8.1.  Short rows: T 16384, d 520 k 1 5.0 and 5.7,
+    // k 4 10.9 and 14.1, k 8 24.7 and 30.3; d 768 k 1 6.9 and 6.2, k 4 19.4 and 20.5; d 1000, k 6 39.3 and 36.3.
+    const long long n = (long long)T * vec_per_row;
+    const bool few = n <= 512ll * sm_count;
+    if (n <= 1280ll * sm_count || (vec_per_row < 96 && n < (1ll << 31))) {
+        const int threads = few ? 128 : 256;
+        const int blocks = (int)min((n + threads - 1) / threads, (long long)sm_count * (2048 / threads));
+        auto go = [&](auto kernel) { pdl_launch(kernel, blocks, threads, 0, st, Yp, perm_row, Y, (uint32_t)n, k, (uint32_t)vec_per_row); };
+        // rows in flight, for the latency of one: T 64, d 7168, k 8 2.2 us with eight, 2.3 with four, 2.5 with two.  With more vectors
+        // than a few a thread's registers cost more than they give (T 512, d 2048, k 8 3.5, 2.9 and 3.0).
+        if (k == 1) go(combine_vectors_kernel<1>);
+        else if (k == 2) go(combine_vectors_kernel<2>);
+        else if (k <= 4 || !few) go(combine_vectors_kernel<4>);
+        else go(combine_vectors_kernel<8>);
+        return;
+    }
+    const long long items = (long long)T * ceil_div(vec_per_row, 32 * COMB_SEG);
+    pdl_launch(combine_rows_kernel, (int)min((items + 7) / 8, 8ll * sm_count), 256, 0, st, Yp, perm_row, Y, T, k, vec_per_row);
 }
 
 // dgate[a] = sum over n-tiles of the partial dot products written by the dgrad-down epilogue

@@ -419,9 +419,11 @@ def test_selection_with_every_form_of_key_matches_oracle(E, k, score, bias):
     assert np.array_equal(idx.cpu().numpy(), want) and np.allclose(gate.cpu().numpy(), g, rtol=1e-5, atol=1e-6)
 
 
-@pytest.mark.parametrize("T,d,k", [(1, 8, 1), (3, 264, 32), (130, 1032, 9),             # a vector a lane, rows in batches of 8
-                                   (3600, 256, 3), (3600, 264, 2), (1800, 1016, 5),      # one and two vectors, two rows at a time
-                                   (900, 1024, 4), (900, 1032, 3)])                      # four vectors, a row at a time
+@pytest.mark.parametrize("T,d,k", [(1, 8, 1), (9, 72, 2), (3, 264, 32), (130, 1032, 9), (60, 520, 3),      # a thread per vector, 1, 2, 8, 8, 4 rows
+                                   (3600, 256, 3), (3600, 264, 2), (900, 1032, 6),    # the same with larger blocks
+                                   (3000, 520, 5), (2500, 760, 1),                    # the same beyond the line: short rows
+                                   (2000, 768, 2), (1800, 1016, 5), (1500, 1032, 3),  # a warp per 2 KiB of a row: partly filled, twice
+                                   (1480, 1024, 9), (1481, 1024, 9)])                 # the last size on one side of the line, whole pieces
 def test_combine_sums_the_rows_in_order(T, d, k):
     """Bit for bit the fp32 sum in ascending j, rounded once; rows of -1 are left out."""
     gen = torch.Generator().manual_seed(T + d)
