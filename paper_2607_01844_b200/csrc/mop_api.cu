@@ -1139,8 +1139,8 @@ mop_status mop_moe_route_bwd(mop_ctx* c, const float* logits, const float* bias,
         if ((r = after_launch(c)) != MOP_OK) return r;
     }
     const int dwr_w = dwr_warps(dwr_blocks, c->sm_count);
-    const long long dx_items = (long long)s.T * ceil_div(s.d, 256);
-    const int dx_blocks = (int)min((dx_items + dwr_w - 1) / dwr_w, (long long)c->sm_count * (64 / dwr_w));
+    const int dx_segs = ceil_div(s.d, 256);            // whole sets of blocks, one for each 256 columns
+    const int dx_blocks = dx_segs * min(ceil_div(s.T, dwr_w), max(1, c->sm_count * (64 / dwr_w) / dx_segs));
     float* db = (dbias_opt && s.bias_mode == MOP_BIAS_PRE_LOGIT) ? dbias_opt : nullptr;
     if (dbias_opt && !db) CUDA_OK(cudaMemsetAsync(dbias_opt, 0, (size_t)s.E * 4, st));
     LAUNCH(c, "route_bwd_dwr_dx", st,

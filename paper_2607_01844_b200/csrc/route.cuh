@@ -828,41 +828,61 @@ __global__ void __launch_bounds__(256) route_bwd_dz_kernel(const float* __restri
     }
 }
 
-// dX[t,:] += dz[t,:] W_r^T = sum_j dz[t,j] * W_r^T[e_j,:]: a warp takes 256 columns of a token, eight a lane, and the k rows of W_r^T
-// (contiguous, L2-resident) four at a time; dX is read, updated in fp32 and rounded back to bf16.  d is a multiple of 8.
+// dX[t,:] += dz[t,:] W_r^T = sum_j dz[t,j] * W_r^T[e_j,:]: a block takes 256 columns (of blocks `block`, `block` + segments, ..) and its
+// warps a token each, twice four columns a lane (neighbouring lanes read neighbouring 16 bytes), with the k rows of W_r^T four at a
+// time; dX is read, updated in fp32 and rounded back to bf16.  d is a multiple of 8.
+// Bound by what the rows of W_r^T cost: k fp32 columns for each bf16 one of dX.  With the columns fixed, E KiB of them pass through an
+// SM's L1 again and again, instead of all E rows through L2.
 __device__ __forceinline__ void route_bwd_dx(const float* __restrict__ W_rT, const int32_t* __restrict__ idx,
-                                             const float* __restrict__ dz_sel, bf16* __restrict__ dX, int T, int d, int k,
-                                             int warp, int warps) {
-    const int lane = threadIdx.x % 32, segs = (d + 255) / 256;
-    const long long items = (long long)T * segs;
-    for (long long it = warp; it < items; it += warps) {
-        const int t = (int)(it / segs), i = (int)(it - (long long)t * segs) * 256 + lane * 8;
-        int e = 0;
-        float dz = 0.0f;
-        if (lane < k) { e = idx[(size_t)t * k + lane]; dz = dz_sel[(size_t)t * k + lane]; }
-        uint4* px = reinterpret_cast<uint4*>(dX + (size_t)t * d + i);
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (i < d) v = *px;
-        float a[8];
+                                             const float* __restrict__ dz_sel, bf16* __restrict__ dX, int T, int d, int k, int block,
+                                             int blocks) {
+    const int lane = threadIdx.x % 32, warps = blockDim.x / 32, segs = (d + 255) / 256;
+    const int i = (block % segs) * 256 + lane * 4;
+    const bool in[2] = {i < d, i + 128 < d};
+    const long long t0 = (long long)(block / segs) * warps + threadIdx.x / 32, step = (long long)(blocks / segs) * warps;
+    int e_next;
+    float dz_next;
+    uint2 v_next[2];
+    auto fetch = [&](long long t) {
+        e_next = 0; dz_next = 0.0f;
+        v_next[0] = v_next[1] = make_uint2(0, 0);
+        if (t >= T) return;
+        if (lane < k) { e_next = idx[(size_t)t * k + lane]; dz_next = dz_sel[(size_t)t * k + lane]; }
+        const bf16* px = dX + (size_t)t * d + i;
+        if (in[0]) v_next[0] = *reinterpret_cast<const uint2*>(px);
+        if (in[1]) v_next[1] = *reinterpret_cast<const uint2*>(px + 128);
+    };
+    fetch(t0);
+    for (long long t = t0; t < T; t += step) {
+        const int e = e_next;
+        const float dz = dz_next;
+        uint2 v[2] = {v_next[0], v_next[1]};
+        fetch(t + step);
+        bf16* px = dX + (size_t)t * d + i;
+        float a[2][4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = 0.0f;
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[h][q] = 0.0f;
 #pragma unroll 4
         for (int j = 0; j < k; ++j) {
             const float* w = W_rT + (size_t)__shfl_sync(0xffffffffu, e, j) * d + i;
             const float s = __shfl_sync(0xffffffffu, dz, j);
-            if (i < d) {
-                const float4 w0 = *reinterpret_cast<const float4*>(w), w1 = *reinterpret_cast<const float4*>(w + 4);
-                a[0] = fmaf(s, w0.x, a[0]); a[1] = fmaf(s, w0.y, a[1]); a[2] = fmaf(s, w0.z, a[2]); a[3] = fmaf(s, w0.w, a[3]);
-                a[4] = fmaf(s, w1.x, a[4]); a[5] = fmaf(s, w1.y, a[5]); a[6] = fmaf(s, w1.z, a[6]); a[7] = fmaf(s, w1.w, a[7]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (in[h]) {
+                    const float4 u = *reinterpret_cast<const float4*>(w + 128 * h);
+                    a[h][0] = fmaf(s, u.x, a[h][0]); a[h][1] = fmaf(s, u.y, a[h][1]);
+                    a[h][2] = fmaf(s, u.z, a[h][2]); a[h][3] = fmaf(s, u.w, a[h][3]);
+                }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (in[h]) {
+                v[h].x = pack_bf16x2(bf16_lo(v[h].x) + a[h][0], bf16_hi(v[h].x) + a[h][1]);
+                v[h].y = pack_bf16x2(bf16_lo(v[h].y) + a[h][2], bf16_hi(v[h].y) + a[h][3]);
+                *reinterpret_cast<uint2*>(px + 128 * h) = v[h];
             }
-        }
-        if (i < d) {
-            v.x = pack_bf16x2(bf16_lo(v.x) + a[0], bf16_hi(v.x) + a[1]);
-            v.y = pack_bf16x2(bf16_lo(v.y) + a[2], bf16_hi(v.y) + a[3]);
-            v.z = pack_bf16x2(bf16_lo(v.z) + a[4], bf16_hi(v.z) + a[5]);
-            v.w = pack_bf16x2(bf16_lo(v.w) + a[6], bf16_hi(v.w) + a[7]);
-            *px = v;
-        }
     }
 }
 
@@ -882,7 +902,7 @@ __global__ void __launch_bounds__(1024) route_bwd_dwr_dx_kernel(const bf16* __re
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, W = blockDim.x / 32;
     const int across = (d + 255) / 256, dwr_blocks = across * E;
     if ((int)blockIdx.x >= dwr_blocks) {
-        route_bwd_dx(W_rT, idx, dz_sel, dX, T, d, k, ((int)blockIdx.x - dwr_blocks) * W + warp, ((int)gridDim.x - dwr_blocks) * W);
+        route_bwd_dx(W_rT, idx, dz_sel, dX, T, d, k, (int)blockIdx.x - dwr_blocks, (int)gridDim.x - dwr_blocks);
         return;
     }
     const int e = blockIdx.x / across, c0 = (blockIdx.x - e * across) * 256, i = c0 + lane * 8;

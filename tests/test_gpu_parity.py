@@ -692,7 +692,8 @@ def test_router_backward_matches_oracle(w):
 
 @pytest.mark.parametrize("T,d,E,k", [(100, 328, 160, 4),      # 16 warps per block of dW_r, the last block of columns partly filled
                                      (150, 264, 300, 3),      # 8 warps, experts with fewer rows than warps
-                                     (900, 264, 300, 7)],     # 8 warps, up to 40 rows per expert: more than four per warp for some
+                                     (900, 264, 300, 7),      # 8 warps, up to 40 rows per expert: more than four per warp for some
+                                     (1, 392, 4, 4), (33, 136, 3, 2), (5000, 264, 6, 2)],  # dX: fewer tokens than warps, half a piece, many rounds
                          ids=lambda v: str(v))
 def test_router_backward_with_many_blocks_matches_oracle(T, d, E, k):
     test_router_backward_matches_oracle(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=64, bias_mode=2, backward=True, seed=34))
