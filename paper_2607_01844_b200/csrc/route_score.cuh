@@ -33,14 +33,16 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, bool ok
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
 }
 
-template <int RT, int RE, int LT, int CW>
+template <int RT, int RE, int LT, int CW, bool TWO>
 struct ScoreShape {
     static constexpr bool PAIRS = RE > 1;                       // chains in pairs of experts; else plain chains, and W transposed
     static constexpr int LE = 32 / LT;
     static constexpr int TT = CW * LT * RT, TE = LE * RE;
     static constexpr int TK = 64;                               // steps per stage
-    static constexpr int THREADS = 64 * CW, LOADERS = 32 * CW;  // warps 0 .. CW - 1 multiply, the others load
-    static constexpr int AHEAD = PAIRS ? 2 : 8;                 // stages in flight from global memory
+    // TWO: two blocks of 64 x 64 on an SM, so that one's multiplications fill the other's waits (registers: six warps of 168; shared
+    // memory: four slots of 25 KiB).  A step of theirs takes long enough to load one stage ahead, by half as many warps.
+    static constexpr int LOADERS = TWO ? 16 * CW : 32 * CW, THREADS = 32 * CW + LOADERS;   // warps 0 .. CW - 1 multiply, the others load
+    static constexpr int AHEAD = TWO ? 1 : PAIRS ? 2 : 8;       // stages in flight from global memory
     static constexpr int READY = 2;                             // stages handed to the multiplying warps
     static constexpr int SLOTS = AHEAD + 1 + READY;             // (filled AHEAD stages early; READY back may still be read; one just released)
     static constexpr int X_PITCH = TK * 2 + 16;                 // neighbouring tokens 16 bytes apart in the banks
@@ -55,11 +57,11 @@ __device__ __forceinline__ void lds_b128(uint32_t addr, uint32_t (&v)[4]) {
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
 }
 
-template <int RT, int RE, int LT, int CW>
-__global__ void __launch_bounds__(64 * CW) route_score_kernel(const bf16* __restrict__ x, const float* __restrict__ W_r,
-                                                              float* __restrict__ z, int T, int d, int E,
-                                                              int32_t* __restrict__ status) {
-    using Sh = ScoreShape<RT, RE, LT, CW>;
+template <int RT, int RE, int LT, int CW, bool TWO>
+__global__ void __launch_bounds__(ScoreShape<RT, RE, LT, CW, TWO>::THREADS, TWO ? 2 : 0)
+route_score_kernel(const bf16* __restrict__ x, const float* __restrict__ W_r, float* __restrict__ z, int T, int d, int E,
+                   int32_t* __restrict__ status) {
+    using Sh = ScoreShape<RT, RE, LT, CW, TWO>;
     constexpr bool PAIRS = Sh::PAIRS;
     constexpr int LE = Sh::LE, TT = Sh::TT, TE = Sh::TE, TK = Sh::TK, AHEAD = Sh::AHEAD, READY = Sh::READY, SLOTS = Sh::SLOTS;
     constexpr int LOADERS = Sh::LOADERS;
@@ -75,7 +77,7 @@ __global__ void __launch_bounds__(64 * CW) route_score_kernel(const bf16* __rest
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sc_smem + 16 * READY);
     const int tid = threadIdx.x, warp = warp_index(), lane = tid % 32;
     if (tid == 0) {
-        for (int s = 0; s < READY; ++s) { mbar_init(full_bar(s), CW); mbar_init(empty_bar(s), CW); }
+        for (int s = 0; s < READY; ++s) { mbar_init(full_bar(s), LOADERS / 32); mbar_init(empty_bar(s), CW); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -88,7 +90,7 @@ __global__ void __launch_bounds__(64 * CW) route_score_kernel(const bf16* __rest
         // ===================================================================== loading warps
         // A thread's copies of a stage lie at fixed distances, so that a stage costs about an addition per copy.  Tokens past T,
         // experts past E and steps past d are zeros (copies of no bytes: many lanes that read one address instead take turns).
-        const int lt = tid - LOADERS;
+        const int lt = tid - 32 * CW;
         constexpr int XN = TT * (TK / 8) / LOADERS, XR = LOADERS / (TK / 8);      // 16 bytes = 8 steps of one token
         const int xt = lt / (TK / 8), xc = (lt % (TK / 8)) * 8;
         const bf16* xs = x + (size_t)(t0 + xt) * d + xc;
@@ -271,31 +273,35 @@ __global__ void __launch_bounds__(64 * CW) route_score_kernel(const bf16* __rest
     }
 }
 
-template <int RT, int RE, int LT, int CW>
+template <int RT, int RE, int LT, int CW, bool TWO>
 inline bool route_score_attr() {
-    return cudaFuncSetAttribute(route_score_kernel<RT, RE, LT, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                ScoreShape<RT, RE, LT, CW>::SMEM) == cudaSuccess;
+    return cudaFuncSetAttribute(route_score_kernel<RT, RE, LT, CW, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                ScoreShape<RT, RE, LT, CW, TWO>::SMEM) == cudaSuccess;
 }
 inline bool route_score_init() {
-    return route_score_attr<2, 1, 4, 2>() && route_score_attr<2, 1, 4, 4>() && route_score_attr<2, 4, 4, 4>() &&
-           route_score_attr<4, 4, 4, 4>() && route_score_attr<4, 8, 4, 4>();
+    return route_score_attr<2, 1, 4, 2, false>() && route_score_attr<2, 1, 4, 4, false>() && route_score_attr<2, 4, 4, 4, false>() &&
+           route_score_attr<4, 4, 4, 4, false>() && route_score_attr<4, 8, 4, 4, false>() && route_score_attr<4, 8, 4, 4, true>();
 }
-template <int RT, int RE, int LT, int CW>
+template <int RT, int RE, int LT, int CW, bool TWO>
 inline void launch_route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int32_t* status, cudaStream_t st) {
-    using Sh = ScoreShape<RT, RE, LT, CW>;
+    using Sh = ScoreShape<RT, RE, LT, CW, TWO>;
     dim3 grid(ceil_div(T, Sh::TT), ceil_div(E, Sh::TE));
-    pdl_launch(route_score_kernel<RT, RE, LT, CW>, grid, Sh::THREADS, Sh::SMEM, st, x, W_r, z, T, d, E, status);
+    pdl_launch(route_score_kernel<RT, RE, LT, CW, TWO>, grid, Sh::THREADS, Sh::SMEM, st, x, W_r, z, T, d, E, status);
 }
 // Shape choice: the least estimated cycles per step on the fullest SM, first + more * (blocks on it - 1), as measured at
 // d = 7168 (one block alone on an SM; each further one).  us, with every thread loading and multiplying by turns and now:
 // T 64, d 7168, E 256 (16 x 8) 44 and 33; T 1537, d 1000, E 20 (32 x 8) 10.8 and 8.4; T 512, d 7168, E 256 (32 x 32) 101 and 66;
-// T 4096, d 2048, E 64 (64 x 32) 39 and 31, E 61 49 and 33; T 2048, d 7168, E 96 (64 x 32) 130 and 102; T 2048, d 7168, E 256
-// (64 x 64) 202 and 185; T 16384, d 7168, E 256 1219 and 1283, E 255 1546 and 1362.  The packed multiply-adds alone, three different
-// operands each, take 2.8 cycles a warp and scheduler: 53 TFLOP/s.
+// T 4096, d 2048, E 64 (64 x 32) 39 and 31, E 61 49 and 33; T 2048, d 7168, E 96 (64 x 32) 130 and 102; d 7168, E 256 (64 x 64)
+// T 2368 208 and 191, T 16576 1225 and 1189, E 255 1552 and 1374.  The packed multiply-adds alone, three different operands each, take
+// 2.8 cycles a warp and scheduler: 53 TFLOP/s.
+// 64 x 64 as two blocks on an SM, or as one with twice the loading warps where E is odd and W_r comes in by 4 bytes: d 7168, one
+// block's worth per SM (T 2368) E 256 191 and 193 us, E 255 247 and 203; seven (T 16576) E 256 1189 and 1292, E 252 1190 and 1337,
+// E 255 1355 and 1374.
 inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d, int E, int sm_count, int32_t* status,
                         cudaStream_t st) {
+    const bool two = E % 2 == 0;
     const struct { int tt, te; float first, more; } shape[5] = {
-        {16, 8, 8.8f, 4.5f}, {32, 8, 11.f, 7.6f}, {32, 32, 16.9f, 13.2f}, {64, 32, 27.8f, 24.8f}, {64, 64, 47.6f, 48.5f}};
+        {16, 8, 8.8f, 4.5f}, {32, 8, 11.f, 7.6f}, {32, 32, 16.9f, 13.2f}, {64, 32, 27.8f, 24.8f}, {64, 64, 47.6f, two ? 43.5f : 48.5f}};
     int pick = 0;
     float best = 0.0f;
     for (int i = 0; i < 5; ++i) {
@@ -303,11 +309,12 @@ inline void route_score(const bf16* x, const float* W_r, float* z, int T, int d,
         const float cost = shape[i].first + shape[i].more * (float)((blocks + sm_count - 1) / sm_count - 1);
         if (i == 0 || cost <= best) { best = cost; pick = i; }
     }
-    if (pick == 0) launch_route_score<2, 1, 4, 2>(x, W_r, z, T, d, E, status, st);
-    else if (pick == 1) launch_route_score<2, 1, 4, 4>(x, W_r, z, T, d, E, status, st);
-    else if (pick == 2) launch_route_score<2, 4, 4, 4>(x, W_r, z, T, d, E, status, st);
-    else if (pick == 3) launch_route_score<4, 4, 4, 4>(x, W_r, z, T, d, E, status, st);
-    else launch_route_score<4, 8, 4, 4>(x, W_r, z, T, d, E, status, st);
+    if (pick == 0) launch_route_score<2, 1, 4, 2, false>(x, W_r, z, T, d, E, status, st);
+    else if (pick == 1) launch_route_score<2, 1, 4, 4, false>(x, W_r, z, T, d, E, status, st);
+    else if (pick == 2) launch_route_score<2, 4, 4, 4, false>(x, W_r, z, T, d, E, status, st);
+    else if (pick == 3) launch_route_score<4, 4, 4, 4, false>(x, W_r, z, T, d, E, status, st);
+    else if (two) launch_route_score<4, 8, 4, 4, true>(x, W_r, z, T, d, E, status, st);
+    else launch_route_score<4, 8, 4, 4, false>(x, W_r, z, T, d, E, status, st);
 }
 
 }  // namespace mop

@@ -786,7 +786,9 @@ def test_exact_scoring_shapes_give_the_contract_chains(T, d, E):
 @pytest.mark.parametrize("T,d,E", [(40, 1000, 9),                        # 16 x 8: the ring of stages around, the last one partly filled
                                    (1500, 776, 17), (4000, 8, 8),        # 32 x 8, and a single stage of 8 steps
                                    (1300, 520, 40), (1300, 456, 41),     # 32 x 32
-                                   (4100, 392, 62), (8200, 328, 65)])    # 64 x 32 and 64 x 64
+                                   (4100, 392, 62), (8200, 328, 65),     # 64 x 32
+                                   (9472, 328, 64), (9000, 456, 34),     # 64 x 64, two blocks on an SM
+                                   (12000, 456, 127)])                   # 64 x 64, one
 def test_exact_scoring_with_more_steps_than_its_ring_holds(T, d, E):
     test_exact_scoring_shapes_give_the_contract_chains(T, d, E)
 
