@@ -46,17 +46,15 @@ constexpr int TN_STAGE_BYTES = 2 * TN_SUB_BYTES;
 constexpr int TN_EPI_WARPS = 8;
 constexpr int TN_EPI_BYTES = 4096;                   // per epilogue warp
 constexpr int TN_SMEM_BYTES = TN_STAGES * TN_STAGE_BYTES + 1024 /*align*/ + TC_BAR_BYTES + TN_EPI_WARPS * TN_EPI_BYTES;
-// The SwiGLU backward has, per pair of epilogue warps, buffers of the stash's three tensors (16 tokens x 64 features) beside the gates
-// of a tile, and a stage less for two of them (TN_B2) or two stages less for three (TN_B2S: where K is short the epilogue is the
-// longer part).
+// The SwiGLU backward has two forms of its epilogue.  TN_B2 stages by warps like the others.  TN_B2S, where K is short and the epilogue
+// the longer part, has three buffers per pair of warps of the stash's three tensors (16 tokens x 64 features) beside the gates of a
+// tile, and two stages less.
 constexpr int TN_STASH_BYTES = 16 * 128;             // of one tensor
-__host__ __device__ constexpr int tn_stash_bufs(int kind) { return kind == TN_B2S ? 3 : 2; }
-__host__ __device__ constexpr int tn_stages(int kind) { return kind == TN_B2S ? 4 : kind == TN_B2 ? 5 : TN_STAGES; }
-__host__ __device__ constexpr int tn_stash_pair_bytes(int kind) { return tn_stash_bufs(kind) * 3 * TN_STASH_BYTES; }
-__host__ __device__ constexpr int tn_b2_smem(int kind) {
-    return tn_stages(kind) * TN_STAGE_BYTES + 1024 + TC_BAR_BYTES + 4 * tn_stash_pair_bytes(kind) + TN_EPI_WARPS * 1024;
-}
-static_assert(tn_b2_smem(TN_B2) <= TN_SMEM_BYTES && tn_b2_smem(TN_B2S) <= TN_SMEM_BYTES, "shared memory");
+constexpr int TN_STASH_BUFS = 3;
+constexpr int TN_STASH_PAIR_BYTES = TN_STASH_BUFS * 3 * TN_STASH_BYTES;
+__host__ __device__ constexpr int tn_stages(int kind) { return kind == TN_B2S ? 4 : TN_STAGES; }
+static_assert(tn_stages(TN_B2S) * TN_STAGE_BYTES + 1024 + TC_BAR_BYTES + 4 * TN_STASH_PAIR_BYTES + TN_EPI_WARPS * 1024 <= TN_SMEM_BYTES,
+              "shared memory");
 constexpr int TN_THREADS = 64 + 32 * TN_EPI_WARPS;
 constexpr int TN_RING = 16;                          // work items announced to the roles of a cluster
 constexpr int TN_SIGNALS = 4;                        // requests for further items
@@ -65,7 +63,7 @@ constexpr int TN_BOXES = 8;                          // token boxes of 16, 32, .
 struct TnMaps {
     CUtensorMap a0, a1;                // weights (F1: gate, up; B4: gate, up)
     CUtensorMap b[TN_BOXES];           // token rows, box of 16 (i + 1) rows
-    CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows; B2: [0..2] the stash G, U, H, [3..5] dG, dU, gH (16 rows)
+    CUtensorMap b1[TN_BOXES];          // B4: the second phase's token rows; B2S: [0..2] the stash G, U, H, [3..5] dG, dU, gH (16 rows)
 };
 
 // A tile's columns of the MMA, and the box (index into TnMaps) that holds one CTA's half of them.
@@ -196,6 +194,51 @@ __device__ __forceinline__ void tn_write_rows(bf16* __restrict__ dst, int ldo, u
     }
 }
 
+// SwiGLU backward of 16 tokens x 32 features in the accumulator's fragments: frag holds G, U, H and becomes dG, dU, gate * H; dot are
+// this lane's shares of <dHu, H> of its tokens.  gates: shared memory, of the step's first token on.
+__device__ __forceinline__ void tn_swiglu_backward(uint32_t (&frag)[3][2][4], const float (&v0)[8], const float (&v1)[8], uint32_t gates,
+                                                   int tpair, float (&dot)[2][2]) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        dot[j][0] = dot[j][1] = 0.0f;
+        const float2 gt = lds64f(gates + 4u * (8 * j + tpair));
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {          // features 8 m + lane / 4
+            float dG[2], dU[2], gH[2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {      // tokens tpair, tpair + 1
+                const float G = p ? bf16_hi(frag[0][j][m]) : bf16_lo(frag[0][j][m]);
+                const float U = p ? bf16_hi(frag[1][j][m]) : bf16_lo(frag[1][j][m]);
+                const float H = p ? bf16_hi(frag[2][j][m]) : bf16_lo(frag[2][j][m]);
+                const float gate = p ? gt.y : gt.x;
+                const float dhu = m < 2 ? v0[4 * j + 2 * m + p] : v1[4 * j + 2 * (m - 2) + p];
+                dot[j][p] = fmaf(dhu, H, dot[j][p]);
+                const float dh = gate * dhu;
+                const float sg = sigmoidf_fast(G);
+                dG[p] = dh * U * sg * (1.0f + G * (1.0f - sg));
+                dU[p] = dh * (G * sg);
+                gH[p] = gate * H;
+            }
+            frag[0][j][m] = pack_bf16x2(dG[0], dG[1]);
+            frag[1][j][m] = pack_bf16x2(dU[0], dU[1]);
+            frag[2][j][m] = pack_bf16x2(gH[0], gH[1]);
+        }
+    }
+}
+// The 32 features' dot products: the 8 lanes with the same lane % 4 hold the shares of the same tokens.
+__device__ __forceinline__ void tn_write_dots(const EpiArgs& ep, float (&dot)[2][2], int row0, int rows_left, int tpair, int fcol, int Mw,
+                                              int lane) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) dot[j][p] += __shfl_xor_sync(0xffffffffu, dot[j][p], off);
+            const int tok = 8 * j + tpair + p;
+            if (lane < 4 && tok < rows_left && fcol < Mw) ep.part[(size_t)(fcol >> 5) * ep.M_total + row0 + tok] = dot[j][p];
+        }
+}
+
 // An epilogue warp's walk over the cluster's items: items n with n % 2 == group are drained, the others passed over.
 // next(n): item n is there; false: none is left, or the wait for it gave up.  wait(n): its accumulator is ready, or the wait gave up.
 // PAIRED: drain(n) meets a partner warp at barriers.  Two warps may see the CTA give up at different items, or one of them while
@@ -223,11 +266,11 @@ template <int KIND, bool ONCE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TN_THREADS, 1)
 tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
     constexpr int S = tn_stages(KIND), STAGE_BYTES = TN_STAGE_BYTES;
-    constexpr int BUFS = tn_stash_bufs(KIND), PAIR_BYTES = tn_stash_pair_bytes(KIND);
+    constexpr int BUFS = TN_STASH_BUFS;
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * STAGE_BYTES);
-    constexpr int STASH_BARS = tn_is_b2(KIND) ? 4 * BUFS : 0;
+    constexpr int STASH_BARS = KIND == TN_B2S ? 4 * BUFS : 0;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4 + TN_RING + TN_SIGNALS + STASH_BARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -259,7 +302,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&maps.a0);
         if (KIND != TN_F2 && !tn_is_b2(KIND)) tma_prefetch_desc(&maps.a1);
-        if (tn_is_b2(KIND))
+        if (KIND == TN_B2S)
             for (int i = 0; i < 6; ++i) tma_prefetch_desc(&maps.b1[i]);
     }
     if (warp == 1) tmem2_alloc(smem_u32(tmem_slot), 512);
@@ -457,16 +500,16 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         const uint32_t wb = epi_base + (uint32_t)(warp - 2) * TN_EPI_BYTES;   // this warp's staging
         const uint32_t fo = frag_off(lane);
         const int tpair = 2 * (lane & 3);             // this thread's tokens within a run of 8: tpair, tpair + 1
-        // F1: a gate warp and its up warp; B2: two warps that share 128-byte lines of the stash
-        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G || tn_is_b2(KIND);
-        const int pair_bar = 1 + 2 * group + (tn_is_b2(KIND) ? quarter >> 1 : quarter & 1);
+        // F1: a gate warp and its up warp; B2S: two warps that share 128-byte lines of the stash
+        constexpr bool PAIRED = KIND == TN_F1 || KIND == TN_F1G || KIND == TN_B2S;
+        const int pair_bar = 1 + 2 * group + (KIND == TN_B2S ? quarter >> 1 : quarter & 1);
         const int buf = group;
-        const uint32_t gbuf = tn_is_b2(KIND) ? epi_base + 4 * PAIR_BYTES + (uint32_t)(warp - 2) * 1024 : wb + 3072;
+        const uint32_t gbuf = KIND == TN_B2S ? epi_base + 4 * TN_STASH_PAIR_BYTES + (uint32_t)(warp - 2) * 1024 : wb + 3072;
         Tile ti = {0, 0, 0, 0};
-        // B2: the pair's buffers, its steps so far (16 tokens each; the buffers and their barriers' phases alternate) and the warp
+        // B2S: the pair's buffers, its steps so far (16 tokens each; the buffers and their barriers' phases alternate) and the warp
         // that copies for both
         const int stash_pair = (warp - 2) >> 1;
-        const uint32_t stash = epi_base + (uint32_t)stash_pair * PAIR_BYTES;
+        const uint32_t stash = epi_base + (uint32_t)stash_pair * TN_STASH_PAIR_BYTES;
         const bool el = elect_one();
         const bool copies = (quarter & 1) == 0 && el;
         int steps = 0;
@@ -483,7 +526,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
         // (the lanes give up together: a lane that left alone would be missed at the shuffles below)
         auto next = [&](int n) { return !gone && __all_sync(0xffffffffu, next_item(n, ti)) != 0; };
         auto wait = [&](int n) {
-            if constexpr (tn_is_b2(KIND)) {       // the stash of the tile's first steps as well
+            if constexpr (KIND == TN_B2S) {       // the stash of the tile's first steps as well
                 if (copies) {
                     tma_store_wait_read<0>();
 #pragma unroll
@@ -575,12 +618,62 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                     tn_write_rows<2>(args.ep.out0, args.ep.ldo, sb, row0 + c + t_own, rows_left - t_own, fcol, args.Mw, lane);
                     bar_pair_sync(pair_bar);     // the partner has read this warp's half
                 }
-            } else if constexpr (tn_is_b2(KIND)) {
-                // 16 tokens at a time.  The stash (G, U, H) and the results (dG, dU, gH) travel as boxes of 64 features, whole 128-byte
-                // lines, between global and shared memory, in the buffers' place; a warp works on its 32 of them in the layout of the
-                // accumulator's fragments (ldmatrix.trans, stmatrix.trans).  With 16-byte loads and stores of half lines, one step
-                // ahead, they were more than half of a tile's time (30 thousand cycles for 192 tokens, 12 without them; d = 2048,
-                // f = 1408, 64 experts of 384 rows 205 us, now 194).
+            } else if constexpr (KIND == TN_B2) {
+                // 16 tokens at a time: the stash (G, U, H) comes in as 16-byte pieces of token rows one step ahead, is staged and
+                // read back as fragments (ldmatrix.trans) that match the accumulator's; the results leave the same way.
+                const int fcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first f column of this warp
+                const int col = fcol + (lane & 3) * 8;
+                const bf16* const src[3] = {args.ep.in0, args.ep.in1, args.ep.in2};
+                bf16* const dst[3] = {args.ep.out0, args.ep.out1, args.ep.out2};
+                uint4 pre[3][2];
+                auto fetch = [&](int c) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int tok = c + 8 * i + (lane >> 2);
+                        const bool okk = tok < rows && col < args.Mw;
+                        const size_t o = (size_t)(row0 + tok) * args.ep.ldo + col;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+                            pre[a][i] = okk ? *reinterpret_cast<const uint4*>(src[a] + o) : make_uint4(0, 0, 0, 0);
+                    }
+                };
+                fetch(0);
+#pragma unroll 1
+                for (int c = 0; c < nmma; c += 16) {
+                    float v0[8], v1[8];
+                    tmem_frag2(taddr + c, v0);
+                    tmem_frag2(taddr + (16u << 16) + c, v1);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) sts128(wb + 1024 * a + 512 * i + piece_off(lane), pre[a][i]);
+                    __syncwarp();
+                    if (c + 16 < nmma) fetch(c + 16);
+                    uint32_t frag[3][2][4];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) ldmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j]);
+                    tmem_frag_wait(v0, v1);
+                    float dot[2][2];
+                    tn_swiglu_backward(frag, v0, v1, gbuf + 4u * c, tpair, dot);
+                    __syncwarp();                              // every lane has its fragments of the stash
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            stmatrix4_trans(wb + 1024 * a + 512 * j + fo, frag[a][j][0], frag[a][j][1], frag[a][j][2], frag[a][j][3]);
+                    __syncwarp();
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        tn_write_rows<2>(dst[a], args.ep.ldo, wb + 1024 * a, row0 + c, rows - c, fcol, args.Mw, lane);
+                    tn_write_dots(args.ep, dot, row0 + c, rows - c, tpair, fcol, args.Mw, lane);
+                    __syncwarp();
+                }
+            } else if constexpr (KIND == TN_B2S) {
+                // The same with the stash and the results travelling as boxes of 64 features, whole 128-byte lines, between global and
+                // shared memory, in the buffers' place; a warp works on its 32 of them.  Where K is short, 16-byte loads and stores of
+                // half lines, one step ahead, are more than half of a tile's time.
                 const int fcol = ti.mt * 256 + 128 * (int)rank + 32 * quarter;      // first f column of this warp
                 const int sub = 4 * (quarter & 1);                                  // its first 16-byte piece of a line
                 const uint32_t fo2 = (uint32_t)((lane & 7) * 128 + (((sub + (lane >> 3)) ^ (lane & 7)) << 4));
@@ -604,32 +697,8 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                         fetch_stash(steps + BUFS - 1, row0 + c + 16 * (BUFS - 1));
                     }
                     tmem_frag_wait(v0, v1);
-                    float dot[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const float2 gt = lds64f(gbuf + 4u * (c + 8 * j + tpair));
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {          // features 8 m + lane / 4
-                            float dG[2], dU[2], gH[2];
-#pragma unroll
-                            for (int p = 0; p < 2; ++p) {      // tokens tpair, tpair + 1
-                                const float G = p ? bf16_hi(frag[0][j][m]) : bf16_lo(frag[0][j][m]);
-                                const float U = p ? bf16_hi(frag[1][j][m]) : bf16_lo(frag[1][j][m]);
-                                const float H = p ? bf16_hi(frag[2][j][m]) : bf16_lo(frag[2][j][m]);
-                                const float gate = p ? gt.y : gt.x;
-                                const float dhu = m < 2 ? v0[4 * j + 2 * m + p] : v1[4 * j + 2 * (m - 2) + p];
-                                dot[j][p] = fmaf(dhu, H, dot[j][p]);
-                                const float dh = gate * dhu;
-                                const float sg = sigmoidf_fast(G);
-                                dG[p] = dh * U * sg * (1.0f + G * (1.0f - sg));
-                                dU[p] = dh * (G * sg);
-                                gH[p] = gate * H;
-                            }
-                            frag[0][j][m] = pack_bf16x2(dG[0], dG[1]);
-                            frag[1][j][m] = pack_bf16x2(dU[0], dU[1]);
-                            frag[2][j][m] = pack_bf16x2(gH[0], gH[1]);
-                        }
-                    }
+                    float dot[2][2];
+                    tn_swiglu_backward(frag, v0, v1, gbuf + 4u * c, tpair, dot);
                     __syncwarp();                              // every lane has its fragments of the stash
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
@@ -659,17 +728,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
                             if (f0 < args.Mw) tma_store_2d(&maps.b1[3 + a], st + a * TN_STASH_BYTES, f0, row0 + c);
                         tma_store_commit();
                     }
-                    // the 32 features' dot products: the 8 lanes with the same lane % 4 hold the shares of the same tokens
-#pragma unroll
-                    for (int j = 0; j < 2; ++j)
-#pragma unroll
-                        for (int p = 0; p < 2; ++p) {
-#pragma unroll
-                            for (int off = 4; off < 32; off <<= 1) dot[j][p] += __shfl_xor_sync(0xffffffffu, dot[j][p], off);
-                            const int tok = c + 8 * j + tpair + p;
-                            if (lane < 4 && tok < rows && fcol < args.Mw)
-                                args.ep.part[(size_t)(fcol >> 5) * args.ep.M_total + row0 + tok] = dot[j][p];
-                        }
+                    tn_write_dots(args.ep, dot, row0 + c, rows - c, tpair, fcol, args.Mw, lane);
                     if (!ok) { gone = true; break; }
                 }
             } else {
@@ -699,7 +758,7 @@ tn_gemm_kernel(const __grid_constant__ TnMaps maps, const TnArgs args) {
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_bar(buf) & T2_PEER_MASK);
         });
-        if (tn_is_b2(KIND) && copies) tma_store_wait_all();
+        if (KIND == TN_B2S && copies) tma_store_wait_all();
     }
 
     tc_fence_before();
@@ -846,19 +905,21 @@ inline mop_status tn_dgrad_down(TcPlan* p, const TcBwdArgs& a, int32_t* tiles, i
     const uint64_t M = tc_rows(p);
     TnMaps m;
     if (!tc_map_3d(p, &m.a0, a.W_down, s.E, s.f, s.d, 128) || !tn_token_maps(p, m.b, a.dYp, M, s.d)) return MOP_ERR_CUDA;
+    TnArgs g = tn_base_args(p, tiles, TN_B2, status);
+    g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
+    g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH; g.ep.in0 = a.G_save; g.ep.in1 = a.U_save; g.ep.in2 = a.H;
+    g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
+    g.gemm_follows = true;
+    // Boxes where the epilogue (by the rows of a tile) is long beside the main loop (by d).  us, by warps and by boxes: d 512, f 1024,
+    // 64 experts of 28 rows 29.3 and 29.0, 64 rows 39.0 and 37.1, 256 rows 86 and 72; d 1000, f 1416, 28 rows 55.5 and 56.4, 64 rows 67.8
+    // and 65.9, 256 rows 152 and 119; d 2048, f 1408, 64 rows 91 and 97, 128 rows 106.9 and 109.8, 160 rows 117.1 and 117.5, 200 rows 133
+    // and 129, 256 rows 160 and 150.  Longer K, with two buffers and a stage more: d 4096, f 1024, 200 rows 152 and 158; d 7168,
+    // f 2048, 32 experts of 96 rows 189 and 197, 600 rows 476 and 493.
+    if (s.d > 2048 || (uint64_t)s.T * s.k * 16 <= (uint64_t)s.d * s.E) return tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
     const void* const boxes[6] = {a.G_save, a.U_save, a.H, a.dG, a.dU, a.gH};
     for (int i = 0; i < 6; ++i)
         if (!tc_map_2d(p, &m.b1[i], boxes[i], M, s.f, 16)) return MOP_ERR_CUDA;
-    // Three stash buffers where K is short and the rows are more than a box or two: d 512, f 1024, 1024 rows per expert 94 us, two buffers
-    // 118; d 1024, f 2048, 2048 rows 212 and 239; d 2048, f 1408, 384 rows 194 and 198; d 2048, f 768, 28 rows 82 and 78.
-    const bool brief = s.d <= 2048 && (uint64_t)s.T * s.k >= 64ull * s.E;
-    TnArgs g = tn_base_args(p, tiles, TN_B2, status);
-    g.tiles_m = ceil_div(s.f, 256); g.kblocks = ceil_div(s.d, TN_BK); g.Mw = s.f;
-    g.ep.out0 = a.dG; g.ep.out1 = a.dU; g.ep.out2 = a.gH;
-    g.ep.gate = a.gate; g.ep.row_src = a.row_src; g.ep.part = a.part; g.ep.ldo = s.f; g.ep.M_total = (int)M;
-    g.gemm_follows = true;
-    return brief ? tn_launch<TN_B2S>(p, "gemm_dgrad_down_dswiglu", m, g, st)
-                 : tn_launch<TN_B2>(p, "gemm_dgrad_down_dswiglu", m, g, st);
+    return tn_launch<TN_B2S>(p, "gemm_dgrad_down_dswiglu", m, g, st);
 }
 
 }  // namespace mop

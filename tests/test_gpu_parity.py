@@ -311,12 +311,15 @@ def test_an_overflowing_expert_does_not_reach_its_neighbours_gradients():
         assert torch.equal(clean.dX[~mine], bad.dX[~mine]) and torch.equal(clean.dgate[~mine], bad.dgate[~mine])
 
 
-@pytest.mark.parametrize("T,d,E,k,f", [(50, 2048, 2, 1, 72),       # 25 rows: two steps, the second partly filled; f ends inside a box
+@pytest.mark.parametrize("T,d,E,k,f", [(50, 384, 2, 1, 72),       # boxes.  25 rows: two steps, the second partly filled; f ends inside a box
                                        (700, 256, 3, 2, 320),     # two tiles per expert, steps beyond every buffer
-                                       (130, 2056, 2, 2, 136),    # longer K: two buffers
-                                       (40, 512, 8, 2, 200)],     # fewer rows than a tile's smallest box asks for
+                                       (40, 128, 8, 2, 200),      # fewer rows than a tile's smallest box asks for
+                                       (130, 2048, 1, 1, 136),    # one more row per expert than the line asks for at the longest K
+                                       (128, 2048, 1, 1, 136),    # by warps: on the line
+                                       (50, 2048, 2, 1, 72), (40, 512, 8, 2, 200),
+                                       (600, 2056, 2, 2, 136)],   # longer K, three tiles per expert
                          ids=lambda v: str(v))
-def test_swiglu_backward_with_two_and_three_stash_buffers(T, d, E, k, f):
+def test_swiglu_backward_by_warps_and_by_boxes(T, d, E, k, f):
     check_layer(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=f, backward=True, seed=T), binding.GEMM_AUTO)
 
 
