@@ -62,8 +62,8 @@ __device__ __forceinline__ void pdl_begin_gemm(bool gemm_follows, const PdlNote&
 //    takes the grid's wait.
 //  - What A reads may only be overwritten, and what A writes only be read, by kernels after this one: it waits for A before it
 //    leaves (pdl_end_beside), so that its end is the end of both.
-__device__ __forceinline__ void pdl_begin_beside(const PdlNote& note) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+__device__ __forceinline__ void pdl_begin_beside(bool gemm_follows, const PdlNote& note) {
+    if (gemm_follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int32_t v = note.value;
     if (threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(note.word) : "memory");
     if (!__syncthreads_and(v == note.value)) asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -207,7 +207,7 @@ tc_gemm2_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     // dX runs beside the weight gradient of its block: both read the logit gradients, neither what the other writes.
-    if constexpr (KIND == TC_VX) pdl_begin_beside(args.note);
+    if constexpr (KIND == TC_VX) pdl_begin_beside(args.gemm_follows, args.note);
     else pdl_begin_gemm(args.gemm_follows, args.note);
 
     const int row_tiles = KIND == TC_VW ? args.tiles_m_fixed : *args.n_mtiles;

@@ -1661,6 +1661,7 @@ mop_status mop_vocab_loss_bwd(int device, int32_t N, int32_t H, int32_t V, const
             // makes 896 tiles of either, 12.1 for each of 74 pairs of CTAs, and 25 rounds of both together instead of 26.
             TcArgs g = base;
             g.note = note;
+            g.gemm_follows = c0 + L.vc < V;      // after the last block comes the conversion, whose small blocks must not pile up
             g.tiles_n = ceil_div(H, 256); g.kblocks = ceil_div(cw, TC_BK); g.N = H; g.kb_base = c0;
             g.ep.outf = dx32; g.ep.accumulate = c0 > 0 ? 1 : 0;
             if ((r = tc2_launch<TC_VX>(p, "vocab_dgrad", mdYk, mdYk, mWk, mWk, g, st)) != MOP_OK) return r;

@@ -142,6 +142,9 @@ def test_kernels_launched_beside_their_predecessor_wait_or_acquire_what_they_rea
     assert order(function("pdl_begin_gemm"), "griddepcontrol.wait", "st.release.gpu", "__syncthreads()", "griddepcontrol.launch_dependents")
     assert order(function("pdl_begin_beside"), "ld.acquire.gpu", "__syncthreads_and", "griddepcontrol.wait", "fence.proxy.async.global")
     assert "griddepcontrol.wait" in function("pdl_end_beside")
+    # a GEMM lets only a GEMM start early: smaller blocks would pile up on the SMs that empty first
+    for name in ("pdl_begin_gemm", "pdl_begin_beside"):
+        assert function(name).count("griddepcontrol.launch_dependents") == function(name).count('if (gemm_follows) asm volatile("griddepcontrol.launch_dependents') == 1
     for name, text in texts.items():
         assert text.count("pdl_begin_beside(") == text.count("pdl_end_beside("), name
 
