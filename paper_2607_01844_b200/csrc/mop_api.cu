@@ -28,7 +28,7 @@ struct mop_ctx {
     char* ws;
     size_t ws_bytes;
     float* z;            // [T,E] logits
-    int32_t* partial;    // [units,E] histogram partials -> unit bases
+    int32_t* partial;    // [units,E] histogram partials -> unit bases (where the permutation takes three kernels)
     int32_t* tiles;      // tile tables of the grouped GEMMs
     int32_t* status;     // device status word
     float* part;         // [ntile_max, M] partial dot products for dgate
@@ -123,7 +123,7 @@ Layout make_layout(const mop_moe_shape& s) {
     auto take = [&](size_t bytes) { size_t r = o; o += align_up(bytes); band(); return r; };
     const size_t T = s.T, d = s.d, E = s.E, k = s.k, f = s.f, M = T * k;
     L.z = take(T * E * 4);
-    L.partial = take((size_t)perm_units(s) * E * 4 + 4);
+    if (!perm_cluster_fits(M)) L.partial = take((size_t)perm_units(s) * E * 4 + 4);
     L.tiles = take(tc_tables_bytes(s.T * s.k, s.E));
     L.status = take(256);
     if (route_fast(s)) {
@@ -313,7 +313,7 @@ mop_status mop_create(mop_ctx** out, const mop_moe_shape* shape, int device) {
     if (cudaMalloc(&c->ws, L.total) != cudaSuccess) { cudaGetLastError(); delete c; return MOP_ERR_WORKSPACE; }
     char* w = c->ws;
     c->z = reinterpret_cast<float*>(w + L.z);
-    c->partial = reinterpret_cast<int32_t*>(w + L.partial);
+    c->partial = perm_cluster_fits((long long)shape->T * shape->k) ? nullptr : reinterpret_cast<int32_t*>(w + L.partial);
     c->tiles = reinterpret_cast<int32_t*>(w + L.tiles);
     c->status = reinterpret_cast<int32_t*>(w + L.status);
     c->fast_route = false;

@@ -63,6 +63,13 @@ def test_only_layers_that_score_on_the_tensor_cores_hold_its_buffers(lib, T, d, 
     assert exact < forced and auto == (forced if tensor else exact)
 
 
+def test_only_layers_whose_permutation_takes_three_kernels_hold_its_partial_counts(lib):
+    """One token more: 8 KiB of logits and rows, and from the line on a count per expert and 512 assignments as well."""
+    from paper_2607_01844_b200.binding import MopShape
+    at = {T: lib.mop_workspace_bytes(ctypes.byref(MopShape(T, 8, 1024, 1, 8, 0, 0, 0, 0, 0, 0))) for T in (98303, 98304, 98305)}
+    assert 0 <= at[98304] - at[98303] < 16384 and at[98305] - at[98304] > 193 * 1024 * 4
+
+
 def test_the_current_stream_without_torchs_private_accessor(monkeypatch):
     import types
 
