@@ -323,12 +323,14 @@ def test_swiglu_backward_by_warps_and_by_boxes(T, d, E, k, f):
     check_layer(synth.small("c3_trillion", T=T, d=d, E=E, k=k, f=f, backward=True, seed=T), binding.GEMM_AUTO)
 
 
-@pytest.mark.parametrize("T,k,E", [(2048, 2, 24), (2049, 2, 24), (4096, 1, 1024), (1025, 4, 7), (4609, 1, 3)])
-def test_permutation_tables_on_both_sides_of_the_single_block_limit(T, k, E):
-    """Up to 8 units of 512 assignments the permutation runs in one block, beyond that in three kernels: the tables
-    must be the oracle's on both sides of that limit (and where the single block would not have the memory)."""
+@pytest.mark.parametrize("T,k,E", [(2048, 2, 24), (2049, 2, 24), (4096, 1, 1024), (1025, 4, 7), (4609, 1, 3),
+                                   (49152, 2, 257), (98304, 1, 1024), (24576, 4, 5),          # one launch: its longest runs
+                                   (49153, 2, 257), (98305, 1, 1024), (33000, 3, 3)])         # three kernels
+def test_permutation_tables_and_rows_on_both_sides_of_the_single_launch_limit(T, k, E):
+    """Up to 98304 assignments the permutation is one cluster launch, beyond that three kernels: tables and copied rows must be the
+    oracle's on both sides of that limit, with few experts and with many."""
     gen = torch.Generator().manual_seed(T + E)
-    idx = torch.stack([torch.randperm(E, generator=gen)[:k] for _ in range(T)]).to(torch.int32)
+    idx = torch.rand((T, E), generator=gen).topk(k, 1).indices.to(torch.int32)
     counts, offsets, perm_row, row_src = oracle.permute(idx.numpy(), E)
     ctx = binding.Context(T, 64, E, k, 64)
     dev = {n: torch.empty(s, dtype=torch.int32, device="cuda") for n, s in
@@ -363,6 +365,12 @@ def test_permutation_in_one_launch_with_indices_out_of_range(T, k, E):
     assert np.array_equal(got["counts"], counts) and np.array_equal(got["offsets"], np.concatenate(([0], np.cumsum(counts))))
     assert np.array_equal(got["perm_row"], perm_row) and np.array_equal(got["row_src"][:order.size], order)
     assert (got["row_src"][order.size:] == -7).all()
+
+
+@pytest.mark.parametrize("T,d,E,k", [(24576, 64, 40, 4), (24577, 64, 40, 4), (98400, 64, 7, 1)])
+def test_forward_on_both_sides_of_the_single_launch_permutation(T, d, E, k):
+    """The token tiles come from the permutation or from a block beside the row copy: the same bits as the separate calls'."""
+    test_small_forward_in_one_call_equals_the_separate_calls(T, d, E, k, 0, 0)
 
 
 @pytest.mark.parametrize("T,d,E,k,score,bias", [(1, 64, 256, 32, 1, 1), (7, 64, 3, 3, 0, 0), (9, 1032, 65, 4, 1, 2),     # one block, eight
