@@ -22,6 +22,7 @@
 //          lies in memory, rows of d on M), two K phases into one accumulator, dXp token-major.
 //   TN_B2  dHu^T = W_down[e] dYp^T (weights K-major, rows of f on M); the epilogue runs the SwiGLU
 //          backward in the accumulator's layout: dG, dU, gate*H out, and one dgate partial per 32 columns of f.
+//   TN_B2S the same where K is short: the epilogue's six tensors travel by TMA, with two pipeline stages less.
 //
 // Epilogues: the accumulator is read with tcgen05.ld.16x256b, whose layout is that of an mma fragment (a thread holds two
 // neighbouring tokens of a feature), packed to bf16 pairs and turned token-major by stmatrix.trans: a block of 32 features x 32

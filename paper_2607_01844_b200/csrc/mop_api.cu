@@ -105,10 +105,12 @@ __global__ void guard_check_kernel(const char* ws, GuardList g, unsigned long lo
 
 int perm_units(const mop_moe_shape& s) { return ceil_div(s.T * s.k, PERM_SEG); }
 // The tensor-core scoring path needs 64-wide K blocks of x and 64-wide column chunks of W_r.  AUTO takes it once the scoring is
-// large: small layers keep the fp32 chains, and their contexts hold none of its buffers.  The line is a safe one and not where the
-// two paths cross: router, us, exact and tensor, at T 4096, d 2048, E 64 (1.1 GFLOP) 52 and 57, T 512, d 7168, E 256 (1.9) 116 and
-// 129, T 4096, d 7168, E 64 (3.8) 144 and 113, T 16384, d 2048, E 64 (4.3) 136 and 82, T 2048, d 7168, E 256 (7.5) 220 and 135,
-// T 8192, d 7168, E 128 (15) 394 and 147, T 16384, d 7168, E 256 (60) 1271 and 221; the crossing is near 3 GFLOP.
+// large: small layers keep the fp32 chains, and their contexts hold none of its buffers (8 T E bytes and more).  Router, us, exact and
+// tensor, normal inputs, sigmoid with a bias, k 8: T 4096, d 2048, E 64 (1.1 GFLOP) 34 and 42, T 512, d 7168, E 256 (1.9) 69 and 109,
+// T 8192, d 2048, E 64 (2.1) 61 and 55, T 4096, d 7168, E 64 (3.8) 106 and 120, T 16384, d 2048, E 64 (4.3) 111 and 76, T 2048,
+// d 7168, E 256 (7.5) 189 and 114, T 8192, d 7168, E 128 (15) 357 and 131, T 16384, d 7168, E 256 (60) 1206 and 201.  They cross
+// between 2 and 4 GFLOP on such inputs; the line lies above that because the tensor path pays for inputs whose order is in doubt
+// (up to 0.28 ms more at 60 GFLOP where every token is), which the exact path does not.
 bool route_fast(const mop_moe_shape& s) {
     if (s.route_path == MOP_ROUTE_EXACT || s.T <= 0 || s.d % 64 || s.E % 64 || !tc_shape_supported(s.d, s.f)) return false;
     return s.route_path == MOP_ROUTE_TENSOR || 2.0 * s.T * s.d * s.E >= 2e10;

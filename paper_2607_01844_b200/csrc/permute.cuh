@@ -1,6 +1,6 @@
 // Count / prefix-sum permutation of token-expert assignments into expert-contiguous rows, and the
-// row movers (scatter x -> Xp, k-row combine Yp -> Y).  No atomics anywhere: the order inside an
-// expert is the assignment id, fixed by a two-level (warp segment, expert) prefix sum.
+// row movers (scatter x -> Xp, k-row combine Yp -> Y).  The order inside an expert is the assignment id: only counts, whose
+// order does not matter, are ever made with atomics (of integers, in shared memory).
 #pragma once
 #include "tiles.cuh"
 
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(PERM_WARPS * 32) perm_rank_kernel(const int32_
 // its CTA, the CTAs read each other's totals through distributed shared memory, every CTA scans the experts for itself, and the
 // warps walk their runs again in order.  Same tables as the three kernels above.  tile_table: the token tiles of the GEMMs too.
 // Bounded by latency, and by the scattered row_src entries (a store of 32 of them takes 32 cycles of an SM, and there are eight SMs)
-// where there are many: us a call in a graph, three kernels (one block with a single cluster's work below 4097 assignments) and this
+// where there are many: us a call in a graph, three kernels (up to 4096 assignments one block doing their work) and this
 // one: M 32, E 8 4.4 and 2.4; 512, 256 11.0 and 3.6; 4096, 64 11.4 and 4.8; 4611, 20 13.0 and 4.6; 24576, 64 15.7 and 6.9; 16384,
 // 1024 20.8 and 10.0; 131072, 256 21.9 and 24.0; 262144, 64 25.4 and 37.5.  Hence the line, PC_MAX_M.
 constexpr int PC_WARPS = 32;

@@ -9,8 +9,8 @@ namespace mop {
 // experts are distinct, so that its k lanes count and rank side by side), the permutation goes on as in perm_cluster_kernel, and
 // the CTA copies the rows of its tokens.  Same tables and gates as the separate kernels.
 // What it saves is two launches; what it costs is that eight SMs copy slower than all.  A whole forward, us, separate and in one:
-// T 16, d 2048, E 64, k 6 160 and 156; T 256, d 256, E 8, k 2 26.1 and 25.4; 1 MiB of rows 52.1 and 49.8 (T 64, d 1024, k 8), 38.0
-// and 37.8 (T 256, d 512, k 4); 4 MiB 57.7 and 62.3 (T 256, d 1024, k 8); four tokens a warp 53 and 55 (T 1000, d 512, k 4).
+// T 16, d 2048, E 64, k 6 152 and 149; T 256, d 256, E 8, k 2 22.6 and 21.0; 1 MiB of rows 33.6 and 31.4 (T 64, d 1024, k 8), 26.7
+// and 26.2 (T 256, d 512, k 4), 31.6 and 31.7 (T 256, d 1024, k 2); 4 MiB 36.0 and 40.6 (T 256, d 1024, k 8; all f 64 but the first two).
 constexpr int RP_MAX_T = PC_MAX_CTAS * PC_WARPS;
 constexpr int RP_MAX_E = 256;
 constexpr long long RP_MAX_BYTES = 1 << 20;        // of the copied rows
